@@ -162,7 +162,11 @@ typedef struct {
  *   state are those of TVBX_SERIES_KEEP, bit for bit. */
 #define TVBX_SERIES_KEEP 0
 #define TVBX_SERIES_STREAM 1
-#define TVBX_KERNEL_AUTO     0 /* fastest kernel that fits the sweep */
+#define TVBX_KERNEL_AUTO     0 /* fastest kernel that fits the sweep: without zero delays,
+                                  several steps per launch with no thread waiting for
+                                  another (tvbx_last_kernel then gives
+                                  TVBX_KERNEL_DIRECT: its state is in registers and its
+                                  coupling read straight from the ring) */
 #define TVBX_KERNEL_DIRECT 100 /* register tiles for connectomes too large for the
                                   prefetch buffer (up to 768 regions): 4 sets of
                                   one region per thread, 16-byte ring gathers;

@@ -28,7 +28,7 @@ NVCC_FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "--expt-r
 # the compiler, so that one set per thread and two sets in a packed register
 # pair round every operation identically (the code writes each intended
 # fused multiply-add explicitly).
-FILE_FLAGS = {"sim.cu": ["-fmad=false"], "sim_fast.cu": ["-fmad=false"]}
+FILE_FLAGS = {"sim.cu": ["-fmad=false"], "sim_fast.cu": ["-fmad=false"], "sim_window.cu": ["-fmad=false"]}
 
 
 def nvcc() -> str:

@@ -207,7 +207,9 @@ struct Group {
     double speed;
     std::vector<int64_t> sets;      // external indices
     int32_t H = 0;
+    int32_t d_min = INT32_MAX;      // shortest delay of a nonzero weight
     std::vector<int32_t> row_ptr;
+    std::vector<int32_t> row_near;  // first entry of each row with a delay below WIN_FAR
     std::vector<int32_t> row_mid;   // first zero-delay entry of each row
     std::vector<uint32_t> col_dly;
     std::vector<float> w;
@@ -243,11 +245,15 @@ struct tvbx_sweep {
     uint64_t gen = 0;               // incremented by every run preparation
     int64_t steps_done = 0;         // steps integrated since the initial state
     bool resumable = false;         // state, ring and OU state hold step steps_done
-    int64_t ring_floats = 0;        // size of the ring allocation in use
+    int64_t ring_floats = 0;        // ring size in the [H][N][stride] layout (that of checkpoints)
+    WindowPlan win;                 // of the last run (steps 0: another kernel)
+    std::vector<GroupDev> ring_groups;   // groups of the last run (device pointers, ring geometry)
+    std::vector<int32_t> ring_H0;   // their ring depths in the checkpoint layout
 
     DevBuf d_prm, d_ext, d_state, d_status, d_ring, d_series, d_ou_table, d_ou_state;
     DevBuf d_csr_row, d_csr_cd, d_csr_w, d_groups, d_tiles;
     DevBuf d_blocks, d_fc, d_chi, d_meanfc, d_vec, d_fcd, d_tmp, d_perm, d_inv, d_mean_e, d_mean_i, d_error;
+    DevBuf d_far;                   // windowed kernels: far sums
     DevBuf d_fcacc, d_shift;        // streamed series: FC moments over the run, fixed shift [N][P]
     DevBuf d_series_i;              // I series (layout sl) when the run keeps it
     SeriesLayout sl{4, 0, 0};      // layout of d_series and d_series_i: set-blocked
@@ -257,7 +263,7 @@ struct tvbx_sweep {
         DevBuf* all[] = {&d_prm, &d_ext, &d_state, &d_status, &d_ring, &d_series, &d_ou_table,
                          &d_ou_state, &d_csr_row, &d_csr_cd, &d_csr_w, &d_groups, &d_tiles,
                          &d_blocks, &d_fc, &d_chi, &d_meanfc, &d_vec, &d_fcd, &d_tmp, &d_perm,
-                         &d_inv, &d_mean_e, &d_mean_i, &d_error, &d_fcacc, &d_shift, &d_series_i};
+                         &d_inv, &d_mean_e, &d_mean_i, &d_error, &d_fcacc, &d_shift, &d_series_i, &d_far};
         for (DevBuf* b : all) b->release();
         for (cudaEvent_t e : ev) cudaEventDestroy(e);
     }
@@ -409,8 +415,23 @@ tvbx_status build_groups(tvbx_sweep* h, double dt, std::vector<Group>& groups)
         groups[it->second].sets.push_back(p);
     }
     const int N = h->N;
+    // delay in steps: rint (ties to even) of length / (speed dt), in FP64
+    int32_t d_min = INT32_MAX;
+    for (Group& g : groups) {
+        for (size_t i = 0; i < h->W.size(); ++i) {
+            if (h->W[i] == 0.0) continue;
+            const double steps = rint(h->L[i] / (g.speed * dt));
+            if (steps > 65533.0) return fail(TVBX_E_UNSUPPORTED, "delay of %g steps exceeds 65533", steps);
+            g.d_min = std::min(g.d_min, steps < 0 ? 0 : (int32_t)steps);
+        }
+        d_min = std::min(d_min, g.d_min);
+    }
+    // short delays somewhere in the sweep: the far entries of each row go first,
+    // in every kernel, so that all of them sum in one order
+    const int64_t far = d_min >= 1 && d_min < WIN_NEAR_BELOW ? WIN_FAR : 0;
     for (Group& g : groups) {
         g.row_ptr.assign(N + 1, 0);
+        g.row_near.assign(N, 0);
         g.row_mid.assign(N, 0);
         int64_t dmax = 1;   // ring of at least 3 slots (the padding entries use d = 1)
         for (int k = 0; k < N; ++k) {
@@ -420,19 +441,20 @@ tvbx_status build_groups(tvbx_sweep* h, double dt, std::vector<Group>& groups)
                 g.w.push_back(0.0f);
             }
             g.row_ptr[k] = (int32_t)g.col_dly.size();
-            std::vector<std::pair<uint32_t, float>> zero;   // zero-delay entries go last
+            std::vector<std::pair<uint32_t, float>> near, zero;   // zero-delay entries go last
             for (int j = 0; j < N; ++j) {
                 const double w = h->W[(size_t)k * N + j];
                 if (w == 0.0) continue;
-                // delay in steps: rint (ties to even) of length / (speed dt), in FP64
                 const double steps = rint(h->L[(size_t)k * N + j] / (g.speed * dt));
-                if (steps > 65533.0) return fail(TVBX_E_UNSUPPORTED, "delay of %g steps exceeds 65533", steps);
                 const int64_t d = steps < 0 ? 0 : (int64_t)steps;
                 dmax = std::max(dmax, d);
                 const uint32_t cd = ((uint32_t)d << 16) | (uint32_t)j;
                 if (d == 0) zero.emplace_back(cd, (float)w);
+                else if (d < far) near.emplace_back(cd, (float)w);
                 else { g.col_dly.push_back(cd); g.w.push_back((float)w); }
             }
+            g.row_near[k] = (int32_t)g.col_dly.size();
+            for (auto& z : near) { g.col_dly.push_back(z.first); g.w.push_back(z.second); }
             g.row_mid[k] = (int32_t)g.col_dly.size();
             for (auto& z : zero) { g.col_dly.push_back(z.first); g.w.push_back(z.second); }
         }
@@ -533,6 +555,7 @@ tvbx_status tvbx_sweep_info(const tvbx_sweep* h, int64_t* n_sets, int32_t* n_reg
 struct RunPlan {
     SimArgs a;
     int variant = -1;
+    WindowPlan win;
     int pb = 16;
     int32_t n_tiles = 0;
     int nnz_max = 0;
@@ -546,7 +569,8 @@ struct RunPlan {
 // ring buffers and OU state are kept; the series and the running sums start
 // afresh for the new samples).
 static tvbx_status prepare_run(tvbx_sweep* h, const tvbx_run_cfg& c, cudaStream_t s, int general_pb,
-                               bool device_init, RunPlan& plan, bool direct_body = false, int64_t n_base = 0)
+                               bool device_init, RunPlan& plan, bool direct_body = false, int64_t n_base = 0,
+                               bool windows = true)
 {
     if (!(c.dt_ms > 0.0) || !isfinite(c.dt_ms)) return fail(TVBX_E_INVALID_ARG, "dt_ms must be > 0");
     if (c.n_steps < 0 || n_base + c.n_steps > ((int64_t)1 << 32) - 2)
@@ -580,12 +604,15 @@ static tvbx_status prepare_run(tvbx_sweep* h, const tvbx_run_cfg& c, cudaStream_
 
     // internal order: sets grouped by speed
     h->perm.clear();
-    int64_t ring_floats = 0;
+    int64_t ring_floats = 0, largest_group = 0;
+    int32_t d_min = INT32_MAX;
     for (Group& g : groups) {
         g.p_base = (int32_t)h->perm.size();
         ring_floats = (ring_floats + 63) / 64 * 64;   // 256-byte aligned ring per group
         g.ring_offset = ring_floats;
         ring_floats += (int64_t)g.H * N * ring_stride(g.sets.size());
+        largest_group = std::max<int64_t>(largest_group, (int64_t)g.sets.size());
+        d_min = std::min(d_min, g.d_min);
         for (int64_t e : g.sets) h->perm.push_back(e);
     }
     h->identity = true;
@@ -606,10 +633,21 @@ static tvbx_status prepare_run(tvbx_sweep* h, const tvbx_run_cfg& c, cudaStream_
         (c.kernel < TVBX_KERNEL_AUTO || c.kernel >= TVBX_KERNEL_PREFETCH + sim_fast_variants()))
         return fail(TVBX_E_INVALID_ARG, "unknown kernel %d", c.kernel);
     if (c.withhold_step < 0) return fail(TVBX_E_INVALID_ARG, "withhold_step must be >= 0");
-    int variant = -1;   // prefetch variant, -1 = general kernel, -2 = register-tile kernel
+    int variant = -1;   // prefetch variant, -1 = general kernel, -2 = register-tile kernels
+    WindowPlan win;
+    // a continued run keeps the ring layout it finds
+    if (n_base > 0 && h->win.steps == 0) windows = false;
+    if (windows && general_pb == 0 && c.kernel == TVBX_KERNEL_AUTO && sim_direct_pb(N) > 0) {
+        int dev = 0, sms = 0;
+        CK(cudaGetDevice(&dev), "device");
+        CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "device");
+        if (!sim_window_plan(d_min, N, largest_group, h->model.tau_e == h->model.tau_i, sms, win)) win = WindowPlan{};
+    }
     if (general_pb > 0) {
         // batch: the batch's body and tile width
         if (direct_body) variant = -2;
+    } else if (win.steps > 0) {
+        variant = -2;
     } else if (c.kernel == TVBX_KERNEL_AUTO) {
         // preference order from measurement on the 32,768-set, 68-region sweep
         // (the packed kernels, slower there, need the reduced transfer
@@ -637,6 +675,8 @@ static tvbx_status prepare_run(tvbx_sweep* h, const tvbx_run_cfg& c, cudaStream_
             return fail(TVBX_E_UNSUPPORTED, "n_regions %d too large", N);
     } else if (variant >= 0) {
         pb = sim_fast_pb(variant);
+    } else if (win.steps > 0) {
+        pb = win.pb;
     } else if (variant == -2) {
         pb = sim_direct_pb(N);
     } else {
@@ -645,6 +685,20 @@ static tvbx_status prepare_run(tvbx_sweep* h, const tvbx_run_cfg& c, cudaStream_
     }
     h->pb = pb;
     h->variant = variant;
+    h->win = win;
+    // rings: [H][N][stride] per group, or the windowed kernels' [tile][N][H + WIN_FAR][pb]
+    h->ring_floats = ring_floats;
+    h->ring_H0.clear();
+    for (const Group& g : groups) h->ring_H0.push_back(g.H);
+    if (win.steps > 0) {
+        ring_floats = 0;
+        for (Group& g : groups) {
+            g.H += win.steps - 1;
+            g.ring_offset = ring_floats;
+            const int64_t columns = ((int64_t)g.sets.size() + pb - 1) / pb * pb;
+            ring_floats += (columns * N * (g.H + WIN_FAR) + 63) / 64 * 64;
+        }
+    }
     std::vector<TileDev> tiles;
     std::vector<GroupDev> gdev(groups.size());
     std::vector<int32_t> all_row;
@@ -657,6 +711,7 @@ static tvbx_status prepare_run(tvbx_sweep* h, const tvbx_run_cfg& c, cudaStream_
         nz_off[gi] = (int64_t)all_cd.size();
         all_row.insert(all_row.end(), g.row_ptr.begin(), g.row_ptr.end());
         all_row.insert(all_row.end(), g.row_mid.begin(), g.row_mid.end());
+        all_row.insert(all_row.end(), g.row_near.begin(), g.row_near.end());
         all_cd.insert(all_cd.end(), g.col_dly.begin(), g.col_dly.end());
         all_w.insert(all_w.end(), g.w.begin(), g.w.end());
         const int32_t Pg = (int32_t)g.sets.size();
@@ -685,7 +740,15 @@ static tvbx_status prepare_run(tvbx_sweep* h, const tvbx_run_cfg& c, cudaStream_
     CK(h->d_inv.ensure(sizeof(int64_t) * P), "set index");
     CK(h->d_state.ensure(sizeof(float) * (size_t)SV_COUNT * N * P), "state");
     CK(h->d_status.ensure(sizeof(uint32_t) * P), "status");
-    CK(h->d_ring.ensure(sizeof(float) * (size_t)std::max<int64_t>(ring_floats, 1)), "ring buffers");
+    cudaError_t ring_e = h->d_ring.ensure(sizeof(float) * (size_t)std::max<int64_t>(ring_floats, 1));
+    if (ring_e == cudaSuccess && win.far) ring_e = h->d_far.ensure(sizeof(float) * tiles.size() * WIN_FAR * N * pb);
+    if (ring_e != cudaSuccess && win.steps > 0) {
+        // the windowed layout is larger: without room for it the other kernels still run
+        h->d_far.release();
+        (void)cudaGetLastError();
+        return prepare_run(h, c, s, general_pb, device_init, plan, direct_body, n_base, false);
+    }
+    CK(ring_e, "ring buffers");
     // set-blocked series: groups of 4 sets, [ceil(P / 4)][series_T][N][4]
     const int64_t P4 = (P + 3) / 4 * 4;
     h->sl = layout_blocked(N, std::max<int64_t>(series_T, 1));
@@ -709,6 +772,7 @@ static tvbx_status prepare_run(tvbx_sweep* h, const tvbx_run_cfg& c, cudaStream_
         d.ring = h->d_ring.as<float>() + groups[gi].ring_offset;
         d.row_ptr = h->d_csr_row.as<int32_t>() + row_off[gi];
         d.row_mid = h->d_csr_row.as<int32_t>() + row_off[gi] + N + 1;
+        d.row_near = d.row_mid + N;
         d.col_dly = h->d_csr_cd.as<uint32_t>() + nz_off[gi];
         d.w = h->d_csr_w.as<float>() + nz_off[gi];
         d.H = groups[gi].H;
@@ -736,7 +800,7 @@ static tvbx_status prepare_run(tvbx_sweep* h, const tvbx_run_cfg& c, cudaStream_
         CK(cudaMemcpyAsync(h->d_tiles.ptr, tiles.data(), sizeof(TileDev) * tiles.size(), cudaMemcpyHostToDevice, s), "upload");
     if (n_base == 0) CK(cudaMemsetAsync(h->d_ou_state.ptr, 0, sizeof(float) * N, s), "OU state");
     CK(cudaMemsetAsync(h->d_error.ptr, 0, sizeof(uint32_t), s), "error word");
-    h->ring_floats = ring_floats;
+    h->ring_groups = gdev;
 
     if (!c.noise_per_set) CK(h->d_ou_table.ensure(sizeof(float) * (size_t)chunk * N), "OU table");
 
@@ -785,10 +849,15 @@ static tvbx_status prepare_run(tvbx_sweep* h, const tvbx_run_cfg& c, cudaStream_
     if (device_init) {
         CK(launch_init_state(a, s), "init state");
         for (size_t gi = 0; gi < groups.size(); ++gi)
-            CK(launch_init_ring(gdev[gi].ring, (int64_t)gdev[gi].H * N * gdev[gi].stride, a.m.E0, s), "init ring");
+            CK(launch_init_ring(gdev[gi].ring,
+                                win.steps > 0 ? (gdev[gi].P_g + pb - 1) / pb * (int64_t)pb * N * (gdev[gi].H + WIN_FAR)
+                                              : (int64_t)gdev[gi].H * N * gdev[gi].stride,
+                                a.m.E0, s),
+               "init ring");
     }
     plan.a = a;
     plan.variant = variant;
+    plan.win = win;
     plan.pb = pb;
     plan.n_tiles = (int32_t)tiles.size();
     plan.nnz_max = nnz_max;
@@ -884,6 +953,18 @@ static tvbx_status run_chunks(tvbx_sweep* h, const tvbx_run_cfg& c, const RunPla
             CK(cudaEventRecord(h->ev[h->ev_used], s), "profiling event");
         }
         if (variant >= 0) CK(launch_sim_fast(a, variant, plan.n_tiles, plan.nnz_max, s), "simulation chunk");
+        else if (plan.win.steps > 0) {
+            SimArgs aw = a;
+            for (int64_t w0 = 0; w0 < a.n_chunk; w0 += aw.n_chunk) {
+                // a window stays within the steps whose far sums are at hand
+                const int64_t row = plan.win.far ? w0 % WIN_FAR : 0;
+                const int64_t most = plan.win.far ? WIN_FAR - row : a.n_chunk;
+                aw.n0 = n0 + w0;
+                aw.n_chunk = (int32_t)std::min({(int64_t)plan.win.steps, a.n_chunk - w0, most});
+                CK(launch_sim_window(aw, plan.win, plan.n_tiles, w0, h->d_far.as<float>(), (int32_t)row, s),
+                   "simulation window");
+            }
+        }
         else if (variant == -2) CK(launch_sim_direct(a, plan.n_tiles, plan.pb, s), "simulation chunk");
         else CK(launch_sim_chunk(a, plan.n_tiles, plan.pb, s), "simulation chunk");
         if (h->profiling) {
@@ -975,6 +1056,35 @@ uint64_t sweep_fingerprint(const tvbx_sweep* h)
     return x;
 }
 
+// The ring of a windowed run to (out) or from its checkpoint layout in host
+// memory, through a staging buffer of whole slots.
+tvbx_status convert_ring(tvbx_sweep* h, bool out, int64_t n, unsigned char* host)
+{
+    int64_t off = 0;   // floats into the checkpoint's ring
+    for (size_t gi = 0; gi < h->ring_groups.size(); ++gi) {
+        const GroupDev& g = h->ring_groups[gi];
+        const int32_t H0 = h->ring_H0[gi];
+        const int64_t row = (int64_t)h->N * g.stride;
+        off = (off + 63) / 64 * 64;
+        const int32_t nf = (int32_t)std::min<int64_t>(H0, std::max<int64_t>(1, ((int64_t)16 << 20) / row));
+        CK(h->d_tmp.ensure(sizeof(float) * (size_t)(nf * row)), "ring staging");
+        float* rows = h->d_tmp.as<float>();
+        for (int32_t f = 0; f < H0; f += nf) {
+            const int32_t m = std::min(nf, H0 - f);
+            unsigned char* at = host + sizeof(float) * (size_t)(off + f * row);
+            const size_t bytes = sizeof(float) * (size_t)(m * row);
+            if (!out) CK(cudaMemcpy(rows, at, bytes, cudaMemcpyHostToDevice), "ring staging");
+            CK(launch_ring_convert(out, g.ring, h->win, g.H, h->N, g.P_g, g.stride, H0, n, f, m, (float)h->model.E0,
+                                   rows, nullptr),
+               "ring layout");
+            if (out) CK(cudaMemcpy(at, rows, bytes, cudaMemcpyDeviceToHost), "ring staging");
+        }
+        off += H0 * row;
+    }
+    CK(cudaStreamSynchronize(nullptr), "ring layout");
+    return TVBX_OK;
+}
+
 size_t ckpt_bytes(int64_t N, int64_t P, int64_t ring_floats)
 {
     return sizeof(CkptHeader) + sizeof(float) * ((size_t)SV_COUNT * N * P + (size_t)ring_floats + (size_t)N) +
@@ -1029,7 +1139,11 @@ tvbx_status tvbx_checkpoint(tvbx_sweep* h, void* host_buf, uint64_t bytes)
     off += b_state;
     CK(cudaMemcpy(out + off, h->d_status.ptr, b_status, cudaMemcpyDeviceToHost), "checkpoint status");
     off += b_status;
-    if (b_ring) CK(cudaMemcpy(out + off, h->d_ring.ptr, b_ring, cudaMemcpyDeviceToHost), "checkpoint ring");
+    if (h->win.steps > 0) {
+        if (tvbx_status e = convert_ring(h, true, h->steps_done, out + off)) return e;
+    } else if (b_ring) {
+        CK(cudaMemcpy(out + off, h->d_ring.ptr, b_ring, cudaMemcpyDeviceToHost), "checkpoint ring");
+    }
     off += b_ring;
     CK(cudaMemcpy(out + off, h->d_ou_state.ptr, b_ou, cudaMemcpyDeviceToHost), "checkpoint OU state");
     h->d2h += need - sizeof hd;
@@ -1078,7 +1192,11 @@ tvbx_status tvbx_restore(tvbx_sweep* h, const void* host_buf, uint64_t bytes)
     in += b_state;
     CK(cudaMemcpy(h->d_status.ptr, in, b_status, cudaMemcpyHostToDevice), "restore status");
     in += b_status;
-    if (b_ring) CK(cudaMemcpy(h->d_ring.ptr, in, b_ring, cudaMemcpyHostToDevice), "restore ring");
+    if (h->win.steps > 0) {
+        if (tvbx_status e = convert_ring(h, false, hd.steps_done, const_cast<unsigned char*>(in))) return e;
+    } else if (b_ring) {
+        CK(cudaMemcpy(h->d_ring.ptr, in, b_ring, cudaMemcpyHostToDevice), "restore ring");
+    }
     in += b_ring;
     CK(cudaMemcpy(h->d_ou_state.ptr, in, b_ou, cudaMemcpyHostToDevice), "restore OU state");
     h->h2d += b_state + b_status + b_ring + b_ou;

@@ -59,15 +59,18 @@ struct DevModel {
 
 // One speed group: sets sharing a delay matrix and a ring buffer.
 struct GroupDev {
-    float* ring;               // [H][N][P_g], E of the group's sets
+    float* ring;               // [H][N][stride], E of the group's sets (the windowed
+                               // kernel's own layout: sim_window.cu)
     const int32_t* row_ptr;    // [N + 1] CSR rows of the nonzero weights u_kj; each row
                                // starts at an index of the parity of k (padded with a
                                // zero-weight self entry of delay 1) and ends with its
                                // zero-delay entries
+    const int32_t* row_near;   // [N] first entry of each row with a delay below WIN_FAR (when
+                               // the shortest delay is below WIN_NEAR_BELOW)
     const int32_t* row_mid;    // [N] first zero-delay entry of each row
     const uint32_t* col_dly;   // [nnz] (delay << 16) | j
     const float* w;            // [nnz] u_kj
-    int32_t H;                 // ring depth (max delay + 2)
+    int32_t H;                 // ring depth (max delay + 2; windowed: + 1 + steps per window)
     int32_t P_g;               // sets in the group
     int32_t p_base;            // first internal set index of the group
     int32_t stride;            // ring row stride in floats (P_g rounded up to 32)
@@ -146,6 +149,31 @@ int sim_fast_pb(int variant);
 bool sim_fast_packed(int variant);   // FP32x2 kernel (needs tau_e == tau_i)
 int sim_fast_variants();
 size_t sim_fast_smem_bytes(int variant, int N, int nnz);
+// Windowed kernels (sim_window.cu): launches of `steps` steps of every pair.
+constexpr int WIN_MAX_STEPS = 32;
+// Sweeps whose shortest delay is below WIN_NEAR_BELOW steps sum the entries of
+// WIN_FAR steps and more for WIN_FAR steps at once (they come first in a row).
+constexpr int WIN_NEAR_BELOW = 8;
+constexpr int WIN_FAR = 16;
+struct WindowPlan {
+    int32_t steps = 0;     // steps per launch (0: no window)
+    int32_t pb = 0;        // sets per tile
+    int32_t threads = 0;   // per CTA
+    bool packed = false;   // two sets per thread
+    bool far = false;      // far entries summed apart
+};
+// d_min: shortest delay of a nonzero weight in steps; P: sets of the largest
+// speed group. False when the sweep has no window.
+bool sim_window_plan(int32_t d_min, int32_t N, int64_t P, bool reduced, int sms, WindowPlan& w);
+// far: buffer [n_tiles][WIN_FAR][N][pb] of the far sums (w.far); far_row: the
+// window's first step in it (0: the far sums are formed first).
+cudaError_t launch_sim_window(const SimArgs& a, const WindowPlan& w, int32_t n_tiles, int64_t table_step, float* far,
+                              int32_t far_row, cudaStream_t s);
+// Rows of slots [f0, f0 + nf) of a group's ring in the layout [H0][N][stride]
+// at step n, from (out) or to the windowed kernel's layout.
+cudaError_t launch_ring_convert(bool out, float* ring, const WindowPlan& w, int32_t H, int32_t N, int32_t P_g,
+                                int32_t stride, int32_t H0, int64_t n, int32_t f0, int32_t nf, float E0, float* rows,
+                                cudaStream_t s);
 int sim_threads(int N, int pb);
 size_t sim_smem_bytes(int N, int pb);
 

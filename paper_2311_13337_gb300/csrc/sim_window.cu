@@ -1,0 +1,394 @@
+// Windowed simulation kernels of the tvbx engine (arXiv 2311.13337, the
+// lock-step integration of Eq. 1-5 with forward Euler).
+//
+// No coupling reads a value younger than the shortest delay d_min of the
+// connectome, so over a window of B <= d_min steps every (set, region) pair
+// is independent of the others: the coupling sums of all B steps can be formed
+// from the ring before the first of them is taken. One launch advances every
+// pair by one window; launch order is the only synchronisation, so nothing
+// waits at a barrier, any number of regions or sets fills the chip evenly, and
+// each row entry is read once per window instead of once per step.
+//
+// A thread owns one region of one set (float) or of two adjacent sets (float2,
+// packed FP32x2). It
+//  1. forms the coupling sums of the window, up to 8 steps at a time, in CSR
+//     order (the sums of the other kernels, bit for bit): independent loads
+//     that do not wait for the sums;
+//  2. loads its state, takes the B steps in registers, and writes E of each
+//     step to the ring; then stores the state.
+//
+// Ring layout: [tile][N][H + WIN_FAR][pb], a tile of pb sets holding the H last
+// steps of a region contiguously, with the first WIN_FAR slots repeated after
+// slot H - 1: the rows an entry reads are one run that never wraps.
+// H = d_max + 1 + B, so that the window's own writes never meet a row that
+// another thread of the same launch may still read.
+//
+// Short delays (d_min < 8, large connectomes at high speeds): a window of d_min
+// steps alone would read each row entry for a few steps only. The entries with
+// d >= WIN_FAR then go first in each CSR row and sim_far_kernel sums them for
+// WIN_FAR steps at once into a buffer [tile][WIN_FAR][N][pb]; the windows of
+// d_min steps start from those sums and add the few nearer entries.
+//
+// Zero delays (which read the current step) have no window; such sweeps take
+// the other kernels.
+
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+#include <type_traits>
+
+#include "internal.h"
+#include "model_device.cuh"
+
+namespace tvbx {
+
+namespace {
+
+// 128 threads and 128 registers: four CTAs per SM. Five or six (102, 85
+// registers, more spills) and three measured slower (32,768 x 68 sweep, 500
+// steps: 23.5 ms against 27.3, 31.5 and 25.4).
+constexpr int WIN_THREADS = 128;
+
+template <class V> struct VSets;
+template <> struct VSets<float> { static constexpr int n = 1; };
+template <> struct VSets<float2> { static constexpr int n = 2; };
+
+__device__ __forceinline__ void load_v(float& x, const float* p, bool, bool) { x = *p; }
+__device__ __forceinline__ void load_v(float2& x, const float* p, bool, bool act1)
+{
+    x.x = p[0];
+    x.y = act1 ? p[1] : 0.0f;
+}
+__device__ __forceinline__ void store_v(float* p, float x, bool) { *p = x; }
+__device__ __forceinline__ void store_v(float* p, float2 x, bool act1)
+{
+    p[0] = x.x;
+    if (act1) p[1] = x.y;
+}
+
+__device__ __noinline__ float next_ou(const DevModel& m, uint64_t seed, uint32_t n, uint32_t k, uint32_t p, float OU)
+{
+    const float xi = std_normal(seed, n, k, p);
+    return fmaf(m.ou_a, m.ou_mu - OU, fmaf(m.ou_b, xi, OU));
+}
+
+// Coupling sums of G steps from row `at` on: row entries [e0, e1) added to acc.
+// ring: row (j, slot) at (j HR + slot) pb. Four entries' loads are in flight
+// together (one: 27.1 ms, two: 23.5 ms, four: 21.9 ms on the sweep above).
+template <int G, class V>
+__device__ __forceinline__ void gather(V (&acc)[G], const GroupDev& grp, const float* ring, int e0, int e1, int at,
+                                       int H, int HR, int pb)
+{
+    const uint32_t* __restrict__ cd_p = grp.col_dly;
+    const float* __restrict__ w_p = grp.w;
+#pragma unroll 4
+    for (int e = e0; e < e1; ++e) {
+        const uint32_t cd = __ldg(cd_p + e);
+        const V w = vbc<V>(__ldg(w_p + e));
+        int sl = at - (int)(cd >> 16);
+        sl += sl < 0 ? H : 0;
+        const float* row = ring + (uint32_t)(((cd & 0xffffu) * (uint32_t)HR + (uint32_t)sl) * (uint32_t)pb);
+#pragma unroll
+        for (int b = 0; b < G; ++b) acc[b] = vfma(w, *reinterpret_cast<const V*>(row + b * pb), acc[b]);
+    }
+}
+
+// The pair of the calling thread: region k of sets tile.q0 + q (and + 1).
+struct WinSlot {
+    int k, q;
+    bool act1;
+};
+template <int S>
+__device__ __forceinline__ WinSlot win_slot(const TileDev& tile, int32_t blocks_per_tile)
+{
+    const int width = (tile.nq + S - 1) / S;   // threads per region
+    const int i = (blockIdx.x % blocks_per_tile) * blockDim.x + threadIdx.x;
+    WinSlot w;
+    w.k = i / width;
+    w.q = (i - w.k * width) * S;
+    w.act1 = w.q + 1 < tile.nq;
+    return w;
+}
+
+// Sums of the entries with d >= WIN_FAR over the WIN_FAR steps from a.n0 on.
+// Bound by the L2 reads of the rows (4 B per weight and step); a launch covers
+// WIN_FAR steps so that the rows that different regions read are mostly the
+// same ones.
+template <class V, int PB>
+__global__ void __launch_bounds__(WIN_THREADS, 4)
+sim_far_kernel(const __grid_constant__ SimArgs a, int32_t pb_rt, int32_t blocks_per_tile, float* __restrict__ far)
+{
+    const int pb = PB > 0 ? PB : pb_rt;
+    const int32_t ti = blockIdx.x / blocks_per_tile;
+    const TileDev tile = a.tiles[ti];
+    const GroupDev& grp = a.groups[tile.group];
+    const int N = a.N;
+    const WinSlot w = win_slot<VSets<V>::n>(tile, blocks_per_tile);
+    if (w.k >= N) return;
+    const int H = grp.H, HR = H + WIN_FAR;
+    V acc[WIN_FAR];
+#pragma unroll
+    for (int b = 0; b < WIN_FAR; ++b) acc[b] = vbc<V>(0.0f);
+    gather<WIN_FAR>(acc, grp, grp.ring + (int64_t)tile.q0 * N * HR + w.q, grp.row_ptr[w.k], grp.row_near[w.k],
+                    (int)((uint32_t)a.n0 % (uint32_t)H), H, HR, pb);
+    float* out = far + ((int64_t)ti * WIN_FAR * N + w.k) * pb + w.q;
+#pragma unroll
+    for (int b = 0; b < WIN_FAR; ++b) *reinterpret_cast<V*>(out + (int64_t)b * N * pb) = acc[b];
+}
+
+// One window of a.n_chunk steps. PB: sets per tile (0: the runtime width
+// pb_rt). NEAR: the sums start from far (row 0: the window's first step) and
+// add the nearer entries.
+template <class V, int PB, bool NEAR>
+__global__ void __launch_bounds__(WIN_THREADS, 4)
+sim_window_kernel(const __grid_constant__ SimArgs a, int32_t pb_rt, int32_t blocks_per_tile, int64_t table_step,
+                  const float* __restrict__ far)
+{
+    constexpr int S = VSets<V>::n;
+    const int pb = PB > 0 ? PB : pb_rt;
+    extern __shared__ __align__(16) unsigned char win_smem[];
+    V* stash = reinterpret_cast<V*>(win_smem) + threadIdx.x;   // coupling of step b at stash[b * blockDim.x]
+    const int32_t ti = blockIdx.x / blocks_per_tile;
+    const TileDev tile = a.tiles[ti];
+    const GroupDev& grp = a.groups[tile.group];
+    const int N = a.N;
+    const WinSlot ws = win_slot<S>(tile, blocks_per_tile);
+    const int k = ws.k, q = ws.q;
+    const bool act1 = ws.act1;
+    if (k >= N) return;
+    const int H = grp.H, HR = H + WIN_FAR;
+    const uint32_t n0 = (uint32_t)a.n0;
+    const int steps = a.n_chunk;
+    const int slot0 = (int)(n0 % (uint32_t)H);
+    float* ring = grp.ring + (int64_t)tile.q0 * N * HR + q;
+
+    // 1. coupling sums of the window
+    {
+        const int e0 = NEAR ? grp.row_near[k] : grp.row_ptr[k], e1 = grp.row_mid[k];
+        const float* far_k = NEAR ? far + ((int64_t)ti * WIN_FAR * N + k) * pb + q : nullptr;
+        int b0 = 0;
+        auto pass = [&](auto g_c) {
+            constexpr int G = decltype(g_c)::value;
+            for (; b0 + G <= steps; b0 += G) {
+                V acc[G];
+#pragma unroll
+                for (int b = 0; b < G; ++b)
+                    acc[b] = NEAR ? *reinterpret_cast<const V*>(far_k + (int64_t)(b0 + b) * N * pb) : vbc<V>(0.0f);
+                int at = slot0 + b0;
+                at -= at >= H ? H : 0;
+                gather<G>(acc, grp, ring, e0, e1, at, H, HR, pb);
+#pragma unroll
+                for (int b = 0; b < G; ++b) stash[(b0 + b) * blockDim.x] = acc[b];
+            }
+        };
+        pass(std::integral_constant<int, 8>{});
+        pass(std::integral_constant<int, 4>{});
+        pass(std::integral_constant<int, 2>{});
+        pass(std::integral_constant<int, 1>{});
+    }
+
+    // 2. the window's steps
+    const DevModel& m = a.m;
+    const int64_t NP = (int64_t)N * a.P;
+    const int64_t p = grp.p_base + tile.q0 + q;
+    float* st = a.state + (int64_t)k * a.P + p;
+    ParamsV<V> sp;
+    {
+        const float* prm = a.prm + p;
+        load_v(sp.g, prm + (int64_t)TVBX_AXIS_G * a.P, true, act1);
+        load_v(sp.b_e, prm + (int64_t)TVBX_AXIS_B_E * a.P, true, act1);
+        load_v(sp.inv_tw, prm + (int64_t)TVBX_AXIS_TAU_W_E * a.P, true, act1);
+        sp.inv_tw = vmap(sp.inv_tw, [](float u) { return 1.0f / u; });
+        load_v(sp.ELe, prm + (int64_t)TVBX_AXIS_E_L_E * a.P, true, act1);
+        load_v(sp.ELi, prm + (int64_t)TVBX_AXIS_E_L_I * a.P, true, act1);
+        load_v(sp.a_e, prm + (int64_t)TVBX_AXIS_A_E * a.P, true, act1);
+        load_v(sp.wn, prm + (int64_t)TVBX_AXIS_W_NOISE * a.P, true, act1);
+        load_v(sp.cFee, prm + (int64_t)TVBX_AXIS_CF_EE * a.P, true, act1);
+        load_v(sp.cFei, prm + (int64_t)TVBX_AXIS_CF_EI * a.P, true, act1);
+        load_v(sp.cFie, prm + (int64_t)TVBX_AXIS_CF_IE * a.P, true, act1);
+        load_v(sp.cFii, prm + (int64_t)TVBX_AXIS_CF_II * a.P, true, act1);
+    }
+    PairV<V> x;
+    V accE, accI, ou;
+    load_v(x.E, st + SV_E * NP, true, act1);
+    load_v(x.I, st + SV_I * NP, true, act1);
+    load_v(x.Cee, st + SV_CEE * NP, true, act1);
+    load_v(x.Cei, st + SV_CEI * NP, true, act1);
+    load_v(x.Cii, st + SV_CII * NP, true, act1);
+    load_v(x.We, st + SV_WE * NP, true, act1);
+    load_v(x.Wi, st + SV_WI * NP, true, act1);
+    load_v(x.cWe, st + SV_CWE * NP, true, act1);
+    load_v(x.cWi, st + SV_CWI * NP, true, act1);
+    load_v(accE, st + SV_ACC_E * NP, true, act1);
+    load_v(accI, st + SV_ACC_I * NP, true, act1);
+    uint32_t pn[2] = {0u, 0u};
+    if (a.noise_per_set) {
+        load_v(ou, st + SV_OU * NP, true, act1);
+        pn[0] = (uint32_t)(a.p_offset + a.ext_index[p]);
+        if (S > 1 && act1) pn[1] = (uint32_t)(a.p_offset + a.ext_index[p + 1]);
+    } else {
+        ou = vbc<V>(0.0f);
+    }
+    Track<V> trk = track_init<V>();
+    const float inv_ts = 1.0f / (float)a.ts;
+    // samples are the means of ts post-step states: steps left to the next one, and its index
+    int left = a.ts - (int)(n0 % (uint32_t)a.ts);
+    int64_t t = n0 / (uint32_t)a.ts;
+    int slot_w = slot0;
+    float* const ring_k = ring + (uint32_t)(k * HR) * (uint32_t)pb;
+    const float* ou_p = a.ou_table + (a.noise_per_set ? 0 : table_step * N + k);
+    for (int b = 0; b < steps; ++b) {
+        const V OU = a.noise_per_set ? ou : vbc<V>(__ldg(ou_p));
+        ou_p += a.noise_per_set ? 0 : N;
+        pair_step(m, sp, x, stash[b * blockDim.x], OU, trk);
+        if (a.noise_per_set) {
+#pragma unroll
+            for (int l = 0; l < S; ++l)
+                set_lane(ou, l, next_ou(m, a.seed, n0 + (uint32_t)b, (uint32_t)k, pn[l], lane(OU, l)));
+        }
+        ++slot_w;
+        slot_w -= slot_w == H ? H : 0;
+        float* dst = ring_k + slot_w * pb;
+        store_v(dst, x.E, act1);
+        if (slot_w < WIN_FAR) store_v(dst + H * pb, x.E, act1);
+        accE = vadd(accE, x.E);
+        accI = vadd(accI, x.I);
+        if (--left == 0) {
+            if (t < a.T) {
+                const V xE = vmul(accE, vbc<V>(inv_ts)), xI = vmul(accI, vbc<V>(inv_ts));
+#pragma unroll
+                for (int l = 0; l < S; ++l) {
+                    if (l && !act1) continue;
+                    const int64_t so = series_index(a.sl, t, k, p + l);
+                    a.series[so] = lane(xE, l);
+                    if (a.series_i) a.series_i[so] = lane(xI, l);
+                    if (t >= a.transient) {
+                        float sE = st[SV_SUM_E * NP + l], cE = st[SV_CMP_E * NP + l];
+                        float sI = st[SV_SUM_I * NP + l], cI = st[SV_CMP_I * NP + l];
+                        kahan_add(sE, cE, lane(xE, l));
+                        kahan_add(sI, cI, lane(xI, l));
+                        st[SV_SUM_E * NP + l] = sE;
+                        st[SV_CMP_E * NP + l] = cE;
+                        st[SV_SUM_I * NP + l] = sI;
+                        st[SV_CMP_I * NP + l] = cI;
+                    }
+                }
+            }
+            left = a.ts;
+            ++t;
+            accE = vbc<V>(0.0f);
+            accI = vbc<V>(0.0f);
+        }
+    }
+    store_v(st + SV_E * NP, x.E, act1);
+    store_v(st + SV_I * NP, x.I, act1);
+    store_v(st + SV_CEE * NP, x.Cee, act1);
+    store_v(st + SV_CEI * NP, x.Cei, act1);
+    store_v(st + SV_CII * NP, x.Cii, act1);
+    store_v(st + SV_WE * NP, x.We, act1);
+    store_v(st + SV_WI * NP, x.Wi, act1);
+    store_v(st + SV_CWE * NP, x.cWe, act1);
+    store_v(st + SV_CWI * NP, x.cWi, act1);
+    store_v(st + SV_ACC_E * NP, accE, act1);
+    store_v(st + SV_ACC_I * NP, accI, act1);
+    if (a.noise_per_set) store_v(st + SV_OU * NP, ou, act1);
+#pragma unroll
+    for (int l = 0; l < S; ++l) {
+        const uint32_t f = track_flags(m, trk, l);
+        if (f && (l == 0 || act1)) atomicOr(a.status + p + l, f);
+    }
+}
+
+// [tile][N][H + WIN_FAR][pb] <-> slots [f0, f0 + nf) of [H0][N][stride], whose slot f
+// holds the latest step t <= n with t = f mod H0.
+template <bool OUT>
+__global__ void ring_convert_kernel(float* __restrict__ ring, int32_t H, int32_t pb, int32_t N, int32_t P_g,
+                                    int32_t stride, int32_t H0, int64_t n, int32_t f0, int32_t nf, float E0,
+                                    float* __restrict__ rows)
+{
+    const int64_t total = (int64_t)nf * N * stride;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
+        const int c = (int)(i % stride);
+        const int j = (int)(i / stride % N);
+        const int f = f0 + (int)(i / stride / N);
+        if (c >= P_g) {
+            if (OUT) rows[i] = E0;
+            continue;
+        }
+        int64_t back = (n - f) % H0;
+        back += back < 0 ? H0 : 0;
+        int64_t slot = (n - back) % H;
+        slot += slot < 0 ? H : 0;
+        const int tile = c / pb;
+        float* at = ring + (((int64_t)tile * N + j) * (H + WIN_FAR) + slot) * pb + (c - tile * pb);
+        if (OUT) {
+            rows[i] = *at;
+        } else {
+            *at = rows[i];
+            if (slot < WIN_FAR) at[(int64_t)H * pb] = rows[i];
+        }
+    }
+}
+
+template <class V, int PB>
+cudaError_t launch_v(const SimArgs& a, const WindowPlan& w, int32_t n_tiles, int64_t table_step, float* far,
+                     int32_t far_row, cudaStream_t s)
+{
+    constexpr int S = VSets<V>::n;
+    const int64_t per_tile = (int64_t)a.N * ((w.pb + S - 1) / S);
+    const int32_t bpt = (int32_t)((per_tile + w.threads - 1) / w.threads);
+    const unsigned grid = (unsigned)((int64_t)n_tiles * bpt);
+    const size_t smem = sizeof(V) * (size_t)w.threads * a.n_chunk;
+    if (w.far) {
+        if (far_row == 0) {
+            note_launch();
+            sim_far_kernel<V, PB><<<grid, w.threads, 0, s>>>(a, w.pb, bpt, far);
+        }
+        note_launch();
+        sim_window_kernel<V, PB, true><<<grid, w.threads, smem, s>>>(a, w.pb, bpt, table_step,
+                                                                     far + (int64_t)far_row * a.N * w.pb);
+    } else {
+        note_launch();
+        sim_window_kernel<V, PB, false><<<grid, w.threads, smem, s>>>(a, w.pb, bpt, table_step, nullptr);
+    }
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+bool sim_window_plan(int32_t d_min, int32_t N, int64_t P, bool reduced, int sms, WindowPlan& w)
+{
+    if (d_min < 1) return false;
+    w.far = d_min < WIN_NEAR_BELOW;
+    w.steps = d_min < WIN_MAX_STEPS ? d_min : WIN_MAX_STEPS;
+    // packed pairs of sets (fewer instructions per step, half the threads) when
+    // they still give every SM four warps per scheduler
+    w.packed = reduced && (int64_t)N * P >= (int64_t)sms * 4 * WIN_THREADS;
+    w.pb = 64;
+    while (w.pb > 2 && w.pb / 2 >= P) w.pb /= 2;
+    const int64_t threads = (int64_t)N * (w.packed ? (P + 1) / 2 : P);
+    // smaller CTAs spread a sweep that cannot fill the chip over more SMs
+    w.threads = threads >= (int64_t)sms * WIN_THREADS ? WIN_THREADS : (threads >= (int64_t)sms * 64 ? 64 : 32);
+    return true;
+}
+
+cudaError_t launch_sim_window(const SimArgs& a, const WindowPlan& w, int32_t n_tiles, int64_t table_step, float* far,
+                              int32_t far_row, cudaStream_t s)
+{
+    if (n_tiles <= 0 || a.n_chunk <= 0) return cudaSuccess;
+    if (w.packed) return w.pb == 64 ? launch_v<float2, 64>(a, w, n_tiles, table_step, far, far_row, s)
+                                    : launch_v<float2, 0>(a, w, n_tiles, table_step, far, far_row, s);
+    return launch_v<float, 0>(a, w, n_tiles, table_step, far, far_row, s);
+}
+
+cudaError_t launch_ring_convert(bool out, float* ring, const WindowPlan& w, int32_t H, int32_t N, int32_t P_g,
+                                int32_t stride, int32_t H0, int64_t n, int32_t f0, int32_t nf, float E0, float* rows,
+                                cudaStream_t s)
+{
+    note_launch();
+    auto kern = out ? ring_convert_kernel<true> : ring_convert_kernel<false>;
+    kern<<<2048, 256, 0, s>>>(ring, H, w.pb, N, P_g, stride, H0, n, f0, nf, E0, rows);
+    return cudaGetLastError();
+}
+
+}  // namespace tvbx

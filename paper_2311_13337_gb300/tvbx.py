@@ -487,7 +487,7 @@ def transfer_function(pop: int, x_e, x_i, W, E_L, C=None, model: Model | None = 
     return out
 
 
-KERNEL_NAMES = {KERNEL_GENERAL: "sim_chunk_kernel", KERNEL_DIRECT: "sim_direct_kernel"}
+KERNEL_NAMES = {KERNEL_GENERAL: "sim_chunk_kernel", KERNEL_DIRECT: "sim_window_kernel or sim_direct_kernel"}
 KERNEL_NAMES.update({KERNEL_PREFETCH + v: ("sim_pack_kernel" if v in PACKED_VARIANTS else "sim_tma_kernel" if 12 <= v <= 14 else
                                           "sim_bulk_kernel" if v in (4, 5) else "sim_fast_kernel") + f" (variant {v})"
                      for v in range(N_PREFETCH_VARIANTS)})
