@@ -1225,6 +1225,12 @@ static tvbx_status run_fc(tvbx_sweep* h, int32_t precision, int32_t fcd_window, 
         n_blocks = (int32_t)((Tn + blk - 1) / blk);
         m = fcd_window / fcd_step;
         nw = (int32_t)((Tn - fcd_window) / fcd_step + 1);
+    } else if (precision == TVBX_FC_FP32 && h->cfg.series_mode != TVBX_SERIES_STREAM) {
+        n_blocks = fc_moment_split(N, P, Tn);
+        if (n_blocks > 1) {
+            blk = (int32_t)((Tn + n_blocks - 1) / n_blocks);
+            n_blocks = (int32_t)((Tn + blk - 1) / blk);
+        }
     }
     const size_t stride_b = (size_t)N * N + N;
     if (h->cfg.series_mode == TVBX_SERIES_STREAM) {
@@ -1386,6 +1392,12 @@ tvbx_status tvbx_fc_series(const float* series, int32_t n_regions, int64_t n_set
         n_blocks = (int32_t)((Tn + blk - 1) / blk);
         m = cfg->fcd_window / cfg->fcd_step;
         nw = (int32_t)((Tn - cfg->fcd_window) / cfg->fcd_step + 1);
+    } else if (cfg->precision == TVBX_FC_FP32) {
+        n_blocks = fc_moment_split(N, P, Tn);
+        if (n_blocks > 1) {
+            blk = (int32_t)((Tn + n_blocks - 1) / n_blocks);
+            n_blocks = (int32_t)((Tn + blk - 1) / blk);
+        }
     }
     cudaStream_t s = (cudaStream_t)cuda_stream;
     const size_t stride_b = (size_t)N * N + N;

@@ -20,124 +20,243 @@
 #include <stdint.h>
 
 #include "internal.h"
+#include "ptx_async.cuh"
 
 namespace tvbx {
 
-constexpr int FC_SETS = 8;        // sets per CTA (one 32-byte sector per (t, k) row)
-constexpr int FC_THREADS = 256;
-constexpr int FC_TASKS_PER_THREAD = 5;
+// ---------------------------------------------------------------------------
+// Gram block moments in FP32. A CTA owns m groups of 4 sets (the 16-byte pieces
+// of a sample), one moment block of samples and a range of 8 x 8 tiles of the
+// upper triangle; a thread owns one tile of one set in registers. Chunks of Tt
+// samples, copied a chunk ahead by cp.async into slots of their own threads, go
+// minus the shift to one of two shared buffers [set][Tt][Npad] (regions fastest): a thread reads 16 values for 64
+// multiply-adds, and the threads of a row of tiles share 8 of them. Column N of
+// the buffer is 1, so the row sums are the Gram column N. Bound by the FP32
+// pipe: 45 tiles per set at 68 regions, 81% of whose products are needed.
+// Measured 4.16 ms on 4,096 x 68 x 5,000 (FMA pipe 51% busy; staging and shared
+// memory take the rest); 4 x 4 tiles of 8 sets took 30 ms.
+// ---------------------------------------------------------------------------
+constexpr int FCR_MAXB = 12;      // most moment blocks the reductions take in registers
+constexpr int FM_TILE = 8;
+constexpr int FM_THREADS = 192;   // at most; two CTAs per SM (a third needs 96 registers, with spills)
+constexpr int FM_LOADS = 6;       // 16-byte pieces a thread copies per chunk
 
-// Gram block moments. grid = (P / FC_SETS, task chunks). Each thread owns up to
-// FC_TASKS_PER_THREAD 4x4 tiles (set q, row tile kb <= column tile jb).
-__global__ void __launch_bounds__(FC_THREADS)
-fc_moments_kernel(const __grid_constant__ FcArgs a, int32_t Npad, int32_t Tt, int32_t tasks_per_set,
-                  int32_t tasks_per_chunk)
+struct FmPlan {
+    int32_t npad;             // regions and the column of ones, rounded up to the tile
+    int32_t tasks_per_set;    // tiles of the upper triangle
+    int32_t m;                // groups of 4 sets per CTA
+    int32_t chunks, per_chunk;// CTAs that share a group's tiles, tiles of each
+    int32_t threads;
+    int32_t Tt;               // samples per chunk
+    size_t smem;
+};
+
+static FmPlan fm_plan(int32_t N, int64_t P)
 {
-    extern __shared__ float xs[];             // [FC_SETS][Tt][Npad]
-    __shared__ float shift[FC_SETS * 384];    // N <= 384
-    const int N = a.N;
-    const int p0 = blockIdx.x * FC_SETS;
-    const int nsets = min(FC_SETS, a.P - p0);
+    FmPlan f;
+    f.npad = (N + 1 + FM_TILE - 1) / FM_TILE * FM_TILE;
+    const int nt = f.npad / FM_TILE;
+    f.tasks_per_set = nt * (nt + 1) / 2;
+    const int64_t groups = (P + 3) / 4;
+    // few regions: several groups fill a CTA, as long as there are CTAs for every SM
+    f.m = 1;
+    while (f.m < 8 && 2 * f.m * 4 * f.tasks_per_set <= FM_THREADS && groups / (2 * f.m) >= 304) f.m *= 2;
+    const int total = 4 * f.m * f.tasks_per_set;
+    f.chunks = (total + FM_THREADS - 1) / FM_THREADS;
+    f.per_chunk = (total + f.chunks - 1) / f.chunks;
+    f.threads = (f.per_chunk + 31) / 32 * 32;
+    if (f.threads < 64) f.threads = 64;
+    f.Tt = FM_LOADS * f.threads / (N * f.m);
+    f.Tt = f.Tt < 1 ? 1 : (f.Tt > 16 ? 16 : f.Tt);
+    f.smem = sizeof(float) * (size_t)(4 * f.m) * (2 * (size_t)f.Tt * f.npad + N) +
+             sizeof(float4) * (size_t)FM_LOADS * f.threads;
+    return f;
+}
+
+__device__ __forceinline__ void cp_async4(float* dst, const float* src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+
+// two FP32 values in a register pair; fma.rn.f32x2 rounds each lane as fmaf
+__device__ __forceinline__ uint64_t pair2(float lo, float hi)
+{
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void unpair2(uint64_t v, float& lo, float& hi)
+{
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ void fma2(uint64_t& d, uint64_t x, uint64_t y)
+{
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(x), "l"(y));
+}
+
+// position of region k in a row of the buffer: 16-byte pieces 8 apart swap with
+// their neighbour, so that the 32-byte strides of a warp's tiles meet every bank
+__device__ __forceinline__ int fm_pos(int k)
+{
+    const int c = k >> 2;
+    return ((c ^ ((c >> 3) & 1)) << 2) | (k & 3);
+}
+
+template <bool VEC>
+__global__ void __launch_bounds__(FM_THREADS, 2)
+fc_moments_kernel(const __grid_constant__ FcArgs a, const __grid_constant__ FmPlan f)
+{
+    extern __shared__ __align__(16) float fm_smem[];
+    const int N = a.N, npad = f.npad, Tt = f.Tt, sets = 4 * f.m;
+    const int tid = threadIdx.x, nthr = blockDim.x;
+    float* xs = fm_smem;                                       // [2][sets][Tt][npad]
+    const int buf = sets * Tt * npad;
+    float4* sh = reinterpret_cast<float4*>(xs + 2 * buf);      // [m][N], the 4 sets of a group
+    const int64_t b = blockIdx.x % a.n_blocks;
+    const int64_t g0 = blockIdx.x / a.n_blocks * f.m;          // first group
     const int64_t Tn = a.t_end - a.t_begin;
-    const int nb = Npad / 4;
-
-    for (int i = threadIdx.x; i < FC_SETS * N; i += blockDim.x) {
-        const int q = i / N, k = i - q * N;
-        float mval = 0.0f;
-        if (q < nsets && Tn > 0) {
-            const int64_t p = p0 + q;
-            if (a.state) mval = a.state[(int64_t)SV_SUM_E * N * a.P + (int64_t)k * a.P + p] / (float)Tn;
-            else if (a.shift) mval = a.shift[(int64_t)k * a.P + p];
-        }
-        shift[q * N + k] = mval;
-    }
-
-    // this thread's tasks
-    int tq[FC_TASKS_PER_THREAD], tk[FC_TASKS_PER_THREAD], tj[FC_TASKS_PER_THREAD];
-    int ntask = 0;
-    const int chunk0 = blockIdx.y * tasks_per_chunk;
-    for (int i = 0; i < FC_TASKS_PER_THREAD; ++i) {
-        const int task = chunk0 + threadIdx.x + i * FC_THREADS;
-        tq[i] = -1;
-        if (task < chunk0 + tasks_per_chunk && task < tasks_per_set * FC_SETS) {
-            const int q = task / tasks_per_set;
-            int r = task - q * tasks_per_set;
-            int kb = 0;
-            while (r >= nb - kb) { r -= nb - kb; ++kb; }
-            if (q < nsets) { tq[i] = q; tk[i] = kb; tj[i] = kb + r; ntask = i + 1; }
-        }
-    }
-    float acc[FC_TASKS_PER_THREAD][16];
-    float rs[FC_TASKS_PER_THREAD][4];
-#pragma unroll
-    for (int i = 0; i < FC_TASKS_PER_THREAD; ++i) {
-#pragma unroll
-        for (int c = 0; c < 16; ++c) acc[i][c] = 0.0f;
-#pragma unroll
-        for (int c = 0; c < 4; ++c) rs[i][c] = 0.0f;
-    }
     const int64_t blk = a.blk > 0 ? a.blk : Tn;
-    const int64_t stride_b = (int64_t)N * N + N;
-    __syncthreads();
+    const int64_t t_lo = a.t_begin + b * blk;
+    const int64_t len = (t_lo + blk < a.t_end ? t_lo + blk : a.t_end) - t_lo;
 
-    for (int64_t t0 = 0; t0 < Tn; t0 += Tt) {
-        const int len = (int)(Tn - t0 < (int64_t)Tt ? Tn - t0 : (int64_t)Tt);
-        // stage rows x[t][k][p0 .. p0 + FC_SETS) minus the shift, transposed to [q][t][k]
-        for (int i = threadIdx.x; i < len * Npad * FC_SETS; i += blockDim.x) {
-            const int q = i % FC_SETS;
-            const int rem = i / FC_SETS;
-            const int k = rem % Npad;
-            const int tt = rem / Npad;
-            float v = 0.0f;
-            if (k < N && q < nsets)
-                v = a.series[series_index(a.sl, a.t_begin + t0 + tt, k, p0 + q)] - shift[q * N + k];
-            xs[((int64_t)q * Tt + tt) * Npad + k] = v;
+    for (int i = tid; i < 2 * buf; i += nthr) xs[i] = 0.0f;
+    for (int i = tid; i < f.m * N; i += nthr) {
+        const int g = i / N, k = i - g * N;
+        float v[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+        for (int q = 0; q < 4; ++q) {
+            const int64_t p = 4 * (g0 + g) + q;
+            if (p >= a.P) continue;
+            if (a.state) v[q] = a.state[(int64_t)SV_SUM_E * N * a.P + (int64_t)k * a.P + p] / (float)Tn;
+            else if (a.shift) v[q] = a.shift[(int64_t)k * a.P + p];
         }
-        __syncthreads();
-        for (int tt = 0; tt < len; ++tt) {
+        sh[i] = make_float4(v[0], v[1], v[2], v[3]);
+    }
+    __syncthreads();
+    for (int i = tid; i < 2 * sets * Tt; i += nthr) xs[i * npad + fm_pos(N)] = 1.0f;
+
+    // this thread's tile
+    const int task = blockIdx.y * f.per_chunk + tid;
+    const bool works = tid < f.per_chunk && task < sets * f.tasks_per_set;
+    int q = 0, kb = 0, jb = 0;
+    if (works) {
+        q = task / f.tasks_per_set;
+        int r = task - q * f.tasks_per_set;
+        const int nt = npad / FM_TILE;
+        while (r >= nt - kb) { r -= nt - kb; ++kb; }
+        jb = kb + r;
+    }
+    const int64_t p = 4 * g0 + q;
+    const int ck0 = fm_pos(FM_TILE * kb), ck1 = fm_pos(FM_TILE * kb + 4);
+    const int cj0 = fm_pos(FM_TILE * jb), cj1 = fm_pos(FM_TILE * jb + 4);
+    uint64_t acc2[FM_TILE][FM_TILE / 2];   // two neighbouring columns each
 #pragma unroll
-            for (int i = 0; i < FC_TASKS_PER_THREAD; ++i) {
-                if (i < ntask && tq[i] >= 0) {
-                    const float4 xk = *reinterpret_cast<const float4*>(xs + ((int64_t)tq[i] * Tt + tt) * Npad + 4 * tk[i]);
-                    const float4 xj = *reinterpret_cast<const float4*>(xs + ((int64_t)tq[i] * Tt + tt) * Npad + 4 * tj[i]);
-                    const float kv[4] = {xk.x, xk.y, xk.z, xk.w};
-                    const float jv[4] = {xj.x, xj.y, xj.z, xj.w};
+    for (int r = 0; r < FM_TILE; ++r)
 #pragma unroll
-                    for (int r = 0; r < 4; ++r) {
+        for (int c = 0; c < FM_TILE / 2; ++c) acc2[r][c] = 0;
+
+    // 16-byte pieces (row = group and sample, region) of a chunk, dealt to the
+    // threads in turn, a chunk ahead: VEC by cp.async into slots of their own
+    // threads, else (rows that are not 16-byte aligned) in registers
+    const int row_first = tid / N, k_first = tid - row_first * N, row_step = nthr / N, k_step = nthr - row_step * N;
+    const int rows = f.m * Tt;
+    float4* raw = reinterpret_cast<float4*>(sh + f.m * N) + tid;   // [FM_LOADS][threads]
+    float4 v[VEC ? 1 : FM_LOADS];
+    const float* base = a.series + g0 * a.sl.sg + t_lo * a.sl.st;
+    auto fetch = [&](int64_t t0) {
+        const int n = len - t0 < Tt ? (int)(len - t0) : Tt;
+        const float* chunk = base + t0 * a.sl.st;
+        int row = row_first, k = k_first;
 #pragma unroll
-                        for (int c = 0; c < 4; ++c) acc[i][r * 4 + c] = fmaf(kv[r], jv[c], acc[i][r * 4 + c]);
-                        rs[i][r] += kv[r];
-                    }
+        for (int u = 0; u < FM_LOADS; ++u) {
+            const int g = f.m > 1 ? row / Tt : 0, t = f.m > 1 ? row - g * Tt : row;
+            const int left = (int)(a.P - 4 * g0) - 4 * g;   // sets from this group on (a.P < 2^31)
+            if (row < rows && t < n && left > 0) {
+                const float* src = chunk + t * a.sl.st + k * a.sl.sk;
+                if (f.m > 1) src += g * a.sl.sg;
+                if constexpr (VEC) {
+                    if (left >= 4) cp_async16(raw + u * nthr, src);
+                    else
+                        for (int c = 0; c < left; ++c) cp_async4(reinterpret_cast<float*>(raw + u * nthr) + c, src + c);
+                } else {
+                    v[u].x = src[0];
+                    if (left > 1) v[u].y = src[1];
+                    if (left > 2) v[u].z = src[2];
+                    if (left > 3) v[u].w = src[3];
                 }
             }
-            // end of a moment block: write it out and restart
-            const int64_t tg = t0 + tt + 1;
-            if (tg % blk == 0 || tg == Tn) {
-                const int64_t b = (tg - 1) / blk;
+            row += row_step;
+            k += k_step;
+            if (k >= N) { k -= N; ++row; }
+        }
+        if constexpr (VEC) cp_async_commit();
+    };
+    auto put = [&](float* dst) {
+        int row = row_first, k = k_first;
 #pragma unroll
-                for (int i = 0; i < FC_TASKS_PER_THREAD; ++i) {
-                    if (i < ntask && tq[i] >= 0) {
-                        float* G = a.blocks + ((int64_t)(p0 + tq[i]) * a.n_blocks + b) * stride_b;
-                        for (int r = 0; r < 4; ++r) {
-                            const int k = 4 * tk[i] + r;
-                            if (k >= N) continue;
-                            for (int c = 0; c < 4; ++c) {
-                                const int j = 4 * tj[i] + c;
-                                if (j >= N) continue;
-                                G[(int64_t)k * N + j] = acc[i][r * 4 + c];
-                                G[(int64_t)j * N + k] = acc[i][r * 4 + c];
-                            }
-                            if (tk[i] == tj[i]) G[(int64_t)N * N + k] = rs[i][r];
-                        }
+        for (int u = 0; u < FM_LOADS; ++u) {
+            if (row < rows) {
+                const int g = f.m > 1 ? row / Tt : 0;
+                const float4 s4 = sh[g * N + k], x = VEC ? raw[u * nthr] : v[VEC ? 0 : u];
+                float* at = dst + (3 * g * Tt + row) * npad + fm_pos(k);   // row 4 g Tt + t
+                at[0] = x.x - s4.x;
+                at[Tt * npad] = x.y - s4.y;
+                at[2 * Tt * npad] = x.z - s4.z;
+                at[3 * Tt * npad] = x.w - s4.w;
+            }
+            row += row_step;
+            k += k_step;
+            if (k >= N) { k -= N; ++row; }
+        }
+    };
+    fetch(0);
+    float* cur = xs + buf;
+    for (int64_t t0 = 0; t0 < len; t0 += Tt) {
+        cur = cur == xs ? xs + buf : xs;
+        if constexpr (VEC) cp_async_wait_all();
+        put(cur);
+        if (t0 + Tt < len) fetch(t0 + Tt);
+        __syncthreads();   // chunk visible; every read of the other buffer's last chunk done
+        if (!works) continue;
+        const int n = len - t0 < Tt ? (int)(len - t0) : Tt;
+        const float* row = cur + q * Tt * npad;
+#pragma unroll 2
+        for (int t = 0; t < n; ++t, row += npad) {
+            const float4 x0 = *reinterpret_cast<const float4*>(row + ck0), x1 = *reinterpret_cast<const float4*>(row + ck1);
+            const float4 y0 = *reinterpret_cast<const float4*>(row + cj0), y1 = *reinterpret_cast<const float4*>(row + cj1);
+            const float x[FM_TILE] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
+            const uint64_t y[FM_TILE / 2] = {pair2(y0.x, y0.y), pair2(y0.z, y0.w), pair2(y1.x, y1.y), pair2(y1.z, y1.w)};
 #pragma unroll
-                        for (int c = 0; c < 16; ++c) acc[i][c] = 0.0f;
+            for (int r = 0; r < FM_TILE; ++r) {
+                const uint64_t xr = pair2(x[r], x[r]);
 #pragma unroll
-                        for (int c = 0; c < 4; ++c) rs[i][c] = 0.0f;
-                    }
-                }
+                for (int c = 0; c < FM_TILE / 2; ++c) fma2(acc2[r][c], xr, y[c]);
             }
         }
-        __syncthreads();
+    }
+    float acc[FM_TILE][FM_TILE];
+#pragma unroll
+    for (int r = 0; r < FM_TILE; ++r)
+#pragma unroll
+        for (int c = 0; c < FM_TILE / 2; ++c) unpair2(acc2[r][c], acc[r][2 * c], acc[r][2 * c + 1]);
+    if (!works || p >= a.P) return;
+    float* G = a.blocks + (p * a.n_blocks + b) * ((int64_t)N * N + N);
+    const bool whole = kb < jb && FM_TILE * (jb + 1) <= N && N % 4 == 0;   // inside the triangle, rows 16-byte aligned
+#pragma unroll
+    for (int r = 0; r < FM_TILE; ++r) {
+        const int k = FM_TILE * kb + r;
+        if (k >= N) continue;
+        float* at = G + (int64_t)k * N + FM_TILE * jb;
+        if (whole) {
+            reinterpret_cast<float4*>(at)[0] = make_float4(acc[r][0], acc[r][1], acc[r][2], acc[r][3]);
+            reinterpret_cast<float4*>(at)[1] = make_float4(acc[r][4], acc[r][5], acc[r][6], acc[r][7]);
+        } else {
+#pragma unroll
+            for (int c = 0; c < FM_TILE; ++c) {
+                const int j = FM_TILE * jb + c;
+                if (j < N && j >= k) at[c] = acc[r][c];
+                else if (j == N) G[(int64_t)N * N + k] = acc[r][c];
+            }
+        }
     }
 }
 
@@ -254,22 +373,28 @@ __global__ void summary_kernel(const float* __restrict__ state, int32_t N, int32
 cudaError_t launch_fc_moments(const FcArgs& a, cudaStream_t s)
 {
     if (a.N > 384) return cudaErrorInvalidValue;
-    const int Npad = (a.N + 3) / 4 * 4;
-    const int nb = Npad / 4;
-    const int tasks_per_set = nb * (nb + 1) / 2;
-    const int total = tasks_per_set * FC_SETS;
-    const int per_chunk = FC_THREADS * FC_TASKS_PER_THREAD;
-    const int chunks = (total + per_chunk - 1) / per_chunk;
-    int Tt = 16384 / (FC_SETS * Npad);
-    Tt = Tt < 4 ? 4 : (Tt > 32 ? 32 : Tt);
-    const size_t smem = sizeof(float) * (size_t)FC_SETS * Tt * Npad;
-    cudaError_t e = cudaFuncSetAttribute(fc_moments_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+    const FmPlan f = fm_plan(a.N, a.P);
+    const bool vec = a.sl.sk % 4 == 0 && a.sl.st % 4 == 0 && a.sl.sg % 4 == 0 &&
+                     (reinterpret_cast<uintptr_t>(a.series) & 15) == 0;
+    auto kern = vec ? fc_moments_kernel<true> : fc_moments_kernel<false>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)f.smem);
     if (e != cudaSuccess) return e;
-    dim3 grid((a.P + FC_SETS - 1) / FC_SETS, chunks);
+    const int64_t groups = ((a.P + 3) / 4 + f.m - 1) / f.m;
     note_launch();
-    fc_moments_kernel<<<grid, FC_THREADS, smem, s>>>(a, Npad, Tt, tasks_per_set, per_chunk);
+    kern<<<dim3((unsigned)(groups * a.n_blocks), f.chunks), f.threads, f.smem, s>>>(a, f);
     return cudaGetLastError();
+}
+
+// Moment blocks of an FC without windows: one, or as many (at most 12, of at
+// least 64 samples) as give every SM four CTAs of a few sets' moments.
+int32_t fc_moment_split(int32_t N, int64_t P, int64_t Tn)
+{
+    if (N > 384) return 1;
+    const FmPlan f = fm_plan(N, P);
+    const int64_t ctas = ((P + 3) / 4 + f.m - 1) / f.m * f.chunks;
+    int64_t n = 608 / ctas;
+    n = n < 1 ? 1 : (n > FCR_MAXB ? FCR_MAXB : n);
+    return (int32_t)(n > Tn / 64 ? (Tn / 64 > 1 ? Tn / 64 : 1) : n);
 }
 
 // Shift of each (region, set): mean of up to 64 evenly spaced samples of
@@ -336,8 +461,8 @@ cudaError_t launch_fc_shift(const float* series, const SeriesLayout& sl, int32_t
 }
 
 // Per set, from the block moments: Pearson FC over all samples, chi, mean
-// off-diagonal FC and, when nw > 0, the FCD over nw windows of m blocks
-// (Lw samples each) in one pass. One CTA per set; one warp per FC row; the
+// off-diagonal FC and the FCD over nw > 0 windows of m blocks (Lw samples
+// each) in one pass. One CTA per set; one warp per FC row; the
 // window FC vectors (upper triangles) stay in shared memory. MW > 0: m == MW
 // and n_blocks <= FCR_MAXB, block values in registers with compile-time
 // indices; MW == 0: any m and n_blocks, block values re-read.
@@ -348,7 +473,6 @@ cudaError_t launch_fc_shift(const float* series, const SeriesLayout& sl, int32_t
 // column r + 1 on, along the row (coalesced).
 constexpr int RED_THREADS = 512;
 constexpr int RED_WARPS = RED_THREADS / 32;
-constexpr int FCR_MAXB = 12;
 
 // Work items of the row pass: (row r, first column of a 32-column chunk right
 // of the diagonal), row by row; their number is sum over L = 1 .. N-1 of
@@ -365,9 +489,98 @@ static __device__ __forceinline__ float warp_sum(float x)
     return x;
 }
 
+// The same without windows, any N: 32 x 32 tiles of the upper triangle, read
+// along the rows; a tile's transpose goes through shared memory, so that both
+// triangles of the FC are written along their rows (column writes measured
+// 1.62 ms on 32,768 x 68 and 2.79 ms on 4,096 x 360).
+constexpr int FIN_THREADS = 256;
+constexpr int FIN_WARPS = FIN_THREADS / 32;
+
+__global__ void __launch_bounds__(FIN_THREADS, 4)
+fc_finish_kernel(const __grid_constant__ FcArgs a)
+{
+    extern __shared__ float sm[];
+    const int N = a.N, nb = a.n_blocks;
+    const int64_t p = blockIdx.x;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int64_t stride_b = (int64_t)N * N + N;
+    const float* B = a.blocks + p * nb * stride_b;
+    const int64_t Tn = a.t_end - a.t_begin;
+    float* sS = sm;                        // [N] row sums
+    float* isd = sS + N;                   // [N] 1 / sd (0 if sd = 0)
+    float (*tr)[32][33] = reinterpret_cast<float (*)[32][33]>(isd + N);   // [2] tiles
+    __shared__ float red[3][FIN_WARPS];
+    const float invT = Tn > 0 ? 1.0f / (float)Tn : 0.0f;
+    float* fc = a.fc ? a.fc + p * N * N : nullptr;
+
+    float s_all = 0.0f, s_diag = 0.0f, s_fc = 0.0f;
+    bool zero = false;
+    for (int k = tid; k < N; k += FIN_THREADS) {
+        float g = 0.0f, sk = 0.0f;
+        for (int b = 0; b < nb; ++b) {
+            g += B[b * stride_b + (int64_t)k * N + k];
+            sk += B[b * stride_b + (int64_t)N * N + k];
+        }
+        const float v = g - sk * sk * invT;
+        sS[k] = sk;
+        isd[k] = v > 0.0f ? rsqrtf(v) : 0.0f;
+        s_all += v;
+        s_diag += v;
+        if (!(v > 0.0f)) zero = true;
+    }
+    if (zero) atomicOr(a.status + p, TVBX_SET_ZERO_VAR);
+    __syncthreads();
+    const int nt = (N + 31) / 32;
+    int parity = 0;
+    for (int ti = 0; ti < nt; ++ti)
+        for (int tj = ti; tj < nt; ++tj, parity ^= 1) {
+            const int j = 32 * tj + lane;
+            const float sj = j < N ? sS[j] : 0.0f, ij = j < N ? isd[j] : 0.0f;
+#pragma unroll
+            for (int u = 0; u < 32 / FIN_WARPS; ++u) {
+                const int rr = warp + u * FIN_WARPS, r = 32 * ti + rr;
+                if (r >= N || j >= N || j < r) continue;
+                if (j == r) {
+                    if (fc) fc[(int64_t)r * N + r] = 1.0f;
+                    tr[parity][rr][lane] = 1.0f;
+                    continue;
+                }
+                float g = 0.0f;
+                for (int b = 0; b < nb; ++b) g += B[b * stride_b + (int64_t)r * N + j];
+                const float c = g - sS[r] * sj * invT;
+                const float x = c * isd[r] * ij;
+                s_all += 2.0f * c;
+                s_fc += 2.0f * x;
+                if (fc) fc[(int64_t)r * N + j] = x;
+                tr[parity][rr][lane] = x;
+            }
+            if (!fc) continue;
+            __syncthreads();   // the tile is whole; the other buffer's readers are done with the tile before
+            const int c0 = 32 * ti + lane;
+#pragma unroll
+            for (int u = 0; u < 32 / FIN_WARPS; ++u) {
+                const int rr = warp + u * FIN_WARPS, r = 32 * tj + rr;
+                if (r < N && c0 < r) fc[(int64_t)r * N + c0] = tr[parity][lane][rr];
+            }
+        }
+    s_all = warp_sum(s_all);
+    s_diag = warp_sum(s_diag);
+    s_fc = warp_sum(s_fc);
+    if (lane == 0) { red[0][warp] = s_all; red[1][warp] = s_diag; red[2][warp] = s_fc; }
+    __syncthreads();
+    if (tid == 0) {
+        float A = 0.0f, D = 0.0f, F = 0.0f;
+        for (int w = 0; w < FIN_WARPS; ++w) { A += red[0][w]; D += red[1][w]; F += red[2][w]; }
+        const float num = A / ((float)N * (float)N), den = D / (float)N;
+        a.chi[p] = den > 0.0f ? sqrtf(fmaxf(num / den, 0.0f)) : 0.0f;
+        a.mean_fc[p] = N > 1 ? F / ((float)N * (float)(N - 1)) : 0.0f;
+    }
+}
+
 template <int MW>
 __global__ void __launch_bounds__(RED_THREADS)
-fc_reduce_kernel(const __grid_constant__ FcArgs a, int32_t m, int32_t nw, int64_t Lw, float* __restrict__ fcd)
+fc_reduce_kernel(const __grid_constant__ FcArgs a, int32_t m, int32_t nw, int64_t Lw, float* __restrict__ fcd,
+                 int32_t with_tri)
 {
     extern __shared__ float sm[];
     const int N = a.N, nb = a.n_blocks;
@@ -386,6 +599,8 @@ fc_reduce_kernel(const __grid_constant__ FcArgs a, int32_t m, int32_t nw, int64_
     float* red = V + (size_t)nw * M;        // [48] sums, [nw] inverse norms
     int* items = reinterpret_cast<int*>(red + 48 + nw);   // row-pass items
     const int n_items = fc_reduce_items(N);
+    // [M] the FC's upper triangle, written out along the rows after the row pass
+    float* tri = with_tri ? reinterpret_cast<float*>(items + n_items) : nullptr;
     const float invT = Tn > 0 ? 1.0f / (float)Tn : 0.0f;
     const float invL = Lw > 0 ? 1.0f / (float)Lw : 0.0f;
 
@@ -420,7 +635,7 @@ fc_reduce_kernel(const __grid_constant__ FcArgs a, int32_t m, int32_t nw, int64_
         s_all += cdg[k];
         s_diag += cdg[k];
         if (!(isd[k] > 0.0f)) zero = true;
-        if (fc) fc[(int64_t)k * N + k] = 1.0f;
+        if (fc && !tri) fc[(int64_t)k * N + k] = 1.0f;
     }
     // the row pass: items (row, 32-column chunk) dealt to the warps in turn,
     // so every warp gets the same number of chunks up to one
@@ -448,7 +663,9 @@ fc_reduce_kernel(const __grid_constant__ FcArgs a, int32_t m, int32_t nw, int64_
             const float f = c * ir * isd[jj];
             s_all += 2.0f * c;
             s_fc += 2.0f * f;
-            if (fc) {
+            if (tri) {
+                tri[e0 + jj] = f;
+            } else if (fc) {
                 fc[(int64_t)r * N + jj] = f;
                 fc[(int64_t)jj * N + r] = f;
             }
@@ -487,7 +704,12 @@ fc_reduce_kernel(const __grid_constant__ FcArgs a, int32_t m, int32_t nw, int64_
         a.chi[p] = den > 0.0f ? sqrtf(fmaxf(num / den, 0.0f)) : 0.0f;
         a.mean_fc[p] = N > 1 ? F / ((float)N * (float)(N - 1)) : 0.0f;
     }
-    if (nw == 0) return;
+    if (fc && tri)
+        for (int r = warp; r < N; r += RED_WARPS)
+            for (int c = lane; c < N; c += 32) {
+                const int lo = c < r ? c : r, hi = c < r ? r : c;
+                fc[(int64_t)r * N + c] = lo == hi ? 1.0f : tri[lo * N - lo * (lo + 1) / 2 - lo - 1 + hi];
+            }
 
     // FCD: centre and normalise each window vector (a warp per window), then
     // the products of window u with up to four windows v > u per warp item
@@ -553,16 +775,21 @@ template <int MW>
 static cudaError_t launch_reduce_mw(const FcArgs& a, int32_t m, int32_t nw, int64_t Lw, float* fcd, size_t smem,
                                     cudaStream_t s)
 {
+    // the triangle buffer where it fits beside the window vectors
+    const size_t tri = sizeof(float) * (size_t)a.N * (a.N - 1) / 2;
+    const bool with_tri = smem + tri <= 200 * 1024;
+    if (with_tri) smem += tri;
     cudaError_t e = cudaFuncSetAttribute(fc_reduce_kernel<MW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     note_launch();
-    fc_reduce_kernel<MW><<<a.P, RED_THREADS, smem, s>>>(a, m, nw, Lw, fcd);
+    fc_reduce_kernel<MW><<<a.P, RED_THREADS, smem, s>>>(a, m, nw, Lw, fcd, with_tri ? 1 : 0);
     return cudaGetLastError();
 }
 
 cudaError_t launch_fc_reduce(const FcArgs& a, int32_t m, int32_t nw, int64_t Lw, float* vec_scratch, float* fcd,
                              cudaStream_t s)
 {
+    if (nw == 0) return launch_fc_finalize(a, s);
     const size_t smem = fc_reduce_smem(a.N, a.n_blocks, nw);
     if (smem > 200 * 1024) {
         // window vectors too large for shared memory: the FC pass without
@@ -572,8 +799,7 @@ cudaError_t launch_fc_reduce(const FcArgs& a, int32_t m, int32_t nw, int64_t Lw,
         return launch_fcd(a.blocks, a.P, a.N, a.n_blocks, m, nw, Lw, vec_scratch, fcd, s);
     }
     if (a.n_blocks <= FCR_MAXB) {
-        const int mw = nw == 0 ? 1 : m;   // without windows only the block sum is used
-        switch (mw) {
+        switch (m) {
         case 1: return launch_reduce_mw<1>(a, m, nw, Lw, fcd, smem, s);
         case 2: return launch_reduce_mw<2>(a, m, nw, Lw, fcd, smem, s);
         case 3: return launch_reduce_mw<3>(a, m, nw, Lw, fcd, smem, s);
@@ -586,9 +812,12 @@ cudaError_t launch_fc_reduce(const FcArgs& a, int32_t m, int32_t nw, int64_t Lw,
 
 cudaError_t launch_fc_finalize(const FcArgs& a, cudaStream_t s)
 {
-    const size_t smem = fc_reduce_smem(a.N, a.n_blocks, 0);
-    return a.n_blocks <= FCR_MAXB ? launch_reduce_mw<1>(a, 0, 0, 0, nullptr, smem, s)
-                                  : launch_reduce_mw<0>(a, 0, 0, 0, nullptr, smem, s);
+    const size_t smem = sizeof(float) * (2 * (size_t)a.N + 2 * 32 * 33);
+    cudaError_t e = cudaFuncSetAttribute(fc_finish_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    note_launch();
+    fc_finish_kernel<<<a.P, FIN_THREADS, smem, s>>>(a);
+    return cudaGetLastError();
 }
 
 size_t fc_reduce_needs_vec_scratch(int N, int nb, int nw) { return fc_reduce_smem(N, nb, nw) > 200 * 1024; }

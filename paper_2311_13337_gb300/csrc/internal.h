@@ -215,6 +215,7 @@ struct FcArgs {
 };
 // Block moments (SIMT, FP32 CUDA-core FMAs).
 cudaError_t launch_fc_moments(const FcArgs& a, cudaStream_t s);
+int32_t fc_moment_split(int32_t N, int64_t P, int64_t Tn);   // moment blocks of an FP32 FC without windows
 // From the block moments: Pearson FC, chi, mean FC and (nw > 0) the FCD over
 // nw windows of m blocks of Lw samples, in one kernel when its shared memory
 // fits; vec_scratch ([P][nw][N(N-1)/2]) is used only when it does not.
