@@ -14,16 +14,16 @@
 //    UP / DOWN runs against that mean (rounded to FP32); the forward DFT of
 //    the mean-removed row (in place in one shared-memory buffer: the row is
 //    stored digit-reversed and transformed by decimation-in-time stages of
-//    radix 2, 3, 4, 5; twiddles from a host FP64 table; for even T' as a
-//    complex transform of length T'/2 of the sample pairs, untangled into the
-//    spectrum of the real row); the periodogram on
-//    the PSD band; the analytic signal (one-sided spectrum doubled) by the
-//    inverse DFT (decimation in frequency, in place, read back through the
-//    digit reversal), written to scratch;
-//  * an_pli_kernel, one CTA per set: time tiles of the N analytic signals in
+//    radix 2, 3, 4, 5; twiddles from a host FP64 table); the periodogram on
+//    the PSD band; the analytic signal (real part: the row; imaginary part: the
+//    inverse transform of -i times the positive-frequency spectrum, decimation
+//    in frequency, in place, read back through the digit reversal), written to
+//    scratch; for even T' both transforms are complex ones of length T'/2 of
+//    the sample pairs;
+//  * an_pli_kernel, one CTA per (time slice, set): time tiles of the N analytic signals in
 //    shared memory; a thread owns a 4 x 4 block of region pairs and counts
-//    sign(Im(z_k conj(z_j))) by comparing the two rounded products, so
-//    identical signals give exactly 0;
+//    sign(Im(z_k conj(z_j))) from the differences of the two rounded products,
+//    so identical signals give exactly 0;
 //  * an_finalize_kernel, one CTA per set: region-mean PSD, its peak on the
 //    band, the least-squares fit of log10 PSD on log10 f (FP64), the pooled
 //    UP / DOWN durations.
@@ -37,6 +37,7 @@
 #include <vector>
 
 #include "internal.h"
+#include "ptx_async.cuh"
 #include "tvbx.h"
 
 namespace tvbx {
@@ -45,11 +46,11 @@ namespace {
 constexpr int AN_MAX_T = 8192;
 constexpr int AN_MAX_STAGES = 16;
 constexpr int AN_THREADS = 256;
-// samples per time tile of the PLI kernel: TT (64, or 32 when the tiles of
-// many regions would not fit); padded row stride of a tile plane TT + 2 floats
+// samples per time tile of the PLI kernel: TT (64; 32 or 8 when the two buffers of
+// many regions would not fit); padded row stride of a tile plane TT + 4 floats
 constexpr int PLI_TT_MAX = 64;
-constexpr int PLI_TT_MIN = 32;
-constexpr int PLI_THREADS = 256;
+constexpr int PLI_TT_MIN = 8;
+constexpr int PLI_THREADS = 160;   // 153 blocks of pairs at 68 regions
 
 struct FftPlan {
     int n;
@@ -58,6 +59,10 @@ struct FftPlan {
     // stage s (radix[s], DIT or DIF) has L1 = radix[0] ... radix[s-1]:
     // magic[s] = ceil(2^32 / L1) (0 for L1 = 1), so idx / L1 = umulhi(idx, magic)
     uint32_t magic[AN_MAX_STAGES];
+    // twiddles of stage s in the plan's table: w_L^{j q} (L = L1 radix[s]) at
+    // tw_off[s] + (q - 1) L1 + j, so that neighbouring butterflies read
+    // neighbouring entries
+    int tw_off[AN_MAX_STAGES];
 };
 
 __device__ __forceinline__ float2 cmul(float2 a, float2 b)
@@ -118,12 +123,12 @@ __device__ __forceinline__ void butterfly(const float2 (&u)[R], float2 (&v)[R], 
 
 // In-place decimation-in-time stage of radix R on a (length n, input in
 // digit-reversed order): butterfly j of a block of span L = L1 R combines
-// a[blk L + j + q L1], twiddled by w_L^{j q} before the R-point DFT.
+// a[blk L + j + q L1], twiddled by w_L^{j q} before the R-point DFT. tw: the
+// stage's twiddles.
 template <int R>
-__device__ void dit_stage(float2* a, int n, int L1, uint32_t magic, const float2* __restrict__ tw, bool inv,
-                          int tws)
+__device__ void dit_stage(float2* a, int n, int L1, uint32_t magic, const float2* __restrict__ tw, bool inv)
 {
-    const int L = L1 * R, nl = n / L, m = n / R;
+    const int L = L1 * R, m = n / R;
     const float sg = inv ? 1.0f : -1.0f;
     for (int idx = threadIdx.x; idx < m; idx += blockDim.x) {
         const int blk = magic ? (int)__umulhi((uint32_t)idx, magic) : idx;   // idx / L1
@@ -133,7 +138,7 @@ __device__ void dit_stage(float2* a, int n, int L1, uint32_t magic, const float2
 #pragma unroll
         for (int q = 0; q < R; ++q) {
             const float2 y = p[q * L1];
-            u[q] = (q == 0 || j == 0) ? y : cmul(y, twiddle(tw, tws * nl * j * q, inv));
+            u[q] = (q == 0 || j == 0) ? y : cmul(y, twiddle(tw, (q - 1) * L1 + j, inv));
         }
         butterfly<R>(u, v, sg);
 #pragma unroll
@@ -147,7 +152,7 @@ __device__ void dit_stage(float2* a, int n, int L1, uint32_t magic, const float2
 template <int R>
 __device__ void dif_stage(float2* a, int n, int L1, uint32_t magic, const float2* __restrict__ tw, bool inv)
 {
-    const int L = L1 * R, nl = n / L, m = n / R;
+    const int L = L1 * R, m = n / R;
     const float sg = inv ? 1.0f : -1.0f;
     for (int idx = threadIdx.x; idx < m; idx += blockDim.x) {
         const int blk = magic ? (int)__umulhi((uint32_t)idx, magic) : idx;   // idx / L1
@@ -158,24 +163,25 @@ __device__ void dif_stage(float2* a, int n, int L1, uint32_t magic, const float2
         for (int q = 0; q < R; ++q) u[q] = p[q * L1];
         butterfly<R>(u, v, sg);
 #pragma unroll
-        for (int k = 0; k < R; ++k) p[k * L1] = (k == 0 || j == 0) ? v[k] : cmul(v[k], twiddle(tw, nl * j * k, inv));
+        for (int k = 0; k < R; ++k)
+            p[k * L1] = (k == 0 || j == 0) ? v[k] : cmul(v[k], twiddle(tw, (k - 1) * L1 + j, inv));
     }
 }
 
 // Forward transform in place: a holds the input in digit-reversed order
-// (a[perm[t]] = x[t]) and ends in natural order. tw holds the twiddles of a
-// transform tws times longer than the plan's (every tws-th one is used).
-__device__ void fft_dit(float2* a, const FftPlan& plan, const float2* __restrict__ tw, bool inv, int tws = 1)
+// (a[perm[t]] = x[t]) and ends in natural order. tw: the plan's table.
+__device__ void fft_dit(float2* a, const FftPlan& plan, const float2* __restrict__ tw, bool inv)
 {
     int L1 = 1;
     for (int s = 0; s < plan.n_stages; ++s) {
         const int r = plan.radix[s];
         const uint32_t mg = plan.magic[s];
+        const float2* ts = tw + plan.tw_off[s];
         switch (r) {
-        case 2: dit_stage<2>(a, plan.n, L1, mg, tw, inv, tws); break;
-        case 3: dit_stage<3>(a, plan.n, L1, mg, tw, inv, tws); break;
-        case 4: dit_stage<4>(a, plan.n, L1, mg, tw, inv, tws); break;
-        default: dit_stage<5>(a, plan.n, L1, mg, tw, inv, tws); break;
+        case 2: dit_stage<2>(a, plan.n, L1, mg, ts, inv); break;
+        case 3: dit_stage<3>(a, plan.n, L1, mg, ts, inv); break;
+        case 4: dit_stage<4>(a, plan.n, L1, mg, ts, inv); break;
+        default: dit_stage<5>(a, plan.n, L1, mg, ts, inv); break;
         }
         __syncthreads();
         L1 *= r;
@@ -191,11 +197,12 @@ __device__ void fft_dif(float2* a, const FftPlan& plan, const float2* __restrict
         const int r = plan.radix[s];
         const int L1 = L / r;
         const uint32_t mg = plan.magic[s];
+        const float2* ts = tw + plan.tw_off[s];
         switch (r) {
-        case 2: dif_stage<2>(a, plan.n, L1, mg, tw, inv); break;
-        case 3: dif_stage<3>(a, plan.n, L1, mg, tw, inv); break;
-        case 4: dif_stage<4>(a, plan.n, L1, mg, tw, inv); break;
-        default: dif_stage<5>(a, plan.n, L1, mg, tw, inv); break;
+        case 2: dif_stage<2>(a, plan.n, L1, mg, ts, inv); break;
+        case 3: dif_stage<3>(a, plan.n, L1, mg, ts, inv); break;
+        case 4: dif_stage<4>(a, plan.n, L1, mg, ts, inv); break;
+        default: dif_stage<5>(a, plan.n, L1, mg, ts, inv); break;
         }
         __syncthreads();
         L = L1;
@@ -222,137 +229,147 @@ __device__ __forceinline__ T block_sum(T v, T* red)
 //
 // HALF (n even): the real row goes through a complex transform of length
 // M = n / 2, z_m = x_2m + i x_2m+1 stored digit-reversed for the half plan
-// (a[perm_h[m]] = z_m); with E, O the transforms of the even and odd samples,
+// (a[perm[m]] = z_m); with E, O the transforms of the even and odd samples,
 // E_k = (Z_k + conj Z_{M-k}) / 2, O_k = -i (Z_k - conj Z_{M-k}) / 2, and
 // X_k = E_k + w^k O_k, X_{M-k} = conj(E_k - w^k O_k), X_M = E_0 - O_0
-// (w = exp(-2 pi i / n)); the spectrum is untangled in place, pair by pair.
+// (w = exp(-2 pi i / n)). The analytic signal's real part is the mean-removed
+// row itself, so only its imaginary part y, a real row with the spectrum
+// -i X_k (0 < k < M; 0 at k = 0, M), is transformed back, again at half the
+// length: with e = E_k and t = w^k O_k, the packed spectrum of y is
+// -i t + e w^-k at k and i conj(t) - conj(e) w^k at M - k. Both untanglings
+// are one pass over the pairs (k, M - k), in place.
+//
+// z_out: per (set, region) the real and then the imaginary part of the
+// analytic signal, ns floats each (n rounded up to 4, zeros at the end).
+// UP / DOWN: with the transitions t_1 < ... < t_m (samples whose state differs
+// from the one before), the complete runs are [t_i, t_{i+1}). Their number in
+// a state is the number of transitions into it, without the last one, and
+// their samples are all samples of that state in [t_1, t_m); so sums, a
+// minimum and a maximum over the samples give them, with no run followed.
+//
+// Bound by the L1 / shared-memory data path (the FFT passes and their
+// twiddles): full-length inverse transforms, twiddles gathered from one
+// natural-order table and a pass that followed the runs measured 6.0 ms on
+// 1,024 x 68 x 5,000.
 template <bool HALF>
 __global__ void __launch_bounds__(AN_THREADS)
 an_series_kernel(const float* __restrict__ series, int N, int64_t T, FftPlan plan, FftPlan plan_h,
-                 const float2* __restrict__ tw, const int* __restrict__ perm, const int* __restrict__ perm_h,
+                 const float2* __restrict__ tw, const float2* __restrict__ tws, const int* __restrict__ perm,
                  int band_lo, int band_n, float psd_scale, int64_t p0, float* __restrict__ psd_out,
-                 int* __restrict__ ud_out, float2* __restrict__ z_out)
+                 int* __restrict__ ud_out, float* __restrict__ z_out, int ns)
 {
     extern __shared__ float2 an_smem[];
     __shared__ double red_d[AN_THREADS / 32];
-    __shared__ int chunk_last[AN_THREADS];
-    __shared__ int warp_last[AN_THREADS / 32];
-    __shared__ int red_i[4][AN_THREADS / 32];
+    __shared__ int red_i[5][AN_THREADS / 32];
     const int n = plan.n, M = n / 2;
     float2* a = an_smem;
     const int b = blockIdx.x / N, k = blockIdx.x - b * N;
     const float* row = series + ((p0 + b) * (int64_t)N + k) * T + (T - n);
-    double s = 0.0;
+    // mean: a thread's samples in two floats (error-free additions), the threads in FP64
+    float hi = 0.0f, lo = 0.0f;
+    for (int t = threadIdx.x; t < n; t += blockDim.x) {
+        const float x = row[t], sum = __fadd_rn(hi, x), bb = __fsub_rn(sum, hi);
+        lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(sum, bb)), __fsub_rn(x, bb)));
+        hi = sum;
+    }
+    double total = block_sum((double)hi + (double)lo, red_d);
+    if (!isfinite(total)) {   // infinities, or a sum beyond FP32: in FP64 throughout
+        double s = 0.0;
+        for (int t = threadIdx.x; t < n; t += blockDim.x) s += (double)row[t];
+        total = block_sum(s, red_d);
+    }
+    const float theta = (float)(total / (double)n);
+    // the mean-removed row in digit-reversed order, and the UP / DOWN counts
+    int ups = 0, into_up = 0, into_dn = 0, first = n, last = -1;
+    auto count = [&](int t, bool up, float before) {
+        ups += up;
+        if (t == 0 || up == (before > theta)) return;
+        into_up += up;
+        into_dn += !up;
+        first = min(first, t);
+        last = max(last, t);
+    };
     if constexpr (HALF) {
         for (int m = threadIdx.x; m < M; m += blockDim.x) {
             const float x0 = row[2 * m], x1 = row[2 * m + 1];
-            a[__ldg(perm_h + m)] = make_float2(x0, x1);
-            s += (double)x0 + (double)x1;
+            a[__ldg(perm + m)] = make_float2(x0 - theta, x1 - theta);
+            count(2 * m, x0 > theta, m > 0 ? row[2 * m - 1] : 0.0f);
+            count(2 * m + 1, x1 > theta, x0);
         }
     } else {
         for (int t = threadIdx.x; t < n; t += blockDim.x) {
             const float x = row[t];
-            a[__ldg(perm + t)] = make_float2(x, 0.0f);
-            s += (double)x;
+            a[__ldg(perm + t)] = make_float2(x - theta, 0.0f);
+            count(t, x > theta, t > 0 ? row[t - 1] : 0.0f);
         }
     }
-    const float theta = (float)(block_sum(s, red_d) / (double)n);
-    // sample t of the raw row
-    auto raw = [&](int t) -> float {
-        if constexpr (HALF) {
-            const float2 v = a[__ldg(perm_h + (t >> 1))];
-            return (t & 1) ? v.y : v.x;
-        } else {
-            return a[__ldg(perm + t)].x;
-        }
-    };
-
-    // UP / DOWN: runs between consecutive transitions (a transition at t >= 1
-    // where the state differs from t - 1); thread c scans [c0, c1)
-    const int per = (n + blockDim.x - 1) / blockDim.x;
-    const int c0 = threadIdx.x * per, c1 = min(n, c0 + per);
-    int first = -1, last = -1, nu = 0, su = 0, nd = 0, sd = 0;
-    const int tb = max(c0, 1);
-    bool was = tb < c1 ? raw(tb - 1) > theta : false;   // the state at tb - 1
-    for (int t = tb; t < c1; ++t) {
-        const bool up = raw(t) > theta;
-        if (up != was) {
-            if (last >= 0) {   // complete run [last, t) in state `was`
-                if (was) { ++nu; su += t - last; } else { ++nd; sd += t - last; }
-            }
-            if (first < 0) first = t;
-            last = t;
-        }
-        was = up;
-    }
-    // the run that ends at this chunk's first transition starts at the last
-    // transition of the nearest preceding chunk that has one: an exclusive
-    // max-scan over the chunks finds it
-    chunk_last[threadIdx.x] = last;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int pv = first >= 0 ? (int)threadIdx.x : -1;
-    for (int o = 1; o < 32; o <<= 1) {
-        const int v = __shfl_up_sync(0xffffffffu, pv, o);
-        if (lane >= o) pv = max(pv, v);
+    ups = __reduce_add_sync(0xffffffffu, ups);
+    into_up = __reduce_add_sync(0xffffffffu, into_up);
+    into_dn = __reduce_add_sync(0xffffffffu, into_dn);
+    first = __reduce_min_sync(0xffffffffu, first);
+    last = __reduce_max_sync(0xffffffffu, last);
+    if (lane == 0) {
+        red_i[0][warp] = ups;
+        red_i[1][warp] = into_up;
+        red_i[2][warp] = into_dn;
+        red_i[3][warp] = first;
+        red_i[4][warp] = last;
     }
-    if (lane == 31) warp_last[warp] = pv;
-    __syncthreads();
-    int prev_chunk = __shfl_up_sync(0xffffffffu, pv, 1);
-    if (lane == 0) prev_chunk = -1;
-    for (int w = 0; w < warp; ++w) prev_chunk = max(prev_chunk, warp_last[w]);
-    if (first >= 0 && prev_chunk >= 0) {
-        const int prev = chunk_last[prev_chunk];
-        if (raw(prev) > theta) { ++nu; su += first - prev; } else { ++nd; sd += first - prev; }
-    }
-    // the four counts summed over the CTA in one pass (thread 0 writes them)
-    for (int o = 16; o > 0; o >>= 1) {
-        nu += __shfl_xor_sync(0xffffffffu, nu, o);
-        su += __shfl_xor_sync(0xffffffffu, su, o);
-        nd += __shfl_xor_sync(0xffffffffu, nd, o);
-        sd += __shfl_xor_sync(0xffffffffu, sd, o);
-    }
-    if (lane == 0) { red_i[0][warp] = nu; red_i[1][warp] = su; red_i[2][warp] = nd; red_i[3][warp] = sd; }
-    __syncthreads();   // also: the raw row was read above
+    __syncthreads();   // also: the row is whole
     if (threadIdx.x == 0) {
-        int tot[4] = {0, 0, 0, 0};
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w)
-            for (int c = 0; c < 4; ++c) tot[c] += red_i[c][w];
+        for (int w = 1; w < AN_THREADS / 32; ++w) {
+            ups += red_i[0][w];
+            into_up += red_i[1][w];
+            into_dn += red_i[2][w];
+            first = min(first, red_i[3][w]);
+            last = max(last, red_i[4][w]);
+        }
+        int nu = 0, su = 0, nd = 0, sd = 0;
+        if (last > first) {   // at least two transitions
+            const bool up_first = row[first] > theta, up_last = row[last] > theta;
+            nu = into_up - up_last;
+            nd = into_dn - !up_last;
+            su = ups - (up_first ? 0 : first) - (up_last ? n - last : 0);
+            sd = last - first - su;
+        }
         int* u = ud_out + ((int64_t)b * N + k) * 4;
-        u[0] = tot[0]; u[1] = tot[1]; u[2] = tot[2]; u[3] = tot[3];
+        u[0] = nu; u[1] = su; u[2] = nd; u[3] = sd;
     }
     float* pr = psd_out + ((int64_t)b * N + k) * band_n;
     if constexpr (HALF) {
-        for (int i = threadIdx.x; i < M; i += blockDim.x) a[i] = make_float2(a[i].x - theta, a[i].y - theta);
-        __syncthreads();
-        fft_dit(a, plan_h, tw, false, 2);
-        // untangle pairs (i, M - i); periodogram of the band bins; analytic
-        // weights h_0 = h_M = 1, h_i = 2 for 0 < i < M, 0 above M
+        fft_dit(a, plan_h, tws, false);
         for (int i = threadIdx.x; i <= M / 2; i += blockDim.x) {
             if (i == 0) {
-                const float2 z0 = a[0];
-                a[0] = make_float2(z0.x + z0.y, 0.0f);
-                a[M] = make_float2(z0.x - z0.y, 0.0f);
+                a[0] = make_float2(0.0f, 0.0f);
                 continue;
             }
-            const float2 zk = a[i], zm = a[M - i];
+            const float2 zk = a[i], zm = a[M - i], w = __ldg(tw + i);
             const float2 e = make_float2(0.5f * (zk.x + zm.x), 0.5f * (zk.y - zm.y));   // (Z_i + conj Z_{M-i}) / 2
             const float2 o = make_float2(0.5f * (zk.y + zm.y), -0.5f * (zk.x - zm.x));  // -i (Z_i - conj Z_{M-i}) / 2
-            const float2 t = cmul(__ldg(tw + i), o);
-            const float2 xk = cadd(e, t);
-            const float2 xm = make_float2(e.x - t.x, t.y - e.y);                         // conj(e - t)
+            const float2 t = cmul(w, o);
+            const float2 xk = cadd(e, t), xm = csub(e, t);                               // X_i, conj X_{M-i}
             if (i >= band_lo && i < band_lo + band_n) pr[i - band_lo] = psd_scale * fmaf(xk.x, xk.x, xk.y * xk.y);
             if (M - i != i && M - i >= band_lo && M - i < band_lo + band_n)
                 pr[M - i - band_lo] = psd_scale * fmaf(xm.x, xm.x, xm.y * xm.y);
-            a[i] = make_float2(2.0f * xk.x, 2.0f * xk.y);
-            a[M - i] = make_float2(2.0f * xm.x, 2.0f * xm.y);
+            const float2 c = cmul(e, make_float2(w.x, -w.y));                            // e w^-i
+            a[i] = make_float2(c.x + t.y, c.y - t.x);
+            if (M - i != i) a[M - i] = make_float2(t.y - c.x, t.x + c.y);                // i conj(t) - conj(c)
         }
-        for (int i = M + 1 + threadIdx.x; i < n; i += blockDim.x) a[i] = make_float2(0.0f, 0.0f);
         __syncthreads();
+        fft_dif(a, plan_h, tws, true);
+        const float inv_m = 1.0f / (float)M;
+        float* xr = z_out + ((int64_t)b * N + k) * 2 * ns;
+        float2* yr = reinterpret_cast<float2*>(xr + ns);
+        for (int m = threadIdx.x; m < M; m += blockDim.x) {
+            const float2 v = a[__ldg(perm + m)];
+            yr[m] = make_float2(v.x * inv_m, v.y * inv_m);
+        }
+        for (int t = threadIdx.x; t < n; t += blockDim.x) xr[t] = row[t] - theta;
+        for (int t = n + threadIdx.x; t < ns; t += blockDim.x) xr[t] = xr[ns + t] = 0.0f;
+        return;
     } else {
-        // mean-removed row
-        for (int t = threadIdx.x; t < n; t += blockDim.x) a[t].x -= theta;
-        __syncthreads();
-        fft_dit(a, plan, tw, false);
+        fft_dit(a, plan, tws, false);
         for (int i = threadIdx.x; i < band_n; i += blockDim.x) {
             const float2 v = a[band_lo + i];
             pr[i] = psd_scale * fmaf(v.x, v.x, v.y * v.y);
@@ -368,55 +385,78 @@ an_series_kernel(const float* __restrict__ series, int N, int64_t T, FftPlan pla
         }
         __syncthreads();
     }
-    fft_dif(a, plan, tw, true);
+    fft_dif(a, plan, tws, true);
     const float inv_n = 1.0f / (float)n;
-    float2* zr = z_out + ((int64_t)b * N + k) * n;
-    for (int t = threadIdx.x; t < n; t += blockDim.x) {
-        const float2 v = a[__ldg(perm + t)];
-        zr[t] = make_float2(v.x * inv_n, v.y * inv_n);
+    float* xr = z_out + ((int64_t)b * N + k) * 2 * ns;
+    for (int t = threadIdx.x; t < ns; t += blockDim.x) {
+        const float2 v = t < n ? a[__ldg(perm + t)] : make_float2(0.0f, 0.0f);
+        xr[t] = v.x * inv_n;
+        xr[ns + t] = v.y * inv_n;
     }
 }
 
+// Packed products with a zero addend: a zero product is +0, never -0, so the
+// differences below are +0 for equal products whatever their signs.
 __device__ __forceinline__ uint64_t mul_f32x2(uint64_t a, uint64_t b)
 {
     uint64_t d;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(0ull));
     return d;
 }
-// sign(p - q) summed over both lanes, by comparison: the packed products are
-// not subtracted, because a packed subtraction of two packed products may be
+// c - a b in each lane. With b = 1 it is the rounded difference of two already
+// rounded products; a packed subtraction of two packed products may be
 // contracted into a fused multiply-add (observed), which leaves the rounding
-// error of one product instead of an exact 0 for identical signals. For
-// distinct finite p and q, p - q is never 0, so the comparison is sign(p - q).
-__device__ __forceinline__ int sign_diff2(uint64_t p, uint64_t q)
+// error of one product instead of an exact 0 for identical signals.
+__device__ __forceinline__ uint64_t diff_f32x2(uint64_t c, uint64_t a)
 {
-    const float p0 = __uint_as_float((uint32_t)p), p1 = __uint_as_float((uint32_t)(p >> 32));
-    const float q0 = __uint_as_float((uint32_t)q), q1 = __uint_as_float((uint32_t)(q >> 32));
-    return (p0 > q0) - (p0 < q0) + (p1 > q1) - (p1 < q1);
+    uint64_t d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(0xbf800000bf800000ull), "l"(c));
+    return d;
+}
+// sign bits of both lanes shifted into w
+__device__ __forceinline__ void take_signs(uint32_t& w, uint64_t d)
+{
+    w = __funnelshift_l((uint32_t)d, w, 1);
+    w = __funnelshift_l((uint32_t)(d >> 32), w, 1);
 }
 
-// One CTA per set: mean over k < j of |mean_t sign(Im(z_k conj(z_j)))|.
-// The tile holds the real and imaginary parts in separate planes, time
-// fastest, so one 8-byte load gives two consecutive samples and the packed
-// two-lane FP32 products handle two samples of a pair per instruction (each
-// lane rounds like the scalar product).
+// One CTA per (time slice, set): cnt[k][j] += sum_t sign(Im(z_k conj(z_j))) for
+// k < j over the slice (slices of a set balance the CTAs over the SMs: one CTA
+// per set left a third of the last wave). Time tiles of the planes of real and imaginary parts come by cp.async into
+// one of two buffers while the other is used. A thread owns a 4 x 4 block of
+// region pairs: per pair and two samples two packed products p, q and the
+// packed differences p - q and q - p, whose sign bits are shifted into two
+// words (a zero has neither) and counted every 32 samples. Bound by the FMA
+// and ALU pipes, about 4 issue slots per pair and sample (comparisons and
+// adds with predicates took 17: 4.98 ms per 1,024 x 68 x 5,000 in all).
 template <int PLI_TT>
-__global__ void __launch_bounds__(PLI_THREADS)
-an_pli_kernel(const float2* __restrict__ z_all, int N, int n, float* __restrict__ pli_out)
+__global__ void __maxnreg__(128)   // 16 warps per SM: three CTAs of five
+an_pli_kernel(const float* __restrict__ z_all, int N, int ns, int slice, int slices, int* __restrict__ cnt_all)
 {
-    constexpr int PLI_TS = PLI_TT + 2;
-    // planes [2][(r mod 4) * NB + r / 4][PLI_TS]: the rows a half-warp reads
-    // together (4 apart in r) are adjacent, and the stride (2 mod 32 words)
-    // puts their 8-byte pieces in distinct banks
-    extern __shared__ float tile[];
-    __shared__ float red[PLI_THREADS / 32];
-    const int b = blockIdx.x;
-    const float2* z = z_all + (int64_t)b * N * n;
+    constexpr int PLI_TS = PLI_TT + 4;
+    // buffers [2][plane][(r mod 4) * NB + r / 4][PLI_TS]: the rows the lanes of a
+    // quarter-warp read together (4 apart in r) are adjacent, and the stride
+    // (4 mod 32 words) puts their 16-byte pieces in distinct banks
+    extern __shared__ __align__(16) float tile[];
+    const int b = blockIdx.x / slices;
+    const int t_lo = (blockIdx.x - b * slices) * slice, t_hi = min(ns, t_lo + slice);   // multiples of 4
+    const float* z = z_all + (int64_t)b * N * 2 * ns;
     const int NB = (N + 3) / 4, NR = NB * 4;
-    float* TX = tile;
-    float* TY = tile + NR * PLI_TS;
+    const int plane = NR * PLI_TS, buf = 2 * plane;
     const int nbp = NB * (NB + 1) / 2;
-    float acc = 0.0f;
+    for (int r = N; r < NR; ++r)   // padded rows stay 0
+        for (int i = threadIdx.x; i < 4 * PLI_TS; i += blockDim.x)
+            tile[i / PLI_TS * plane + ((r & 3) * NB + (r >> 2)) * PLI_TS + i % PLI_TS] = 0.0f;
+    auto fetch = [&](int t0, float* dst) {
+        constexpr int C = PLI_TT / 4;   // 16-byte pieces per row
+        for (int i = threadIdx.x; i < 2 * N * C; i += blockDim.x) {
+            const int rp = i / C, c = i - rp * C, r = rp >> 1, pl = rp & 1;
+            if (t0 + 4 * c < t_hi)
+                cp_async16(dst + pl * plane + ((r & 3) * NB + (r >> 2)) * PLI_TS + 4 * c,
+                           z + (int64_t)rp * ns + t0 + 4 * c);
+        }
+        cp_async_commit();
+    };
     for (int base = 0; base < nbp; base += blockDim.x) {
         const int bp = base + threadIdx.x;
         int bk = 0, bj = 0;
@@ -426,41 +466,61 @@ an_pli_kernel(const float2* __restrict__ z_all, int N, int n, float* __restrict_
             bj = bk + rem;
         }
         int cnt[4][4];
+        uint32_t wp[4][4], wn[4][4];
 #pragma unroll
         for (int u = 0; u < 4; ++u)
 #pragma unroll
-            for (int v = 0; v < 4; ++v) cnt[u][v] = 0;
-        for (int t0 = 0; t0 < n; t0 += PLI_TT) {
-            const int tl = min(PLI_TT, n - t0);
-            __syncthreads();
-            for (int i = threadIdx.x; i < NR * PLI_TT; i += blockDim.x) {
-                const int r = i / PLI_TT, t = i - r * PLI_TT;
-                const float2 v = (r < N && t < tl) ? z[(int64_t)r * n + t0 + t] : make_float2(0.0f, 0.0f);
-                const int o = ((r & 3) * NB + (r >> 2)) * PLI_TS + t;
-                TX[o] = v.x;
-                TY[o] = v.y;
-            }
-            __syncthreads();
+            for (int v = 0; v < 4; ++v) cnt[u][v] = 0, wp[u][v] = wn[u][v] = 0u;
+        __syncthreads();   // the buffers are free
+        fetch(t_lo, tile);
+        float* cur = tile;
+        for (int t0 = t_lo; t0 < t_hi; t0 += PLI_TT) {
+            cp_async_wait_all();
+            __syncthreads();   // this tile is whole, the other buffer's last reads are done
+            float* next = cur == tile ? tile + buf : tile;
+            if (t0 + PLI_TT < t_hi) fetch(t0 + PLI_TT, next);
+            const int tl = min(PLI_TT, t_hi - t0);
             if (bp < nbp) {
-                // padded samples are 0 and add sign(0) = 0
-                for (int t = 0; t < PLI_TT; t += 2) {
-                    uint64_t xk[4], yk[4], xj[4], yj[4];
+                const float* xk0 = cur + bk * PLI_TS;
+                const float* xj0 = cur + bj * PLI_TS;
+                int since = 0;
+                for (int t = 0; t < tl; t += 4) {
+                    ulonglong2 xk[4], yk[4];
 #pragma unroll
                     for (int u = 0; u < 4; ++u) {
-                        xk[u] = *reinterpret_cast<const uint64_t*>(TX + (u * NB + bk) * PLI_TS + t);
-                        yk[u] = *reinterpret_cast<const uint64_t*>(TY + (u * NB + bk) * PLI_TS + t);
-                        xj[u] = *reinterpret_cast<const uint64_t*>(TX + (u * NB + bj) * PLI_TS + t);
-                        yj[u] = *reinterpret_cast<const uint64_t*>(TY + (u * NB + bj) * PLI_TS + t);
+                        xk[u] = *reinterpret_cast<const ulonglong2*>(xk0 + u * NB * PLI_TS + t);
+                        yk[u] = *reinterpret_cast<const ulonglong2*>(xk0 + plane + u * NB * PLI_TS + t);
                     }
 #pragma unroll
-                    for (int u = 0; u < 4; ++u)
+                    for (int v = 0; v < 4; ++v) {
+                        const ulonglong2 xj = *reinterpret_cast<const ulonglong2*>(xj0 + v * NB * PLI_TS + t);
+                        const ulonglong2 yj = *reinterpret_cast<const ulonglong2*>(xj0 + plane + v * NB * PLI_TS + t);
 #pragma unroll
-                        for (int v = 0; v < 4; ++v) {
+                        for (int u = 0; u < 4; ++u) {
                             // Im(z_k conj(z_j)) = y_k x_j - x_k y_j, each product rounded
-                            cnt[u][v] += sign_diff2(mul_f32x2(yk[u], xj[v]), mul_f32x2(xk[u], yj[v]));
+                            uint64_t p = mul_f32x2(yk[u].x, xj.x), q = mul_f32x2(xk[u].x, yj.x);
+                            take_signs(wn[u][v], diff_f32x2(p, q));
+                            take_signs(wp[u][v], diff_f32x2(q, p));
+                            p = mul_f32x2(yk[u].y, xj.y);
+                            q = mul_f32x2(xk[u].y, yj.y);
+                            take_signs(wn[u][v], diff_f32x2(p, q));
+                            take_signs(wp[u][v], diff_f32x2(q, p));
                         }
+                    }
+                    since += 4;
+                    if (since == 32 || t + 4 >= tl) {
+                        since = 0;
+#pragma unroll
+                        for (int u = 0; u < 4; ++u)
+#pragma unroll
+                            for (int v = 0; v < 4; ++v) {
+                                cnt[u][v] += __popc(wp[u][v]) - __popc(wn[u][v]);
+                                wp[u][v] = wn[u][v] = 0u;
+                            }
+                    }
                 }
             }
+            cur = next;
         }
         if (bp < nbp) {
 #pragma unroll
@@ -468,17 +528,16 @@ an_pli_kernel(const float2* __restrict__ z_all, int N, int n, float* __restrict_
 #pragma unroll
                 for (int v = 0; v < 4; ++v) {
                     const int kk = bk * 4 + u, jj = bj * 4 + v;
-                    if (kk < jj && jj < N) acc += (float)abs(cnt[u][v]) / (float)n;
+                    if (kk < jj && jj < N) atomicAdd(cnt_all + ((int64_t)b * N + kk) * N + jj, cnt[u][v]);
                 }
         }
     }
-    const float tot = block_sum(acc, red);
-    if (threadIdx.x == 0) pli_out[b] = N > 1 ? tot / (float)(N * (N - 1) / 2) : __int_as_float(0x7fc00000);
 }
 
-// One CTA per set: PSD mean over regions, peak, fit; UP / DOWN means.
+// One CTA per set: mean phase lag index (the mean over k < j of |cnt| / n), PSD
+// mean over regions, peak, fit; UP / DOWN means.
 __global__ void __launch_bounds__(AN_THREADS)
-an_finalize_kernel(const float* __restrict__ psd, const int* __restrict__ ud, const float* __restrict__ pli, int N,
+an_finalize_kernel(const float* __restrict__ psd, const int* __restrict__ ud, const int* __restrict__ cnt, int N, int n,
                    int band_lo, int band_n, double df, double dt_ms, int64_t p0, float* __restrict__ out)
 {
     extern __shared__ float an_psd[];   // [band_n]
@@ -486,7 +545,13 @@ an_finalize_kernel(const float* __restrict__ psd, const int* __restrict__ ud, co
     __shared__ float s_best[AN_THREADS];
     __shared__ int s_besti[AN_THREADS];
     __shared__ int s_pos;
+    __shared__ float red_f[AN_THREADS / 32];
     const int b = blockIdx.x;
+    float lag = 0.0f;
+    const int* cb = cnt + (int64_t)b * N * N;
+    for (int k = threadIdx.x >> 5; k < N; k += AN_THREADS / 32)
+        for (int j = k + 1 + (threadIdx.x & 31); j < N; j += 32) lag += (float)abs(cb[k * N + j]) / (float)n;
+    lag = block_sum(lag, red_f);
     const float* pb = psd + (int64_t)b * N * band_n;
     for (int i = threadIdx.x; i < band_n; i += blockDim.x) {
         float s = 0.0f;
@@ -529,7 +594,7 @@ an_finalize_kernel(const float* __restrict__ psd, const int* __restrict__ ud, co
         }
         const float nan = __int_as_float(0x7fc00000);
         float* o = out + (p0 + b) * (int64_t)TVBX_AN_COUNT;
-        o[TVBX_AN_MEAN_PLI] = pli[b];
+        o[TVBX_AN_MEAN_PLI] = N > 1 ? lag / (float)(N * (N - 1) / 2) : nan;
         o[TVBX_AN_PSD_FMAX] = bix >= 0 ? (float)((double)(band_lo + bix) * df) : nan;
         o[TVBX_AN_PSD_AMPMAX] = bix >= 0 ? bv : nan;
         const double nb = (double)band_n;
@@ -708,12 +773,40 @@ bool make_plan(int n, FftPlan& p)
     }
     if (r != 1) return false;
     uint64_t L1 = 1;
+    int off = 0;
     for (int s = 0; s < p.n_stages; ++s) {
+        p.tw_off[s] = off;
+        off += (p.radix[s] - 1) * (int)L1;
         // idx < 2^13 and L1 < 2^13: floor(idx * ceil(2^32 / L1) / 2^32) = floor(idx / L1)
         p.magic[s] = L1 == 1 ? 0u : (uint32_t)((((uint64_t)1 << 32) + L1 - 1) / L1);
         L1 *= (uint64_t)p.radix[s];
     }
     return true;
+}
+
+// exp(-2 pi i e / n) for 0 <= e < n, from FP64.
+std::vector<float2> roots(int n)
+{
+    std::vector<float2> w(n);
+    for (int e = 0; e < n; ++e) {
+        const double ang = -2.0 * 3.14159265358979323846 * (double)e / (double)n;
+        w[e] = make_float2((float)std::cos(ang), (float)std::sin(ang));
+    }
+    return w;
+}
+
+// The plan's twiddle table (FftPlan::tw_off) from the roots of a multiple of its length.
+std::vector<float2> stage_twiddles(const FftPlan& p, const std::vector<float2>& w)
+{
+    std::vector<float2> t;
+    int L1 = 1;
+    for (int s = 0; s < p.n_stages; ++s) {
+        const int step = (int)w.size() / (L1 * p.radix[s]);
+        for (int q = 1; q < p.radix[s]; ++q)
+            for (int j = 0; j < L1; ++j) t.push_back(w[(size_t)step * j * q]);
+        L1 *= p.radix[s];
+    }
+    return t;
 }
 
 // Digit reversal of the plan: the decimation-in-time stages (radix[0] first)
@@ -838,57 +931,45 @@ extern "C" tvbx_status tvbx_series_analysis(const float* series, int32_t n_regio
     }
     const int band_n = band_lo < 0 ? 0 : band_hi - band_lo + 1;
     cudaStream_t s = (cudaStream_t)cuda_stream;
-    // batch of sets: analytic signals of B sets in at most ~2 GiB, B a whole
-    // number of waves of the phase-lag kernel (one CTA per set) when the
-    // budget allows, so no SM runs more of its CTAs than another
-    const int64_t per_set = (int64_t)N * n * 8;
+    // batch of sets: analytic signals and pair counts of B sets in at most ~2 GiB
+    const int ns = (n + 3) / 4 * 4;
+    const int64_t per_set = (int64_t)N * ns * 8 + (int64_t)N * N * 4;
     int64_t B = std::max<int64_t>(1, std::min<int64_t>(P, ((int64_t)1 << 31) / std::max<int64_t>(per_set, 1)));
-    const size_t pli_row = sizeof(float) * 2 * (size_t)((N + 3) / 4 * 4);
-    const bool wide_tiles = pli_row * (PLI_TT_MAX + 2) <= 64 * 1024;
-    const size_t smem_pli = pli_row * (size_t)((wide_tiles ? PLI_TT_MAX : PLI_TT_MIN) + 2);
+    const size_t pli_row = sizeof(float) * 4 * (size_t)((N + 3) / 4 * 4);   // two buffers of two planes
+    const int tt = pli_row * (PLI_TT_MAX + 4) <= 110 * 1024 ? PLI_TT_MAX : (pli_row * 36 <= 200 * 1024 ? 32 : PLI_TT_MIN);
+    const size_t smem_pli = pli_row * (size_t)(tt + 4);
     if (smem_pli > 200 * 1024) return report_error(TVBX_E_INVALID_ARG, "too many regions for the PLI tile");
-    auto pli_kernel = wide_tiles ? an_pli_kernel<PLI_TT_MAX> : an_pli_kernel<PLI_TT_MIN>;
+    auto pli_kernel = tt == PLI_TT_MAX ? an_pli_kernel<PLI_TT_MAX>
+                                       : (tt == 32 ? an_pli_kernel<32> : an_pli_kernel<PLI_TT_MIN>);
     ACK(cudaFuncSetAttribute(pli_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_pli),
         "analysis shared memory");
-    {
-        int dev = 0, sms = 0, per_sm = 0;
-        ACK(cudaGetDevice(&dev), "device");
-        ACK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "device");
-        ACK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, pli_kernel, PLI_THREADS, smem_pli),
-            "occupancy");
-        const int64_t wave = (int64_t)sms * std::max(per_sm, 1);
-        if (B < P && B >= wave) B = B / wave * wave;
-    }
-    std::vector<float2> htw(n);
-    for (int e = 0; e < n; ++e) {
-        const double ang = -2.0 * 3.14159265358979323846 * (double)e / (double)n;
-        htw[e] = make_float2((float)std::cos(ang), (float)std::sin(ang));
-    }
+    // time slices of about 640 samples, whole tiles
+    const int slice = std::min((ns + PLI_TT_MAX - 1) / PLI_TT_MAX * PLI_TT_MAX, 10 * PLI_TT_MAX);
+    const int slices = (ns + slice - 1) / slice;
+    const std::vector<float2> htw = roots(n);
     AnScratch scr(s);
-    float2 *tw, *z;
-    float *psd, *pli;
-    int* ud;
-    ACK(scr.get(&tw, n), "analysis twiddles");
-    int* perm;
-    ACK(scr.get(&perm, n), "analysis digit reversal");
-    const std::vector<int> hperm = digit_reversal(plan);
-    ACK(cudaMemcpyAsync(perm, hperm.data(), sizeof(int) * n, cudaMemcpyHostToDevice, s), "analysis digit reversal");
-    // even lengths: the forward transform as a complex one of half the length
+    float2* tw;
+    float *z, *psd;
+    int *ud, *cnt;
+    // even lengths: complex transforms of half the length
     FftPlan plan_h = plan;
     const bool half = n % 2 == 0 && n >= 4 && make_plan(n / 2, plan_h);
-    int* perm_h = perm;
-    if (half) {
-        ACK(scr.get(&perm_h, n / 2), "analysis digit reversal");
-        const std::vector<int> hperm_h = digit_reversal(plan_h);
-        ACK(cudaMemcpyAsync(perm_h, hperm_h.data(), sizeof(int) * (n / 2), cudaMemcpyHostToDevice, s),
-            "analysis digit reversal");
-    }
-    ACK(scr.get(&z, (size_t)B * N * n), "analysis signals");
+    const FftPlan& used = half ? plan_h : plan;
+    const std::vector<float2> htws = stage_twiddles(used, htw);
+    const std::vector<int> hperm = digit_reversal(used);
+    float2* tws;
+    int* perm;
+    ACK(scr.get(&tw, n), "analysis twiddles");
+    ACK(scr.get(&tws, htws.size()), "analysis twiddles");
+    ACK(scr.get(&perm, used.n), "analysis digit reversal");
+    ACK(cudaMemcpyAsync(perm, hperm.data(), sizeof(int) * used.n, cudaMemcpyHostToDevice, s), "analysis digit reversal");
+    ACK(cudaMemcpyAsync(tws, htws.data(), sizeof(float2) * htws.size(), cudaMemcpyHostToDevice, s), "analysis twiddles");
+    ACK(scr.get(&z, (size_t)B * N * 2 * ns), "analysis signals");
     ACK(scr.get(&psd, (size_t)B * N * std::max(band_n, 1)), "analysis PSD");
-    ACK(scr.get(&pli, (size_t)B), "analysis PLI");
+    ACK(scr.get(&cnt, (size_t)B * N * N), "analysis PLI");
     ACK(scr.get(&ud, (size_t)B * N * 4), "analysis UP/DOWN");
     ACK(cudaMemcpyAsync(tw, htw.data(), sizeof(float2) * n, cudaMemcpyHostToDevice, s), "analysis twiddles");
-    const size_t smem_series = sizeof(float2) * (size_t)n;
+    const size_t smem_series = sizeof(float2) * (size_t)(half ? n / 2 : n);
     auto series_kernel = half ? an_series_kernel<true> : an_series_kernel<false>;
     ACK(cudaFuncSetAttribute(series_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_series),
         "analysis shared memory");
@@ -928,14 +1009,15 @@ extern "C" tvbx_status tvbx_series_analysis(const float* series, int32_t n_regio
             in_p0 = 0;
         }
         note_launch(3);
-        series_kernel<<<(unsigned)(nb * N), AN_THREADS, smem_series, s>>>(in, N, T, plan, plan_h, tw, perm, perm_h,
+        series_kernel<<<(unsigned)(nb * N), AN_THREADS, smem_series, s>>>(in, N, T, plan, plan_h, tw, tws, perm,
                                                                         band_lo, band_n, psd_scale, in_p0, psd,
-                                                                        ud, z);
+                                                                        ud, z, ns);
         ACK(cudaGetLastError(), "analysis series");
         if (host_in) ACK(cudaEventRecord(hp.ev[3 + slot], s), "analysis events");   // the slot was read
-        pli_kernel<<<(unsigned)nb, PLI_THREADS, smem_pli, s>>>(z, N, n, pli);
+        ACK(cudaMemsetAsync(cnt, 0, sizeof(int) * (size_t)nb * N * N, s), "analysis PLI");
+        pli_kernel<<<(unsigned)(nb * slices), PLI_THREADS, smem_pli, s>>>(z, N, ns, slice, slices, cnt);
         ACK(cudaGetLastError(), "analysis PLI");
-        an_finalize_kernel<<<(unsigned)nb, AN_THREADS, smem_fin, s>>>(psd, ud, pli, N, band_lo, band_n, df, dt_ms,
+        an_finalize_kernel<<<(unsigned)nb, AN_THREADS, smem_fin, s>>>(psd, ud, cnt, N, n, band_lo, band_n, df, dt_ms,
                                                                        p0, out);
         ACK(cudaGetLastError(), "analysis finalize");
     }
@@ -970,20 +1052,16 @@ extern "C" tvbx_status tvbx_phfcd(const float* bold, int32_t n_regions, int64_t 
     cudaStream_t s = (cudaStream_t)cuda_stream;
     const int64_t per_set = (int64_t)Tp * N * 8;
     const int64_t B = std::max<int64_t>(1, std::min<int64_t>(P, ((int64_t)1 << 30) / std::max<int64_t>(per_set, 1)));
-    std::vector<float2> htw(n);
-    for (int e = 0; e < n; ++e) {
-        const double ang = -2.0 * 3.14159265358979323846 * (double)e / (double)n;
-        htw[e] = make_float2((float)std::cos(ang), (float)std::sin(ang));
-    }
+    const std::vector<float2> htw = stage_twiddles(plan, roots(n));
     AnScratch scr(s);
     float2 *tw, *U;
-    ACK(scr.get(&tw, n), "phFCD twiddles");
+    ACK(scr.get(&tw, htw.size()), "phFCD twiddles");
     int* perm;
     ACK(scr.get(&perm, n), "phFCD digit reversal");
     const std::vector<int> hperm = digit_reversal(plan);
     ACK(cudaMemcpyAsync(perm, hperm.data(), sizeof(int) * n, cudaMemcpyHostToDevice, s), "phFCD digit reversal");
     ACK(scr.get(&U, (size_t)B * Tp * N), "phFCD phasors");
-    ACK(cudaMemcpyAsync(tw, htw.data(), sizeof(float2) * n, cudaMemcpyHostToDevice, s), "phFCD twiddles");
+    ACK(cudaMemcpyAsync(tw, htw.data(), sizeof(float2) * htw.size(), cudaMemcpyHostToDevice, s), "phFCD twiddles");
     const size_t smem_phase = sizeof(float2) * (size_t)n;
     ACK(cudaFuncSetAttribute(an_phase_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_phase),
         "phFCD shared memory");

@@ -1,0 +1,57 @@
+"""Table 2 metrics at the edges of the phase-lag tiles and of the UP / DOWN
+counts: region counts on both sides of a block, tile sizes for many regions,
+odd and short lengths, rows that repeat, are constant, or leave a state once,
+against the FP64 oracle."""
+import numpy as np
+import pytest
+
+from gpu_common import require_gpu
+from oracle import analysis as A
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def tvbx():
+    return require_gpu()
+
+
+def mean_pli(x):
+    """Mean phase lag index with every row transformed on its own: a batched
+    transform may round identical rows differently, and their lag sign is 0."""
+    z = np.stack([A.analytic_signal(row) for row in x])
+    n = x.shape[1]
+    lag = [abs(np.sign(z[k].imag * z[k + 1:].real - z[k].real * z[k + 1:].imag).sum(axis=1)) / n
+           for k in range(len(z) - 1)]
+    return np.concatenate(lag).mean()
+
+
+@pytest.mark.parametrize("n_regions,n_samples", [(2, 2), (3, 4), (5, 33), (8, 100), (9, 6), (101, 130), (197, 64),
+                                                 (360, 40), (752, 12), (21, 8191), (4, 1025)])
+def test_metrics_at_edges(tvbx, n_regions, n_samples):
+    import torch
+    rng = np.random.default_rng(n_regions + n_samples)
+    x = (5e-3 + 1e-3 * rng.standard_normal((3, n_regions, n_samples))).astype(np.float32)
+    x[1, 0] = 2e-3                      # no transition
+    x[1, -1] = x[1, n_regions // 2]     # identical rows: lag sign 0
+    x[2, 0] = np.where(np.arange(n_samples) < n_samples // 2, 1e-3, 4e-3)   # one transition
+    out, used = tvbx.series_analysis(torch.from_numpy(x).cuda(), 1.0)
+    got = out.cpu().numpy().astype(np.float64)
+    for p in range(3):
+        want = A.table2_metrics(x[p], 1.0)
+        assert used == want["n_samples"]
+        want["mean_pli"] = mean_pli(x[p].astype(np.float64)[:, n_samples - used:])
+        for i, name in enumerate(tvbx.AN_FIELDS):
+            g, w = got[p, i], want[name]
+            if np.isnan(w):
+                assert np.isnan(g), name
+            elif name in ("n_up", "up_samples", "n_down", "down_samples"):
+                assert g == w, name
+            elif name == "mean_pli":
+                # a sign may flip where |sin| of the phase difference is below the transforms'
+                # relative error (about 1e-6): one of n samples of one pair in 1e5
+                assert abs(g - w) < 1e-3, name
+            elif name == "psd_b":
+                assert abs(g - w) <= 1e-3 * abs(w), name
+            else:
+                assert abs(g - w) <= 1e-4 * abs(w) + 1e-7, name
