@@ -169,8 +169,9 @@ __device__ void dif_stage(float2* a, int n, int L1, uint32_t magic, const float2
 }
 
 // Forward transform in place: a holds the input in digit-reversed order
-// (a[perm[t]] = x[t]) and ends in natural order. tw: the plan's table.
-__device__ void fft_dit(float2* a, const FftPlan& plan, const float2* __restrict__ tw, bool inv)
+// (a[perm[t]] = x[t]) and ends in natural order. tw: the plan's table. total:
+// points of all the series that lie one after the other in a.
+__device__ void fft_dit(float2* a, const FftPlan& plan, const float2* __restrict__ tw, bool inv, int total)
 {
     int L1 = 1;
     for (int s = 0; s < plan.n_stages; ++s) {
@@ -178,10 +179,10 @@ __device__ void fft_dit(float2* a, const FftPlan& plan, const float2* __restrict
         const uint32_t mg = plan.magic[s];
         const float2* ts = tw + plan.tw_off[s];
         switch (r) {
-        case 2: dit_stage<2>(a, plan.n, L1, mg, ts, inv); break;
-        case 3: dit_stage<3>(a, plan.n, L1, mg, ts, inv); break;
-        case 4: dit_stage<4>(a, plan.n, L1, mg, ts, inv); break;
-        default: dit_stage<5>(a, plan.n, L1, mg, ts, inv); break;
+        case 2: dit_stage<2>(a, total, L1, mg, ts, inv); break;
+        case 3: dit_stage<3>(a, total, L1, mg, ts, inv); break;
+        case 4: dit_stage<4>(a, total, L1, mg, ts, inv); break;
+        default: dit_stage<5>(a, total, L1, mg, ts, inv); break;
         }
         __syncthreads();
         L1 *= r;
@@ -190,7 +191,7 @@ __device__ void fft_dit(float2* a, const FftPlan& plan, const float2* __restrict
 
 // Transform in place from natural order to digit-reversed order (result t at
 // a[perm[t]]): the stages in reverse radix order.
-__device__ void fft_dif(float2* a, const FftPlan& plan, const float2* __restrict__ tw, bool inv)
+__device__ void fft_dif(float2* a, const FftPlan& plan, const float2* __restrict__ tw, bool inv, int total)
 {
     int L = plan.n;
     for (int s = plan.n_stages - 1; s >= 0; --s) {
@@ -199,10 +200,10 @@ __device__ void fft_dif(float2* a, const FftPlan& plan, const float2* __restrict
         const uint32_t mg = plan.magic[s];
         const float2* ts = tw + plan.tw_off[s];
         switch (r) {
-        case 2: dif_stage<2>(a, plan.n, L1, mg, ts, inv); break;
-        case 3: dif_stage<3>(a, plan.n, L1, mg, ts, inv); break;
-        case 4: dif_stage<4>(a, plan.n, L1, mg, ts, inv); break;
-        default: dif_stage<5>(a, plan.n, L1, mg, ts, inv); break;
+        case 2: dif_stage<2>(a, total, L1, mg, ts, inv); break;
+        case 3: dif_stage<3>(a, total, L1, mg, ts, inv); break;
+        case 4: dif_stage<4>(a, total, L1, mg, ts, inv); break;
+        default: dif_stage<5>(a, total, L1, mg, ts, inv); break;
         }
         __syncthreads();
         L = L1;
@@ -338,7 +339,7 @@ an_series_kernel(const float* __restrict__ series, int N, int64_t T, FftPlan pla
     }
     float* pr = psd_out + ((int64_t)b * N + k) * band_n;
     if constexpr (HALF) {
-        fft_dit(a, plan_h, tws, false);
+        fft_dit(a, plan_h, tws, false, M);
         for (int i = threadIdx.x; i <= M / 2; i += blockDim.x) {
             if (i == 0) {
                 a[0] = make_float2(0.0f, 0.0f);
@@ -357,7 +358,7 @@ an_series_kernel(const float* __restrict__ series, int N, int64_t T, FftPlan pla
             if (M - i != i) a[M - i] = make_float2(t.y - c.x, t.x + c.y);                // i conj(t) - conj(c)
         }
         __syncthreads();
-        fft_dif(a, plan_h, tws, true);
+        fft_dif(a, plan_h, tws, true, M);
         const float inv_m = 1.0f / (float)M;
         float* xr = z_out + ((int64_t)b * N + k) * 2 * ns;
         float2* yr = reinterpret_cast<float2*>(xr + ns);
@@ -369,7 +370,7 @@ an_series_kernel(const float* __restrict__ series, int N, int64_t T, FftPlan pla
         for (int t = n + threadIdx.x; t < ns; t += blockDim.x) xr[t] = xr[ns + t] = 0.0f;
         return;
     } else {
-        fft_dit(a, plan, tws, false);
+        fft_dit(a, plan, tws, false, n);
         for (int i = threadIdx.x; i < band_n; i += blockDim.x) {
             const float2 v = a[band_lo + i];
             pr[i] = psd_scale * fmaf(v.x, v.x, v.y * v.y);
@@ -385,7 +386,7 @@ an_series_kernel(const float* __restrict__ series, int N, int64_t T, FftPlan pla
         }
         __syncthreads();
     }
-    fft_dif(a, plan, tws, true);
+    fft_dif(a, plan, tws, true, n);
     const float inv_n = 1.0f / (float)n;
     float* xr = z_out + ((int64_t)b * N + k) * 2 * ns;
     for (int t = threadIdx.x; t < ns; t += blockDim.x) {
@@ -628,49 +629,73 @@ an_finalize_kernel(const float* __restrict__ psd, const int* __restrict__ ud, co
 constexpr int PF_TILE = 64;
 constexpr int PF_THREADS = 256;
 
-// One CTA per (set in batch, region): unit phasors of the band-limited
-// analytic signal of the region's BOLD series, U[b][t][k] for the T' kept
-// samples.
+// Unit phasors of the band-limited analytic signals, U[b][k][t] for the T' kept
+// samples. A CTA takes S adjacent sets of a region (S a power of two, S n <=
+// AN_MAX_T): a short BOLD series alone leaves most threads of a stage idle, and
+// the sets of a sample are neighbours in memory (one series per CTA and
+// 8-byte writes at stride N: 441 us on 512 x 68 x 300).
 __global__ void __launch_bounds__(AN_THREADS)
 an_phase_kernel(const float* __restrict__ bold, int N, int64_t P, int64_t Tb, FftPlan plan,
                 const float2* __restrict__ tw, const int* __restrict__ perm, int band_lo, int band_hi, int discard,
-                int64_t p0, float2* __restrict__ U)
+                int64_t p0, int nb, int S, float2* __restrict__ U)
 {
     extern __shared__ float2 an_smem[];
-    __shared__ double red_d[AN_THREADS / 32];
+    __shared__ double part[AN_THREADS];
+    __shared__ float mean[AN_THREADS];
     const int n = plan.n, Tp = n - 2 * discard;
-    float2* a = an_smem;   // the series in digit-reversed order, transformed in place
-    const int b = blockIdx.x / N, k = blockIdx.x - b * N;
+    float2* a = an_smem;   // [S][n], each series in digit-reversed order, transformed in place
+    const int b0 = blockIdx.x / N * S, k = blockIdx.x % N;
     const int64_t NP = (int64_t)N * P;
-    const float* col = bold + (Tb - n) * NP + (int64_t)k * P + p0 + b;
+    const float* col = bold + (Tb - n) * NP + (int64_t)k * P + p0 + b0;
+    const int q = threadIdx.x % S;   // this thread's series, times threadIdx.x / S, + AN_THREADS / S, ...
     double s = 0.0;
-    for (int t = threadIdx.x; t < n; t += blockDim.x) {
-        const float x = col[(int64_t)t * NP];
-        a[__ldg(perm + t)] = make_float2(x, 0.0f);
+    for (int t = threadIdx.x / S; t < n; t += AN_THREADS / S) {
+        const float x = b0 + q < nb ? col[(int64_t)t * NP + q] : 0.0f;
+        a[q * n + __ldg(perm + t)] = make_float2(x, 0.0f);
         s += (double)x;
     }
-    const float mean = (float)(block_sum(s, red_d) / (double)n);
-    for (int t = threadIdx.x; t < n; t += blockDim.x) a[t].x -= mean;
+    part[threadIdx.x] = s;
     __syncthreads();
-    fft_dit(a, plan, tw, false);
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    for (int h = AN_THREADS / 2; h >= S; h >>= 1) {
+        if (threadIdx.x < h) part[threadIdx.x] += part[threadIdx.x + h];
+        __syncthreads();
+    }
+    if (threadIdx.x < S) mean[threadIdx.x] = (float)(part[threadIdx.x] / (double)n);
+    __syncthreads();
+    const float mu = mean[q];
+    for (int t = threadIdx.x / S; t < n; t += AN_THREADS / S) a[q * n + t].x -= mu;
+    __syncthreads();
+    fft_dit(a, plan, tw, false, S * n);
+    for (int i = threadIdx.x / S; i < n; i += AN_THREADS / S) {
         const float h = (i >= band_lo && i <= band_hi) ? 2.0f : 0.0f;
-        a[i] = make_float2(h * a[i].x, h * a[i].y);
+        a[q * n + i] = make_float2(h * a[q * n + i].x, h * a[q * n + i].y);
     }
     __syncthreads();
-    fft_dif(a, plan, tw, true);
-    float2* Ub = U + (int64_t)b * Tp * N;
-    for (int t = threadIdx.x; t < Tp; t += blockDim.x) {
-        const float2 v = a[__ldg(perm + t + discard)];
-        const float r = hypotf(v.x, v.y);
-        Ub[(int64_t)t * N + k] = r > 0.0f ? make_float2(v.x / r, v.y / r) : make_float2(1.0f, 0.0f);
+    fft_dif(a, plan, tw, true, S * n);
+    for (int i = threadIdx.x; i < S * Tp; i += AN_THREADS) {
+        const int r = i / Tp, t = i - r * Tp;
+        if (b0 + r >= nb) break;
+        const float2 v = a[r * n + __ldg(perm + t + discard)];
+        const float len = hypotf(v.x, v.y);
+        U[((int64_t)(b0 + r) * N + k) * Tp + t] = len > 0.0f ? make_float2(v.x / len, v.y / len) : make_float2(1.0f, 0.0f);
     }
+}
+
+// (x, x) (c, d) + acc in both lanes
+__device__ __forceinline__ void fma_f32x2(uint64_t& acc, float x, uint64_t cd)
+{
+    uint64_t xx;
+    asm("mov.b64 %0, {%1, %1};" : "=l"(xx) : "f"(x));
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(xx), "l"(cd));
 }
 
 // One CTA per (tile pair ta <= tc of 64 x 64 times, set in batch). Tiles are
 // stored region-major in shared memory; thread (m, q) owns times
 // ta*64 + q + 16 i and tc*64 + m + 16 j (i, j < 4), so a half-warp reads 16
-// consecutive 8-byte phasors.
+// consecutive 8-byte phasors. With the four real sums xx, xy, yx, yy over the
+// regions, |sum u u'|^2 + |sum u conj u'|^2 = 2 (xx^2 + xy^2 + yx^2 + yy^2):
+// two packed multiply-adds per pair and region where the two complex sums took
+// eight scalar ones (832 us on 512 x 68 x 300).
 __global__ void __launch_bounds__(PF_THREADS)
 an_phfcd_kernel(const float2* __restrict__ U, int N, int Tp, int64_t p0, int64_t M2, float* __restrict__ out)
 {
@@ -683,12 +708,12 @@ an_phfcd_kernel(const float2* __restrict__ U, int N, int Tp, int64_t p0, int64_t
     while (rem >= nt - ta) { rem -= nt - ta; ++ta; }
     const int tc = ta + rem;
     const int b = blockIdx.y;
-    const float2* Ub = U + (int64_t)b * Tp * N;
+    const float2* Ub = U + (int64_t)b * N * Tp;
     for (int i = threadIdx.x; i < PF_TILE * N; i += blockDim.x) {
-        const int r = i / N, k = i - r * N;
+        const int k = i / PF_TILE, r = i % PF_TILE;
         const int t1 = ta * PF_TILE + r, t2 = tc * PF_TILE + r;
-        Ua[k * PF_TILE + r] = t1 < Tp ? Ub[(int64_t)t1 * N + k] : make_float2(0.0f, 0.0f);
-        Uc[k * PF_TILE + r] = t2 < Tp ? Ub[(int64_t)t2 * N + k] : make_float2(0.0f, 0.0f);
+        Ua[i] = t1 < Tp ? Ub[(int64_t)k * Tp + t1] : make_float2(0.0f, 0.0f);
+        Uc[i] = t2 < Tp ? Ub[(int64_t)k * Tp + t2] : make_float2(0.0f, 0.0f);
     }
     __syncthreads();
     // |V(t)| from S = sum_k u_k^2: |V|^2 = ((|S|^2 - N) + N^2 - N) / 4
@@ -707,27 +732,26 @@ an_phfcd_kernel(const float2* __restrict__ U, int N, int Tp, int64_t p0, int64_t
     }
     __syncthreads();
     const int q = threadIdx.x >> 4, m = threadIdx.x & 15;
-    float ax[4][4], ay[4][4], bx[4][4], by[4][4];
+    uint64_t xv[4][4], yv[4][4];   // (xx, xy), (yx, yy)
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) ax[i][j] = ay[i][j] = bx[i][j] = by[i][j] = 0.0f;
+        for (int j = 0; j < 4; ++j) xv[i][j] = yv[i][j] = 0;
+#pragma unroll 2
     for (int k = 0; k < N; ++k) {
-        float2 ua[4], uc[4];
+        float2 ua[4];
+        uint64_t uc[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             ua[i] = Ua[k * PF_TILE + q + 16 * i];
-            uc[i] = Uc[k * PF_TILE + m + 16 * i];
+            uc[i] = *reinterpret_cast<const uint64_t*>(Uc + k * PF_TILE + m + 16 * i);
         }
 #pragma unroll
         for (int i = 0; i < 4; ++i)
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
-                // A += ua uc, B += ua conj(uc)
-                ax[i][j] = fmaf(ua[i].x, uc[j].x, fmaf(-ua[i].y, uc[j].y, ax[i][j]));
-                ay[i][j] = fmaf(ua[i].x, uc[j].y, fmaf(ua[i].y, uc[j].x, ay[i][j]));
-                bx[i][j] = fmaf(ua[i].x, uc[j].x, fmaf(ua[i].y, uc[j].y, bx[i][j]));
-                by[i][j] = fmaf(ua[i].y, uc[j].x, fmaf(-ua[i].x, uc[j].y, by[i][j]));
+                fma_f32x2(xv[i][j], ua[i].x, uc[j]);
+                fma_f32x2(yv[i][j], ua[i].y, uc[j]);
             }
     }
     const float fN = (float)N;
@@ -739,8 +763,9 @@ an_phfcd_kernel(const float2* __restrict__ U, int N, int Tp, int64_t p0, int64_t
             const int ra = q + 16 * i, rc = m + 16 * j;
             const int t1 = ta * PF_TILE + ra, t2 = tc * PF_TILE + rc;
             if (t1 < t2 && t2 < Tp) {
-                const float dot = 0.25f * ((fmaf(ax[i][j], ax[i][j], ay[i][j] * ay[i][j]) - fN) +
-                                           (fmaf(bx[i][j], bx[i][j], by[i][j] * by[i][j]) - fN));
+                const float xx = __uint_as_float((uint32_t)xv[i][j]), xy = __uint_as_float((uint32_t)(xv[i][j] >> 32));
+                const float yx = __uint_as_float((uint32_t)yv[i][j]), yy = __uint_as_float((uint32_t)(yv[i][j] >> 32));
+                const float dot = 0.5f * (fmaf(xx, xx, yy * yy) + fmaf(xy, xy, yx * yx) - fN);
                 const int64_t e = (int64_t)t1 * Tp - (int64_t)t1 * (t1 + 1) / 2 + (t2 - t1 - 1);
                 o[e] = dot / (nrm_a[ra] * nrm_c[rc]);
             }
@@ -1062,7 +1087,9 @@ extern "C" tvbx_status tvbx_phfcd(const float* bold, int32_t n_regions, int64_t 
     ACK(cudaMemcpyAsync(perm, hperm.data(), sizeof(int) * n, cudaMemcpyHostToDevice, s), "phFCD digit reversal");
     ACK(scr.get(&U, (size_t)B * Tp * N), "phFCD phasors");
     ACK(cudaMemcpyAsync(tw, htw.data(), sizeof(float2) * htw.size(), cudaMemcpyHostToDevice, s), "phFCD twiddles");
-    const size_t smem_phase = sizeof(float2) * (size_t)n;
+    int S = 1;   // sets per CTA of the phase kernel
+    while (S < 8 && 2 * S * n <= AN_MAX_T / 2 && 2 * S <= P) S *= 2;
+    const size_t smem_phase = sizeof(float2) * (size_t)n * S;
     ACK(cudaFuncSetAttribute(an_phase_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_phase),
         "phFCD shared memory");
     const size_t smem_pf = sizeof(float2) * 2 * (size_t)N * PF_TILE;
@@ -1074,8 +1101,8 @@ extern "C" tvbx_status tvbx_phfcd(const float* bold, int32_t n_regions, int64_t 
     for (int64_t p0 = 0; p0 < P; p0 += B) {
         const int64_t nb = std::min<int64_t>(B, P - p0);
         note_launch(2);
-        an_phase_kernel<<<(unsigned)(nb * N), AN_THREADS, smem_phase, s>>>(bold, N, P, n_tr, plan, tw, perm, band_lo,
-                                                                          band_hi, discard, p0, U);
+        an_phase_kernel<<<(unsigned)((nb + S - 1) / S * N), AN_THREADS, smem_phase, s>>>(
+            bold, N, P, n_tr, plan, tw, perm, band_lo, band_hi, discard, p0, (int)nb, S, U);
         ACK(cudaGetLastError(), "phFCD phases");
         an_phfcd_kernel<<<dim3((unsigned)(nt * (nt + 1) / 2), (unsigned)nb), PF_THREADS, smem_pf, s>>>(U, N, Tp, p0,
                                                                                                        M2, out);
