@@ -1,0 +1,40 @@
+"""BOLD of short and uneven lengths (the rates are fetched in blocks of eight
+samples) and of drives on both sides of the short series' bounds, against the
+FP64 oracle, and in two pieces bit for bit."""
+import numpy as np
+import pytest
+
+from gpu_common import require_gpu
+from oracle import bold as B
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def tvbx():
+    return require_gpu()
+
+
+@pytest.mark.parametrize("n_samples", [1, 7, 8, 9, 16, 17, 31, 4001])
+@pytest.mark.parametrize("n_sets", [2, 3])
+def test_bold_lengths(tvbx, n_samples, n_sets):
+    import torch
+    rng = np.random.default_rng(n_samples)
+    # set 0 at 5 Hz, the others from rest to 150 Hz (f - 1 from 0 to 0.37)
+    X = 5e-3 * rng.uniform(0.5, 1.5, (n_samples, 3, n_sets))
+    X[:, :, 1:] += np.linspace(0.0, 0.15, n_samples)[:, None, None]
+    X = X.astype(np.float32)
+    x = torch.from_numpy(X).cuda()
+    st = torch.zeros((4, 3, n_sets), device="cuda")
+    y = tvbx.bold(x, 1.0, 1, state=st, reset_state=True)
+    for p in range(n_sets):
+        want, state = B.bold(X[:, :, p].T, 1.0, 1)
+        state[1:] -= 1.0
+        # Euler steps of FP32 roundings: 4,000 steps of 2^-24 of the largest term
+        assert np.abs(y[:, :, p].cpu().numpy().T - want).max() <= 1e-4 * np.abs(want).max() + 1e-12
+        assert np.abs(st[:, :, p].cpu().numpy() - state).max() <= 1e-4 * np.abs(state).max() + 1e-12
+    half = n_samples // 2
+    st2 = torch.zeros_like(st)
+    parts = [tvbx.bold(x[:half].contiguous(), 1.0, 1, state=st2, reset_state=True)] if half else []
+    parts.append(tvbx.bold(x[half:].contiguous(), 1.0, 1, state=st2, reset_state=not half))
+    assert torch.equal(torch.cat(parts), y) and torch.equal(st, st2)
