@@ -435,9 +435,10 @@ tvbx_status build_groups(tvbx_sweep* h, double dt, std::vector<Group>& groups)
         g.row_mid.assign(N, 0);
         int64_t dmax = 1;   // ring of at least 3 slots (the padding entries use d = 1)
         for (int k = 0; k < N; ++k) {
-            // rows start at an index of the parity of k (zero-weight self entry pads)
+            // rows start at an index of the parity of k; a zero-weight entry pads the end of
+            // row k - 1 with its own region (0 x NaN must not reach another region)
             if ((int)(g.col_dly.size() & 1) != (k & 1)) {
-                g.col_dly.push_back((1u << 16) | (uint32_t)k);
+                g.col_dly.push_back((1u << 16) | (uint32_t)(k - 1));
                 g.w.push_back(0.0f);
             }
             g.row_ptr[k] = (int32_t)g.col_dly.size();
