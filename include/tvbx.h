@@ -502,6 +502,9 @@ tvbx_status tvbx_batch_create(tvbx_sweep* const* jobs, const tvbx_run_cfg* cfgs,
  * then two of the register-tile body (threads 512 and 768: each job with
  * N <= threads gets pb = 4 floor(threads / N) sets per CTA, 4 sets of one
  * region per thread; larger jobs keep the general body with a 200 KB budget).
+ * Where no job has a zero delay and all share one model, the windowed body
+ * (several steps of a tile between two CTA barriers) is timed besides, outside
+ * the reported trials; it reads as (128, 64 KB).
  * Runs are shortened to trial_steps steps per job. threads_out, smem_kb_out:
  * the choice (smem_kb_out is the general body's budget); trial_ms [n_trials]
  * (host, nullable; 8 entries, INFINITY where a candidate does not fit).

@@ -552,7 +552,8 @@ tvbx_status tvbx_sweep_info(const tvbx_sweep* h, int64_t* n_sets, int32_t* n_reg
 // checks, delay groups, internal set order, kernel and tile choice, device
 // buffers and uploads; with device_init also the state and ring
 // initialisation on stream s. general_pb > 0 forces the general kernel (or,
-// with direct_body, the register-tile body) with that tile width (batches).
+// with direct_body, the register-tile body) with that tile width (batches);
+// windows: the windowed kernels may be chosen, with general_pb > 0 they must be.
 struct RunPlan {
     SimArgs a;
     int variant = -1;
@@ -566,12 +567,18 @@ struct RunPlan {
     std::vector<int64_t> tile_nnz;   // weights per row of the tile's group (cost model)
 };
 
+// Floats of a group's ring.
+static int64_t group_ring_floats(const GroupDev& g, const WindowPlan& w, int N)
+{
+    return w.steps > 0 ? (int64_t)(g.P_g + w.pb - 1) / w.pb * w.pb * N * (g.H + WIN_FAR)
+                       : (int64_t)g.H * N * g.stride;
+}
+
 // n_base > 0: the run continues a trajectory at global step n_base (state,
 // ring buffers and OU state are kept; the series and the running sums start
 // afresh for the new samples).
 static tvbx_status prepare_run(tvbx_sweep* h, const tvbx_run_cfg& c, cudaStream_t s, int general_pb,
-                               bool device_init, RunPlan& plan, bool direct_body = false, int64_t n_base = 0,
-                               bool windows = true)
+                               bool device_init, RunPlan& plan, bool direct_body, int64_t n_base, bool windows)
 {
     if (!(c.dt_ms > 0.0) || !isfinite(c.dt_ms)) return fail(TVBX_E_INVALID_ARG, "dt_ms must be > 0");
     if (c.n_steps < 0 || n_base + c.n_steps > ((int64_t)1 << 32) - 2)
@@ -638,13 +645,18 @@ static tvbx_status prepare_run(tvbx_sweep* h, const tvbx_run_cfg& c, cudaStream_
     WindowPlan win;
     // a continued run keeps the ring layout it finds
     if (n_base > 0 && h->win.steps == 0) windows = false;
-    if (windows && general_pb == 0 && c.kernel == TVBX_KERNEL_AUTO && sim_direct_pb(N) > 0) {
+    if (windows && (general_pb > 0 || c.kernel == TVBX_KERNEL_AUTO) && sim_direct_pb(N) > 0) {
         int dev = 0, sms = 0;
         CK(cudaGetDevice(&dev), "device");
         CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "device");
         if (!sim_window_plan(d_min, N, largest_group, h->model.tau_e == h->model.tau_i, sms, win)) win = WindowPlan{};
     }
-    if (general_pb > 0) {
+    if (windows && general_pb > 0) {
+        if (win.steps == 0) return fail(TVBX_E_UNSUPPORTED, "no window of steps without coupling");
+        win.pb = general_pb;
+        win.packed = h->model.tau_e == h->model.tau_i;
+        variant = -2;
+    } else if (general_pb > 0) {
         // batch: the batch's body and tile width
         if (direct_body) variant = -2;
     } else if (win.steps > 0) {
@@ -672,7 +684,7 @@ static tvbx_status prepare_run(tvbx_sweep* h, const tvbx_run_cfg& c, cudaStream_
     int pb = 16;
     if (general_pb > 0) {
         pb = general_pb;
-        if (!direct_body && sim_smem_bytes(N, pb) > 227 * 1024)
+        if (!direct_body && !windows && sim_smem_bytes(N, pb) > 227 * 1024)
             return fail(TVBX_E_UNSUPPORTED, "n_regions %d too large", N);
     } else if (variant >= 0) {
         pb = sim_fast_pb(variant);
@@ -743,7 +755,7 @@ static tvbx_status prepare_run(tvbx_sweep* h, const tvbx_run_cfg& c, cudaStream_
     CK(h->d_status.ensure(sizeof(uint32_t) * P), "status");
     cudaError_t ring_e = h->d_ring.ensure(sizeof(float) * (size_t)std::max<int64_t>(ring_floats, 1));
     if (ring_e == cudaSuccess && win.far) ring_e = h->d_far.ensure(sizeof(float) * tiles.size() * WIN_FAR * N * pb);
-    if (ring_e != cudaSuccess && win.steps > 0) {
+    if (ring_e != cudaSuccess && win.steps > 0 && general_pb == 0) {
         // the windowed layout is larger: without room for it the other kernels still run
         h->d_far.release();
         (void)cudaGetLastError();
@@ -850,11 +862,7 @@ static tvbx_status prepare_run(tvbx_sweep* h, const tvbx_run_cfg& c, cudaStream_
     if (device_init) {
         CK(launch_init_state(a, s), "init state");
         for (size_t gi = 0; gi < groups.size(); ++gi)
-            CK(launch_init_ring(gdev[gi].ring,
-                                win.steps > 0 ? (gdev[gi].P_g + pb - 1) / pb * (int64_t)pb * N * (gdev[gi].H + WIN_FAR)
-                                              : (int64_t)gdev[gi].H * N * gdev[gi].stride,
-                                a.m.E0, s),
-               "init ring");
+            CK(launch_init_ring(gdev[gi].ring, group_ring_floats(gdev[gi], win, N), a.m.E0, s), "init ring");
     }
     plan.a = a;
     plan.variant = variant;
@@ -985,7 +993,7 @@ tvbx_status tvbx_run(tvbx_sweep* h, const tvbx_run_cfg* cfg, void* cuda_stream)
     const tvbx_run_cfg c = *cfg;
     cudaStream_t s = (cudaStream_t)cuda_stream;
     RunPlan plan;
-    tvbx_status st = prepare_run(h, c, s, 0, true, plan);
+    tvbx_status st = prepare_run(h, c, s, 0, true, plan, false, 0, true);
     if (st != TVBX_OK) return st;
     if ((st = run_chunks(h, c, plan, 0, s)) != TVBX_OK) return st;
     finish_run(h, c, 0, true);
@@ -1007,7 +1015,7 @@ tvbx_status tvbx_run_continue(tvbx_sweep* h, int64_t n_steps, int32_t transient_
     const int64_t n_base = h->steps_done;
     cudaStream_t s = (cudaStream_t)cuda_stream;
     RunPlan plan;
-    tvbx_status st = prepare_run(h, c, s, 0, false, plan, false, n_base);
+    tvbx_status st = prepare_run(h, c, s, 0, false, plan, false, n_base, true);
     if (st != TVBX_OK) return st;
     if ((st = run_chunks(h, c, plan, n_base, s)) != TVBX_OK) return st;
     finish_run(h, c, n_base, true);
@@ -1179,7 +1187,7 @@ tvbx_status tvbx_restore(tvbx_sweep* h, const void* host_buf, uint64_t bytes)
     // and the default stream used
     CK(cudaDeviceSynchronize(), "restore");
     RunPlan plan;
-    tvbx_status st = prepare_run(h, c, nullptr, 0, false, plan);
+    tvbx_status st = prepare_run(h, c, nullptr, 0, false, plan, false, 0, true);
     if (st != TVBX_OK) return st;
     if (h->ring_floats != hd.ring_floats) return fail(TVBX_E_INVALID_ARG, "checkpoint ring layout differs");
     const int64_t N = h->N, P = h->P;
@@ -1686,6 +1694,12 @@ struct tvbx_batch {
     int32_t threads = 512;
     size_t smem_budget = 200 * 1024;
     bool direct = false;                // register-tile bodies where a job fits
+    bool window = true;                 // windowed kernels (every job must have windows, and one model):
+                                        // the graph holds the initialisation, the turns are launched after it
+    bool packed = false;
+    std::vector<BatchJob> round_jobs;   // [round][job]
+    std::vector<RunPlan> plans;
+    int64_t rounds = 0;
     bool only_direct = false;           // every job on register tiles
     DevBuf d_jobs, d_items, d_head, d_ou;
     int32_t n_items = 0, grid = 0;
@@ -1741,7 +1755,7 @@ tvbx_status batch_adopt_jobs(tvbx_batch* b)
     return TVBX_OK;
 }
 
-tvbx_status batch_build(tvbx_batch* b, int32_t threads, size_t budget, int64_t trial_steps, bool direct)
+tvbx_status batch_build(tvbx_batch* b, int32_t threads, size_t budget, int64_t trial_steps, bool direct, bool window)
 {
     b->drop_graph();
     if (tvbx_status st = batch_adopt_jobs(b)) return st;
@@ -1779,15 +1793,17 @@ tvbx_status batch_build(tvbx_batch* b, int32_t threads, size_t budget, int64_t t
         const int N = b->jobs[j]->N;
         // register tiles: as many 4-set quads per region as the CTA has threads for
         const bool dj = direct && N <= threads;
-        const int pb = dj ? 4 * (threads / N) : batch_pb(N, budget, threads);
+        const int pb = window ? WIN_BATCH_PB : dj ? 4 * (threads / N) : batch_pb(N, budget, threads);
         if (!pb) return fail(TVBX_E_UNSUPPORTED, "batch job %zu: %d regions do not fit %zu bytes of shared memory", j,
                              N, budget);
         pbs[j] = pb;
         dirs[j] = dj ? 1 : 0;
-        smem = std::max(smem, dj ? sizeof(float) * 11 * (size_t)pb : sim_smem_bytes(N, pb));
+        if (!window) smem = std::max(smem, dj ? sizeof(float) * 11 * (size_t)pb : sim_smem_bytes(N, pb));
         c.chunk_steps = c.series_mode == TVBX_SERIES_STREAM ? (int32_t)S : 0;
-        tvbx_status st = prepare_run(b->jobs[j], c, b->stream, pb, false, plans[j], dj);
+        tvbx_status st = prepare_run(b->jobs[j], c, b->stream, pb, false, plans[j], dj, 0, window);
         if (st != TVBX_OK) return st;
+        if (window && (memcmp(&plans[j].a.m, &plans[0].a.m, sizeof(DevModel)) != 0))
+            return fail(TVBX_E_UNSUPPORTED, "windowed batch: job %zu has another model", j);
         if (!c.noise_per_set) {
             ou_off[j] = ou_floats;
             ou_floats += ((int64_t)c.n_steps * b->jobs[j]->N + 63) / 64 * 64;
@@ -1802,6 +1818,12 @@ tvbx_status batch_build(tvbx_batch* b, int32_t threads, size_t budget, int64_t t
     struct Cost { double c; int32_t job, tile; };
     std::vector<BatchItem> items;
     std::vector<int64_t> item_off((size_t)R + 1, 0);
+    int32_t win_steps = 1;
+    bool packed = true;
+    for (const RunPlan& p : plans) {
+        win_steps = std::max(win_steps, p.win.steps);
+        packed = packed && p.win.packed;
+    }
     for (int64_t r = 0; r < R; ++r) {
         std::vector<Cost> costs;
         for (size_t j = 0; j < nj; ++j) {
@@ -1812,9 +1834,17 @@ tvbx_status batch_build(tvbx_batch* b, int32_t threads, size_t budget, int64_t t
             a.ou_table = ou_off[j] >= 0 ? b->d_ou.as<float>() + ou_off[j] + n0 * b->jobs[j]->N : nullptr;
             if (run_cfgs[j].series_mode == TVBX_SERIES_STREAM)
                 a.series = series_at(b->jobs[j]->d_series.ptr, n0 / run_cfgs[j].tavg_steps, b->jobs[j]->sl);
-            jobs[(size_t)r * nj + j] = BatchJob{a, pbs[j], dirs[j]};
+            jobs[(size_t)r * nj + j] = BatchJob{a, pbs[j], dirs[j], plans[j].win.steps, 0,
+                                               plans[j].win.far ? b->jobs[j]->d_far.as<float>() : nullptr};
             if (nc <= 0) continue;
             const int N = b->jobs[j]->N;
+            if (window) {
+                // one list of blocks for all rounds, the jobs with the longest windows first
+                const int32_t bpt = sim_batch_window_blocks(N, packed);
+                for (int32_t t = 0; t < plans[j].n_tiles * bpt && r == 0; ++t)
+                    costs.push_back(Cost{(double)plans[j].win.steps, (int32_t)j, t});
+                continue;
+            }
             for (int32_t t = 0; t < plans[j].n_tiles; ++t) {
                 const double per_step = (double)N * 40.0 + (double)plans[j].tile_nnz[t];   // TF work + gathers
                 costs.push_back(Cost{per_step * (double)nc * plans[j].tiles[t].nq, (int32_t)(r * nj + j), t});
@@ -1838,12 +1868,16 @@ tvbx_status batch_build(tvbx_batch* b, int32_t threads, size_t budget, int64_t t
     CK(cudaGetDevice(&dev), "device");
     CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "device");
     b->only_direct = std::all_of(dirs.begin(), dirs.end(), [](int d) { return d != 0; });
-    const int per_sm = sim_batch_ctas_per_sm(threads, smem, b->only_direct);
+    const int per_sm = window ? 4 : sim_batch_ctas_per_sm(threads, smem, b->only_direct);
     if (per_sm < 1) return fail(TVBX_E_UNSUPPORTED, "batch kernel does not fit %d threads / %zu bytes", threads, smem);
     b->grid = (int32_t)std::max<int64_t>(1, std::min<int64_t>((int64_t)sms * per_sm, (int64_t)items.size()));
     b->threads = threads;
     b->smem_budget = budget;
     b->direct = direct;
+    b->window = window;
+    b->packed = packed;
+    b->rounds = R;
+    b->round_jobs.swap(jobs);
     CK(cudaStreamSynchronize(b->stream), "batch upload");
 
     // capture the device work of one run
@@ -1853,12 +1887,12 @@ tvbx_status batch_build(tvbx_batch* b, int32_t threads, size_t budget, int64_t t
     int64_t kernels = 0;
     for (size_t j = 0; j < nj && ce == cudaSuccess; ++j) {
         tvbx_sweep* h = b->jobs[j];
-        const SimArgs& a = jobs[j].a;   // round 0
+        const SimArgs& a = b->round_jobs[j].a;   // round 0
         if ((ce = cudaMemsetAsync(h->d_error.ptr, 0, sizeof(uint32_t), b->stream)) != cudaSuccess) break;
         if ((ce = launch_init_state(a, b->stream)) != cudaSuccess) break;
         ++kernels;
         for (const GroupDev& g : plans[j].gdev) {
-            if ((ce = launch_init_ring(g.ring, (int64_t)g.H * h->N * g.stride, a.m.E0, b->stream)) != cudaSuccess) break;
+            if ((ce = launch_init_ring(g.ring, group_ring_floats(g, plans[j].win, h->N), a.m.E0, b->stream)) != cudaSuccess) break;
             ++kernels;
         }
         if (ce != cudaSuccess) break;
@@ -1875,7 +1909,7 @@ tvbx_status batch_build(tvbx_batch* b, int32_t threads, size_t budget, int64_t t
     }
     if (ce == cudaSuccess) ce = cudaMemsetAsync(b->d_head.ptr, 0, sizeof(int32_t) * (size_t)R, b->stream);
     std::vector<char> shift_set(nj, 0);
-    for (int64_t r = 0; r < R && ce == cudaSuccess && fst == TVBX_OK; ++r) {
+    for (int64_t r = 0; r < R && !window && ce == cudaSuccess && fst == TVBX_OK; ++r) {
         const int64_t n_r = item_off[(size_t)r + 1] - item_off[(size_t)r];
         if (n_r > 0) {
             const int32_t grid_r = (int32_t)std::max<int64_t>(1, std::min<int64_t>((int64_t)sms * per_sm, n_r));
@@ -1885,7 +1919,7 @@ tvbx_status batch_build(tvbx_batch* b, int32_t threads, size_t budget, int64_t t
             ++kernels;
         }
         for (size_t j = 0; j < nj && ce == cudaSuccess && fst == TVBX_OK; ++j) {
-            const SimArgs& a = jobs[(size_t)r * nj + j].a;
+            const SimArgs& a = b->round_jobs[(size_t)r * nj + j].a;
             if (run_cfgs[j].series_mode != TVBX_SERIES_STREAM || a.n_chunk <= 0) continue;
             bool ss = shift_set[j] != 0;
             kernels += ss ? 2 : 3;   // (shift,) moments, accumulation
@@ -1908,9 +1942,50 @@ tvbx_status batch_build(tvbx_batch* b, int32_t threads, size_t budget, int64_t t
     b->graph_nodes = (int64_t)nodes;
     b->graph_kernels = kernels;
     b->cfgs_run = run_cfgs;
+    b->plans.swap(plans);
     b->gens.resize(nj);
     for (size_t j = 0; j < nj; ++j) b->gens[j] = b->jobs[j]->gen;
     b->built = true;
+    return TVBX_OK;
+}
+
+// Enqueue one run of a built batch on its stream: the graph and, windowed, the
+// turns of every round, each followed by its streamed jobs' FC folds.
+tvbx_status batch_enqueue(tvbx_batch* b)
+{
+    CK(cudaGraphLaunch(b->exec, b->stream), "batch launch");
+    note_launch(b->graph_kernels);
+    if (!b->window) return TVBX_OK;
+    const size_t nj = b->jobs.size();
+    std::vector<char> shift_set(nj, 0);
+    for (int64_t r = 0; r < b->rounds; ++r) {
+        const BatchJob* dev = b->d_jobs.as<BatchJob>() + (size_t)r * nj;
+        const BatchJob* host = b->round_jobs.data() + (size_t)r * nj;
+        int32_t turns = 0, steps = 1;
+        for (size_t j = 0; j < nj; ++j) {
+            turns = std::max(turns, sim_batch_window_turns(host[j].win_steps, host[j].far != nullptr, host[j].a.n_chunk));
+            steps = std::max(steps, host[j].win_steps);
+        }
+        for (int32_t t = 0; t < turns; ++t) {
+            bool due = false;   // a job starts a far block with this turn
+            for (size_t j = 0; j < nj && !due; ++j)
+                due = host[j].far && t % ((WIN_FAR + host[j].win_steps - 1) / host[j].win_steps) == 0 &&
+                      t < sim_batch_window_turns(host[j].win_steps, true, host[j].a.n_chunk);
+            const BatchItem* blocks = b->d_items.as<BatchItem>();
+            if (due)
+                CK(launch_sim_batch_window(host[0].a.m, b->packed, true, dev, blocks, b->n_items, t, steps, b->stream),
+                   "batch far sums");
+            CK(launch_sim_batch_window(host[0].a.m, b->packed, false, dev, blocks, b->n_items, t, steps, b->stream),
+               "batch window");
+        }
+        for (size_t j = 0; j < nj; ++j) {
+            const SimArgs& a = host[j].a;
+            if (b->cfgs_run[j].series_mode != TVBX_SERIES_STREAM || a.n_chunk <= 0) continue;
+            bool ss = shift_set[j] != 0;
+            if (tvbx_status st = stream_fc_chunk(b->jobs[j], a, a.n0, a.n_chunk, ss, b->stream)) return st;
+            shift_set[j] = ss ? 1 : 0;
+        }
+    }
     return TVBX_OK;
 }
 
@@ -1948,45 +2023,49 @@ tvbx_status tvbx_batch_tune(tvbx_batch* b, int64_t trial_steps, int32_t* threads
 {
     if (!b) return fail(TVBX_E_INVALID_ARG, "NULL batch");
     if (trial_steps < 1) return fail(TVBX_E_INVALID_ARG, "trial_steps must be >= 1");
-    // general body under shared-memory budgets, and register tiles (general
-    // body only for jobs with more regions than threads)
-    struct Cand { int32_t threads; size_t budget; bool direct; };
-    const Cand cands[] = {{256, 100 * 1024, false}, {512, 100 * 1024, false}, {256, 200 * 1024, false},
-                          {512, 200 * 1024, false}, {128, 64 * 1024, false},  {256, 64 * 1024, false},
-                          {512, 200 * 1024, true},  {768, 200 * 1024, true}};
+    // general body under shared-memory budgets, register tiles (general body
+    // only for jobs with more regions than threads), and the windowed body
+    // (not among the reported trials)
+    struct Cand { int32_t threads; size_t budget; bool direct, window; };
+    const Cand cands[] = {{256, 100 * 1024, false, false}, {512, 100 * 1024, false, false},
+                          {256, 200 * 1024, false, false}, {512, 200 * 1024, false, false},
+                          {128, 64 * 1024, false, false},  {256, 64 * 1024, false, false},
+                          {512, 200 * 1024, true, false},  {768, 200 * 1024, true, false},
+                          {128, 64 * 1024, false, true}};
     float best = INFINITY;
-    Cand win{0, 0, false};
+    Cand win{0, 0, false, false};
     int32_t k = 0;
     cudaEvent_t e0, e1;
     CK(cudaEventCreate(&e0), "event");
     CK(cudaEventCreate(&e1), "event");
     for (const Cand& c : cands) {
         float ms = INFINITY;
-        if (batch_build(b, c.threads, c.budget, trial_steps, c.direct) == TVBX_OK) {
-            cudaError_t e = cudaGraphLaunch(b->exec, b->stream);   // warm-up
-            if (e == cudaSuccess) e = cudaEventRecord(e0, b->stream);
-            if (e == cudaSuccess) e = cudaGraphLaunch(b->exec, b->stream);
+        if (batch_build(b, c.threads, c.budget, trial_steps, c.direct, c.window) == TVBX_OK) {
+            tvbx_status st = batch_enqueue(b);   // warm-up
+            cudaError_t e = cudaEventRecord(e0, b->stream);
+            if (st == TVBX_OK) st = batch_enqueue(b);
             if (e == cudaSuccess) e = cudaEventRecord(e1, b->stream);
             if (e == cudaSuccess) e = cudaEventSynchronize(e1);
             if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
-            if (e != cudaSuccess) {
+            if (st != TVBX_OK || e != cudaSuccess) {
                 cudaEventDestroy(e0);
                 cudaEventDestroy(e1);
-                return cuda_fail(e, "batch trial");
+                return st != TVBX_OK ? st : cuda_fail(e, "batch trial");
             }
-            note_launch(2 * b->graph_kernels);
         } else {
             (void)cudaGetLastError();
         }
-        if (trial_ms) trial_ms[k] = ms;
-        ++k;
+        if (!c.window) {
+            if (trial_ms) trial_ms[k] = ms;
+            ++k;
+        }
         if (ms < best) { best = ms; win = c; }
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (!(best < INFINITY)) return fail(TVBX_E_UNSUPPORTED, "no batch configuration fits every job");
     if (n_trials) *n_trials = k;
-    tvbx_status st = batch_build(b, win.threads, win.budget, 0, win.direct);
+    tvbx_status st = batch_build(b, win.threads, win.budget, 0, win.direct, win.window);
     if (st != TVBX_OK) return st;
     if (threads_out) *threads_out = win.threads;
     if (smem_kb_out) *smem_kb_out = (int32_t)(win.budget / 1024);
@@ -2001,11 +2080,16 @@ tvbx_status tvbx_batch_run(tvbx_batch* b)
     for (size_t j = 0; j < b->jobs.size() && !stale; ++j) stale = b->jobs[j]->gen != b->gens[j];
     for (size_t j = 0; j < b->jobs.size() && !stale; ++j) stale = b->cfgs_run[j].n_steps != b->cfgs[j].n_steps;
     if (stale) {
-        tvbx_status st = batch_build(b, b->threads, b->smem_budget, 0, b->direct);
+        // untuned: windowed bodies where every job has them, else the general body
+        tvbx_status st = batch_build(b, b->window ? 128 : b->threads, b->smem_budget, 0, b->direct, b->window);
+        if (st != TVBX_OK && b->window) {
+            (void)cudaGetLastError();
+            b->window = false;
+            st = batch_build(b, b->threads, b->smem_budget, 0, b->direct, false);
+        }
         if (st != TVBX_OK) return st;
     }
-    CK(cudaGraphLaunch(b->exec, b->stream), "batch launch");
-    note_launch(b->graph_kernels);
+    if (tvbx_status st = batch_enqueue(b)) return st;
     for (size_t j = 0; j < b->jobs.size(); ++j) {
         b->jobs[j]->stream = b->stream;
         finish_run(b->jobs[j], b->cfgs_run[j]);

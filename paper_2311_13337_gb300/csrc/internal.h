@@ -184,6 +184,9 @@ struct BatchJob {
     SimArgs a;
     int32_t pb;       // tile width of the job
     int32_t direct;   // 1: register-tile body (N pb / 4 <= blockDim), 0: general body
+    int32_t win_steps;   // windowed batches: steps per window
+    int32_t pad;
+    float* far;          // and the far sums' buffer (null: none)
 };
 struct BatchItem {
     int32_t job, tile;
@@ -194,6 +197,16 @@ int sim_direct_pb(int N);
 cudaError_t launch_sim_direct(const SimArgs& a, int32_t n_tiles, int32_t pb, cudaStream_t s);
 cudaError_t launch_sim_batch(const BatchJob* jobs, const BatchItem* items, int32_t n_items, int32_t* head,
                              int32_t grid, int32_t threads, size_t smem, bool only_direct, cudaStream_t s);
+// Batches whose jobs all have windows and the model m (sim_window.cu), in tiles
+// of WIN_BATCH_PB sets: blocks per tile, windows ("turns") of a job per round of
+// n_chunk steps, and one turn of every job (far: the far sums it needs); steps:
+// the longest window.
+constexpr int WIN_BATCH_PB = 64;
+int32_t sim_batch_window_blocks(int32_t N, bool packed);
+int32_t sim_batch_window_turns(int32_t steps, bool far, int32_t n_chunk);
+cudaError_t launch_sim_batch_window(const DevModel& m, bool packed, bool far, const BatchJob* jobs,
+                                    const BatchItem* blocks, int32_t n_blocks, int32_t turn, int32_t steps,
+                                    cudaStream_t s);
 int sim_batch_ctas_per_sm(int32_t threads, size_t smem, bool only_direct);
 
 struct FcArgs {

@@ -99,10 +99,9 @@ struct WinSlot {
     bool act1;
 };
 template <int S>
-__device__ __forceinline__ WinSlot win_slot(const TileDev& tile, int32_t blocks_per_tile)
+__device__ __forceinline__ WinSlot win_slot(const TileDev& tile, int i)   // i: the pair within the tile
 {
-    const int width = (tile.nq + S - 1) / S;   // threads per region
-    const int i = (blockIdx.x % blocks_per_tile) * blockDim.x + threadIdx.x;
+    const int width = (tile.nq + S - 1) / S;   // pairs per region
     WinSlot w;
     w.k = i / width;
     w.q = (i - w.k * width) * S;
@@ -110,10 +109,27 @@ __device__ __forceinline__ WinSlot win_slot(const TileDev& tile, int32_t blocks_
     return w;
 }
 
-// Sums of the entries with d >= WIN_FAR over the WIN_FAR steps from a.n0 on.
-// Bound by the L2 reads of the rows (4 B per weight and step); a launch covers
-// WIN_FAR steps so that the rows that different regions read are mostly the
-// same ones.
+// Sums of a pair's entries with d >= WIN_FAR over the WIN_FAR steps from n0 on,
+// to the tile's far buffer.
+template <class V, int PB>
+__device__ __forceinline__ void far_pair(const SimArgs& a, const TileDev& tile, const GroupDev& grp, const WinSlot ws,
+                                         int pb, uint32_t n0, float* far)
+{
+    const int N = a.N, H = grp.H, HR = H + WIN_FAR;
+    V acc[WIN_FAR];
+#pragma unroll
+    for (int b = 0; b < WIN_FAR; ++b) acc[b] = vbc<V>(0.0f);
+    gather<WIN_FAR>(acc, grp, grp.ring + (int64_t)tile.q0 * N * HR + ws.q, grp.row_ptr[ws.k], grp.row_near[ws.k],
+                    (int)(n0 % (uint32_t)H), H, HR, pb);
+    float* out = far + (int64_t)ws.k * pb + ws.q;
+#pragma unroll
+    for (int b = 0; b < WIN_FAR; ++b) *reinterpret_cast<V*>(out + (int64_t)b * N * pb) = acc[b];
+}
+
+// The far sums of every pair from step a.n0 on. Bound by the L2 reads of the
+// rows (4 B per weight and step; 72% of the L2 rate on 1,024 x 360); a launch
+// covers WIN_FAR steps so that the rows that different regions read are mostly
+// the same ones (85% L2 hits).
 template <class V, int PB>
 __global__ void __launch_bounds__(WIN_THREADS, 4)
 sim_far_kernel(const __grid_constant__ SimArgs a, int32_t pb_rt, int32_t blocks_per_tile, float* __restrict__ far)
@@ -121,51 +137,34 @@ sim_far_kernel(const __grid_constant__ SimArgs a, int32_t pb_rt, int32_t blocks_
     const int pb = PB > 0 ? PB : pb_rt;
     const int32_t ti = blockIdx.x / blocks_per_tile;
     const TileDev tile = a.tiles[ti];
-    const GroupDev& grp = a.groups[tile.group];
-    const int N = a.N;
-    const WinSlot w = win_slot<VSets<V>::n>(tile, blocks_per_tile);
-    if (w.k >= N) return;
-    const int H = grp.H, HR = H + WIN_FAR;
-    V acc[WIN_FAR];
-#pragma unroll
-    for (int b = 0; b < WIN_FAR; ++b) acc[b] = vbc<V>(0.0f);
-    gather<WIN_FAR>(acc, grp, grp.ring + (int64_t)tile.q0 * N * HR + w.q, grp.row_ptr[w.k], grp.row_near[w.k],
-                    (int)((uint32_t)a.n0 % (uint32_t)H), H, HR, pb);
-    float* out = far + ((int64_t)ti * WIN_FAR * N + w.k) * pb + w.q;
-#pragma unroll
-    for (int b = 0; b < WIN_FAR; ++b) *reinterpret_cast<V*>(out + (int64_t)b * N * pb) = acc[b];
+    const WinSlot ws = win_slot<VSets<V>::n>(tile, (blockIdx.x % blocks_per_tile) * blockDim.x + threadIdx.x);
+    if (ws.k >= a.N) return;
+    far_pair<V, PB>(a, tile, a.groups[tile.group], ws, pb, (uint32_t)a.n0, far + (int64_t)ti * WIN_FAR * a.N * pb);
 }
 
-// One window of a.n_chunk steps. PB: sets per tile (0: the runtime width
-// pb_rt). NEAR: the sums start from far (row 0: the window's first step) and
-// add the nearer entries.
+// One window of `steps` steps of one thread's pair (region ws.k of sets
+// tile.q0 + ws.q, + 1) from step n0. NEAR: the sums start from far (the
+// tile's row of the window's first step) and add the nearer entries. m: the
+// model, in constant memory. stash: this thread's coupling sums, a step every
+// WIN_THREADS.
 template <class V, int PB, bool NEAR>
-__global__ void __launch_bounds__(WIN_THREADS, 4)
-sim_window_kernel(const __grid_constant__ SimArgs a, int32_t pb_rt, int32_t blocks_per_tile, int64_t table_step,
-                  const float* __restrict__ far)
+__device__ __forceinline__ void window_pair(const SimArgs& a, const DevModel& m, const TileDev& tile,
+                                            const GroupDev& grp, const WinSlot ws, int pb, uint32_t n0, int steps,
+                                            int64_t table_step, const float* far, V* stash)
 {
     constexpr int S = VSets<V>::n;
-    const int pb = PB > 0 ? PB : pb_rt;
-    extern __shared__ __align__(16) unsigned char win_smem[];
-    V* stash = reinterpret_cast<V*>(win_smem) + threadIdx.x;   // coupling of step b at stash[b * blockDim.x]
-    const int32_t ti = blockIdx.x / blocks_per_tile;
-    const TileDev tile = a.tiles[ti];
-    const GroupDev& grp = a.groups[tile.group];
-    const int N = a.N;
-    const WinSlot ws = win_slot<S>(tile, blocks_per_tile);
-    const int k = ws.k, q = ws.q;
+    const int N = a.N, k = ws.k, q = ws.q;
     const bool act1 = ws.act1;
-    if (k >= N) return;
     const int H = grp.H, HR = H + WIN_FAR;
-    const uint32_t n0 = (uint32_t)a.n0;
-    const int steps = a.n_chunk;
     const int slot0 = (int)(n0 % (uint32_t)H);
     float* ring = grp.ring + (int64_t)tile.q0 * N * HR + q;
+    const int ts = a.ts;
+    const bool own_noise = a.noise_per_set != 0;
 
     // 1. coupling sums of the window
     {
         const int e0 = NEAR ? grp.row_near[k] : grp.row_ptr[k], e1 = grp.row_mid[k];
-        const float* far_k = NEAR ? far + ((int64_t)ti * WIN_FAR * N + k) * pb + q : nullptr;
+        const float* far_k = NEAR ? far + (int64_t)k * pb + q : nullptr;
         int b0 = 0;
         auto pass = [&](auto g_c) {
             constexpr int G = decltype(g_c)::value;
@@ -178,7 +177,7 @@ sim_window_kernel(const __grid_constant__ SimArgs a, int32_t pb_rt, int32_t bloc
                 at -= at >= H ? H : 0;
                 gather<G>(acc, grp, ring, e0, e1, at, H, HR, pb);
 #pragma unroll
-                for (int b = 0; b < G; ++b) stash[(b0 + b) * blockDim.x] = acc[b];
+                for (int b = 0; b < G; ++b) stash[(b0 + b) * WIN_THREADS] = acc[b];
             }
         };
         pass(std::integral_constant<int, 8>{});
@@ -188,7 +187,6 @@ sim_window_kernel(const __grid_constant__ SimArgs a, int32_t pb_rt, int32_t bloc
     }
 
     // 2. the window's steps
-    const DevModel& m = a.m;
     const int64_t NP = (int64_t)N * a.P;
     const int64_t p = grp.p_base + tile.q0 + q;
     float* st = a.state + (int64_t)k * a.P + p;
@@ -222,7 +220,7 @@ sim_window_kernel(const __grid_constant__ SimArgs a, int32_t pb_rt, int32_t bloc
     load_v(accE, st + SV_ACC_E * NP, true, act1);
     load_v(accI, st + SV_ACC_I * NP, true, act1);
     uint32_t pn[2] = {0u, 0u};
-    if (a.noise_per_set) {
+    if (own_noise) {
         load_v(ou, st + SV_OU * NP, true, act1);
         pn[0] = (uint32_t)(a.p_offset + a.ext_index[p]);
         if (S > 1 && act1) pn[1] = (uint32_t)(a.p_offset + a.ext_index[p + 1]);
@@ -230,18 +228,18 @@ sim_window_kernel(const __grid_constant__ SimArgs a, int32_t pb_rt, int32_t bloc
         ou = vbc<V>(0.0f);
     }
     Track<V> trk = track_init<V>();
-    const float inv_ts = 1.0f / (float)a.ts;
+    const float inv_ts = 1.0f / (float)ts;
     // samples are the means of ts post-step states: steps left to the next one, and its index
-    int left = a.ts - (int)(n0 % (uint32_t)a.ts);
-    int64_t t = n0 / (uint32_t)a.ts;
+    int left = ts - (int)(n0 % (uint32_t)ts);
+    int64_t t = n0 / (uint32_t)ts;
     int slot_w = slot0;
     float* const ring_k = ring + (uint32_t)(k * HR) * (uint32_t)pb;
-    const float* ou_p = a.ou_table + (a.noise_per_set ? 0 : table_step * N + k);
+    const float* ou_p = a.ou_table + (own_noise ? 0 : table_step * N + k);
     for (int b = 0; b < steps; ++b) {
-        const V OU = a.noise_per_set ? ou : vbc<V>(__ldg(ou_p));
-        ou_p += a.noise_per_set ? 0 : N;
-        pair_step(m, sp, x, stash[b * blockDim.x], OU, trk);
-        if (a.noise_per_set) {
+        const V OU = own_noise ? ou : vbc<V>(__ldg(ou_p));
+        ou_p += own_noise ? 0 : N;
+        pair_step(m, sp, x, stash[b * WIN_THREADS], OU, trk);
+        if (own_noise) {
 #pragma unroll
             for (int l = 0; l < S; ++l)
                 set_lane(ou, l, next_ou(m, a.seed, n0 + (uint32_t)b, (uint32_t)k, pn[l], lane(OU, l)));
@@ -274,7 +272,7 @@ sim_window_kernel(const __grid_constant__ SimArgs a, int32_t pb_rt, int32_t bloc
                     }
                 }
             }
-            left = a.ts;
+            left = ts;
             ++t;
             accE = vbc<V>(0.0f);
             accI = vbc<V>(0.0f);
@@ -291,11 +289,94 @@ sim_window_kernel(const __grid_constant__ SimArgs a, int32_t pb_rt, int32_t bloc
     store_v(st + SV_CWI * NP, x.cWi, act1);
     store_v(st + SV_ACC_E * NP, accE, act1);
     store_v(st + SV_ACC_I * NP, accI, act1);
-    if (a.noise_per_set) store_v(st + SV_OU * NP, ou, act1);
+    if (own_noise) store_v(st + SV_OU * NP, ou, act1);
 #pragma unroll
     for (int l = 0; l < S; ++l) {
         const uint32_t f = track_flags(m, trk, l);
         if (f && (l == 0 || act1)) atomicOr(a.status + p + l, f);
+    }
+}
+
+// One window of a.n_chunk steps from step a.n0. PB: sets per tile (0: the
+// runtime width pb_rt).
+template <class V, int PB, bool NEAR>
+__global__ void __launch_bounds__(WIN_THREADS, 4)
+sim_window_kernel(const __grid_constant__ SimArgs a, int32_t pb_rt, int32_t blocks_per_tile, int64_t table_step,
+                  const float* __restrict__ far)
+{
+    extern __shared__ __align__(16) unsigned char win_smem[];
+    const int pb = PB > 0 ? PB : pb_rt;
+    const int32_t ti = blockIdx.x / blocks_per_tile;
+    const TileDev tile = a.tiles[ti];
+    const WinSlot ws = win_slot<VSets<V>::n>(tile, (blockIdx.x % blocks_per_tile) * blockDim.x + threadIdx.x);
+    if (ws.k >= a.N) return;
+    window_pair<V, PB, NEAR>(a, a.m, tile, a.groups[tile.group], ws, pb, (uint32_t)a.n0, a.n_chunk, table_step,
+                             NEAR ? far + (int64_t)ti * WIN_FAR * a.N * pb : nullptr,
+                             reinterpret_cast<V*>(win_smem) + threadIdx.x);
+}
+
+// Window `turn` of a job: its first step within the round, its length (0: the
+// round is over) and its first row of the far sums. A window stays within the
+// WIN_FAR steps whose far sums are at hand.
+struct WinTurn {
+    int w0, len, row;
+};
+__host__ __device__ __forceinline__ WinTurn win_turn(int turn, int steps, bool far, int n_chunk)
+{
+    WinTurn t;
+    t.row = 0;
+    if (far) {
+        const int per = (WIN_FAR + steps - 1) / steps;   // windows per far block
+        t.row = turn % per * steps;
+        t.w0 = turn / per * WIN_FAR + t.row;
+        t.len = WIN_FAR - t.row < steps ? WIN_FAR - t.row : steps;
+    } else {
+        t.w0 = turn * steps;
+        t.len = steps;
+    }
+    if (t.len > n_chunk - t.w0) t.len = n_chunk - t.w0 > 0 ? n_chunk - t.w0 : 0;
+    return t;
+}
+
+// A batch of sweeps that all have windows and share the model m: one launch
+// takes every job through its window `turn` (FAR: forms the far sums of the
+// jobs that start a far block with it). blocks[i] names block i's job and its
+// index among the job's blocks. The register-tile body, whose CTAs keep a tile
+// of 4 to 28 sets through a whole round, took 19.4 ms of an eight-job batch of
+// 64 to 1,024 sets; a windowed body over such tiles reads rows of 16 bytes and
+// took 34 ms.
+template <class V, bool FAR>
+__global__ void __launch_bounds__(WIN_THREADS, 4)
+sim_batch_window_kernel(const __grid_constant__ DevModel m, const BatchJob* __restrict__ jobs,
+                        const BatchItem* __restrict__ blocks, int32_t turn)
+{
+    extern __shared__ __align__(16) unsigned char win_smem[];
+    __shared__ BatchJob s_job;
+    constexpr int S = VSets<V>::n;
+    const BatchItem bi = blocks[blockIdx.x];
+    const uint32_t* src = reinterpret_cast<const uint32_t*>(jobs + bi.job);
+    uint32_t* dst = reinterpret_cast<uint32_t*>(&s_job);
+    for (int w = threadIdx.x; w < (int)(sizeof(BatchJob) / 4); w += WIN_THREADS) dst[w] = src[w];
+    __syncthreads();
+    const SimArgs& a = s_job.a;
+    const WinTurn t = win_turn(turn, s_job.win_steps, s_job.far != nullptr, a.n_chunk);
+    if (t.len == 0 || (FAR && (!s_job.far || t.row != 0))) return;
+    const int N = a.N, bpt = (N * (WIN_BATCH_PB / S) + WIN_THREADS - 1) / WIN_THREADS;
+    const int ti = bi.tile / bpt;
+    const TileDev tile = a.tiles[ti];
+    const GroupDev grp = a.groups[tile.group];
+    const WinSlot ws = win_slot<S>(tile, (bi.tile - ti * bpt) * WIN_THREADS + threadIdx.x);
+    if (ws.k >= N) return;
+    const uint32_t n0 = (uint32_t)a.n0 + (uint32_t)t.w0;
+    float* far = s_job.far ? s_job.far + (int64_t)ti * WIN_FAR * N * WIN_BATCH_PB : nullptr;
+    V* stash = reinterpret_cast<V*>(win_smem) + threadIdx.x;
+    if constexpr (FAR) {
+        far_pair<V, WIN_BATCH_PB>(a, tile, grp, ws, WIN_BATCH_PB, n0, far);
+    } else if (far) {
+        window_pair<V, WIN_BATCH_PB, true>(a, m, tile, grp, ws, WIN_BATCH_PB, n0, t.len, t.w0,
+                                           far + (int64_t)t.row * N * WIN_BATCH_PB, stash);
+    } else {
+        window_pair<V, WIN_BATCH_PB, false>(a, m, tile, grp, ws, WIN_BATCH_PB, n0, t.len, t.w0, nullptr, stash);
     }
 }
 
@@ -338,7 +419,7 @@ cudaError_t launch_v(const SimArgs& a, const WindowPlan& w, int32_t n_tiles, int
     const int64_t per_tile = (int64_t)a.N * ((w.pb + S - 1) / S);
     const int32_t bpt = (int32_t)((per_tile + w.threads - 1) / w.threads);
     const unsigned grid = (unsigned)((int64_t)n_tiles * bpt);
-    const size_t smem = sizeof(V) * (size_t)w.threads * a.n_chunk;
+    const size_t smem = sizeof(V) * (size_t)WIN_THREADS * a.n_chunk;
     if (w.far) {
         if (far_row == 0) {
             note_launch();
@@ -379,6 +460,31 @@ cudaError_t launch_sim_window(const SimArgs& a, const WindowPlan& w, int32_t n_t
     if (w.packed) return w.pb == 64 ? launch_v<float2, 64>(a, w, n_tiles, table_step, far, far_row, s)
                                     : launch_v<float2, 0>(a, w, n_tiles, table_step, far, far_row, s);
     return launch_v<float, 0>(a, w, n_tiles, table_step, far, far_row, s);
+}
+
+int32_t sim_batch_window_blocks(int32_t N, bool packed)
+{
+    return (N * (packed ? WIN_BATCH_PB / 2 : WIN_BATCH_PB) + WIN_THREADS - 1) / WIN_THREADS;
+}
+
+int32_t sim_batch_window_turns(int32_t steps, bool far, int32_t n_chunk)
+{
+    if (n_chunk <= 0) return 0;
+    if (!far) return (n_chunk + steps - 1) / steps;
+    const int32_t per = (WIN_FAR + steps - 1) / steps, rest = n_chunk % WIN_FAR;
+    return n_chunk / WIN_FAR * per + (rest + steps - 1) / steps;
+}
+
+cudaError_t launch_sim_batch_window(const DevModel& m, bool packed, bool far, const BatchJob* jobs,
+                                    const BatchItem* blocks, int32_t n_blocks, int32_t turn, int32_t steps,
+                                    cudaStream_t s)
+{
+    if (n_blocks <= 0) return cudaSuccess;
+    auto kern = packed ? (far ? sim_batch_window_kernel<float2, true> : sim_batch_window_kernel<float2, false>)
+                       : (far ? sim_batch_window_kernel<float, true> : sim_batch_window_kernel<float, false>);
+    note_launch();
+    kern<<<n_blocks, WIN_THREADS, far ? 0 : (packed ? 8 : 4) * (size_t)WIN_THREADS * steps, s>>>(m, jobs, blocks, turn);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_ring_convert(bool out, float* ring, const WindowPlan& w, int32_t H, int32_t N, int32_t P_g,
