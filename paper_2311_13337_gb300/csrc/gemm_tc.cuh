@@ -13,15 +13,18 @@
 // these K.
 //
 // Layout. A CTA of 128 threads owns a 128 x 128 tile of C. Per chunk of 64
-// K (one 128-byte row of BF16) thread t reads row t of the A tile and row t
-// of the B tile from global memory (any strides: the backward products read
-// transposed operands), splits, and writes the parts to shared memory in the
-// 128-byte swizzled K-major layout; one thread then issues the MMAs of the
-// four 16-wide K slices and commits them to an mbarrier that every thread
-// waits on (bounded) before the next chunk overwrites the operands. The
-// accumulator (128 lanes x up to 128 FP32 columns) is read back by the four
-// warps, each its 32 lanes (rows), and stored with the epilogue. Rows and
-// columns beyond M, N and K are staged as zeros.
+// K (one 128-byte row of BF16) the threads read their shares of the A and B
+// tiles (lanes along K where K is contiguous, else along the rows: the backward
+// products read transposed operands) into registers, split, and write the
+// parts to shared memory in the 128-byte swizzled K-major layout; one thread
+// then issues the MMAs of the four 16-wide K slices and commits them to an
+// mbarrier; the next chunk is read under them, and every thread waits (bounded)
+// before it overwrites the operands. The accumulator (128 lanes x up to 128
+// FP32 columns) is read back by the four warps, each its 32 lanes (rows), and
+// stored with the epilogue along the rows. Rows and columns beyond M, N and K
+// are staged as zeros. The products are small (1,024 x 256 x 256 per member)
+// and bound by latency: a row per thread, read and written 4 bytes at a time,
+// measured 113, 53 and 31 us for the masked, forward and weight products.
 //
 // Split K. A product with few output tiles and a long K (the weight
 // gradients: K = the mini-batch rows) would occupy a handful of SMs, so its
@@ -60,38 +63,158 @@ static __device__ __forceinline__ uint32_t tcg_pack2(__nv_bfloat16 a, __nv_bfloa
     return (uint32_t)__bfloat16_as_ushort(a) | ((uint32_t)__bfloat16_as_ushort(b) << 16);
 }
 
-// Row r (of R valid rows) of an operand tile, K chunk k0 (of K), split into
-// BF16 parts and written to the swizzled tiles at sh (high) and sl (low).
-template <typename T>
-static __device__ __forceinline__ void tcg_stage_row(const T* X, int64_t s_row, int64_t s_k, int64_t row0, int r,
-                                                     int R, int k0, int K, uint32_t sh, uint32_t sl)
+// Registers of one thread's share of an operand chunk (128 rows x 64 K).
+template <typename T> struct TcgRegs {
+    uint32_t v[16 * sizeof(T)];   // FP32: 64 values; BF16: 64 values in pairs
+};
+
+// Load the chunk [0, 128) x [k0, k0 + 64) of an operand of R valid rows and K
+// columns; zeros beyond. X points at row 0. K-contiguous operands (s_k == 1):
+// lanes along the row, 16 bytes each (vec: rows start 16-byte aligned), else
+// lanes along the rows, which are then neighbours (s_row == 1).
+static __device__ __forceinline__ void tcg_load(TcgRegs<float>& f, const float* X, int64_t s_row, int64_t s_k, bool vec,
+                                                int R, int k0, int K)
 {
-    const bool rok = r < R;
+    const int t = threadIdx.x;
+    if (s_k == 1) {
 #pragma unroll
-    for (int c = 0; c < 8; ++c) {   // 16-byte chunks of 8 BF16
-        uint32_t h[4], l[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            __nv_bfloat16 hv[2], lv[2];
-#pragma unroll
-            for (int u = 0; u < 2; ++u) {
-                const int k = k0 + c * 8 + q * 2 + u;
-                const float x = (rok && k < K) ? ldf(X, (row0 + r) * s_row + (int64_t)k * s_k) : 0.0f;
-                hv[u] = __float2bfloat16_rn(x);
-                lv[u] = __float2bfloat16_rn(x - __bfloat162float(hv[u]));
+        for (int p = 0; p < 16; ++p) {
+            const int r = 8 * p + (t >> 4), k = k0 + 4 * (t & 15);
+            float4 x = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            if (r < R) {
+                const float* at = X + r * s_row + k;
+                if (vec && k + 4 <= K) {
+                    x = *reinterpret_cast<const float4*>(at);
+                } else {
+                    if (k < K) x.x = at[0];
+                    if (k + 1 < K) x.y = at[1];
+                    if (k + 2 < K) x.z = at[2];
+                    if (k + 3 < K) x.w = at[3];
+                }
             }
-            h[q] = tcg_pack2(hv[0], hv[1]);
-            l[q] = tcg_pack2(lv[0], lv[1]);
+            f.v[4 * p] = __float_as_uint(x.x);
+            f.v[4 * p + 1] = __float_as_uint(x.y);
+            f.v[4 * p + 2] = __float_as_uint(x.z);
+            f.v[4 * p + 3] = __float_as_uint(x.w);
         }
-        const uint32_t off = tcg_sw_off(r, c * 8);
-        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};\n" ::"r"(sh + off), "r"(h[0]), "r"(h[1]), "r"(h[2]),
-                     "r"(h[3])
-                     : "memory");
-        if (sl) {
-            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};\n" ::"r"(sl + off), "r"(l[0]), "r"(l[1]),
-                         "r"(l[2]), "r"(l[3])
-                         : "memory");
+    } else {
+#pragma unroll
+        for (int k = 0; k < TCG_K; ++k)
+            f.v[k] = t < R && k0 + k < K ? __float_as_uint(X[t * s_row + (k0 + k) * s_k]) : 0u;
+    }
+}
+static __device__ __forceinline__ void tcg_load(TcgRegs<__nv_bfloat16>& f, const __nv_bfloat16* X, int64_t s_row,
+                                                int64_t s_k, bool vec, int R, int k0, int K)
+{
+    const int t = threadIdx.x;
+    const uint16_t* U = reinterpret_cast<const uint16_t*>(X);
+    if (s_k == 1) {
+#pragma unroll
+        for (int p = 0; p < 8; ++p) {
+            const int r = 16 * p + (t >> 3), k = k0 + 8 * (t & 7);
+            uint4 x = make_uint4(0u, 0u, 0u, 0u);
+            if (r < R) {
+                const uint16_t* at = U + r * s_row + k;
+                if (vec && k + 8 <= K) {
+                    x = *reinterpret_cast<const uint4*>(at);
+                } else {
+                    uint32_t w[4];
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+                        w[q] = (k + 2 * q < K ? at[2 * q] : 0u) | (k + 2 * q + 1 < K ? (uint32_t)at[2 * q + 1] << 16 : 0u);
+                    x = make_uint4(w[0], w[1], w[2], w[3]);
+                }
+            }
+            f.v[4 * p] = x.x;
+            f.v[4 * p + 1] = x.y;
+            f.v[4 * p + 2] = x.z;
+            f.v[4 * p + 3] = x.w;
         }
+    } else {
+        // lanes along K, two K of eight neighbouring rows each: 4 pairs (k, k + 1)
+        // of row group (t >> 5) + 4 p, in f.v[8 p + row]
+#pragma unroll
+        for (int p = 0; p < 4; ++p) {
+            const int r = 8 * ((t >> 5) + 4 * p), k = k0 + 2 * (t & 31);
+            uint32_t w[2][4];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const uint16_t* at = U + r + (k + h) * s_k;
+                if (k + h >= K) {
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) w[h][q] = 0u;
+                } else if (vec && r + 8 <= R) {
+                    const uint4 x = *reinterpret_cast<const uint4*>(at);
+                    w[h][0] = x.x; w[h][1] = x.y; w[h][2] = x.z; w[h][3] = x.w;
+                } else {
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+                        w[h][q] = (r + 2 * q < R ? at[2 * q] : 0u) | (r + 2 * q + 1 < R ? (uint32_t)at[2 * q + 1] << 16 : 0u);
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                f.v[8 * p + 2 * q] = __byte_perm(w[0][q], w[1][q], 0x5410);
+                f.v[8 * p + 2 * q + 1] = __byte_perm(w[0][q], w[1][q], 0x7632);
+            }
+        }
+    }
+}
+
+// Split the loaded values into BF16 parts and write them to the swizzled tiles
+// at sh (high) and sl (low; a BF16 operand has none).
+static __device__ __forceinline__ void tcg_split2(float x, float y, uint32_t& h, uint32_t& l)
+{
+    const __nv_bfloat16 hx = __float2bfloat16_rn(x), hy = __float2bfloat16_rn(y);
+    h = tcg_pack2(hx, hy);
+    l = tcg_pack2(__float2bfloat16_rn(x - __bfloat162float(hx)), __float2bfloat16_rn(y - __bfloat162float(hy)));
+}
+static __device__ __forceinline__ void tcg_store4(uint32_t at, uint32_t a, uint32_t b, uint32_t c, uint32_t d)
+{
+    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};\n" ::"r"(at), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
+}
+static __device__ __forceinline__ void tcg_put(const TcgRegs<float>& f, int64_t s_k, uint32_t sh, uint32_t sl)
+{
+    const int t = threadIdx.x;
+    if (s_k == 1) {
+#pragma unroll
+        for (int p = 0; p < 16; ++p) {
+            uint32_t h[2], l[2];
+            tcg_split2(__uint_as_float(f.v[4 * p]), __uint_as_float(f.v[4 * p + 1]), h[0], l[0]);
+            tcg_split2(__uint_as_float(f.v[4 * p + 2]), __uint_as_float(f.v[4 * p + 3]), h[1], l[1]);
+            const uint32_t off = tcg_sw_off(8 * p + (t >> 4), 4 * (t & 15));
+            asm volatile("st.shared.v2.b32 [%0], {%1, %2};\n" ::"r"(sh + off), "r"(h[0]), "r"(h[1]) : "memory");
+            asm volatile("st.shared.v2.b32 [%0], {%1, %2};\n" ::"r"(sl + off), "r"(l[0]), "r"(l[1]) : "memory");
+        }
+    } else {
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+            uint32_t h[4], l[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                tcg_split2(__uint_as_float(f.v[8 * c + 2 * q]), __uint_as_float(f.v[8 * c + 2 * q + 1]), h[q], l[q]);
+            const uint32_t off = tcg_sw_off(t, 8 * c);
+            tcg_store4(sh + off, h[0], h[1], h[2], h[3]);
+            tcg_store4(sl + off, l[0], l[1], l[2], l[3]);
+        }
+    }
+}
+static __device__ __forceinline__ void tcg_put(const TcgRegs<__nv_bfloat16>& f, int64_t s_k, uint32_t sh, uint32_t)
+{
+    const int t = threadIdx.x;
+    if (s_k == 1) {
+#pragma unroll
+        for (int c = 0; c < 8; ++c)
+            tcg_store4(sh + tcg_sw_off(16 * c + (t >> 3), 8 * (t & 7)), f.v[4 * c], f.v[4 * c + 1], f.v[4 * c + 2],
+                       f.v[4 * c + 3]);
+    } else {
+#pragma unroll
+        for (int p = 0; p < 4; ++p)
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+                asm volatile("st.shared.b32 [%0], %1;\n" ::"r"(sh + tcg_sw_off(8 * ((t >> 5) + 4 * p) + i, 2 * (t & 31))),
+                             "r"(f.v[8 * p + i])
+                             : "memory");
     }
 }
 
@@ -133,13 +256,22 @@ __global__ void __launch_bounds__(TCG_THREADS) mlp_gemm_tc_kernel(const GemmArgs
     tc_fence_after();
     const uint32_t tmem = tmem_slot;
 
+    const TA* Am = A + (int64_t)m0 * g.sam;
+    const TB* Bn = B + (int64_t)n0 * g.sbn;
+    // 16-byte pieces along the contiguous direction
+    const bool a_vec = (reinterpret_cast<uintptr_t>(Am) & 15) == 0 && (g.sak == 1 ? g.sam : g.sak) * sizeof(TA) % 16 == 0;
+    const bool b_vec = (reinterpret_cast<uintptr_t>(Bn) & 15) == 0 && (g.sbk == 1 ? g.sbn : g.sbk) * sizeof(TB) % 16 == 0;
+    TcgRegs<TA> ra;
+    TcgRegs<TB> rb;
+
     uint32_t parity = 0;
     const int n_chunks = (g.K + TCG_K - 1) / TCG_K;
     const int ch0 = split * chunks_per_split, ch1 = min(n_chunks, ch0 + chunks_per_split);   // ch0 < ch1 (host)
+    tcg_load(ra, Am, g.sam, g.sak, a_vec, g.M - m0, ch0 * TCG_K, g.K);
+    tcg_load(rb, Bn, g.sbn, g.sbk, b_vec, g.N - n0, ch0 * TCG_K, g.K);
     for (int ch = ch0; ch < ch1; ++ch) {
-        const int k0 = ch * TCG_K;
-        tcg_stage_row(A, g.sam, g.sak, m0, t, g.M - m0, k0, g.K, sAh, A_SPLIT ? sAl : 0u);
-        tcg_stage_row(B, g.sbn, g.sbk, n0, t, g.N - n0, k0, g.K, sBh, B_SPLIT ? sBl : 0u);
+        tcg_put(ra, g.sak, sAh, sAl);
+        tcg_put(rb, g.sbk, sBh, sBl);
         fence_proxy_async_shared();   // the operand writes, visible to the tensor cores
         __syncthreads();
         if (t == 0 && !abort_flag) {
@@ -154,6 +286,10 @@ __global__ void __launch_bounds__(TCG_THREADS) mlp_gemm_tc_kernel(const GemmArgs
             }
             tc_commit(&mbar);
         }
+        if (ch + 1 < ch1) {   // the next chunk, under the MMAs
+            tcg_load(ra, Am, g.sam, g.sak, a_vec, g.M - m0, (ch + 1) * TCG_K, g.K);
+            tcg_load(rb, Bn, g.sbn, g.sbk, b_vec, g.N - n0, (ch + 1) * TCG_K, g.K);
+        }
         // every thread: wait (bounded) until the MMAs have read the operands
         if (!abort_flag && !mbar_wait_bounded(&mbar, parity, wait_limit)) {
             atomicOr(error, TVBX_DEVERR_TIMEOUT);
@@ -165,8 +301,9 @@ __global__ void __launch_bounds__(TCG_THREADS) mlp_gemm_tc_kernel(const GemmArgs
     }
 
     // epilogue: warp w drains accumulator lanes 32 w .. 32 w + 31 (rows of C)
-    const int warp = t >> 5;
-    const int m = m0 + t;   // = m0 + 32 warp + lane
+    // to the operands' shared memory, 16-byte pieces swizzled by the row, and
+    // writes its rows from there, lanes along the columns
+    const int warp = t >> 5, lane = t & 31;
     float* C = g.C + mem * g.c_mem;
     int64_t ldc = g.ldc;
     if (part) {   // split K: this split's partial tile, [split][member][M][N]
@@ -175,19 +312,60 @@ __global__ void __launch_bounds__(TCG_THREADS) mlp_gemm_tc_kernel(const GemmArgs
         ldc = g.N;
     }
     if (!abort_flag) {
+        auto piece = [&](int row, int c) { return base + (uint32_t)(row * 4 * TCG_N + ((c ^ (row & 31)) << 4)); };
         for (int cb = 0; cb * 16 < nvalid; ++cb) {
             float v[16];
             tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(cb * 16), v);
-            if (m < g.M) {
 #pragma unroll
-                for (int i = 0; i < 16; ++i) {
-                    const int n = n0 + cb * 16 + i;
-                    if (n >= g.N) continue;
-                    float x = v[i];
-                    if (EPI == EPI_BIAS || EPI == EPI_BIAS_RELU) x += g.bias[mem * g.bias_mem + n];
-                    if (EPI == EPI_BIAS_RELU) x = fmaxf(x, 0.0f);
-                    if (EPI == EPI_MASK && !(g.mask[mem * g.mask_mem + (int64_t)m * g.ldm + n] > 0.0f)) x = 0.0f;
-                    C[(int64_t)m * ldc + n] = x;
+            for (int q = 0; q < 4; ++q)
+                tcg_store4(piece(t, 4 * cb + q), __float_as_uint(v[4 * q]), __float_as_uint(v[4 * q + 1]),
+                           __float_as_uint(v[4 * q + 2]), __float_as_uint(v[4 * q + 3]));
+        }
+        __syncwarp();
+        const int n = n0 + 4 * lane;
+        const int left = g.N - n;
+        const float* mask = EPI == EPI_MASK ? g.mask + mem * g.mask_mem + n : nullptr;
+        const bool vec = left >= 4 && ldc % 4 == 0 && (reinterpret_cast<uintptr_t>(C + n) & 15) == 0 &&
+                         (EPI != EPI_MASK || (g.ldm % 4 == 0 && (reinterpret_cast<uintptr_t>(mask) & 15) == 0));
+        float bias[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+        if (EPI == EPI_BIAS || EPI == EPI_BIAS_RELU)
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                if (i < left) bias[i] = g.bias[mem * g.bias_mem + n + i];
+        const int rows = min(32, g.M - m0 - 32 * warp);
+        if (left > 0) {
+#pragma unroll 4
+            for (int r = 0; r < rows; ++r) {
+                const int row = 32 * warp + r;
+                float x[4];
+                asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];\n"
+                             : "=f"(x[0]), "=f"(x[1]), "=f"(x[2]), "=f"(x[3])
+                             : "r"(piece(row, lane)));
+                float* out = C + (int64_t)(m0 + row) * ldc + n;
+                float mk[4] = {1.0f, 1.0f, 1.0f, 1.0f};
+                if (EPI == EPI_MASK) {
+                    const float* at = mask + (int64_t)(m0 + row) * g.ldm;
+                    if (vec) {
+                        const float4 q = *reinterpret_cast<const float4*>(at);
+                        mk[0] = q.x; mk[1] = q.y; mk[2] = q.z; mk[3] = q.w;
+                    } else {
+#pragma unroll
+                        for (int i = 0; i < 4; ++i)
+                            if (i < left) mk[i] = at[i];
+                    }
+                }
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    if (EPI == EPI_BIAS || EPI == EPI_BIAS_RELU) x[i] += bias[i];
+                    if (EPI == EPI_BIAS_RELU) x[i] = fmaxf(x[i], 0.0f);
+                    if (EPI == EPI_MASK && !(mk[i] > 0.0f)) x[i] = 0.0f;
+                }
+                if (vec) {
+                    *reinterpret_cast<float4*>(out) = make_float4(x[0], x[1], x[2], x[3]);
+                } else {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+                        if (i < left) out[i] = x[i];
                 }
             }
         }
@@ -205,6 +383,7 @@ __global__ void mlp_splitk_reduce_kernel(const float* __restrict__ part, int spl
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
         const int64_t mem = i / MN, r = i % MN;
         float acc = 0.0f;
+#pragma unroll 8
         for (int sp = 0; sp < splits; ++sp) acc += part[((int64_t)sp * E + mem) * MN + r];
         C[mem * c_mem + (r / N) * ldc + r % N] = acc;
     }

@@ -141,6 +141,7 @@ __global__ void mlp_bias_grad_kernel(const float* __restrict__ dz, int rows, int
     const int q = threadIdx.x >> 5;
     float s = 0.0f;
     if (o < n_out)
+#pragma unroll 16
         for (int r = q; r < rows; r += 8) s += dz[((int64_t)m * rows + r) * n_out + o];
     __shared__ float red[8][33];
     red[q][threadIdx.x & 31] = s;
