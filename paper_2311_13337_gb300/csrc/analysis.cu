@@ -1088,7 +1088,7 @@ extern "C" tvbx_status tvbx_phfcd(const float* bold, int32_t n_regions, int64_t 
     ACK(scr.get(&U, (size_t)B * Tp * N), "phFCD phasors");
     ACK(cudaMemcpyAsync(tw, htw.data(), sizeof(float2) * htw.size(), cudaMemcpyHostToDevice, s), "phFCD twiddles");
     int S = 1;   // sets per CTA of the phase kernel
-    while (S < 8 && 2 * S * n <= AN_MAX_T / 2 && 2 * S <= P) S *= 2;
+    while (S < 8 && 2 * S * n <= AN_MAX_T / 2) S *= 2;
     const size_t smem_phase = sizeof(float2) * (size_t)n * S;
     ACK(cudaFuncSetAttribute(an_phase_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_phase),
         "phFCD shared memory");

@@ -416,7 +416,6 @@ tvbx_status build_groups(tvbx_sweep* h, double dt, std::vector<Group>& groups)
     }
     const int N = h->N;
     // delay in steps: rint (ties to even) of length / (speed dt), in FP64
-    int32_t d_min = INT32_MAX;
     for (Group& g : groups) {
         for (size_t i = 0; i < h->W.size(); ++i) {
             if (h->W[i] == 0.0) continue;
@@ -424,11 +423,10 @@ tvbx_status build_groups(tvbx_sweep* h, double dt, std::vector<Group>& groups)
             if (steps > 65533.0) return fail(TVBX_E_UNSUPPORTED, "delay of %g steps exceeds 65533", steps);
             g.d_min = std::min(g.d_min, steps < 0 ? 0 : (int32_t)steps);
         }
-        d_min = std::min(d_min, g.d_min);
     }
-    // short delays somewhere in the sweep: the far entries of each row go first,
-    // in every kernel, so that all of them sum in one order
-    const int64_t far = d_min >= 1 && d_min < WIN_NEAR_BELOW ? WIN_FAR : 0;
+    // each row: entries of WIN_FAR steps and more, then the nearer ones, then zero
+    // delays; the order is the group's own, whatever else the sweep holds, and
+    // every kernel sums in it
     for (Group& g : groups) {
         g.row_ptr.assign(N + 1, 0);
         g.row_near.assign(N, 0);
@@ -451,7 +449,7 @@ tvbx_status build_groups(tvbx_sweep* h, double dt, std::vector<Group>& groups)
                 dmax = std::max(dmax, d);
                 const uint32_t cd = ((uint32_t)d << 16) | (uint32_t)j;
                 if (d == 0) zero.emplace_back(cd, (float)w);
-                else if (d < far) near.emplace_back(cd, (float)w);
+                else if (d < WIN_FAR) near.emplace_back(cd, (float)w);
                 else { g.col_dly.push_back(cd); g.w.push_back((float)w); }
             }
             g.row_near[k] = (int32_t)g.col_dly.size();
@@ -1224,7 +1222,7 @@ static tvbx_status run_fc(tvbx_sweep* h, int32_t precision, int32_t fcd_window, 
     const int64_t t0 = h->cfg.transient_samples, t1 = h->T;
     const int64_t Tn = t1 - t0;
     if (Tn < 1) return fail(TVBX_E_BAD_STATE, "the last run produced no samples");
-    int32_t blk = 0, n_blocks = 1, m = 0, nw = 0;
+    int32_t blk = 0, n_blocks = 1, merge = 1, m = 0, nw = 0;
     if (fcd_window > 0) {
         if (fcd_step < 1 || fcd_window % fcd_step != 0)
             return fail(TVBX_E_INVALID_ARG, "fcd_window must be a positive multiple of fcd_step");
@@ -1235,11 +1233,7 @@ static tvbx_status run_fc(tvbx_sweep* h, int32_t precision, int32_t fcd_window, 
         m = fcd_window / fcd_step;
         nw = (int32_t)((Tn - fcd_window) / fcd_step + 1);
     } else if (precision == TVBX_FC_FP32 && h->cfg.series_mode != TVBX_SERIES_STREAM) {
-        n_blocks = fc_moment_split(N, P, Tn);
-        if (n_blocks > 1) {
-            blk = (int32_t)((Tn + n_blocks - 1) / n_blocks);
-            n_blocks = (int32_t)((Tn + blk - 1) / blk);
-        }
+        n_blocks = fc_moment_blocks(N, P, Tn, &blk, &merge);
     }
     const size_t stride_b = (size_t)N * N + N;
     if (h->cfg.series_mode == TVBX_SERIES_STREAM) {
@@ -1283,6 +1277,7 @@ static tvbx_status run_fc(tvbx_sweep* h, int32_t precision, int32_t fcd_window, 
     f.t_end = t1;
     f.blk = blk;
     f.n_blocks = n_blocks;
+    f.merge = merge;
     f.blocks = h->d_blocks.as<float>();
     f.fc = h->d_fc.as<float>();
     f.chi = h->d_chi.as<float>();
@@ -1387,7 +1382,7 @@ tvbx_status tvbx_fc_series(const float* series, int32_t n_regions, int64_t n_set
     if (cfg->precision != TVBX_FC_FP32 && !fc_tc_supported(N, cfg->precision))
         return fail(TVBX_E_INVALID_ARG, "tensor-core FC needs n_regions <= 112 (have %d)", N);
     if (cfg->precision == TVBX_FC_FP32 && N > 384) return fail(TVBX_E_INVALID_ARG, "FC needs n_regions <= 384");
-    int32_t blk = 0, n_blocks = 1, m = 0, nw = 0;
+    int32_t blk = 0, n_blocks = 1, merge = 1, m = 0, nw = 0;
     if (cfg->series_layout != TVBX_LAYOUT_TNP && cfg->series_layout != TVBX_LAYOUT_SET4)
         return fail(TVBX_E_INVALID_ARG, "unknown series_layout %d", cfg->series_layout);
     const SeriesLayout sl = cfg->series_layout == TVBX_LAYOUT_SET4 ? layout_blocked(N, Tn) : layout_tnp(N, P);
@@ -1402,11 +1397,7 @@ tvbx_status tvbx_fc_series(const float* series, int32_t n_regions, int64_t n_set
         m = cfg->fcd_window / cfg->fcd_step;
         nw = (int32_t)((Tn - cfg->fcd_window) / cfg->fcd_step + 1);
     } else if (cfg->precision == TVBX_FC_FP32) {
-        n_blocks = fc_moment_split(N, P, Tn);
-        if (n_blocks > 1) {
-            blk = (int32_t)((Tn + n_blocks - 1) / n_blocks);
-            n_blocks = (int32_t)((Tn + blk - 1) / blk);
-        }
+        n_blocks = fc_moment_blocks(N, P, Tn, &blk, &merge);
     }
     cudaStream_t s = (cudaStream_t)cuda_stream;
     const size_t stride_b = (size_t)N * N + N;
@@ -1453,6 +1444,7 @@ tvbx_status tvbx_fc_series(const float* series, int32_t n_regions, int64_t n_set
         f.t_end = Tn;
         f.blk = blk;
         f.n_blocks = n_blocks;
+        f.merge = merge;
         f.blocks = d_blocks;
         f.fc = d_fc;
         f.chi = d_chi;

@@ -48,6 +48,7 @@ struct FmPlan {
     int32_t chunks, per_chunk;// CTAs that share a group's tiles, tiles of each
     int32_t threads;
     int32_t Tt;               // samples per chunk
+    int32_t merge;            // moment sub-blocks (of FcArgs::blk samples) added up in a stored block
     size_t smem;
 };
 
@@ -59,6 +60,7 @@ static FmPlan fm_plan(int32_t N, int64_t P)
     f.tasks_per_set = nt * (nt + 1) / 2;
     const int64_t groups = (P + 3) / 4;
     // few regions: several groups fill a CTA, as long as there are CTAs for every SM
+    f.merge = 1;
     f.m = 1;
     while (f.m < 8 && 2 * f.m * 4 * f.tasks_per_set <= FM_THREADS && groups / (2 * f.m) >= 304) f.m *= 2;
     const int total = 4 * f.m * f.tasks_per_set;
@@ -116,8 +118,7 @@ fc_moments_kernel(const __grid_constant__ FcArgs a, const __grid_constant__ FmPl
     const int64_t g0 = blockIdx.x / a.n_blocks * f.m;          // first group
     const int64_t Tn = a.t_end - a.t_begin;
     const int64_t blk = a.blk > 0 ? a.blk : Tn;
-    const int64_t t_lo = a.t_begin + b * blk;
-    const int64_t len = (t_lo + blk < a.t_end ? t_lo + blk : a.t_end) - t_lo;
+    int64_t t_lo = a.t_begin + b * blk;   // of the sub-block at hand
 
     for (int i = tid; i < 2 * buf; i += nthr) xs[i] = 0.0f;
     for (int i = tid; i < f.m * N; i += nthr) {
@@ -149,10 +150,6 @@ fc_moments_kernel(const __grid_constant__ FcArgs a, const __grid_constant__ FmPl
     const int ck0 = fm_pos(FM_TILE * kb), ck1 = fm_pos(FM_TILE * kb + 4);
     const int cj0 = fm_pos(FM_TILE * jb), cj1 = fm_pos(FM_TILE * jb + 4);
     uint64_t acc2[FM_TILE][FM_TILE / 2];   // two neighbouring columns each
-#pragma unroll
-    for (int r = 0; r < FM_TILE; ++r)
-#pragma unroll
-        for (int c = 0; c < FM_TILE / 2; ++c) acc2[r][c] = 0;
 
     // 16-byte pieces (row = group and sample, region) of a chunk, dealt to the
     // threads in turn, a chunk ahead: VEC by cp.async into slots of their own
@@ -161,10 +158,10 @@ fc_moments_kernel(const __grid_constant__ FcArgs a, const __grid_constant__ FmPl
     const int rows = f.m * Tt;
     float4* raw = reinterpret_cast<float4*>(sh + f.m * N) + tid;   // [FM_LOADS][threads]
     float4 v[VEC ? 1 : FM_LOADS];
-    const float* base = a.series + g0 * a.sl.sg + t_lo * a.sl.st;
+    int64_t len = 0;
     auto fetch = [&](int64_t t0) {
         const int n = len - t0 < Tt ? (int)(len - t0) : Tt;
-        const float* chunk = base + t0 * a.sl.st;
+        const float* chunk = a.series + g0 * a.sl.sg + (t_lo + t0) * a.sl.st;
         int row = row_first, k = k_first;
 #pragma unroll
         for (int u = 0; u < FM_LOADS; ++u) {
@@ -208,53 +205,66 @@ fc_moments_kernel(const __grid_constant__ FcArgs a, const __grid_constant__ FmPl
             if (k >= N) { k -= N; ++row; }
         }
     };
-    fetch(0);
-    float* cur = xs + buf;
-    for (int64_t t0 = 0; t0 < len; t0 += Tt) {
-        cur = cur == xs ? xs + buf : xs;
-        if constexpr (VEC) cp_async_wait_all();
-        put(cur);
-        if (t0 + Tt < len) fetch(t0 + Tt);
-        __syncthreads();   // chunk visible; every read of the other buffer's last chunk done
-        if (!works) continue;
-        const int n = len - t0 < Tt ? (int)(len - t0) : Tt;
-        const float* row = cur + q * Tt * npad;
-#pragma unroll 2
-        for (int t = 0; t < n; ++t, row += npad) {
-            const float4 x0 = *reinterpret_cast<const float4*>(row + ck0), x1 = *reinterpret_cast<const float4*>(row + ck1);
-            const float4 y0 = *reinterpret_cast<const float4*>(row + cj0), y1 = *reinterpret_cast<const float4*>(row + cj1);
-            const float x[FM_TILE] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
-            const uint64_t y[FM_TILE / 2] = {pair2(y0.x, y0.y), pair2(y0.z, y0.w), pair2(y1.x, y1.y), pair2(y1.z, y1.w)};
-#pragma unroll
-            for (int r = 0; r < FM_TILE; ++r) {
-                const uint64_t xr = pair2(x[r], x[r]);
-#pragma unroll
-                for (int c = 0; c < FM_TILE / 2; ++c) fma2(acc2[r][c], xr, y[c]);
-            }
-        }
-    }
-    float acc[FM_TILE][FM_TILE];
-#pragma unroll
-    for (int r = 0; r < FM_TILE; ++r)
-#pragma unroll
-        for (int c = 0; c < FM_TILE / 2; ++c) unpair2(acc2[r][c], acc[r][2 * c], acc[r][2 * c + 1]);
-    if (!works || p >= a.P) return;
     float* G = a.blocks + (p * a.n_blocks + b) * ((int64_t)N * N + N);
     const bool whole = kb < jb && FM_TILE * (jb + 1) <= N && N % 4 == 0;   // inside the triangle, rows 16-byte aligned
+    float* cur = xs + buf;
+    for (int sub = 0; sub < f.merge; ++sub, t_lo += blk) {
+        len = (t_lo + blk < a.t_end ? t_lo + blk : a.t_end) - t_lo;
+        if (len <= 0) break;
 #pragma unroll
-    for (int r = 0; r < FM_TILE; ++r) {
-        const int k = FM_TILE * kb + r;
-        if (k >= N) continue;
-        float* at = G + (int64_t)k * N + FM_TILE * jb;
-        if (whole) {
-            reinterpret_cast<float4*>(at)[0] = make_float4(acc[r][0], acc[r][1], acc[r][2], acc[r][3]);
-            reinterpret_cast<float4*>(at)[1] = make_float4(acc[r][4], acc[r][5], acc[r][6], acc[r][7]);
-        } else {
+        for (int r = 0; r < FM_TILE; ++r)
 #pragma unroll
-            for (int c = 0; c < FM_TILE; ++c) {
-                const int j = FM_TILE * jb + c;
-                if (j < N && j >= k) at[c] = acc[r][c];
-                else if (j == N) G[(int64_t)N * N + k] = acc[r][c];
+            for (int c = 0; c < FM_TILE / 2; ++c) acc2[r][c] = 0;
+        fetch(0);
+        for (int64_t t0 = 0; t0 < len; t0 += Tt) {
+            cur = cur == xs ? xs + buf : xs;
+            if constexpr (VEC) cp_async_wait_all();
+            put(cur);
+            if (t0 + Tt < len) fetch(t0 + Tt);
+            __syncthreads();   // chunk visible; every read of the other buffer's last chunk done
+            if (!works) continue;
+            const int n = len - t0 < Tt ? (int)(len - t0) : Tt;
+            const float* row = cur + q * Tt * npad;
+#pragma unroll 2
+            for (int t = 0; t < n; ++t, row += npad) {
+                const float4 x0 = *reinterpret_cast<const float4*>(row + ck0), x1 = *reinterpret_cast<const float4*>(row + ck1);
+                const float4 y0 = *reinterpret_cast<const float4*>(row + cj0), y1 = *reinterpret_cast<const float4*>(row + cj1);
+                const float x[FM_TILE] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
+                const uint64_t y[FM_TILE / 2] = {pair2(y0.x, y0.y), pair2(y0.z, y0.w), pair2(y1.x, y1.y), pair2(y1.z, y1.w)};
+#pragma unroll
+                for (int r = 0; r < FM_TILE; ++r) {
+                    const uint64_t xr = pair2(x[r], x[r]);
+#pragma unroll
+                    for (int c = 0; c < FM_TILE / 2; ++c) fma2(acc2[r][c], xr, y[c]);
+                }
+            }
+        }
+        if (!works || p >= a.P) continue;
+        // the first sub-block's sums, or the sums so far and this one's
+#pragma unroll
+        for (int r = 0; r < FM_TILE; ++r) {
+            const int k = FM_TILE * kb + r;
+            if (k >= N) continue;
+            float s[FM_TILE];
+#pragma unroll
+            for (int c = 0; c < FM_TILE / 2; ++c) unpair2(acc2[r][c], s[2 * c], s[2 * c + 1]);
+            float* at = G + (int64_t)k * N + FM_TILE * jb;
+            if (whole) {
+                float4 lo = make_float4(s[0], s[1], s[2], s[3]), hi = make_float4(s[4], s[5], s[6], s[7]);
+                if (sub > 0) {
+                    const float4 l0 = reinterpret_cast<float4*>(at)[0], h0 = reinterpret_cast<float4*>(at)[1];
+                    lo = make_float4(l0.x + lo.x, l0.y + lo.y, l0.z + lo.z, l0.w + lo.w);
+                    hi = make_float4(h0.x + hi.x, h0.y + hi.y, h0.z + hi.z, h0.w + hi.w);
+                }
+                reinterpret_cast<float4*>(at)[0] = lo;
+                reinterpret_cast<float4*>(at)[1] = hi;
+            } else {
+#pragma unroll
+                for (int c = 0; c < FM_TILE; ++c) {
+                    const int j = FM_TILE * jb + c;
+                    float* to = j < N && j >= k ? at + c : (j == N ? G + (int64_t)N * N + k : nullptr);
+                    if (to) *to = sub > 0 ? *to + s[c] : s[c];
+                }
             }
         }
     }
@@ -373,7 +383,8 @@ __global__ void summary_kernel(const float* __restrict__ state, int32_t N, int32
 cudaError_t launch_fc_moments(const FcArgs& a, cudaStream_t s)
 {
     if (a.N > 384) return cudaErrorInvalidValue;
-    const FmPlan f = fm_plan(a.N, a.P);
+    FmPlan f = fm_plan(a.N, a.P);
+    f.merge = a.merge > 0 ? a.merge : 1;
     const bool vec = a.sl.sk % 4 == 0 && a.sl.st % 4 == 0 && a.sl.sg % 4 == 0 &&
                      (reinterpret_cast<uintptr_t>(a.series) & 15) == 0;
     auto kern = vec ? fc_moments_kernel<true> : fc_moments_kernel<false>;
@@ -385,16 +396,23 @@ cudaError_t launch_fc_moments(const FcArgs& a, cudaStream_t s)
     return cudaGetLastError();
 }
 
-// Moment blocks of an FC without windows: one, or as many (at most 12, of at
-// least 64 samples) as give every SM four CTAs of a few sets' moments.
-int32_t fc_moment_split(int32_t N, int64_t P, int64_t Tn)
+// Moment sub-blocks of an FC without windows, of at least 256 samples and at
+// most 12: a function of the samples alone, so that a set's sums do not depend
+// on how many sets there are. Few sets store them as blocks that CTAs of their
+// own form (*merge 1, and the reduction adds them in order); otherwise one CTA
+// adds them up in the same order (*merge: their number).
+int32_t fc_moment_blocks(int32_t N, int64_t P, int64_t Tn, int32_t* blk, int32_t* merge)
 {
-    if (N > 384) return 1;
+    int64_t n = Tn / 256 < 1 ? 1 : (Tn / 256 > FCR_MAXB ? FCR_MAXB : Tn / 256);
+    *blk = 0;
+    *merge = 1;
+    if (N > 384 || n == 1) return 1;
+    *blk = (int32_t)((Tn + n - 1) / n);
+    n = (Tn + *blk - 1) / *blk;
     const FmPlan f = fm_plan(N, P);
-    const int64_t ctas = ((P + 3) / 4 + f.m - 1) / f.m * f.chunks;
-    int64_t n = 608 / ctas;
-    n = n < 1 ? 1 : (n > FCR_MAXB ? FCR_MAXB : n);
-    return (int32_t)(n > Tn / 64 ? (Tn / 64 > 1 ? Tn / 64 : 1) : n);
+    if (((P + 3) / 4 + f.m - 1) / f.m * f.chunks < 4 * 304) return (int32_t)n;   // 304 CTAs are resident
+    *merge = (int32_t)n;
+    return 1;
 }
 
 // Shift of each (region, set): mean of up to 64 evenly spaced samples of

@@ -65,8 +65,7 @@ struct GroupDev {
                                // starts at an index of the parity of k (padded with a
                                // zero-weight self entry of delay 1) and ends with its
                                // zero-delay entries
-    const int32_t* row_near;   // [N] first entry of each row with a delay below WIN_FAR (when
-                               // the shortest delay is below WIN_NEAR_BELOW)
+    const int32_t* row_near;   // [N] first entry of each row with a delay below WIN_FAR
     const int32_t* row_mid;    // [N] first zero-delay entry of each row
     const uint32_t* col_dly;   // [nnz] (delay << 16) | j
     const float* w;            // [nnz] u_kj
@@ -152,7 +151,7 @@ size_t sim_fast_smem_bytes(int variant, int N, int nnz);
 // Windowed kernels (sim_window.cu): launches of `steps` steps of every pair.
 constexpr int WIN_MAX_STEPS = 32;
 // Sweeps whose shortest delay is below WIN_NEAR_BELOW steps sum the entries of
-// WIN_FAR steps and more for WIN_FAR steps at once (they come first in a row).
+// WIN_FAR steps and more for WIN_FAR steps at once (they come first in every row).
 constexpr int WIN_NEAR_BELOW = 8;
 constexpr int WIN_FAR = 16;
 struct WindowPlan {
@@ -217,6 +216,7 @@ struct FcArgs {
     int64_t t_begin, t_end;    // samples used: [t_begin, t_end)
     int32_t blk;               // samples per FCD block (0: one block)
     int32_t n_blocks;
+    int32_t merge;             // FP32 moments: blocks of blk samples added up per stored block (0: 1)
     float* blocks;             // [P][n_blocks][N*N + N] block moments (nullable)
     float* fc;                 // [P][N][N] internal order (nullable)
     float* chi;                // [P]
@@ -228,7 +228,8 @@ struct FcArgs {
 };
 // Block moments (SIMT, FP32 CUDA-core FMAs).
 cudaError_t launch_fc_moments(const FcArgs& a, cudaStream_t s);
-int32_t fc_moment_split(int32_t N, int64_t P, int64_t Tn);   // moment blocks of an FP32 FC without windows
+// Blocks of an FP32 FC without windows, FcArgs::blk and ::merge.
+int32_t fc_moment_blocks(int32_t N, int64_t P, int64_t Tn, int32_t* blk, int32_t* merge);
 // From the block moments: Pearson FC, chi, mean FC and (nw > 0) the FCD over
 // nw windows of m blocks of Lw samples, in one kernel when its shared memory
 // fits; vec_scratch ([P][nw][N(N-1)/2]) is used only when it does not.

@@ -24,8 +24,8 @@
 // another thread of the same launch may still read.
 //
 // Short delays (d_min < 8, large connectomes at high speeds): a window of d_min
-// steps alone would read each row entry for a few steps only. The entries with
-// d >= WIN_FAR then go first in each CSR row and sim_far_kernel sums them for
+// steps alone would read each row entry for a few steps only. sim_far_kernel
+// then sums the entries with d >= WIN_FAR, which come first in each CSR row, for
 // WIN_FAR steps at once into a buffer [tile][WIN_FAR][N][pb]; the windows of
 // d_min steps start from those sums and add the few nearer entries.
 //

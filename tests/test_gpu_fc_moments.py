@@ -41,3 +41,17 @@ def test_fp32_fc_against_fp64(tvbx, n_regions, n_sets, n_samples, layout):
     assert np.array_equal(got, np.swapaxes(got, 1, 2))
     assert np.abs(chi.cpu().numpy()[at] - O.chi(ref)).max() < 5e-5
     assert np.abs(mfc.cpu().numpy()[at] - O.mean_offdiag(want)).max() < 5e-5
+
+
+@pytest.mark.parametrize("n_regions", [16, 68])
+def test_fp32_fc_of_a_set_does_not_depend_on_the_others(tvbx, n_regions):
+    import torch
+    T = 1100
+    x = 5e-3 + 1e-3 * torch.randn((T, n_regions, 5000), device="cuda")
+    out = []
+    for P in (5000, 777, 5):
+        fc, chi = torch.empty((P, n_regions, n_regions), device="cuda"), torch.empty(P, device="cuda")
+        tvbx.fc_series(x[:, :, :P].contiguous(), n_regions, P, T, fc_out=fc, chi=chi)
+        out.append((fc[:5].clone(), chi[:5].clone()))
+    for fc, chi in out[1:]:
+        assert torch.equal(fc, out[0][0]) and torch.equal(chi, out[0][1])

@@ -84,3 +84,15 @@ def test_window_with_several_speeds_restores_from_a_checkpoint(tvbx):
     g = tvbx.Sweep(W, L, points=pts)
     g.run(dt_ms=DT, n_steps=220, tavg_steps=10, seed=2, kernel=tvbx.KERNEL_GENERAL)
     assert np.array_equal(a.state(), g.state())
+
+
+def test_a_set_does_not_depend_on_the_other_speeds(tvbx):
+    """Short delays of one speed change how the sweep runs, not what a set of
+    another speed gives."""
+    W, L, pts = _inputs(tvbx, 40, 30, 3, speeds=(1.0, 4.0))
+    slow = pts[:, tvbx.AXES.index("speed")] == 1.0
+    both, alone = tvbx.Sweep(W, L, points=pts), tvbx.Sweep(W, L, points=pts[slow])
+    for sw in (both, alone):
+        sw.run(dt_ms=DT, n_steps=100, tavg_steps=10, seed=4)
+    assert np.array_equal(both.state()[slow], alone.state())
+    assert np.array_equal(both.series()[slow], alone.series())
