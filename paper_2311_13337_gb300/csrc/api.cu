@@ -647,7 +647,7 @@ static tvbx_status prepare_run(tvbx_sweep* h, const tvbx_run_cfg& c, cudaStream_
         int dev = 0, sms = 0;
         CK(cudaGetDevice(&dev), "device");
         CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "device");
-        if (!sim_window_plan(d_min, N, largest_group, h->model.tau_e == h->model.tau_i, sms, win)) win = WindowPlan{};
+        if (!sim_window_plan(d_min, N, P, largest_group, h->model.tau_e == h->model.tau_i, sms, win)) win = WindowPlan{};
     }
     if (windows && general_pb > 0) {
         if (win.steps == 0) return fail(TVBX_E_UNSUPPORTED, "no window of steps without coupling");

@@ -159,11 +159,12 @@ struct WindowPlan {
     int32_t pb = 0;        // sets per tile
     int32_t threads = 0;   // per CTA
     bool packed = false;   // two sets per thread
+    bool split = false;    // two threads per set and region
     bool far = false;      // far entries summed apart
 };
-// d_min: shortest delay of a nonzero weight in steps; P: sets of the largest
-// speed group. False when the sweep has no window.
-bool sim_window_plan(int32_t d_min, int32_t N, int64_t P, bool reduced, int sms, WindowPlan& w);
+// d_min: shortest delay of a nonzero weight in steps; P: sets of the sweep,
+// P_group: of its largest speed group. False when the sweep has no window.
+bool sim_window_plan(int32_t d_min, int32_t N, int64_t P, int64_t P_group, bool reduced, int sms, WindowPlan& w);
 // far: buffer [n_tiles][WIN_FAR][N][pb] of the far sums (w.far); far_row: the
 // window's first step in it (0: the far sums are formed first).
 cudaError_t launch_sim_window(const SimArgs& a, const WindowPlan& w, int32_t n_tiles, int64_t table_step, float* far,

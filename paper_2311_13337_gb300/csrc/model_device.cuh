@@ -602,16 +602,21 @@ static __device__ __forceinline__ void tf_share(const DevModel& m, V fe, V fi, V
     s.SQ2 = vfma(vmul(caa, fi), vbc<V>(m.sq_i), vmul(vmul(cbb, fe), vbc<V>(m.sq_e)));
 }
 
-// One population (POP 0 = e, 1 = i): F with its gradient in (fe, fi) and
-// l(F); muV receives mu_V. alpha = g_L (E_e - E_L) + W.
-// Coefficient k of population POP's folded polynomial, read as a member (a
+// One population: F with its gradient in (fe, fi) and l(F); muV receives mu_V.
+// alpha = g_L (E_e - E_L) + W. cp(k): coefficient k of the population's folded
+// polynomial; PolyE and PolyI read it as a member of the model (a
 // kernel-parameter constant, not a load through a pointer).
-template <int POP> static __device__ __forceinline__ float cpoly(const DevModel& m, int k);
-template <> __device__ __forceinline__ float cpoly<0>(const DevModel& m, int k) { return m.cp_e[k]; }
-template <> __device__ __forceinline__ float cpoly<1>(const DevModel& m, int k) { return m.cp_i[k]; }
+struct PolyE {
+    const DevModel& m;
+    __device__ __forceinline__ float operator()(int k) const { return m.cp_e[k]; }
+};
+struct PolyI {
+    const DevModel& m;
+    __device__ __forceinline__ float operator()(int k) const { return m.cp_i[k]; }
+};
 
-template <int POP, class V>
-static __device__ __forceinline__ CJ<V> tf_pop(const DevModel& m, const TFShare<V>& s, V alpha, V& muV)
+template <class V, class CP>
+static __device__ __forceinline__ CJ<V> tf_pop(const DevModel& m, CP cp, const TFShare<V>& s, V alpha, V& muV)
 {
     const V ae = vfma(vbc<V>(m.be), s.fi, alpha);
     const V ai = vfma(vbc<V>(-m.dE), s.mu, ae);
@@ -663,20 +668,20 @@ static __device__ __forceinline__ CJ<V> tf_pop(const DevModel& m, const TFShare<
     const V Za = vmul(s.zr, vbc<V>(m.qe)), Zb = vmul(s.zr, vbc<V>(m.qi));
     // d = (V_thre - mu_V) / sqrt(2) and its jet
     const V Z = s.Zv;
-    const V t = vfma(vbc<V>(cpoly<POP>(m, 8)), Z, vfma(vbc<V>(cpoly<POP>(m, 7)), S.v, vfma(vbc<V>(cpoly<POP>(m, 4)), Vj.v, vbc<V>(cpoly<POP>(m, 1)))));
-    const V u = vfma(vbc<V>(cpoly<POP>(m, 9)), Z, vfma(vbc<V>(cpoly<POP>(m, 5)), S.v, vbc<V>(cpoly<POP>(m, 2))));
-    const V w = vfma(vbc<V>(cpoly<POP>(m, 6)), Z, vbc<V>(cpoly<POP>(m, 3)));
+    const V t = vfma(vbc<V>(cp(8)), Z, vfma(vbc<V>(cp(7)), S.v, vfma(vbc<V>(cp(4)), Vj.v, vbc<V>(cp(1)))));
+    const V u = vfma(vbc<V>(cp(9)), Z, vfma(vbc<V>(cp(5)), S.v, vbc<V>(cp(2))));
+    const V w = vfma(vbc<V>(cp(6)), Z, vbc<V>(cp(3)));
     CJ<V> d;
-    d.v = vfma(Vj.v, t, vfma(S.v, u, vfma(Z, w, vbc<V>(cpoly<POP>(m, 0)))));
-    const V gV = vfma(vbc<V>(cpoly<POP>(m, 4)), Vj.v, t);
-    const V gS = vfma(vbc<V>(cpoly<POP>(m, 7)), Vj.v, vfma(vbc<V>(cpoly<POP>(m, 5)), S.v, u));
-    const V gZ = vfma(vbc<V>(cpoly<POP>(m, 8)), Vj.v, vfma(vbc<V>(cpoly<POP>(m, 9)), S.v, vfma(vbc<V>(cpoly<POP>(m, 6)), Z, w)));
+    d.v = vfma(Vj.v, t, vfma(S.v, u, vfma(Z, w, vbc<V>(cp(0)))));
+    const V gV = vfma(vbc<V>(cp(4)), Vj.v, t);
+    const V gS = vfma(vbc<V>(cp(7)), Vj.v, vfma(vbc<V>(cp(5)), S.v, u));
+    const V gZ = vfma(vbc<V>(cp(8)), Vj.v, vfma(vbc<V>(cp(9)), S.v, vfma(vbc<V>(cp(6)), Z, w)));
     d.a = vfma(gV, Vj.a, vfma(gS, S.a, vmul(gZ, Za)));
     d.b = vfma(gV, Vj.b, vfma(gS, S.b, vmul(gZ, Zb)));
-    const V H = vfma(vbc<V>(cpoly<POP>(m, 4)), BVV,
-                     vfma(vbc<V>(cpoly<POP>(m, 5)), BSS,
-                          vfma(vbc<V>(cpoly<POP>(m, 6)), s.BZZ,
-                               vfma(vbc<V>(cpoly<POP>(m, 7)), BVS, vfma(vbc<V>(cpoly<POP>(m, 8)), BVZ, vmul(vbc<V>(cpoly<POP>(m, 9)), BSZ))))));
+    const V H = vfma(vbc<V>(cp(4)), BVV,
+                     vfma(vbc<V>(cp(5)), BSS,
+                          vfma(vbc<V>(cp(6)), s.BZZ,
+                               vfma(vbc<V>(cp(7)), BVS, vfma(vbc<V>(cp(8)), BVZ, vmul(vbc<V>(cp(9)), BSZ))))));
     d.l = vfma(vbc<V>(2.0f), H, vfma(gV, Vj.l, vfma(gS, S.l, vmul(gZ, s.Zl))));
     // y = d / sigma_V, with d(1/sigma_V)/d s2 = k1 = -rs^3/2 and d2 = 3 rs^5 / 4
     const V k1 = vmul(vbc<V>(-0.5f), rs3);
@@ -739,7 +744,7 @@ static __device__ __forceinline__ void transfer_integrator(const DevModel& m, in
     TFShare<float> sh;
     tf_share(m, fe, fi, caa, cab, cbb, sh);
     const float alpha = vadd(vfma(-m.g_L, E_L, m.gLEe), W);
-    const CJ<float> F = pop ? tf_pop<1>(m, sh, alpha, muV) : tf_pop<0>(m, sh, alpha, muV);
+    const CJ<float> F = pop ? tf_pop(m, PolyI{m}, sh, alpha, muV) : tf_pop(m, PolyE{m}, sh, alpha, muV);
     out[0] = F.v;
     out[1] = vmul(de, F.a);
     out[2] = vmul(di, F.b);
@@ -820,7 +825,7 @@ static __device__ __forceinline__ void pair_tf_reduced(const DevModel& m, const 
     TFShare<V> sh;
     tf_share(m, fe, fi, caa, cab, cbb, sh);
     const V gLEe = vbc<V>(m.gLEe), ngL = vbc<V>(-m.g_L);
-    Fe = tf_pop<0>(m, sh, vadd(vfma(ngL, sp.ELe, gLEe), We), muVe);
+    Fe = tf_pop(m, PolyE{m}, sh, vadd(vfma(ngL, sp.ELe, gLEe), We), muVe);
     const V zero = vbc<V>(0.0f);
     Fex = vfma(de, Fe.a, zero);   // products that later meet sums: see the lane arithmetic
     Fey = vfma(di, Fe.b, zero);
@@ -837,7 +842,7 @@ static __device__ __forceinline__ void pair_tf_reduced(const DevModel& m, const 
     }
     tf_inputs(m, xei_, xii_, ce, cx, ci, fe, fi, de, di, caa, cab, cbb);
     tf_share(m, fe, fi, caa, cab, cbb, sh);
-    Fi = tf_pop<1>(m, sh, vadd(vfma(ngL, sp.ELi, gLEe), Wi), muVi);
+    Fi = tf_pop(m, PolyI{m}, sh, vadd(vfma(ngL, sp.ELi, gLEe), Wi), muVi);
     Fix = vfma(de, Fi.a, zero);
     Fiy = vfma(di, Fi.b, zero);
 }
@@ -853,36 +858,14 @@ static __device__ __noinline__ void pair_tf_general(const DevModel& m, float ELe
     transfer_x_lap(m, m.P_i, ELi, Wi, xei, xii, ce, cx, ci, oi, muVi);
 }
 
-// One forward-Euler step of Eq. 1-3 for one pair (or two sets of one region),
-// from the state at step n, the delayed coupling sum_j u_kj E_j(n - d_kj) and
-// the OU value at step n. E and I are clamped to [E_min, E_max] after the
-// update (NaN kept); the events go to the tracker.
+// The Euler update of pair_step from both populations' transfer functions: F
+// and l(F) (Fe.v, Fe.l, ...), the gradients in the input rates and mu_V.
 template <class V>
-static __device__ __forceinline__ void pair_step(const DevModel& m, const ParamsV<V>& sp, PairV<V>& x, V coupling,
-                                                 V OU, Track<V>& trk)
+static __device__ __forceinline__ void pair_update(const DevModel& m, const ParamsV<V>& sp, PairV<V>& x,
+                                                   const CJ<V>& Fe, const CJ<V>& Fi, V Fex, V Fey, V Fix, V Fiy,
+                                                   V muVe, V muVi, Track<V>& trk)
 {
     const V E = x.E, I = x.I, ce = x.Cee, cx = x.Cei, ci = x.Cii, We = x.We, Wi = x.Wi;
-    const V exc = vfma(sp.wn, OU, vfma(sp.g, coupling, E));
-    const V xee = vadd(exc, sp.cFee), xie = vadd(I, sp.cFei);
-    const V xei = vadd(exc, sp.cFie), xii = vadd(I, sp.cFii);
-    CJ<V> Fe, Fi;
-    V Fex, Fey, Fix, Fiy, muVe, muVi;
-    if constexpr (std::is_same<V, float>::value) {
-        if (!m.reduced) {   // general template (tau_e != tau_i)
-            float oe[4], oi[4];
-            pair_tf_general(m, sp.ELe, sp.ELi, We, Wi, ce, cx, ci, xee, xie, xei, xii, oe, oi, muVe, muVi);
-            Fe = CJ<V>{oe[0], 0.0f, 0.0f, oe[3]};
-            Fi = CJ<V>{oi[0], 0.0f, 0.0f, oi[3]};
-            Fex = oe[1];
-            Fey = oe[2];
-            Fix = oi[1];
-            Fiy = oi[2];
-        } else {
-            pair_tf_reduced(m, sp, We, Wi, ce, cx, ci, xee, xie, xei, xii, Fe, Fi, Fex, Fey, Fix, Fiy, muVe, muVi);
-        }
-    } else {
-        pair_tf_reduced(m, sp, We, Wi, ce, cx, ci, xee, xie, xei, xii, Fe, Fi, Fex, Fey, Fix, Fiy, muVe, muVi);
-    }
     const V one = vbc<V>(1.0f), rT = vbc<V>(m.inv_T);
     const V dFe = vsub(Fe.v, E), dFi = vsub(Fi.v, I);
     // Eq. 1
@@ -929,6 +912,71 @@ static __device__ __forceinline__ void pair_step(const DevModel& m, const Params
         set_lane(x.I, i, ci_);
         if (!(ce_ == e && ci_ == ii && cm <= m.C_div)) trk.f[i] |= step_events(m, e, ii, cm);
     }
+}
+
+// One forward-Euler step of Eq. 1-3 for one pair (or two sets of one region),
+// from the state at step n, the delayed coupling sum_j u_kj E_j(n - d_kj) and
+// the OU value at step n. E and I are clamped to [E_min, E_max] after the
+// update (NaN kept); the events go to the tracker.
+template <class V>
+static __device__ __forceinline__ void pair_step(const DevModel& m, const ParamsV<V>& sp, PairV<V>& x, V coupling,
+                                                 V OU, Track<V>& trk)
+{
+    const V E = x.E, I = x.I, ce = x.Cee, cx = x.Cei, ci = x.Cii, We = x.We, Wi = x.Wi;
+    const V exc = vfma(sp.wn, OU, vfma(sp.g, coupling, E));
+    const V xee = vadd(exc, sp.cFee), xie = vadd(I, sp.cFei);
+    const V xei = vadd(exc, sp.cFie), xii = vadd(I, sp.cFii);
+    CJ<V> Fe, Fi;
+    V Fex, Fey, Fix, Fiy, muVe, muVi;
+    if constexpr (std::is_same<V, float>::value) {
+        if (!m.reduced) {   // general template (tau_e != tau_i)
+            float oe[4], oi[4];
+            pair_tf_general(m, sp.ELe, sp.ELi, We, Wi, ce, cx, ci, xee, xie, xei, xii, oe, oi, muVe, muVi);
+            Fe = CJ<V>{oe[0], 0.0f, 0.0f, oe[3]};
+            Fi = CJ<V>{oi[0], 0.0f, 0.0f, oi[3]};
+            Fex = oe[1];
+            Fey = oe[2];
+            Fix = oi[1];
+            Fiy = oi[2];
+        } else {
+            pair_tf_reduced(m, sp, We, Wi, ce, cx, ci, xee, xie, xei, xii, Fe, Fi, Fex, Fey, Fix, Fiy, muVe, muVi);
+        }
+    } else {
+        pair_tf_reduced(m, sp, We, Wi, ce, cx, ci, xee, xie, xei, xii, Fe, Fi, Fex, Fey, Fix, Fiy, muVe, muVi);
+    }
+    pair_update(m, sp, x, Fe, Fi, Fex, Fey, Fix, Fiy, muVe, muVi, trk);
+}
+
+// The same step by two lanes (2i and 2i + 1 of a warp; lanes: all lanes that
+// call), one per population: each evaluates its own transfer function (cp, E_L, W, the
+// inputs' constants cFe and cFi, all of its population), receives the other's,
+// and takes the whole update, so both lanes hold the same state afterwards.
+// The same operations as pair_step in the reduced form, so the same numbers;
+// the chain of a step is about half as long.
+template <class CP>
+static __device__ __forceinline__ void pair_step_split(const DevModel& m, CP cp, int pop, float EL, float cFe, float cFi,
+                                                       const SetParams& sp, PairState& x, float coupling, float OU,
+                                                       Track<float>& trk, uint32_t lanes)
+{
+    const float exc = vfma(sp.wn, OU, vfma(sp.g, coupling, x.E));
+    float fe, fi, de, di, caa, cab, cbb;
+    tf_inputs(m, vadd(exc, cFe), vadd(x.I, cFi), x.Cee, x.Cei, x.Cii, fe, fi, de, di, caa, cab, cbb);
+    TFShare<float> sh;
+    tf_share(m, fe, fi, caa, cab, cbb, sh);
+    float mu;
+    const CJ<float> F = tf_pop(m, cp, sh, vadd(vfma(-m.g_L, EL, m.gLEe), pop ? x.Wi : x.We), mu);
+    const float mine[5] = {F.v, vfma(de, F.a, 0.0f), vfma(di, F.b, 0.0f), F.l, mu};
+    float other[5];
+#pragma unroll
+    for (int i = 0; i < 5; ++i) other[i] = __shfl_xor_sync(lanes, mine[i], 1);
+    float e[5], in[5];
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {
+        e[i] = pop ? other[i] : mine[i];
+        in[i] = pop ? mine[i] : other[i];
+    }
+    pair_update(m, sp, x, CJ<float>{e[0], 0.0f, 0.0f, e[3]}, CJ<float>{in[0], 0.0f, 0.0f, in[3]}, e[1], e[2], in[1],
+                in[2], e[4], in[4], trk);
 }
 
 // Kahan-compensated accumulation s += v with carry c.

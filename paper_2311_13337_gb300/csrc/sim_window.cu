@@ -10,7 +10,8 @@
 // each row entry is read once per window instead of once per step.
 //
 // A thread owns one region of one set (float) or of two adjacent sets (float2,
-// packed FP32x2). It
+// packed FP32x2); in sweeps too small to fill the chip two threads share one.
+// It
 //  1. forms the coupling sums of the window, up to 8 steps at a time, in CSR
 //     order (the sums of the other kernels, bit for bit): independent loads
 //     that do not wait for the sums;
@@ -315,6 +316,127 @@ sim_window_kernel(const __grid_constant__ SimArgs a, int32_t pb_rt, int32_t bloc
                              reinterpret_cast<V*>(win_smem) + threadIdx.x);
 }
 
+// The window of a sweep too small to fill the chip, where the chain of one step
+// bounds it: two lanes per pair, one per population (pair_step_split), each
+// forming the coupling sums of half the steps. Needs the reduced transfer
+// function (tau_e == tau_i).
+template <bool NEAR>
+__global__ void __launch_bounds__(WIN_THREADS, 2)
+sim_window_split_kernel(const __grid_constant__ SimArgs a, int32_t pb, int32_t blocks_per_tile, int64_t table_step,
+                        const float* __restrict__ far)
+{
+    extern __shared__ __align__(16) unsigned char win_smem[];
+    constexpr int PAIRS = WIN_THREADS / 2;
+    const int32_t ti = blockIdx.x / blocks_per_tile;
+    const TileDev tile = a.tiles[ti];
+    const GroupDev& grp = a.groups[tile.group];
+    const DevModel& m = a.m;
+    const int N = a.N, pop = threadIdx.x & 1;
+    const WinSlot ws = win_slot<1>(tile, ((blockIdx.x % blocks_per_tile) * blockDim.x + threadIdx.x) >> 1);
+    const uint32_t lanes = __ballot_sync(0xffffffffu, ws.k < N);
+    if (ws.k >= N) return;
+    const int k = ws.k, q = ws.q, H = grp.H, HR = H + WIN_FAR, steps = a.n_chunk, ts = a.ts;
+    const bool own_noise = a.noise_per_set != 0;
+    const uint32_t n0 = (uint32_t)a.n0;
+    const int slot0 = (int)(n0 % (uint32_t)H);
+    float* ring = grp.ring + (int64_t)tile.q0 * N * HR + q;
+    float* stash = reinterpret_cast<float*>(win_smem) + (threadIdx.x >> 1);   // step b at stash[b * PAIRS]
+
+    // 1. coupling sums: of every 2 G steps a lane takes G
+    {
+        const int e0 = NEAR ? grp.row_near[k] : grp.row_ptr[k], e1 = grp.row_mid[k];
+        const float* far_k = NEAR ? far + ((int64_t)ti * WIN_FAR * N + k) * pb + q : nullptr;
+        int b0 = 0;
+        auto pass = [&](auto g_c) {
+            constexpr int G = decltype(g_c)::value;
+            for (; b0 + 2 * G <= steps || (G == 1 && b0 < steps); b0 += 2 * G) {
+                const int c0 = b0 + pop * G;
+                if (c0 >= steps) continue;   // an odd last step
+                float acc[G];
+#pragma unroll
+                for (int b = 0; b < G; ++b) acc[b] = NEAR ? far_k[(int64_t)(c0 + b) * N * pb] : 0.0f;
+                int at = slot0 + c0;
+                at -= at >= H ? H : 0;
+                gather<G>(acc, grp, ring, e0, e1, at, H, HR, pb);
+#pragma unroll
+                for (int b = 0; b < G; ++b) stash[(c0 + b) * PAIRS] = acc[b];
+            }
+        };
+        pass(std::integral_constant<int, 8>{});
+        pass(std::integral_constant<int, 4>{});
+        pass(std::integral_constant<int, 2>{});
+        pass(std::integral_constant<int, 1>{});
+    }
+    __syncwarp(lanes);
+
+    // 2. the window's steps; the even lane writes
+    const int64_t NP = (int64_t)N * a.P;
+    const int64_t p = grp.p_base + tile.q0 + q;
+    float* st = a.state + (int64_t)k * a.P + p;
+    const SetParams sp = load_set_params(a.prm, a.P, p);
+    const float EL = pop ? sp.ELi : sp.ELe, cFe = pop ? sp.cFie : sp.cFee, cFi = pop ? sp.cFii : sp.cFei;
+    float cp[10];
+#pragma unroll
+    for (int c = 0; c < 10; ++c) cp[c] = pop ? m.cp_i[c] : m.cp_e[c];
+    const auto poly = [&cp](int c) { return cp[c]; };
+    PairState x{st[SV_E * NP],  st[SV_I * NP],  st[SV_CEE * NP], st[SV_CEI * NP], st[SV_CII * NP],
+                st[SV_WE * NP], st[SV_WI * NP], st[SV_CWE * NP], st[SV_CWI * NP]};
+    float accE = st[SV_ACC_E * NP], accI = st[SV_ACC_I * NP], ou = own_noise ? st[SV_OU * NP] : 0.0f;
+    const uint32_t pn = own_noise ? (uint32_t)(a.p_offset + a.ext_index[p]) : 0u;
+    Track<float> trk = track_init<float>();
+    const float inv_ts = 1.0f / (float)ts;
+    int left = ts - (int)(n0 % (uint32_t)ts);
+    int64_t t = n0 / (uint32_t)ts;
+    int slot_w = slot0;
+    float* const ring_k = ring + (uint32_t)(k * HR) * (uint32_t)pb;
+    const float* ou_p = a.ou_table + (own_noise ? 0 : table_step * N + k);
+    for (int b = 0; b < steps; ++b) {
+        const float OU = own_noise ? ou : __ldg(ou_p);
+        ou_p += own_noise ? 0 : N;
+        pair_step_split(m, poly, pop, EL, cFe, cFi, sp, x, stash[b * PAIRS], OU, trk, lanes);
+        if (own_noise) ou = next_ou(m, a.seed, n0 + (uint32_t)b, (uint32_t)k, pn, OU);
+        ++slot_w;
+        slot_w -= slot_w == H ? H : 0;
+        accE = vadd(accE, x.E);
+        accI = vadd(accI, x.I);
+        if (pop == 0) {
+            float* dst = ring_k + slot_w * pb;
+            *dst = x.E;
+            if (slot_w < WIN_FAR) dst[H * pb] = x.E;
+        }
+        if (--left == 0) {
+            if (t < a.T && pop == 0) {
+                const float xE = vmul(accE, inv_ts), xI = vmul(accI, inv_ts);
+                const int64_t so = series_index(a.sl, t, k, p);
+                a.series[so] = xE;
+                if (a.series_i) a.series_i[so] = xI;
+                if (t >= a.transient) {
+                    float sE = st[SV_SUM_E * NP], cE = st[SV_CMP_E * NP];
+                    float sI = st[SV_SUM_I * NP], cI = st[SV_CMP_I * NP];
+                    kahan_add(sE, cE, xE);
+                    kahan_add(sI, cI, xI);
+                    st[SV_SUM_E * NP] = sE;
+                    st[SV_CMP_E * NP] = cE;
+                    st[SV_SUM_I * NP] = sI;
+                    st[SV_CMP_I * NP] = cI;
+                }
+            }
+            left = ts;
+            ++t;
+            accE = 0.0f;
+            accI = 0.0f;
+        }
+    }
+    if (pop) return;
+    const float v[11] = {x.E, x.I, x.Cee, x.Cei, x.Cii, x.We, x.Wi, x.cWe, x.cWi, accE, accI};
+    constexpr int at[11] = {SV_E, SV_I, SV_CEE, SV_CEI, SV_CII, SV_WE, SV_WI, SV_CWE, SV_CWI, SV_ACC_E, SV_ACC_I};
+#pragma unroll
+    for (int c = 0; c < 11; ++c) st[at[c] * NP] = v[c];
+    if (own_noise) st[SV_OU * NP] = ou;
+    const uint32_t f = track_flags(m, trk, 0);
+    if (f) atomicOr(a.status + p, f);
+}
+
 // Window `turn` of a job: its first step within the round, its length (0: the
 // round is over) and its first row of the far sums. A window stays within the
 // WIN_FAR steps whose far sums are at hand.
@@ -411,43 +533,55 @@ __global__ void ring_convert_kernel(float* __restrict__ ring, int32_t H, int32_t
     }
 }
 
-template <class V, int PB>
+// far sums (when due) and the window of every pair; S sets per thread, or (SPLIT) two threads per set
+template <class V, int PB, bool SPLIT = false>
 cudaError_t launch_v(const SimArgs& a, const WindowPlan& w, int32_t n_tiles, int64_t table_step, float* far,
                      int32_t far_row, cudaStream_t s)
 {
     constexpr int S = VSets<V>::n;
     const int64_t per_tile = (int64_t)a.N * ((w.pb + S - 1) / S);
     const int32_t bpt = (int32_t)((per_tile + w.threads - 1) / w.threads);
-    const unsigned grid = (unsigned)((int64_t)n_tiles * bpt);
-    const size_t smem = sizeof(V) * (size_t)WIN_THREADS * a.n_chunk;
+    const int32_t bpt_w = SPLIT ? (int32_t)((2 * per_tile + w.threads - 1) / w.threads) : bpt;
+    const unsigned grid = (unsigned)((int64_t)n_tiles * bpt_w);
+    const size_t smem = sizeof(V) * (size_t)WIN_THREADS * a.n_chunk / (SPLIT ? 2 : 1);
+    float* row = nullptr;
     if (w.far) {
         if (far_row == 0) {
             note_launch();
-            sim_far_kernel<V, PB><<<grid, w.threads, 0, s>>>(a, w.pb, bpt, far);
+            sim_far_kernel<V, PB><<<(unsigned)((int64_t)n_tiles * bpt), w.threads, 0, s>>>(a, w.pb, bpt, far);
         }
-        note_launch();
-        sim_window_kernel<V, PB, true><<<grid, w.threads, smem, s>>>(a, w.pb, bpt, table_step,
-                                                                     far + (int64_t)far_row * a.N * w.pb);
+        row = far + (int64_t)far_row * a.N * w.pb;
+    }
+    note_launch();
+    if constexpr (SPLIT) {
+        if (w.far) sim_window_split_kernel<true><<<grid, w.threads, smem, s>>>(a, w.pb, bpt_w, table_step, row);
+        else sim_window_split_kernel<false><<<grid, w.threads, smem, s>>>(a, w.pb, bpt_w, table_step, row);
     } else {
-        note_launch();
-        sim_window_kernel<V, PB, false><<<grid, w.threads, smem, s>>>(a, w.pb, bpt, table_step, nullptr);
+        if (w.far) sim_window_kernel<V, PB, true><<<grid, w.threads, smem, s>>>(a, w.pb, bpt_w, table_step, row);
+        else sim_window_kernel<V, PB, false><<<grid, w.threads, smem, s>>>(a, w.pb, bpt_w, table_step, row);
     }
     return cudaGetLastError();
 }
 
 }  // namespace
 
-bool sim_window_plan(int32_t d_min, int32_t N, int64_t P, bool reduced, int sms, WindowPlan& w)
+bool sim_window_plan(int32_t d_min, int32_t N, int64_t P, int64_t P_group, bool reduced, int sms, WindowPlan& w)
 {
     if (d_min < 1) return false;
     w.far = d_min < WIN_NEAR_BELOW;
     w.steps = d_min < WIN_MAX_STEPS ? d_min : WIN_MAX_STEPS;
-    // packed pairs of sets (fewer instructions per step, half the threads) when
-    // they still give every SM four warps per scheduler
-    w.packed = reduced && (int64_t)N * P >= (int64_t)sms * 4 * WIN_THREADS;
+    // packed pairs of sets (fewer instructions per step, half the threads) from
+    // four warps per scheduler of single ones on: 1,001 x 68 (448 pairs per SM)
+    // took 1.50 ms packed and 1.45 single, 1,500 x 68 the same either way. Two
+    // lanes per pair while the chain of a step bounds the sweep: 16 x 68 took
+    // 0.99 ms per 1,000 steps against 1.39, 400 x 68 (179 pairs per SM) 0.55
+    // against 0.62, 600 x 68 (268) 0.95 against 0.74.
+    const int64_t pairs = (int64_t)N * P;
+    w.packed = reduced && pairs >= (int64_t)sms * 512;
+    w.split = reduced && pairs <= (int64_t)sms * 192;
     w.pb = 64;
-    while (w.pb > 2 && w.pb / 2 >= P) w.pb /= 2;
-    const int64_t threads = (int64_t)N * (w.packed ? (P + 1) / 2 : P);
+    while (w.pb > 2 && w.pb / 2 >= P_group) w.pb /= 2;
+    const int64_t threads = w.packed ? (pairs + 1) / 2 : (w.split ? 2 * pairs : pairs);
     // smaller CTAs spread a sweep that cannot fill the chip over more SMs
     w.threads = threads >= (int64_t)sms * WIN_THREADS ? WIN_THREADS : (threads >= (int64_t)sms * 64 ? 64 : 32);
     return true;
@@ -459,7 +593,8 @@ cudaError_t launch_sim_window(const SimArgs& a, const WindowPlan& w, int32_t n_t
     if (n_tiles <= 0 || a.n_chunk <= 0) return cudaSuccess;
     if (w.packed) return w.pb == 64 ? launch_v<float2, 64>(a, w, n_tiles, table_step, far, far_row, s)
                                     : launch_v<float2, 0>(a, w, n_tiles, table_step, far, far_row, s);
-    return launch_v<float, 0>(a, w, n_tiles, table_step, far, far_row, s);
+    return w.split ? launch_v<float, 0, true>(a, w, n_tiles, table_step, far, far_row, s)
+                   : launch_v<float, 0>(a, w, n_tiles, table_step, far, far_row, s);
 }
 
 int32_t sim_batch_window_blocks(int32_t N, bool packed)

@@ -56,7 +56,7 @@ def _run(tvbx, inputs, kernel, n_steps, more=0, **kw):
     (5, 1, 1, 40, 4, False), (5, 1, 2, 41, 4, False), (7, 3, 7, 100, 10, True), (68, 2, 9, 130, 10, False),
     (68, 65, 16, 147, 7, False), (33, 131, 40, 90, 1, True), (68, 1203, 5, 63, 9, False), (68, 1251, 19, 50, 10, True),
     (200, 450, 12, 55, 5, False),
-    (200, 401, 3, 50, 10, True), (16, 70, 15, 64, 8, False),
+    (200, 401, 3, 50, 10, True), (16, 70, 15, 64, 8, False), (68, 701, 9, 44, 4, False), (100, 401, 2, 30, 3, True),
 ])
 def test_window_equals_general_kernel(tvbx, n_regions, n_sets, d_min, n_steps, tavg, noise):
     inputs = _inputs(tvbx, n_regions, n_sets, d_min)
@@ -69,6 +69,17 @@ def test_window_equals_general_kernel(tvbx, n_regions, n_sets, d_min, n_steps, t
     # the checkpoint's body (state, rings, noise) does not depend on the kernel
     header = 15 * 8
     assert np.array_equal(ck_want[header:], ck_got[header:])
+
+
+def test_window_of_the_general_template(tvbx):
+    """Unequal synaptic time constants take the template itself, one set per thread."""
+    W, L, pts = _inputs(tvbx, 30, 40, 6)
+    out = []
+    for kernel in (tvbx.KERNEL_GENERAL, tvbx.KERNEL_AUTO):
+        sw = tvbx.Sweep(W, L, points=pts, model=tvbx.make_model({"tau_i": 6.0}))
+        sw.run(dt_ms=DT, n_steps=50, tavg_steps=5, seed=3, kernel=kernel)
+        out.append((sw.state(), sw.series()))
+    assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][1], out[1][1])
 
 
 def test_window_with_several_speeds_restores_from_a_checkpoint(tvbx):
