@@ -507,14 +507,17 @@ static __device__ __forceinline__ float warp_sum(float x)
     return x;
 }
 
-// The same without windows, any N: 32 x 32 tiles of the upper triangle, read
-// along the rows; a tile's transpose goes through shared memory, so that both
-// triangles of the FC are written along their rows (column writes measured
-// 1.62 ms on 32,768 x 68 and 2.79 ms on 4,096 x 360).
+// The same without windows. The upper triangle is read along the rows, and both
+// triangles of the FC are written along theirs: through the whole matrix in
+// shared memory (WHOLE, up to FIN_WHOLE regions), else through the transposes
+// of 32 x 32 tiles (column writes measured 1.62 ms on 32,768 x 68 and 2.79 ms
+// on 4,096 x 360; tiles throughout 0.94 and 1.96).
+constexpr int FIN_WHOLE = 112;   // 50 KB: four CTAs per SM
 constexpr int FIN_THREADS = 256;
 constexpr int FIN_WARPS = FIN_THREADS / 32;
 
-__global__ void __launch_bounds__(FIN_THREADS, 4)
+template <bool WHOLE>
+__global__ void __launch_bounds__(FIN_THREADS, 3)
 fc_finish_kernel(const __grid_constant__ FcArgs a)
 {
     extern __shared__ float sm[];
@@ -526,7 +529,6 @@ fc_finish_kernel(const __grid_constant__ FcArgs a)
     const int64_t Tn = a.t_end - a.t_begin;
     float* sS = sm;                        // [N] row sums
     float* isd = sS + N;                   // [N] 1 / sd (0 if sd = 0)
-    float (*tr)[32][33] = reinterpret_cast<float (*)[32][33]>(isd + N);   // [2] tiles
     __shared__ float red[3][FIN_WARPS];
     const float invT = Tn > 0 ? 1.0f / (float)Tn : 0.0f;
     float* fc = a.fc ? a.fc + p * N * N : nullptr;
@@ -548,39 +550,71 @@ fc_finish_kernel(const __grid_constant__ FcArgs a)
     }
     if (zero) atomicOr(a.status + p, TVBX_SET_ZERO_VAR);
     __syncthreads();
-    const int nt = (N + 31) / 32;
-    int parity = 0;
-    for (int ti = 0; ti < nt; ++ti)
-        for (int tj = ti; tj < nt; ++tj, parity ^= 1) {
-            const int j = 32 * tj + lane;
-            const float sj = j < N ? sS[j] : 0.0f, ij = j < N ? isd[j] : 0.0f;
-#pragma unroll
-            for (int u = 0; u < 32 / FIN_WARPS; ++u) {
-                const int rr = warp + u * FIN_WARPS, r = 32 * ti + rr;
-                if (r >= N || j >= N || j < r) continue;
-                if (j == r) {
-                    if (fc) fc[(int64_t)r * N + r] = 1.0f;
-                    tr[parity][rr][lane] = 1.0f;
-                    continue;
-                }
+    if constexpr (WHOLE) {
+        // the whole FC in shared memory, pitch N | 1 (columns meet every bank)
+        const int pitch = N | 1;
+        float* F = isd + N;
+        for (int r = warp; r < N; r += FIN_WARPS) {
+            const float* Br = B + (int64_t)r * N;
+            const float sr = sS[r], ir = isd[r];
+            if (lane == 0) F[r * pitch + r] = 1.0f;
+#pragma unroll 3
+            for (int j = r + 1 + lane; j < N; j += 32) {
                 float g = 0.0f;
-                for (int b = 0; b < nb; ++b) g += B[b * stride_b + (int64_t)r * N + j];
-                const float c = g - sS[r] * sj * invT;
-                const float x = c * isd[r] * ij;
+                for (int b = 0; b < nb; ++b) g += Br[b * stride_b + j];
+                const float c = g - sr * sS[j] * invT;
+                const float x = c * ir * isd[j];
                 s_all += 2.0f * c;
                 s_fc += 2.0f * x;
-                if (fc) fc[(int64_t)r * N + j] = x;
-                tr[parity][rr][lane] = x;
-            }
-            if (!fc) continue;
-            __syncthreads();   // the tile is whole; the other buffer's readers are done with the tile before
-            const int c0 = 32 * ti + lane;
-#pragma unroll
-            for (int u = 0; u < 32 / FIN_WARPS; ++u) {
-                const int rr = warp + u * FIN_WARPS, r = 32 * tj + rr;
-                if (r < N && c0 < r) fc[(int64_t)r * N + c0] = tr[parity][lane][rr];
+                F[r * pitch + j] = x;
+                F[j * pitch + r] = x;
             }
         }
+        __syncthreads();
+        if (fc)
+            for (int i = tid; i < N * N; i += FIN_THREADS) fc[i] = F[i / N * pitch + i % N];
+    } else {
+        const int nt = (N + 31) / 32;
+        float (*tr)[32][33] = reinterpret_cast<float (*)[32][33]>(isd + N);   // [2] tiles
+        int parity = 0;
+        for (int ti = 0; ti < nt; ++ti)
+            for (int tj = ti; tj < nt; ++tj, parity ^= 1) {
+                const int j = 32 * tj + lane;
+                const float sj = j < N ? sS[j] : 0.0f, ij = j < N ? isd[j] : 0.0f;
+                float g[32 / FIN_WARPS];
+#pragma unroll
+                for (int u = 0; u < 32 / FIN_WARPS; ++u) g[u] = 0.0f;
+                for (int b = 0; b < nb; ++b)
+#pragma unroll
+                    for (int u = 0; u < 32 / FIN_WARPS; ++u) {
+                        const int r = 32 * ti + warp + u * FIN_WARPS;
+                        if (r < N && j < N && j > r) g[u] += B[b * stride_b + (int64_t)r * N + j];
+                    }
+#pragma unroll
+                for (int u = 0; u < 32 / FIN_WARPS; ++u) {
+                    const int rr = warp + u * FIN_WARPS, r = 32 * ti + rr;
+                    if (r >= N || j >= N || j < r) continue;
+                    if (j == r) {
+                        if (fc) fc[(int64_t)r * N + r] = 1.0f;
+                        continue;
+                    }
+                    const float c = g[u] - sS[r] * sj * invT;
+                    const float x = c * isd[r] * ij;
+                    s_all += 2.0f * c;
+                    s_fc += 2.0f * x;
+                    if (fc) fc[(int64_t)r * N + j] = x;
+                    tr[parity][rr][lane] = x;
+                }
+                if (!fc) continue;
+                __syncthreads();   // the tile is whole; the other buffer's readers are done with the tile before
+                const int c0 = 32 * ti + lane;
+#pragma unroll
+                for (int u = 0; u < 32 / FIN_WARPS; ++u) {
+                    const int rr = warp + u * FIN_WARPS, r = 32 * tj + rr;
+                    if (r < N && c0 < r) fc[(int64_t)r * N + c0] = tr[parity][lane][rr];
+                }
+            }
+    }
     s_all = warp_sum(s_all);
     s_diag = warp_sum(s_diag);
     s_fc = warp_sum(s_fc);
@@ -830,11 +864,13 @@ cudaError_t launch_fc_reduce(const FcArgs& a, int32_t m, int32_t nw, int64_t Lw,
 
 cudaError_t launch_fc_finalize(const FcArgs& a, cudaStream_t s)
 {
-    const size_t smem = sizeof(float) * (2 * (size_t)a.N + 2 * 32 * 33);
-    cudaError_t e = cudaFuncSetAttribute(fc_finish_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const bool whole = a.N <= FIN_WHOLE;
+    const size_t smem = sizeof(float) * (2 * (size_t)a.N + (whole ? (size_t)a.N * (a.N | 1) : 2 * 32 * 33));
+    auto kern = whole ? fc_finish_kernel<true> : fc_finish_kernel<false>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     note_launch();
-    fc_finish_kernel<<<a.P, FIN_THREADS, smem, s>>>(a);
+    kern<<<a.P, FIN_THREADS, smem, s>>>(a);
     return cudaGetLastError();
 }
 
