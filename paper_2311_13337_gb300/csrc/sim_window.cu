@@ -318,8 +318,11 @@ sim_window_kernel(const __grid_constant__ SimArgs a, int32_t pb_rt, int32_t bloc
 
 // The window of a sweep too small to fill the chip, where the chain of one step
 // bounds it: two lanes per pair, one per population (pair_step_split), each
-// forming the coupling sums of half the steps. Needs the reduced transfer
-// function (tau_e == tau_i).
+// forming the coupling sums of half the steps. The next step's noise and
+// coupling are read during a step: 16 x 68 took 0.85 ms per 1,000 steps with
+// that and 0.99 without. (In sim_window_kernel, whose warps hide those reads
+// from one another, the extra registers cost more: 32,768 x 68 went from 21.8
+// to 22.4 ms.) Needs the reduced transfer function (tau_e == tau_i).
 template <bool NEAR>
 __global__ void __launch_bounds__(WIN_THREADS, 2)
 sim_window_split_kernel(const __grid_constant__ SimArgs a, int32_t pb, int32_t blocks_per_tile, int64_t table_step,
@@ -390,10 +393,14 @@ sim_window_split_kernel(const __grid_constant__ SimArgs a, int32_t pb, int32_t b
     int slot_w = slot0;
     float* const ring_k = ring + (uint32_t)(k * HR) * (uint32_t)pb;
     const float* ou_p = a.ou_table + (own_noise ? 0 : table_step * N + k);
+    float ou_next = own_noise ? 0.0f : __ldg(ou_p), c_next = stash[0];   // the next step's, on the way
     for (int b = 0; b < steps; ++b) {
-        const float OU = own_noise ? ou : __ldg(ou_p);
-        ou_p += own_noise ? 0 : N;
-        pair_step_split(m, poly, pop, EL, cFe, cFi, sp, x, stash[b * PAIRS], OU, trk, lanes);
+        const float OU = own_noise ? ou : ou_next, c = c_next;
+        if (b + 1 < steps) {
+            if (!own_noise) ou_next = __ldg(ou_p += N);
+            c_next = stash[(b + 1) * PAIRS];
+        }
+        pair_step_split(m, poly, pop, EL, cFe, cFi, sp, x, c, OU, trk, lanes);
         if (own_noise) ou = next_ou(m, a.seed, n0 + (uint32_t)b, (uint32_t)k, pn, OU);
         ++slot_w;
         slot_w -= slot_w == H ? H : 0;
@@ -574,7 +581,7 @@ bool sim_window_plan(int32_t d_min, int32_t N, int64_t P, int64_t P_group, bool 
     // four warps per scheduler of single ones on: 1,001 x 68 (448 pairs per SM)
     // took 1.50 ms packed and 1.45 single, 1,500 x 68 the same either way. Two
     // lanes per pair while the chain of a step bounds the sweep: 16 x 68 took
-    // 0.99 ms per 1,000 steps against 1.39, 400 x 68 (179 pairs per SM) 0.55
+    // 0.85 ms per 1,000 steps against 1.39, 400 x 68 (179 pairs per SM) 0.50
     // against 0.62, 600 x 68 (268) 0.95 against 0.74.
     const int64_t pairs = (int64_t)N * P;
     w.packed = reduced && pairs >= (int64_t)sms * 512;
