@@ -73,6 +73,13 @@ __device__ __noinline__ float next_ou(const DevModel& m, uint64_t seed, uint32_t
     return fmaf(m.ou_a, m.ou_mu - OU, fmaf(m.ou_b, xi, OU));
 }
 
+// The launches below start their blocks as the last ones of the launch before end
+// (launch_next). Until this returns a block reads only its arguments and the
+// plan's tables, which the host wrote. No launch_dependents: with it, the next
+// launch's blocks take slots early and unevenly, and 1,500 x 68 went from 1.31 to
+// 1.50 ms instead of to 1.28.
+__device__ __forceinline__ void after_last_launch() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // Coupling sums of G steps from row `at` on: row entries [e0, e1) added to acc.
 // ring: row (j, slot) at (j HR + slot) pb. Four entries' loads are in flight
 // together (one: 27.1 ms, two: 23.5 ms, four: 21.9 ms on the sweep above).
@@ -139,6 +146,7 @@ sim_far_kernel(const __grid_constant__ SimArgs a, int32_t pb_rt, int32_t blocks_
     const int32_t ti = blockIdx.x / blocks_per_tile;
     const TileDev tile = a.tiles[ti];
     const WinSlot ws = win_slot<VSets<V>::n>(tile, (blockIdx.x % blocks_per_tile) * blockDim.x + threadIdx.x);
+    after_last_launch();
     if (ws.k >= a.N) return;
     far_pair<V, PB>(a, tile, a.groups[tile.group], ws, pb, (uint32_t)a.n0, far + (int64_t)ti * WIN_FAR * a.N * pb);
 }
@@ -310,6 +318,7 @@ sim_window_kernel(const __grid_constant__ SimArgs a, int32_t pb_rt, int32_t bloc
     const int32_t ti = blockIdx.x / blocks_per_tile;
     const TileDev tile = a.tiles[ti];
     const WinSlot ws = win_slot<VSets<V>::n>(tile, (blockIdx.x % blocks_per_tile) * blockDim.x + threadIdx.x);
+    after_last_launch();
     if (ws.k >= a.N) return;
     window_pair<V, PB, NEAR>(a, a.m, tile, a.groups[tile.group], ws, pb, (uint32_t)a.n0, a.n_chunk, table_step,
                              NEAR ? far + (int64_t)ti * WIN_FAR * a.N * pb : nullptr,
@@ -337,6 +346,7 @@ sim_window_split_kernel(const __grid_constant__ SimArgs a, int32_t pb, int32_t b
     const int N = a.N, pop = threadIdx.x & 1;
     const WinSlot ws = win_slot<1>(tile, ((blockIdx.x % blocks_per_tile) * blockDim.x + threadIdx.x) >> 1);
     const uint32_t lanes = __ballot_sync(0xffffffffu, ws.k < N);
+    after_last_launch();
     if (ws.k >= N) return;
     const int k = ws.k, q = ws.q, H = grp.H, HR = H + WIN_FAR, steps = a.n_chunk, ts = a.ts;
     const bool own_noise = a.noise_per_set != 0;
@@ -487,6 +497,7 @@ sim_batch_window_kernel(const __grid_constant__ DevModel m, const BatchJob* __re
     uint32_t* dst = reinterpret_cast<uint32_t*>(&s_job);
     for (int w = threadIdx.x; w < (int)(sizeof(BatchJob) / 4); w += WIN_THREADS) dst[w] = src[w];
     __syncthreads();
+    after_last_launch();
     const SimArgs& a = s_job.a;
     const WinTurn t = win_turn(turn, s_job.win_steps, s_job.far != nullptr, a.n_chunk);
     if (t.len == 0 || (FAR && (!s_job.far || t.row != 0))) return;
@@ -540,6 +551,27 @@ __global__ void ring_convert_kernel(float* __restrict__ ring, int32_t H, int32_t
     }
 }
 
+// Launch whose start overlaps the end of the launch before it on s; kern calls
+// after_last_launch. A window takes 5 to 400 us, a start about 2: 16 x 68
+// went from 0.85 to 0.77 ms per 1,000 steps, 1,001 x 68 at six speeds from 1.47
+// to 1.39, an eight-job batch from 8.9 to 8.4.
+template <class... P, class... A>
+cudaError_t launch_next(void (*kern)(P...), unsigned grid, unsigned threads, size_t smem, cudaStream_t s, A... args)
+{
+    cudaLaunchConfig_t c = {};
+    c.gridDim = dim3(grid);
+    c.blockDim = dim3(threads);
+    c.dynamicSmemBytes = smem;
+    c.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = at;
+    c.numAttrs = 1;
+    note_launch();
+    return cudaLaunchKernelEx(&c, kern, P(args)...);
+}
+
 // far sums (when due) and the window of every pair; S sets per thread, or (SPLIT) two threads per set
 template <class V, int PB, bool SPLIT = false>
 cudaError_t launch_v(const SimArgs& a, const WindowPlan& w, int32_t n_tiles, int64_t table_step, float* far,
@@ -554,20 +586,18 @@ cudaError_t launch_v(const SimArgs& a, const WindowPlan& w, int32_t n_tiles, int
     float* row = nullptr;
     if (w.far) {
         if (far_row == 0) {
-            note_launch();
-            sim_far_kernel<V, PB><<<(unsigned)((int64_t)n_tiles * bpt), w.threads, 0, s>>>(a, w.pb, bpt, far);
+            const cudaError_t e = launch_next(sim_far_kernel<V, PB>, (unsigned)((int64_t)n_tiles * bpt), w.threads, 0, s,
+                                              a, w.pb, bpt, far);
+            if (e != cudaSuccess) return e;
         }
         row = far + (int64_t)far_row * a.N * w.pb;
     }
-    note_launch();
-    if constexpr (SPLIT) {
-        if (w.far) sim_window_split_kernel<true><<<grid, w.threads, smem, s>>>(a, w.pb, bpt_w, table_step, row);
-        else sim_window_split_kernel<false><<<grid, w.threads, smem, s>>>(a, w.pb, bpt_w, table_step, row);
-    } else {
-        if (w.far) sim_window_kernel<V, PB, true><<<grid, w.threads, smem, s>>>(a, w.pb, bpt_w, table_step, row);
-        else sim_window_kernel<V, PB, false><<<grid, w.threads, smem, s>>>(a, w.pb, bpt_w, table_step, row);
-    }
-    return cudaGetLastError();
+    if constexpr (SPLIT)
+        return launch_next(w.far ? sim_window_split_kernel<true> : sim_window_split_kernel<false>, grid, w.threads, smem,
+                           s, a, w.pb, bpt_w, table_step, row);
+    else
+        return launch_next(w.far ? sim_window_kernel<V, PB, true> : sim_window_kernel<V, PB, false>, grid, w.threads,
+                           smem, s, a, w.pb, bpt_w, table_step, row);
 }
 
 }  // namespace
@@ -624,9 +654,8 @@ cudaError_t launch_sim_batch_window(const DevModel& m, bool packed, bool far, co
     if (n_blocks <= 0) return cudaSuccess;
     auto kern = packed ? (far ? sim_batch_window_kernel<float2, true> : sim_batch_window_kernel<float2, false>)
                        : (far ? sim_batch_window_kernel<float, true> : sim_batch_window_kernel<float, false>);
-    note_launch();
-    kern<<<n_blocks, WIN_THREADS, far ? 0 : (packed ? 8 : 4) * (size_t)WIN_THREADS * steps, s>>>(m, jobs, blocks, turn);
-    return cudaGetLastError();
+    return launch_next(kern, n_blocks, WIN_THREADS, far ? 0 : (packed ? 8 : 4) * (size_t)WIN_THREADS * steps, s, m, jobs,
+                       blocks, turn);
 }
 
 cudaError_t launch_ring_convert(bool out, float* ring, const WindowPlan& w, int32_t H, int32_t N, int32_t P_g,
