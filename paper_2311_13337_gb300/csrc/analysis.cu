@@ -414,22 +414,54 @@ __device__ __forceinline__ uint64_t diff_f32x2(uint64_t c, uint64_t a)
     asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(0xbf800000bf800000ull), "l"(c));
     return d;
 }
-// sign bits of both lanes shifted into w
-__device__ __forceinline__ void take_signs(uint32_t& w, uint64_t d)
+// The signs of both lanes as two halves: -1 (negative) or 0 in bits 0-15 and 16-31.
+__device__ __forceinline__ uint32_t sign_halves(uint64_t d)
 {
-    w = __funnelshift_l((uint32_t)d, w, 1);
-    w = __funnelshift_l((uint32_t)(d >> 32), w, 1);
+    uint32_t t;
+    asm("prmt.b32 %0, %1, %2, 0xffbb;" : "=r"(t) : "r"((uint32_t)d), "r"((uint32_t)(d >> 32)));
+    return t;
+}
+// min(m, |d|) over both lanes; NaN once a lane is NaN
+__device__ __forceinline__ float min_abs(float m, uint64_t d)
+{
+    float r;
+    asm("{\n .reg .f32 x, y;\n abs.f32 x, %1;\n abs.f32 y, %2;\n min.NaN.f32 %0, x, y, %3;\n}"
+        : "=f"(r) : "f"(__uint_as_float((uint32_t)d)), "f"(__uint_as_float((uint32_t)(d >> 32))), "f"(m));
+    return r;
+}
+// Negatives among the samples whose sign_halves were summed into s (fewer than
+// 65,536 per half): with l negatives in the low half and h in the high one,
+// -s = 65536 (h - l) + l.
+__device__ __forceinline__ int negatives(uint32_t s)
+{
+    const uint32_t l = -s & 0xffffu, h = (((-s - l) >> 16) + l) & 0xffffu;
+    return (int)(l + h);
+}
+// Samples of a pair without a sign (zero or NaN).
+__device__ __noinline__ int count_signless(const float* xk, const float* yk, const float* xj, const float* yj, int n)
+{
+    int c = 0;
+#pragma unroll 4
+    for (int t = 0; t < n; ++t) {
+        const float p = __fmul_rn(yk[t], xj[t]), q = __fmul_rn(xk[t], yj[t]);
+        c += !(p < q) && !(p > q);
+    }
+    return c;
 }
 
 // One CTA per (time slice, set): cnt[k][j] += sum_t sign(Im(z_k conj(z_j))) for
 // k < j over the slice (slices of a set balance the CTAs over the SMs: one CTA
-// per set left a third of the last wave). Time tiles of the planes of real and imaginary parts come by cp.async into
-// one of two buffers while the other is used. A thread owns a 4 x 4 block of
-// region pairs: per pair and two samples two packed products p, q and the
-// packed differences p - q and q - p, whose sign bits are shifted into two
-// words (a zero has neither) and counted every 32 samples. Bound by the FMA
-// and ALU pipes, about 4 issue slots per pair and sample (comparisons and
-// adds with predicates took 17: 4.98 ms per 1,024 x 68 x 5,000 in all).
+// per set left a third of the last wave). Time tiles of the planes of real and
+// imaginary parts come by cp.async into one of two buffers while the other is
+// used. A thread owns a 4 x 4 block of region pairs: per pair and two samples
+// two packed products p, q and the packed difference p - q, whose signs are
+// summed as halves, two differences to an add, and whose smallest magnitude is
+// kept; only where that is 0 or NaN are the tile's samples without a sign
+// counted (equal rows, silent regions, the zeros after a row's end), the others
+// being positive or negative. Bound by the FMA and ALU pipes, about 3 issue
+// slots per pair and sample, 2.5 ms per 1,024 x 68 x 5,000 (sign bits of p - q and of
+// q - p shifted into words took 4 and 3.2 ms, comparisons and adds with
+// predicates 17 and 4.98 ms).
 template <int PLI_TT>
 __global__ void __maxnreg__(128)   // 16 warps per SM: three CTAs of five
 an_pli_kernel(const float* __restrict__ z_all, int N, int ns, int slice, int slices, int* __restrict__ cnt_all)
@@ -466,12 +498,12 @@ an_pli_kernel(const float* __restrict__ z_all, int N, int ns, int slice, int sli
             while (rem >= NB - bk) { rem -= NB - bk; ++bk; }
             bj = bk + rem;
         }
-        int cnt[4][4];
-        uint32_t wp[4][4], wn[4][4];
+        uint32_t sg[4][4];
+        float least[4][4];   // smallest |p - q| of a tile
 #pragma unroll
         for (int u = 0; u < 4; ++u)
 #pragma unroll
-            for (int v = 0; v < 4; ++v) cnt[u][v] = 0, wp[u][v] = wn[u][v] = 0u;
+            for (int v = 0; v < 4; ++v) sg[u][v] = 0u;
         __syncthreads();   // the buffers are free
         fetch(t_lo, tile);
         float* cur = tile;
@@ -484,7 +516,10 @@ an_pli_kernel(const float* __restrict__ z_all, int N, int ns, int slice, int sli
             if (bp < nbp) {
                 const float* xk0 = cur + bk * PLI_TS;
                 const float* xj0 = cur + bj * PLI_TS;
-                int since = 0;
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+#pragma unroll
+                    for (int v = 0; v < 4; ++v) least[u][v] = 1.0f;   // any positive number
                 for (int t = 0; t < tl; t += 4) {
                     ulonglong2 xk[4], yk[4];
 #pragma unroll
@@ -499,27 +534,22 @@ an_pli_kernel(const float* __restrict__ z_all, int N, int ns, int slice, int sli
 #pragma unroll
                         for (int u = 0; u < 4; ++u) {
                             // Im(z_k conj(z_j)) = y_k x_j - x_k y_j, each product rounded
-                            uint64_t p = mul_f32x2(yk[u].x, xj.x), q = mul_f32x2(xk[u].x, yj.x);
-                            take_signs(wn[u][v], diff_f32x2(p, q));
-                            take_signs(wp[u][v], diff_f32x2(q, p));
-                            p = mul_f32x2(yk[u].y, xj.y);
-                            q = mul_f32x2(xk[u].y, yj.y);
-                            take_signs(wn[u][v], diff_f32x2(p, q));
-                            take_signs(wp[u][v], diff_f32x2(q, p));
+                            const uint64_t d0 = diff_f32x2(mul_f32x2(yk[u].x, xj.x), mul_f32x2(xk[u].x, yj.x));
+                            const uint64_t d1 = diff_f32x2(mul_f32x2(yk[u].y, xj.y), mul_f32x2(xk[u].y, yj.y));
+                            sg[u][v] += sign_halves(d0) + sign_halves(d1);
+                            least[u][v] = min_abs(min_abs(least[u][v], d0), d1);
                         }
                     }
-                    since += 4;
-                    if (since == 32 || t + 4 >= tl) {
-                        since = 0;
-#pragma unroll
-                        for (int u = 0; u < 4; ++u)
-#pragma unroll
-                            for (int v = 0; v < 4; ++v) {
-                                cnt[u][v] += __popc(wp[u][v]) - __popc(wn[u][v]);
-                                wp[u][v] = wn[u][v] = 0u;
-                            }
-                    }
                 }
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+#pragma unroll
+                    for (int v = 0; v < 4; ++v)
+                        if (const int kk = bk * 4 + u, jj = bj * 4 + v; !(least[u][v] > 0.0f) && kk < jj && jj < N) {
+                            const float *rk = xk0 + u * NB * PLI_TS, *rj = xj0 + v * NB * PLI_TS;
+                            const int none = count_signless(rk, rk + plane, rj, rj + plane, tl);
+                            atomicAdd(cnt_all + ((int64_t)b * N + kk) * N + jj, -none);
+                        }
             }
             cur = next;
         }
@@ -529,7 +559,7 @@ an_pli_kernel(const float* __restrict__ z_all, int N, int ns, int slice, int sli
 #pragma unroll
                 for (int v = 0; v < 4; ++v) {
                     const int kk = bk * 4 + u, jj = bj * 4 + v;
-                    if (kk < jj && jj < N) atomicAdd(cnt_all + ((int64_t)b * N + kk) * N + jj, cnt[u][v]);
+                    if (kk < jj && jj < N) atomicAdd(cnt_all + ((int64_t)b * N + kk) * N + jj, t_hi - t_lo - 2 * negatives(sg[u][v]));
                 }
         }
     }

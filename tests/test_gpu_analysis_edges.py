@@ -55,3 +55,20 @@ def test_metrics_at_edges(tvbx, n_regions, n_samples):
                 assert abs(g - w) <= 1e-3 * abs(w), name
             else:
                 assert abs(g - w) <= 1e-4 * abs(w) + 1e-7, name
+
+
+@pytest.mark.parametrize("n_regions,n_samples", [(6, 100), (68, 1301), (101, 64)])
+def test_phase_lag_without_sign(tvbx, n_regions, n_samples):
+    """A region of NaN or infinities has no sign in any pair, like a silent one,
+    and the other pairs keep theirs; a set of silent regions has none."""
+    import torch
+    rng = np.random.default_rng(n_regions)
+    x = (5e-3 + 1e-3 * rng.standard_normal((4, n_regions, n_samples))).astype(np.float32)
+    x[1:] = x[0]
+    x[0, 2] = 2e-3
+    x[1, 2] = np.nan
+    x[2, 2, 7] = np.inf
+    x[3] = 2e-3
+    out, _ = tvbx.series_analysis(torch.from_numpy(x).cuda(), 1.0)
+    lag = out.cpu().numpy()[:, tvbx.AN_FIELDS.index("mean_pli")]
+    assert lag[0] > 0 and lag[1] == lag[0] and lag[2] == lag[0] and lag[3] == 0
