@@ -41,6 +41,7 @@
 
 #include "gemm_simt.cuh"
 #include "internal.h"
+#include "launch_next.cuh"
 #include "ptx_async.cuh"
 
 namespace tvbx {
@@ -255,6 +256,7 @@ __global__ void __launch_bounds__(TCG_THREADS) mlp_gemm_tc_kernel(const GemmArgs
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = tmem_slot;
+    after_last_launch();
 
     const TA* Am = A + (int64_t)m0 * g.sam;
     const TB* Bn = B + (int64_t)n0 * g.sbn;
@@ -375,12 +377,47 @@ __global__ void __launch_bounds__(TCG_THREADS) mlp_gemm_tc_kernel(const GemmArgs
     if (t < 32) tmem_dealloc(tmem, (uint32_t)TCG_N);
 }
 
-// C(member) = sum over splits of the partial tiles, in split order.
-__global__ void mlp_splitk_reduce_kernel(const float* __restrict__ part, int splits, int E, int M, int N,
-                                         float* __restrict__ C, int64_t ldc, int64_t c_mem)
+// Column sums of X [E][rows][n] to out, a member every out_mem (a layer's bias
+// gradient): 8 row-interleaved sums per column.
+struct ColumnSums {
+    const float* X = nullptr;
+    float* out = nullptr;
+    int rows = 0, n = 0;
+    int64_t out_mem = 0;
+};
+__device__ __forceinline__ void column_sums(const ColumnSums& c, int mem, int block)
 {
-    const int64_t MN = (int64_t)M * N, total = (int64_t)E * MN;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
+    const int o = block * 32 + (threadIdx.x & 31);
+    const int q = threadIdx.x >> 5;
+    float s = 0.0f;
+    if (o < c.n)
+#pragma unroll 16
+        for (int r = q; r < c.rows; r += 8) s += c.X[((int64_t)mem * c.rows + r) * c.n + o];
+    __shared__ float red[8][33];
+    red[q][threadIdx.x & 31] = s;
+    __syncthreads();
+    if (q == 0 && o < c.n) {
+        float t = 0.0f;
+        for (int i = 0; i < 8; ++i) t += red[i][threadIdx.x & 31];
+        c.out[mem * c.out_mem + o] = t;
+    }
+}
+
+// The first `sums` blocks: column sums. The others: C(member) = sum over splits
+// of the partial tiles, in split order. Both wait on memory with few loads in
+// flight, so they share a launch; 256 threads.
+__global__ void __launch_bounds__(256)
+mlp_reduce_kernel(const ColumnSums c, int sums, const float* __restrict__ part, int splits, int E, int M, int N,
+                  float* __restrict__ C, int64_t ldc, int64_t c_mem)
+{
+    after_last_launch();
+    if ((int)blockIdx.x < sums) {
+        const int per = sums / E;
+        column_sums(c, blockIdx.x / per, blockIdx.x % per);
+        return;
+    }
+    const int64_t MN = (int64_t)M * N, total = (int64_t)E * MN, step = (int64_t)(gridDim.x - sums) * blockDim.x;
+    for (int64_t i = (int64_t)(blockIdx.x - sums) * blockDim.x + threadIdx.x; i < total; i += step) {
         const int64_t mem = i / MN, r = i % MN;
         float acc = 0.0f;
 #pragma unroll 8
@@ -392,9 +429,11 @@ __global__ void mlp_splitk_reduce_kernel(const float* __restrict__ part, int spl
 // Launch on E members; error: device word that receives TVBX_DEVERR_TIMEOUT
 // when a bounded wait expires (the outputs are then invalid). part / part_cap
 // (floats): scratch for split K (plain-store epilogue only; nullptr: none).
+// sums: column sums to form beside the product (X nullptr: none).
 template <typename TA, typename TB, int EPI>
 static inline cudaError_t gemm_tc(const GemmArgs& g, int E, uint32_t* error, uint32_t wait_limit, cudaStream_t s,
-                                  float* part = nullptr, size_t part_cap = 0)
+                                  float* part = nullptr, size_t part_cap = 0,
+                                  const ColumnSums& sums = {})
 {
     if (g.M <= 0 || g.N <= 0 || g.K <= 0) return cudaSuccess;
     auto kern = mlp_gemm_tc_kernel<TA, TB, EPI>;
@@ -413,14 +452,13 @@ static inline cudaError_t gemm_tc(const GemmArgs& g, int E, uint32_t* error, uin
     const int cps = (n_chunks + splits - 1) / splits;
     splits = (n_chunks + cps - 1) / cps;   // every split owns at least one chunk
     dim3 grid((g.N + TCG_N - 1) / TCG_N, (g.M + TCG_M - 1) / TCG_M, E * splits);
-    note_launch();
-    kern<<<grid, TCG_THREADS, TCG_SMEM, s>>>(g, error, wait_limit, splits, cps, splits > 1 ? part : nullptr);
-    if ((e = cudaGetLastError()) != cudaSuccess || splits == 1) return e;
+    e = launch_next(kern, grid, TCG_THREADS, TCG_SMEM, s, g, error, wait_limit, splits, cps, splits > 1 ? part : nullptr);
+    const int sum_blocks = sums.X ? (sums.n + 31) / 32 * E : 0;
+    if (e != cudaSuccess || (splits == 1 && sum_blocks == 0)) return e;
     const int64_t total = (int64_t)E * g.M * g.N;
-    note_launch();
-    mlp_splitk_reduce_kernel<<<(unsigned)std::min<int64_t>((total + 255) / 256, 4 * 152), 256, 0, s>>>(
-        part, splits, E, g.M, g.N, g.C, g.ldc, g.c_mem);
-    return cudaGetLastError();
+    const int blocks = splits > 1 ? (int)std::min<int64_t>((total + 255) / 256, 4 * 152) : 0;
+    return launch_next(mlp_reduce_kernel, dim3(sum_blocks + blocks), 256, 0, s, sums, sum_blocks, part, splits, E, g.M, g.N,
+                       g.C, g.ldc, g.c_mem);
 }
 
 }  // namespace tvbx

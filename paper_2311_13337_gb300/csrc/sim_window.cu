@@ -39,6 +39,7 @@
 #include <type_traits>
 
 #include "internal.h"
+#include "launch_next.cuh"
 #include "model_device.cuh"
 
 namespace tvbx {
@@ -72,13 +73,6 @@ __device__ __noinline__ float next_ou(const DevModel& m, uint64_t seed, uint32_t
     const float xi = std_normal(seed, n, k, p);
     return fmaf(m.ou_a, m.ou_mu - OU, fmaf(m.ou_b, xi, OU));
 }
-
-// The launches below start their blocks as the last ones of the launch before end
-// (launch_next). Until this returns a block reads only its arguments and the
-// plan's tables, which the host wrote. No launch_dependents: with it, the next
-// launch's blocks take slots early and unevenly, and 1,500 x 68 went from 1.31 to
-// 1.50 ms instead of to 1.28.
-__device__ __forceinline__ void after_last_launch() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // Coupling sums of G steps from row `at` on: row entries [e0, e1) added to acc.
 // ring: row (j, slot) at (j HR + slot) pb. Four entries' loads are in flight
@@ -551,27 +545,10 @@ __global__ void ring_convert_kernel(float* __restrict__ ring, int32_t H, int32_t
     }
 }
 
-// Launch whose start overlaps the end of the launch before it on s; kern calls
-// after_last_launch. A window takes 5 to 400 us, a start about 2: 16 x 68
-// went from 0.85 to 0.77 ms per 1,000 steps, 1,001 x 68 at six speeds from 1.47
-// to 1.39, an eight-job batch from 8.9 to 8.4.
-template <class... P, class... A>
-cudaError_t launch_next(void (*kern)(P...), unsigned grid, unsigned threads, size_t smem, cudaStream_t s, A... args)
-{
-    cudaLaunchConfig_t c = {};
-    c.gridDim = dim3(grid);
-    c.blockDim = dim3(threads);
-    c.dynamicSmemBytes = smem;
-    c.stream = s;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    c.attrs = at;
-    c.numAttrs = 1;
-    note_launch();
-    return cudaLaunchKernelEx(&c, kern, P(args)...);
-}
-
+// A window takes 5 to 400 us: launches that start under the end of the last one
+// (launch_next) took 16 x 68 from 0.85 to 0.77 ms per 1,000 steps, 1,001 x 68 at
+// six speeds from 1.47 to 1.39, an eight-job batch from 8.9 to 8.4.
+//
 // far sums (when due) and the window of every pair; S sets per thread, or (SPLIT) two threads per set
 template <class V, int PB, bool SPLIT = false>
 cudaError_t launch_v(const SimArgs& a, const WindowPlan& w, int32_t n_tiles, int64_t table_step, float* far,

@@ -30,6 +30,7 @@
 #include "internal.h"
 #include "gemm_simt.cuh"
 #include "gemm_tc.cuh"
+#include "launch_next.cuh"
 #include "model_device.cuh"
 #include "tvbx.h"
 
@@ -97,6 +98,7 @@ __global__ void mlp_batch_kernel(const float* __restrict__ X, const float* __res
                                  const float* __restrict__ mu, const float* __restrict__ sd, float* __restrict__ xb,
                                  float* __restrict__ tb)
 {
+    after_last_launch();
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
     const int m = blockIdx.y;
     if (r >= rows) return;
@@ -113,6 +115,7 @@ __global__ void mlp_batch_kernel(const float* __restrict__ X, const float* __res
 __global__ void mlp_loss_kernel(const float* __restrict__ y, const float* __restrict__ t, int rows, int n_out,
                                 float* __restrict__ dz, double* __restrict__ loss)
 {
+    after_last_launch();
     const int m = blockIdx.y;
     const int64_t cnt = (int64_t)rows * n_out;
     const float scale = 2.0f / (float)cnt;
@@ -132,33 +135,13 @@ __global__ void mlp_loss_kernel(const float* __restrict__ y, const float* __rest
     if (threadIdx.x == 0) atomicAdd(loss + m, red[0] / (double)cnt);
 }
 
-// db[o] = sum over rows of dZ[row][o]; grid (ceil(n_out / 32), members).
-__global__ void mlp_bias_grad_kernel(const float* __restrict__ dz, int rows, int n_out, float* __restrict__ g,
-                                     int64_t g_mem)
-{
-    const int m = blockIdx.y;
-    const int o = blockIdx.x * 32 + (threadIdx.x & 31);
-    const int q = threadIdx.x >> 5;
-    float s = 0.0f;
-    if (o < n_out)
-#pragma unroll 16
-        for (int r = q; r < rows; r += 8) s += dz[((int64_t)m * rows + r) * n_out + o];
-    __shared__ float red[8][33];
-    red[q][threadIdx.x & 31] = s;
-    __syncthreads();
-    if (q == 0 && o < n_out) {
-        float t = 0.0f;
-        for (int i = 0; i < 8; ++i) t += red[i][threadIdx.x & 31];
-        g[m * g_mem + o] = t;
-    }
-}
-
 // AdamW on every parameter of every member; decay[j] marks weight entries.
 __global__ void mlp_adamw_kernel(float* __restrict__ p, __nv_bfloat16* __restrict__ pb, float* __restrict__ m1,
                                  float* __restrict__ m2, const float* __restrict__ g,
                                  const uint8_t* __restrict__ decay, int64_t n_par, int E, float lr, float wd,
                                  float b1, float b2, float eps, float bc1, float bc2)
 {
+    after_last_launch();
     const int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (idx >= n_par * E) return;
     const int64_t j = idx % n_par;
@@ -404,30 +387,24 @@ cudaError_t backward(tvbx_surrogate* s, int rows)
     float* dzn = s->dz1.p;
     {
         dim3 grid(std::min(64, (rows * s->n_out + 255) / 256), s->E);
-        note_launch();
-        mlp_loss_kernel<<<grid, 256, 0, s->stream>>>(s->act.p + act_offset(s, L, rows), s->tb.p, rows, s->n_out, dz,
-                                                     s->loss.p);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        e = launch_next(mlp_loss_kernel, grid, 256, 0, s->stream, s->act.p + act_offset(s, L, rows), s->tb.p, rows,
+                        s->n_out, dz, s->loss.p);
+        if (e != cudaSuccess) return e;
     }
     for (int l = L - 1; l >= 0; --l) {
         const int I = s->dims[l], O = s->dims[l + 1];
         const float* a_prev = s->act.p + act_offset(s, l, rows);
-        // dW_l = dZ^T a_prev
+        // dW_l = dZ^T a_prev and db_l = the column sums of dZ
+        ColumnSums db;
+        db.X = dz; db.out = s->g.p + s->b_off[l]; db.rows = rows; db.n = O; db.out_mem = s->n_par;
         GemmArgs gw{};
         gw.A = dz; gw.sam = 1; gw.sak = O; gw.a_mem = (int64_t)rows * O;
         gw.B = a_prev; gw.sbn = 1; gw.sbk = I; gw.b_mem = (int64_t)rows * I;
         gw.C = s->g.p + s->w_off[l]; gw.ldc = I; gw.c_mem = s->n_par;
         gw.M = O; gw.N = I; gw.K = rows;
-        if ((e = gemm_tc<float, float, EPI_STORE>(gw, s->E, s->err.p, kTcWait, s->stream, s->splitk.p, s->splitk.n)) !=
+        if ((e = gemm_tc<float, float, EPI_STORE>(gw, s->E, s->err.p, kTcWait, s->stream, s->splitk.p, s->splitk.n, db)) !=
             cudaSuccess)
             return e;
-        // db_l
-        {
-            dim3 grid((O + 31) / 32, s->E);
-            note_launch();
-            mlp_bias_grad_kernel<<<grid, 256, 0, s->stream>>>(dz, rows, O, s->g.p + s->b_off[l], s->n_par);
-            if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        }
         if (l == 0) break;
         // dZ_{l-1} = (dZ W_l) masked by a_prev > 0
         GemmArgs gd{};
@@ -657,20 +634,18 @@ tvbx_status tvbx_surrogate_train(tvbx_surrogate* s, int32_t mem, const float* X,
         int n_batches = 0;
         for (int64_t start = 0; start < n; start += batch) {
             const int rows = (int)std::min<int64_t>(batch, n - start);
-            note_launch();
-            mlp_batch_kernel<<<dim3((rows + 127) / 128, s->E), 128, 0, s->stream>>>(
-                dX, dY, n, s->n_in, s->n_out, start, rows, shuffle, hb, key, s->lo.p, s->hi.p, s->mu.p,
-                s->sd.p, s->act.p, s->tb.p);
-            SCK(cudaGetLastError(), "batch");
+            SCK(launch_next(mlp_batch_kernel, dim3((rows + 127) / 128, s->E), 128, 0, s->stream, dX, dY, n, s->n_in,
+                            s->n_out, start, rows, shuffle, hb, key, s->lo.p, s->hi.p, s->mu.p, s->sd.p, s->act.p,
+                            s->tb.p),
+                "batch");
             SCK(forward(s, rows), "forward");
             SCK(backward(s, rows), "backward");
             s->step += 1;
             const double bc1 = 1.0 - pow(b1, (double)s->step), bc2 = 1.0 - pow(b2, (double)s->step);
-            note_launch();
-            mlp_adamw_kernel<<<(unsigned)((np + 255) / 256), 256, 0, s->stream>>>(
-                s->p.p, s->pb.p, s->m1.p, s->m2.p, s->g.p, s->decay.p, s->n_par, s->E, lr, weight_decay, (float)b1,
-                (float)b2, 1e-8f, (float)bc1, (float)bc2);
-            SCK(cudaGetLastError(), "AdamW");
+            SCK(launch_next(mlp_adamw_kernel, dim3((unsigned)((np + 255) / 256)), 256, 0, s->stream, s->p.p, s->pb.p,
+                            s->m1.p, s->m2.p, s->g.p, s->decay.p, s->n_par, s->E, lr, weight_decay, (float)b1,
+                            (float)b2, 1e-8f, (float)bc1, (float)bc2),
+                "AdamW");
             ++n_batches;
         }
         if (loss_out) {
