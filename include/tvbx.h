@@ -162,9 +162,9 @@ typedef struct {
  *   state are those of TVBX_SERIES_KEEP, bit for bit. */
 #define TVBX_SERIES_KEEP 0
 #define TVBX_SERIES_STREAM 1
-#define TVBX_KERNEL_AUTO     0 /* fastest kernel that fits the sweep: without zero delays,
-                                  several steps per launch with no thread waiting for
-                                  another (tvbx_last_kernel then gives
+#define TVBX_KERNEL_AUTO     0 /* fastest kernel that fits the sweep: up to 768 regions, one
+                                  step more per launch than the shortest delay, with no
+                                  thread waiting for another (tvbx_last_kernel then gives
                                   TVBX_KERNEL_DIRECT: its state is in registers and its
                                   coupling read straight from the ring) */
 #define TVBX_KERNEL_DIRECT 100 /* register tiles for connectomes too large for the
@@ -472,14 +472,15 @@ tvbx_status tvbx_sweep_destroy(tvbx_sweep* h);
 
 /* ---- Batches of sweeps ----------------------------------------------------
  * Runs several sweeps -- different connectomes (region counts), durations,
- * conduction speeds (delay horizons) and grids -- as one persistent kernel
- * launch captured in a CUDA graph (the batched form of the lock-step
- * integration of Eq. 1-5). Every (job, tile of sets) is a work item; CTAs
- * take items from a global counter, most expensive first, and integrate the
- * tile over the job's whole duration with the general kernel (state in
- * shared memory, any region count). The graph holds the per-job state, ring
- * and OU-table initialisation, the queue reset and the persistent kernel;
- * one tvbx_batch_run is one graph launch. Each job's results are read
+ * conduction speeds (delay horizons) and grids -- together (the batched form
+ * of the lock-step integration of Eq. 1-5). Where all jobs share one model
+ * and have at most 768 regions, one launch per turn takes every job through its next
+ * window of steps, after a graph with the per-job state, ring and OU-table
+ * initialisation. Other batches, and those whose windows' rings do not fit in
+ * device memory, are one persistent launch in that graph: every (job, tile of
+ * sets) is a work item; CTAs take items from a global counter, most expensive
+ * first, and integrate the tile over the job's whole duration with the general
+ * kernel (state in shared memory, any region count). Each job's results are read
  * through its own handle afterwards (tvbx_summary, tvbx_fc, tvbx_series ...),
  * and equal those of tvbx_run with kernel = TVBX_KERNEL_GENERAL bit for bit
  * (the tile width does not change any set's arithmetic). */
@@ -502,9 +503,8 @@ tvbx_status tvbx_batch_create(tvbx_sweep* const* jobs, const tvbx_run_cfg* cfgs,
  * then two of the register-tile body (threads 512 and 768: each job with
  * N <= threads gets pb = 4 floor(threads / N) sets per CTA, 4 sets of one
  * region per thread; larger jobs keep the general body with a 200 KB budget).
- * Where no job has a zero delay and all share one model, the windowed body
- * (several steps of a tile between two CTA barriers) is timed besides, outside
- * the reported trials; it reads as (128, 64 KB).
+ * Where all jobs share one model and have at most 768 regions, windows are timed
+ * besides, outside the reported trials; they read as (128, 64 KB).
  * Runs are shortened to trial_steps steps per job. threads_out, smem_kb_out:
  * the choice (smem_kb_out is the general body's budget); trial_ms [n_trials]
  * (host, nullable; 8 entries, INFINITY where a candidate does not fit).
@@ -512,8 +512,9 @@ tvbx_status tvbx_batch_create(tvbx_sweep* const* jobs, const tvbx_run_cfg* cfgs,
 tvbx_status tvbx_batch_tune(tvbx_batch* b, int64_t trial_steps, int32_t* threads_out, int32_t* smem_kb_out,
                             float* trial_ms, int32_t* n_trials);
 
-/* Run every job (one graph launch; the first call builds the graph with
- * 512 threads and a 200 KB budget unless tvbx_batch_tune chose otherwise).
+/* Run every job (the first call builds the graph; where the batch has no
+ * windows, with 512 threads and a 200 KB budget unless tvbx_batch_tune chose
+ * otherwise).
  * The jobs' later calls run on the batch's stream. Synchronises it. */
 tvbx_status tvbx_batch_run(tvbx_batch* b);
 

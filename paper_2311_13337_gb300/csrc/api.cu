@@ -211,6 +211,7 @@ struct Group {
     std::vector<int32_t> row_ptr;
     std::vector<int32_t> row_near;  // first entry of each row with a delay below WIN_FAR
     std::vector<int32_t> row_mid;   // first zero-delay entry of each row
+    std::vector<int32_t> row_end;   // end of each row without the padding entry
     std::vector<uint32_t> col_dly;
     std::vector<float> w;
     int64_t ring_offset = 0;        // floats into the ring allocation
@@ -431,6 +432,7 @@ tvbx_status build_groups(tvbx_sweep* h, double dt, std::vector<Group>& groups)
         g.row_ptr.assign(N + 1, 0);
         g.row_near.assign(N, 0);
         g.row_mid.assign(N, 0);
+        g.row_end.assign(N, 0);
         int64_t dmax = 1;   // ring of at least 3 slots (the padding entries use d = 1)
         for (int k = 0; k < N; ++k) {
             // rows start at an index of the parity of k; a zero-weight entry pads the end of
@@ -456,6 +458,7 @@ tvbx_status build_groups(tvbx_sweep* h, double dt, std::vector<Group>& groups)
             for (auto& z : near) { g.col_dly.push_back(z.first); g.w.push_back(z.second); }
             g.row_mid[k] = (int32_t)g.col_dly.size();
             for (auto& z : zero) { g.col_dly.push_back(z.first); g.w.push_back(z.second); }
+            g.row_end[k] = (int32_t)g.col_dly.size();
         }
         g.row_ptr[N] = (int32_t)g.col_dly.size();
         g.H = (int32_t)(dmax + 2);
@@ -647,10 +650,10 @@ static tvbx_status prepare_run(tvbx_sweep* h, const tvbx_run_cfg& c, cudaStream_
         int dev = 0, sms = 0;
         CK(cudaGetDevice(&dev), "device");
         CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "device");
-        if (!sim_window_plan(d_min, N, P, largest_group, h->model.tau_e == h->model.tau_i, sms, win)) win = WindowPlan{};
+        sim_window_plan(d_min, N, P, largest_group, h->model.tau_e == h->model.tau_i, sms, win);
     }
     if (windows && general_pb > 0) {
-        if (win.steps == 0) return fail(TVBX_E_UNSUPPORTED, "no window of steps without coupling");
+        if (win.steps == 0) return fail(TVBX_E_UNSUPPORTED, "no windows for %d regions", N);
         win.pb = general_pb;
         win.packed = h->model.tau_e == h->model.tau_i;
         variant = -2;
@@ -723,6 +726,7 @@ static tvbx_status prepare_run(tvbx_sweep* h, const tvbx_run_cfg& c, cudaStream_
         all_row.insert(all_row.end(), g.row_ptr.begin(), g.row_ptr.end());
         all_row.insert(all_row.end(), g.row_mid.begin(), g.row_mid.end());
         all_row.insert(all_row.end(), g.row_near.begin(), g.row_near.end());
+        all_row.insert(all_row.end(), g.row_end.begin(), g.row_end.end());
         all_cd.insert(all_cd.end(), g.col_dly.begin(), g.col_dly.end());
         all_w.insert(all_w.end(), g.w.begin(), g.w.end());
         const int32_t Pg = (int32_t)g.sets.size();
@@ -784,6 +788,7 @@ static tvbx_status prepare_run(tvbx_sweep* h, const tvbx_run_cfg& c, cudaStream_
         d.row_ptr = h->d_csr_row.as<int32_t>() + row_off[gi];
         d.row_mid = h->d_csr_row.as<int32_t>() + row_off[gi] + N + 1;
         d.row_near = d.row_mid + N;
+        d.row_end = d.row_near + N;
         d.col_dly = h->d_csr_cd.as<uint32_t>() + nz_off[gi];
         d.w = h->d_csr_w.as<float>() + nz_off[gi];
         d.H = groups[gi].H;

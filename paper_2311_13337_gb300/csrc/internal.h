@@ -67,6 +67,7 @@ struct GroupDev {
                                // zero-delay entries
     const int32_t* row_near;   // [N] first entry of each row with a delay below WIN_FAR
     const int32_t* row_mid;    // [N] first zero-delay entry of each row
+    const int32_t* row_end;    // [N] end of each row without the padding entry
     const uint32_t* col_dly;   // [nnz] (delay << 16) | j
     const float* w;            // [nnz] u_kj
     int32_t H;                 // ring depth (max delay + 2; windowed: + 1 + steps per window)
@@ -150,7 +151,7 @@ int sim_fast_variants();
 size_t sim_fast_smem_bytes(int variant, int N, int nnz);
 // Windowed kernels (sim_window.cu): launches of `steps` steps of every pair.
 constexpr int WIN_MAX_STEPS = 32;
-// Sweeps whose shortest delay is below WIN_NEAR_BELOW steps sum the entries of
+// Sweeps whose windows are shorter than WIN_NEAR_BELOW steps sum the entries of
 // WIN_FAR steps and more for WIN_FAR steps at once (they come first in every row).
 constexpr int WIN_NEAR_BELOW = 8;
 constexpr int WIN_FAR = 16;
@@ -163,8 +164,8 @@ struct WindowPlan {
     bool far = false;      // far entries summed apart
 };
 // d_min: shortest delay of a nonzero weight in steps; P: sets of the sweep,
-// P_group: of its largest speed group. False when the sweep has no window.
-bool sim_window_plan(int32_t d_min, int32_t N, int64_t P, int64_t P_group, bool reduced, int sms, WindowPlan& w);
+// P_group: of its largest speed group.
+void sim_window_plan(int32_t d_min, int32_t N, int64_t P, int64_t P_group, bool reduced, int sms, WindowPlan& w);
 // far: buffer [n_tiles][WIN_FAR][N][pb] of the far sums (w.far); far_row: the
 // window's first step in it (0: the far sums are formed first).
 cudaError_t launch_sim_window(const SimArgs& a, const WindowPlan& w, int32_t n_tiles, int64_t table_step, float* far,

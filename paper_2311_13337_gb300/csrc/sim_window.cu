@@ -1,10 +1,10 @@
 // Windowed simulation kernels of the tvbx engine (arXiv 2311.13337, the
 // lock-step integration of Eq. 1-5 with forward Euler).
 //
-// No coupling reads a value younger than the shortest delay d_min of the
-// connectome, so over a window of B <= d_min steps every (set, region) pair
-// is independent of the others: the coupling sums of all B steps can be formed
-// from the ring before the first of them is taken. One launch advances every
+// Step n + b reads values of steps up to n + b - d_min, d_min the connectome's
+// shortest delay, and step n's are known: over a window of B <= d_min + 1 steps
+// every (set, region) pair is independent of the others, and the coupling sums
+// of all B steps can be formed from the ring before the first of them is taken. One launch advances every
 // pair by one window; launch order is the only synchronisation, so nothing
 // waits at a barrier, any number of regions or sets fills the chip evenly, and
 // each row entry is read once per window instead of once per step.
@@ -24,14 +24,11 @@
 // H = d_max + 1 + B, so that the window's own writes never meet a row that
 // another thread of the same launch may still read.
 //
-// Short delays (d_min < 8, large connectomes at high speeds): a window of d_min
-// steps alone would read each row entry for a few steps only. sim_far_kernel
-// then sums the entries with d >= WIN_FAR, which come first in each CSR row, for
-// WIN_FAR steps at once into a buffer [tile][WIN_FAR][N][pb]; the windows of
-// d_min steps start from those sums and add the few nearer entries.
-//
-// Zero delays (which read the current step) have no window; such sweeps take
-// the other kernels.
+// Short delays (B < 8, large connectomes at high speeds): a window alone would
+// read each row entry for a few steps only. sim_far_kernel then sums the entries
+// with d >= WIN_FAR, which come first in each CSR row, for WIN_FAR steps at once
+// into a buffer [tile][WIN_FAR][N][pb]; the windows start from those sums and add
+// the few nearer entries. Zero delays read the step before the window's only one.
 
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -166,7 +163,7 @@ __device__ __forceinline__ void window_pair(const SimArgs& a, const DevModel& m,
 
     // 1. coupling sums of the window
     {
-        const int e0 = NEAR ? grp.row_near[k] : grp.row_ptr[k], e1 = grp.row_mid[k];
+        const int e0 = NEAR ? grp.row_near[k] : grp.row_ptr[k], e1 = grp.row_end[k];
         const float* far_k = NEAR ? far + (int64_t)k * pb + q : nullptr;
         int b0 = 0;
         auto pass = [&](auto g_c) {
@@ -351,7 +348,7 @@ sim_window_split_kernel(const __grid_constant__ SimArgs a, int32_t pb, int32_t b
 
     // 1. coupling sums: of every 2 G steps a lane takes G
     {
-        const int e0 = NEAR ? grp.row_near[k] : grp.row_ptr[k], e1 = grp.row_mid[k];
+        const int e0 = NEAR ? grp.row_near[k] : grp.row_ptr[k], e1 = grp.row_end[k];
         const float* far_k = NEAR ? far + ((int64_t)ti * WIN_FAR * N + k) * pb + q : nullptr;
         int b0 = 0;
         auto pass = [&](auto g_c) {
@@ -579,17 +576,23 @@ cudaError_t launch_v(const SimArgs& a, const WindowPlan& w, int32_t n_tiles, int
 
 }  // namespace
 
-bool sim_window_plan(int32_t d_min, int32_t N, int64_t P, int64_t P_group, bool reduced, int sms, WindowPlan& w)
+void sim_window_plan(int32_t d_min, int32_t N, int64_t P, int64_t P_group, bool reduced, int sms, WindowPlan& w)
 {
-    if (d_min < 1) return false;
-    w.far = d_min < WIN_NEAR_BELOW;
-    w.steps = d_min < WIN_MAX_STEPS ? d_min : WIN_MAX_STEPS;
+    // d_min + 1 steps, less those that would need a gather pass of their own: 24 of
+    // 28 steps (32,768 x 68: 20.97 ms against 21.03, 21.70 at 27), 16 of 17 (1,001 x
+    // 68: 1.38 against 1.48), 8 of 13 (500 x 192: 1.67 against 1.84, 1.68 at 12), 4
+    // of 5 (16,384 x 68: 5.45 against 5.65); 6, 4, 3 and 2 beat 5, 3, 2 and 1
+    w.steps = d_min < WIN_MAX_STEPS - 1 ? d_min + 1 : WIN_MAX_STEPS;
+    if (w.steps >= 8) w.steps -= w.steps % 8;
+    else if (w.steps >= 5) w.steps -= w.steps % 2;
+    w.far = w.steps < WIN_NEAR_BELOW;
     // packed pairs of sets (fewer instructions per step, half the threads) from
     // four warps per scheduler of single ones on: 1,001 x 68 (448 pairs per SM)
     // took 1.50 ms packed and 1.45 single, 1,500 x 68 the same either way. Two
     // lanes per pair while the chain of a step bounds the sweep: 16 x 68 took
-    // 0.85 ms per 1,000 steps against 1.39, 400 x 68 (179 pairs per SM) 0.50
-    // against 0.62, 600 x 68 (268) 0.95 against 0.74.
+    // 0.85 ms per 1,000 steps against 1.39 (0.66 with windows of 24 that start
+    // under the last one's end), 400 x 68 (179 pairs per SM) 0.50 against 0.62, 600
+    // x 68 (268) 0.95 against 0.74.
     const int64_t pairs = (int64_t)N * P;
     w.packed = reduced && pairs >= (int64_t)sms * 512;
     w.split = reduced && pairs <= (int64_t)sms * 192;
@@ -598,7 +601,6 @@ bool sim_window_plan(int32_t d_min, int32_t N, int64_t P, int64_t P_group, bool 
     const int64_t threads = w.packed ? (pairs + 1) / 2 : (w.split ? 2 * pairs : pairs);
     // smaller CTAs spread a sweep that cannot fill the chip over more SMs
     w.threads = threads >= (int64_t)sms * WIN_THREADS ? WIN_THREADS : (threads >= (int64_t)sms * 64 ? 64 : 32);
-    return true;
 }
 
 cudaError_t launch_sim_window(const SimArgs& a, const WindowPlan& w, int32_t n_tiles, int64_t table_step, float* far,

@@ -930,7 +930,7 @@ class Surrogate:
 
 
 class Batch:
-    """Several sweeps run as one persistent launch in a CUDA graph
+    """Several sweeps run together, a launch for a window of steps of every job
     (tvbx_batch_*). jobs: list of (Sweep, dict of run settings)."""
 
     def __init__(self, jobs):

@@ -1,5 +1,4 @@
-"""The windowed simulation kernel (the automatic choice when no delay is zero)
-against the general kernel on the edges of its windows, tiles and gather
+"""The windowed simulation kernel (the automatic choice) against the general kernel on the edges of its windows, tiles and gather
 passes: state, series, status and checkpoint equal bit for bit (both sum the
 coupling in the same order and share the integrator)."""
 import numpy as np
@@ -49,14 +48,16 @@ def _run(tvbx, inputs, kernel, n_steps, more=0, **kw):
     return out, ck
 
 
-# d_min: far entries apart with windows of 1, 2, 5 and 7 steps; one window with
-# gather passes of 8, 4, 2 and 1, and the longest; sets: one, odd pairs, tiles
-# of 64 and a rest
+# d_min (windows of up to one step more): zero delays; far entries apart with
+# windows of 2 to 6 steps; windows of 8, 16, 24 and 32 steps and ends with gather
+# passes of 4, 2 and 1; sets: one, odd pairs, tiles of 64 and a rest
 @pytest.mark.parametrize("n_regions,n_sets,d_min,n_steps,tavg,noise", [
     (5, 1, 1, 40, 4, False), (5, 1, 2, 41, 4, False), (7, 3, 7, 100, 10, True), (68, 2, 9, 130, 10, False),
     (68, 65, 16, 147, 7, False), (33, 131, 40, 90, 1, True), (68, 1203, 5, 63, 9, False), (68, 1251, 19, 50, 10, True),
     (200, 450, 12, 55, 5, False),
     (200, 401, 3, 50, 10, True), (16, 70, 15, 64, 8, False), (68, 701, 9, 44, 4, False), (100, 401, 2, 30, 3, True),
+    (5, 1, 0, 40, 4, False), (68, 131, 0, 50, 10, True), (100, 401, 0, 30, 3, False), (200, 450, 0, 45, 5, False),
+    (68, 1203, 6, 48, 8, False), (68, 701, 7, 45, 9, False), (33, 70, 31, 99, 3, False), (33, 70, 30, 99, 3, False),
 ])
 def test_window_equals_general_kernel(tvbx, n_regions, n_sets, d_min, n_steps, tavg, noise):
     inputs = _inputs(tvbx, n_regions, n_sets, d_min)
