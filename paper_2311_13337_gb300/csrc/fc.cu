@@ -631,8 +631,7 @@ fc_finish_kernel(const __grid_constant__ FcArgs a)
 
 template <int MW>
 __global__ void __launch_bounds__(RED_THREADS)
-fc_reduce_kernel(const __grid_constant__ FcArgs a, int32_t m, int32_t nw, int64_t Lw, float* __restrict__ fcd,
-                 int32_t with_tri)
+fc_reduce_kernel(const __grid_constant__ FcArgs a, int32_t m, int32_t nw, int64_t Lw, float* __restrict__ fcd)
 {
     extern __shared__ float sm[];
     const int N = a.N, nb = a.n_blocks;
@@ -651,8 +650,6 @@ fc_reduce_kernel(const __grid_constant__ FcArgs a, int32_t m, int32_t nw, int64_
     float* red = V + (size_t)nw * M;        // [48] sums, [nw] inverse norms
     int* items = reinterpret_cast<int*>(red + 48 + nw);   // row-pass items
     const int n_items = fc_reduce_items(N);
-    // [M] the FC's upper triangle, written out along the rows after the row pass
-    float* tri = with_tri ? reinterpret_cast<float*>(items + n_items) : nullptr;
     const float invT = Tn > 0 ? 1.0f / (float)Tn : 0.0f;
     const float invL = Lw > 0 ? 1.0f / (float)Lw : 0.0f;
 
@@ -687,7 +684,7 @@ fc_reduce_kernel(const __grid_constant__ FcArgs a, int32_t m, int32_t nw, int64_
         s_all += cdg[k];
         s_diag += cdg[k];
         if (!(isd[k] > 0.0f)) zero = true;
-        if (fc && !tri) fc[(int64_t)k * N + k] = 1.0f;
+        if (fc) fc[(int64_t)k * N + k] = 1.0f;
     }
     // the row pass: items (row, 32-column chunk) dealt to the warps in turn,
     // so every warp gets the same number of chunks up to one
@@ -715,9 +712,7 @@ fc_reduce_kernel(const __grid_constant__ FcArgs a, int32_t m, int32_t nw, int64_
             const float f = c * ir * isd[jj];
             s_all += 2.0f * c;
             s_fc += 2.0f * f;
-            if (tri) {
-                tri[e0 + jj] = f;
-            } else if (fc) {
+            if (fc) {
                 fc[(int64_t)r * N + jj] = f;
                 fc[(int64_t)jj * N + r] = f;
             }
@@ -756,12 +751,6 @@ fc_reduce_kernel(const __grid_constant__ FcArgs a, int32_t m, int32_t nw, int64_
         a.chi[p] = den > 0.0f ? sqrtf(fmaxf(num / den, 0.0f)) : 0.0f;
         a.mean_fc[p] = N > 1 ? F / ((float)N * (float)(N - 1)) : 0.0f;
     }
-    if (fc && tri)
-        for (int r = warp; r < N; r += RED_WARPS)
-            for (int c = lane; c < N; c += 32) {
-                const int lo = c < r ? c : r, hi = c < r ? r : c;
-                fc[(int64_t)r * N + c] = lo == hi ? 1.0f : tri[lo * N - lo * (lo + 1) / 2 - lo - 1 + hi];
-            }
 
     // FCD: centre and normalise each window vector (a warp per window), then
     // the products of window u with up to four windows v > u per warp item
@@ -827,14 +816,10 @@ template <int MW>
 static cudaError_t launch_reduce_mw(const FcArgs& a, int32_t m, int32_t nw, int64_t Lw, float* fcd, size_t smem,
                                     cudaStream_t s)
 {
-    // the triangle buffer where it fits beside the window vectors
-    const size_t tri = sizeof(float) * (size_t)a.N * (a.N - 1) / 2;
-    const bool with_tri = smem + tri <= 200 * 1024;
-    if (with_tri) smem += tri;
     cudaError_t e = cudaFuncSetAttribute(fc_reduce_kernel<MW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     note_launch();
-    fc_reduce_kernel<MW><<<a.P, RED_THREADS, smem, s>>>(a, m, nw, Lw, fcd, with_tri ? 1 : 0);
+    fc_reduce_kernel<MW><<<a.P, RED_THREADS, smem, s>>>(a, m, nw, Lw, fcd);
     return cudaGetLastError();
 }
 
