@@ -396,8 +396,9 @@ an_series_kernel(const float* __restrict__ series, int N, int64_t T, FftPlan pla
     }
 }
 
-// Packed products with a zero addend: a zero product is +0, never -0, so the
-// differences below are +0 for equal products whatever their signs.
+// Packed products with a zero addend: a product that is zero is +0, and -0 is
+// left only where a negative one underflows. So of two products without a sign
+// the difference below is +0, but for -0 less +0 (which signless_sums counts).
 __device__ __forceinline__ uint64_t mul_f32x2(uint64_t a, uint64_t b)
 {
     uint64_t d;
@@ -437,16 +438,44 @@ __device__ __forceinline__ int negatives(uint32_t s)
     const uint32_t l = -s & 0xffffu, h = (((-s - l) >> 16) + l) & 0xffffu;
     return (int)(l + h);
 }
-// Samples of a pair without a sign (zero or NaN).
-__device__ __noinline__ int count_signless(const float* xk, const float* yk, const float* xj, const float* yj, int n)
+// Adds to none[u][v] what the n samples of the pairs of rows xk + u row and
+// xj + v row (imaginary parts a plane further) that have no sign (a difference
+// that is zero or NaN) count for as positive or negative ones: 1, or -1 for -0.
+__device__ __noinline__ void signless_sums(const float* xk, const float* xj, int row, int plane, int n, int (&none)[4][4])
 {
-    int c = 0;
-#pragma unroll 4
-    for (int t = 0; t < n; ++t) {
-        const float p = __fmul_rn(yk[t], xj[t]), q = __fmul_rn(xk[t], yj[t]);
-        c += !(p < q) && !(p > q);
+    int c[4][4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int v = 0; v < 4; ++v) c[u][v] = none[u][v];
+#pragma unroll 1
+    for (int t = 0; t < n; t += 4) {
+        ulonglong2 ak[4], bk[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            ak[u] = *reinterpret_cast<const ulonglong2*>(xk + u * row + t);
+            bk[u] = *reinterpret_cast<const ulonglong2*>(xk + plane + u * row + t);
+        }
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+            const ulonglong2 aj = *reinterpret_cast<const ulonglong2*>(xj + v * row + t);
+            const ulonglong2 bj = *reinterpret_cast<const ulonglong2*>(xj + plane + v * row + t);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const uint64_t d[2] = {diff_f32x2(mul_f32x2(bk[u].x, aj.x), mul_f32x2(ak[u].x, bj.x)),
+                                       diff_f32x2(mul_f32x2(bk[u].y, aj.y), mul_f32x2(ak[u].y, bj.y))};
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int x = (int)(uint32_t)(d[i >> 1] >> (i & 1) * 32);
+                    if (!(fabsf(__int_as_float(x)) > 0.0f)) c[u][v] += 1 | (x >> 31);
+                }
+            }
+        }
     }
-    return c;
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int v = 0; v < 4; ++v) none[u][v] = c[u][v];
 }
 
 // One CTA per (time slice, set): cnt[k][j] += sum_t sign(Im(z_k conj(z_j))) for
@@ -456,9 +485,11 @@ __device__ __noinline__ int count_signless(const float* xk, const float* yk, con
 // used. A thread owns a 4 x 4 block of region pairs: per pair and two samples
 // two packed products p, q and the packed difference p - q, whose signs are
 // summed as halves, two differences to an add, and whose smallest magnitude is
-// kept; only where that is 0 or NaN are the tile's samples without a sign
-// counted (equal rows, silent regions, the zeros after a row's end), the others
-// being positive or negative. Bound by the FMA and ALU pipes, about 3 issue
+// kept; only where that is 0 or NaN does a thread go over the tile again for its
+// samples without a sign (equal rows, silent regions, products that underflow, the
+// zeros after a row's end), the others being positive or negative: 1,024 x 68 x
+// 5,000 of silent regions take 14.5 ms with the transforms (16.9 with a count, and
+// an atomic, per pair). Bound by the FMA and ALU pipes, about 3 issue
 // slots per pair and sample, 2.5 ms per 1,024 x 68 x 5,000 (sign bits of p - q and of
 // q - p shifted into words took 4 and 3.2 ms, comparisons and adds with
 // predicates 17 and 4.98 ms).
@@ -504,6 +535,7 @@ an_pli_kernel(const float* __restrict__ z_all, int N, int ns, int slice, int sli
         for (int u = 0; u < 4; ++u)
 #pragma unroll
             for (int v = 0; v < 4; ++v) sg[u][v] = 0u;
+        int none[4][4] = {};   // in local memory
         __syncthreads();   // the buffers are free
         fetch(t_lo, tile);
         float* cur = tile;
@@ -541,15 +573,15 @@ an_pli_kernel(const float* __restrict__ z_all, int N, int ns, int slice, int sli
                         }
                     }
                 }
+                bool any = false;   // pairs with a sample without a sign
 #pragma unroll
                 for (int u = 0; u < 4; ++u)
 #pragma unroll
-                    for (int v = 0; v < 4; ++v)
-                        if (const int kk = bk * 4 + u, jj = bj * 4 + v; !(least[u][v] > 0.0f) && kk < jj && jj < N) {
-                            const float *rk = xk0 + u * NB * PLI_TS, *rj = xj0 + v * NB * PLI_TS;
-                            const int none = count_signless(rk, rk + plane, rj, rj + plane, tl);
-                            atomicAdd(cnt_all + ((int64_t)b * N + kk) * N + jj, -none);
-                        }
+                    for (int v = 0; v < 4; ++v) {
+                        const int kk = bk * 4 + u, jj = bj * 4 + v;
+                        any = any || (!(least[u][v] > 0.0f) && kk < jj && jj < N);
+                    }
+                if (any) signless_sums(xk0, xj0, NB * PLI_TS, plane, tl, none);
             }
             cur = next;
         }
@@ -559,7 +591,9 @@ an_pli_kernel(const float* __restrict__ z_all, int N, int ns, int slice, int sli
 #pragma unroll
                 for (int v = 0; v < 4; ++v) {
                     const int kk = bk * 4 + u, jj = bj * 4 + v;
-                    if (kk < jj && jj < N) atomicAdd(cnt_all + ((int64_t)b * N + kk) * N + jj, t_hi - t_lo - 2 * negatives(sg[u][v]));
+                    if (kk < jj && jj < N)
+                        atomicAdd(cnt_all + ((int64_t)b * N + kk) * N + jj,
+                                  t_hi - t_lo - 2 * negatives(sg[u][v]) - none[u][v]);
                 }
         }
     }

@@ -72,3 +72,31 @@ def test_phase_lag_without_sign(tvbx, n_regions, n_samples):
     out, _ = tvbx.series_analysis(torch.from_numpy(x).cuda(), 1.0)
     lag = out.cpu().numpy()[:, tvbx.AN_FIELDS.index("mean_pli")]
     assert lag[0] > 0 and lag[1] == lag[0] and lag[2] == lag[0] and lag[3] == 0
+
+
+@pytest.mark.parametrize("scale", [1e-19, 1e-21, 1e-22, 1e-23, 1e-24, 1e-30])
+@pytest.mark.parametrize("n_regions,n_samples", [(6, 100), (33, 1301)])
+def test_phase_lag_of_signals_whose_products_underflow(tvbx, scale, n_regions, n_samples):
+    """A sample has a sign where its two products, rounded to FP32, differ: none
+    where both underflow to zero, of either sign."""
+    import torch
+    rng = np.random.default_rng(n_samples)
+    x = (scale * rng.standard_normal((2, n_regions, n_samples))).astype(np.float32)
+    x[1, 0] = 5e-3   # a silent region beside them
+    out, used = tvbx.series_analysis(torch.from_numpy(x).cuda(), 1.0)
+    got = out.cpu().numpy()[:, tvbx.AN_FIELDS.index("mean_pli")]
+    for p in range(2):
+        z = [A.analytic_signal(row) for row in x[p].astype(np.float64)[:, n_samples - used:]]
+        re, im = np.float32([v.real for v in z]), np.float32([v.imag for v in z])
+        if p == 1:
+            re[0] = im[0] = 0.0
+        lag = []
+        for k in range(n_regions - 1):
+            a, b = im[k] * re[k + 1:], re[k] * im[k + 1:]
+            lag.append(abs((a > b).sum(axis=1) - (a < b).sum(axis=1)) / used)
+        want = np.concatenate(lag).mean()
+        # the transforms' relative error (about 1e-6) moves the rounding of one product
+        # of some 1e4 at most (products of 1e-43 are 100 units of the least FP32 number)
+        assert abs(got[p] - want) < 1e-3
+        if scale <= 1e-24:
+            assert got[p] == 0.0
