@@ -546,7 +546,7 @@ fc_finish_kernel(const __grid_constant__ FcArgs a)
         isd[k] = v > 0.0f ? rsqrtf(v) : 0.0f;
         s_all += v;
         s_diag += v;
-        if (!(v > 0.0f)) zero = true;
+        if (!(isd[k] > 0.0f)) zero = true;   // no variance, or one that overflowed
     }
     if (zero) atomicOr(a.status + p, TVBX_SET_ZERO_VAR);
     __syncthreads();

@@ -55,3 +55,19 @@ def test_fp32_fc_of_a_set_does_not_depend_on_the_others(tvbx, n_regions):
         out.append((fc[:5].clone(), chi[:5].clone()))
     for fc, chi in out[1:]:
         assert torch.equal(fc, out[0][0]) and torch.equal(chi, out[0][1])
+
+
+@pytest.mark.parametrize("n_regions", [5, 130])
+@pytest.mark.parametrize("window", [0, 32])
+def test_a_variance_beyond_fp32_is_flagged(tvbx, n_regions, window):
+    """A region whose squares overflow has no FC row, with windows and without."""
+    import torch
+    N, P, T = n_regions, 6, 64   # 64 samples: the shift is the mean of all of them
+    x = 5e-3 + 1e-3 * torch.randn((T, N, P), device="cuda")
+    x[:, 1, 2] = 3e18 * (1.0 - 2.0 * (torch.arange(T, device="cuda") % 2))   # sum of squares 5.8e38, of 32 samples 2.9e38
+    x[:, 1, 3] = 2e-3
+    fc, status = torch.empty((P, N, N), device="cuda"), torch.zeros(P, dtype=torch.int32, device="cuda")
+    fcd = torch.empty((P, 3, 3), device="cuda") if window else None
+    tvbx.fc_series(x, N, P, T, fc_out=fc, fcd_out=fcd, fcd_window=window, fcd_step=window // 2, set_status=status)
+    flagged = (status.cpu().numpy() & tvbx.SET_ZERO_VAR) != 0
+    assert flagged.tolist() == [False, False, True, True, False, False]
