@@ -100,3 +100,23 @@ def test_phase_lag_of_signals_whose_products_underflow(tvbx, scale, n_regions, n
         assert abs(got[p] - want) < 1e-3
         if scale <= 1e-24:
             assert got[p] == 0.0
+
+
+def test_threshold_keeps_the_last_bits_of_the_sum(tvbx):
+    """Three samples of one thread whose FP64 sum, 1 + 2^-24 + 2^-50, lies just
+    above a tie of the threshold's FP32 rounding: the sample at the threshold is
+    not above it."""
+    import torch
+    n = 1024
+    x = np.zeros((1, 2, n), dtype=np.float32)
+    x[0, 0, [0, 256, 512]] = 1.0, 2.0 ** -24, 2.0 ** -50
+    at = np.float32((1.0 + 2.0 ** -23) / n)
+    x[0, 0, [5, 261]] = at, -at
+    x[0, 1, ::3] = 1e-3
+    assert x[0, 0].sum(dtype=np.float64) == 1.0 + 2.0 ** -24 + 2.0 ** -50
+    out, used = tvbx.series_analysis(torch.from_numpy(x).cuda(), 1.0)
+    want = A.table2_metrics(x[0], 1.0)
+    assert used == n
+    got = out.cpu().numpy()[0]
+    for name in ("n_up", "up_samples", "n_down", "down_samples"):
+        assert got[tvbx.AN_FIELDS.index(name)] == want[name], name
