@@ -603,8 +603,8 @@ static int64_t group_ring_floats(const GroupDev& g, const WindowPlan& w, int N)
 // n_base > 0: the run continues a trajectory at global step n_base (state,
 // ring buffers and OU state are kept; the series and the running sums start
 // afresh for the new samples).
-static tvbx_status prepare_run(tvbx_sweep* h, const tvbx_run_cfg& c, cudaStream_t s, int general_pb,
-                               bool device_init, RunPlan& plan, bool direct_body, int64_t n_base, bool windows)
+static tvbx_status prepare_once(tvbx_sweep* h, const tvbx_run_cfg& c, cudaStream_t s, int general_pb,
+                                bool device_init, RunPlan& plan, bool direct_body, int64_t n_base, bool windows)
 {
     if (!(c.dt_ms > 0.0) || !isfinite(c.dt_ms)) return fail(TVBX_E_INVALID_ARG, "dt_ms must be > 0");
     if (c.n_steps < 0 || n_base + c.n_steps > ((int64_t)1 << 32) - 2)
@@ -780,15 +780,8 @@ static tvbx_status prepare_run(tvbx_sweep* h, const tvbx_run_cfg& c, cudaStream_
     CK(h->d_inv.ensure(sizeof(int64_t) * P), "set index");
     CK(h->d_state.ensure(sizeof(float) * (size_t)SV_COUNT * N * P), "state");
     CK(h->d_status.ensure(sizeof(uint32_t) * P), "status");
-    cudaError_t ring_e = h->d_ring.ensure(sizeof(float) * (size_t)std::max<int64_t>(ring_floats, 1));
-    if (ring_e == cudaSuccess && win.far) ring_e = h->d_far.ensure(sizeof(float) * tiles.size() * WIN_FAR * N * pb);
-    if (ring_e != cudaSuccess && win.steps > 0 && general_pb == 0) {
-        // the windowed layout is larger: without room for it the other kernels still run
-        h->d_far.release();
-        (void)cudaGetLastError();
-        return prepare_run(h, c, s, general_pb, device_init, plan, direct_body, n_base, false);
-    }
-    CK(ring_e, "ring buffers");
+    CK(h->d_ring.ensure(sizeof(float) * (size_t)std::max<int64_t>(ring_floats, 1)), "ring buffers");
+    if (win.far) CK(h->d_far.ensure(sizeof(float) * tiles.size() * WIN_FAR * N * pb), "far sums");
     // set-blocked series: groups of 4 sets, [ceil(P / 4)][series_T][N][4]
     const int64_t P4 = (P + 3) / 4 * 4;
     h->sl = layout_blocked(N, std::max<int64_t>(series_T, 1));
@@ -902,6 +895,28 @@ static tvbx_status prepare_run(tvbx_sweep* h, const tvbx_run_cfg& c, cudaStream_
     plan.gdev = gdev;
     plan.tiles = tiles;
     return TVBX_OK;
+}
+
+// Give back the windowed kernels' rings and far sums (of a handle whose
+// trajectory nothing continues), which are larger than the other kernels need.
+static void release_windows(tvbx_sweep* h)
+{
+    h->d_ring.release();
+    h->d_far.release();
+}
+
+// prepare_once; a fresh run that does not fit in device memory again, without
+// windows and what an earlier run's left. (A batch decides for all of its jobs.)
+static tvbx_status prepare_run(tvbx_sweep* h, const tvbx_run_cfg& c, cudaStream_t s, int general_pb,
+                               bool device_init, RunPlan& plan, bool direct_body, int64_t n_base, bool windows)
+{
+    tvbx_status st = prepare_once(h, c, s, general_pb, device_init, plan, direct_body, n_base, windows);
+    if (st == TVBX_E_OOM && general_pb == 0 && n_base == 0) {
+        release_windows(h);
+        plan = RunPlan{};
+        st = prepare_once(h, c, s, general_pb, device_init, plan, direct_body, n_base, false);
+    }
+    return st;
 }
 
 // Mark a handle's run as complete (results may be read). steps_before: the
@@ -1781,6 +1796,9 @@ tvbx_status batch_build(tvbx_batch* b, int32_t threads, size_t budget, int64_t t
 {
     b->drop_graph();
     if (tvbx_status st = batch_adopt_jobs(b)) return st;
+    if (!window)   // room for what fitted without an earlier build's windows
+        for (tvbx_sweep* h : b->jobs)
+            if (h->win.steps > 0 && !h->resumable) release_windows(h);
     const size_t nj = b->jobs.size();
     std::vector<RunPlan> plans(nj);
     std::vector<tvbx_run_cfg> run_cfgs(b->cfgs);
@@ -2054,8 +2072,8 @@ tvbx_status tvbx_batch_tune(tvbx_batch* b, int64_t trial_steps, int32_t* threads
                           {128, 64 * 1024, false, false},  {256, 64 * 1024, false, false},
                           {512, 200 * 1024, true, false},  {768, 200 * 1024, true, false},
                           {128, 64 * 1024, false, true}};
-    float best = INFINITY;
-    Cand win{0, 0, false, false};
+    float best = INFINITY, best_general = INFINITY;
+    Cand win{0, 0, false, false}, general{0, 0, false, false};   // best of all, and without windows
     int32_t k = 0;
     cudaEvent_t e0, e1;
     CK(cudaEventCreate(&e0), "event");
@@ -2082,12 +2100,17 @@ tvbx_status tvbx_batch_tune(tvbx_batch* b, int64_t trial_steps, int32_t* threads
             ++k;
         }
         if (ms < best) { best = ms; win = c; }
+        if (!c.window && ms < best_general) { best_general = ms; general = c; }
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (!(best < INFINITY)) return fail(TVBX_E_UNSUPPORTED, "no batch configuration fits every job");
     if (n_trials) *n_trials = k;
     tvbx_status st = batch_build(b, win.threads, win.budget, 0, win.direct, win.window);
+    if (st == TVBX_E_OOM && win.window && best_general < INFINITY) {   // the whole runs' series leave windows no room
+        win = general;
+        st = batch_build(b, win.threads, win.budget, 0, win.direct, false);
+    }
     if (st != TVBX_OK) return st;
     if (threads_out) *threads_out = win.threads;
     if (smem_kb_out) *smem_kb_out = (int32_t)(win.budget / 1024);

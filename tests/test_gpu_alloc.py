@@ -95,3 +95,112 @@ def test_surrogate_and_batch_on_a_caller_allocator(tvbx, oracle):
         assert not live
     finally:
         tvbx.set_allocator()
+
+
+class CappedAllocator:
+    """Device memory through PyTorch's allocator, refused beyond `cap` live bytes."""
+
+    callbacks = []   # for as long as a handle may hold memory of theirs
+
+    def __init__(self, tvbx, cap=None):
+        self.live, self.cap = {}, cap
+        tvbx.set_allocator(self.alloc, self.free)
+        self.callbacks.append(tvbx._allocator_refs)
+
+    def alloc(self, n):
+        import torch
+        used = sum(self.live.values()) + n
+        if self.cap is not None and used > self.cap:
+            return 0
+        p = torch.cuda.caching_allocator_alloc(n)
+        self.live[p] = n
+        return p
+
+    def free(self, p):
+        import torch
+        del self.live[p]
+        torch.cuda.caching_allocator_delete(p)
+
+
+SLACK = 1 << 16   # small tables whose sizes depend on the tile width
+
+
+def _window_inputs(tvbx, n_regions, n_sets, speed):
+    """Delays of a few steps, where windows need the most memory beside the others."""
+    W, L = synth.connectome(n_regions)
+    m = tvbx.make_model()
+    pts = np.tile(np.array([m.defaults[i] for i in range(tvbx.N_AXES)]), (n_sets, 1))
+    rng = np.random.default_rng(n_sets)
+    pts[:, tvbx.AXES.index("g")] = rng.uniform(0.0, 0.4, n_sets)
+    pts[:, tvbx.AXES.index("b_e")] = rng.uniform(0.0, 120.0, n_sets)
+    pts[:, tvbx.AXES.index("speed")] = speed
+    return W, L, pts
+
+
+def _peak(tvbx, inputs, kernel, kw):
+    """Bytes a run holds, and its results."""
+    mem = CappedAllocator(tvbx)
+    sw = tvbx.Sweep(inputs[0], inputs[1], points=inputs[2]).run(kernel=kernel, **kw)
+    peak = sum(mem.live.values())
+    out = (sw.series(), sw.state()) if kw.get("series_mode", 0) == 0 else (sw.state(),)
+    sw.close()
+    tvbx.set_allocator()
+    return peak, out
+
+
+@pytest.mark.parametrize("speed,streamed", [(100.0, False), (30.0, False), (30.0, True)])
+def test_a_run_that_only_fits_without_windows_runs_without_them(tvbx, speed, streamed):
+    inputs = _window_inputs(tvbx, 68, 640, speed)
+    kw = dict(dt_ms=0.1, n_steps=200, tavg_steps=10, seed=5, keep_i_series=not streamed,
+              series_mode=tvbx.SERIES_STREAM if streamed else tvbx.SERIES_KEEP)
+    try:
+        general, want = _peak(tvbx, inputs, tvbx.KERNEL_GENERAL, kw)
+        windowed, got = _peak(tvbx, inputs, tvbx.KERNEL_AUTO, kw)
+        for a, b in zip(want, got):
+            assert np.array_equal(a, b)
+        assert windowed > general + 2 * SLACK
+        # the rings' own allocation refused, the last one, and between them the series'
+        for cap in (general + SLACK, (general + windowed) // 2, windowed - SLACK):
+            mem = CappedAllocator(tvbx, cap)
+            sw = tvbx.Sweep(inputs[0], inputs[1], points=inputs[2]).run(**kw)
+            mem.cap = None
+            got = (sw.series(), sw.state()) if not streamed else (sw.state(),)
+            for a, b in zip(want, got):
+                assert np.array_equal(a, b)
+            sw.run_continue(50)
+            again = tvbx.Sweep(inputs[0], inputs[1], points=inputs[2]).run(**kw).run_continue(50)
+            assert np.array_equal(sw.state(), again.state())
+            again.close()
+            sw.close()
+            tvbx.set_allocator()
+    finally:
+        tvbx.set_allocator()
+
+
+def test_a_batch_that_only_fits_without_windows_runs_without_them(tvbx):
+    inputs = [_window_inputs(tvbx, n, p, v) for n, p, v in ((68, 640, 100.0), (84, 512, 30.0))]
+    kw = dict(dt_ms=0.1, n_steps=1000, tavg_steps=5, seed=5)
+    try:
+        peaks = [[_peak(tvbx, x, kernel, kw) for kernel in (tvbx.KERNEL_GENERAL, tvbx.KERNEL_AUTO)] for x in inputs]
+        more = sum(w[0] - g[0] for g, w in peaks)
+        assert more > 4 * SLACK
+        for tune in (False, True):
+            cap = None
+            for step in range(2):   # uncapped, then with room for half of what windows need more
+                mem = CappedAllocator(tvbx, cap)
+                sweeps = [tvbx.Sweep(W, L, points=pts) for W, L, pts in inputs]
+                b = tvbx.Batch([(sw, kw) for sw in sweeps])
+                if tune and step:
+                    b.tune(trial_steps=50)
+                b.run()
+                if cap is None:
+                    cap = sum(mem.live.values()) - more // 2
+                mem.cap = None
+                for sw, ((_, want), _) in zip(sweeps, peaks):
+                    assert np.array_equal(sw.series(), want[0]) and np.array_equal(sw.state(), want[1])
+                b.close()
+                for sw in sweeps:
+                    sw.close()
+                tvbx.set_allocator()
+    finally:
+        tvbx.set_allocator()
