@@ -512,13 +512,16 @@ tvbx_status tvbx_batch_create(tvbx_sweep* const* jobs, const tvbx_run_cfg* cfgs,
 tvbx_status tvbx_batch_tune(tvbx_batch* b, int64_t trial_steps, int32_t* threads_out, int32_t* smem_kb_out,
                             float* trial_ms, int32_t* n_trials);
 
-/* Run every job (the first call builds the graph; where the batch has no
- * windows, with 512 threads and a 200 KB budget unless tvbx_batch_tune chose
- * otherwise).
+/* Run every job (the first call builds the graph: with windows where every job
+ * has them and they fit, unless tvbx_batch_tune chose otherwise; else the body
+ * that tvbx_batch_tune found best, untuned with 512 threads and a 200 KB budget).
+ * A build that windows did not fit tries them again when it is next rebuilt.
  * The jobs' later calls run on the batch's stream. Synchronises it. */
 tvbx_status tvbx_batch_run(tvbx_batch* b);
 
-/* Current tiling, work items, persistent grid size and graph nodes. */
+/* Current tiling, work items, persistent grid size and graph nodes. A batch built
+ * with windows reads as (128, 64 KB), its work items and grid as the CTAs of every
+ * turn's launch. */
 tvbx_status tvbx_batch_info(const tvbx_batch* b, int32_t* threads, int32_t* smem_kb, int64_t* n_items,
                             int32_t* grid, int64_t* graph_nodes);
 

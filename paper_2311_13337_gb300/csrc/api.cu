@@ -1728,16 +1728,17 @@ struct tvbx_batch {
     std::vector<uint64_t> gens;     // generation of each job when the graph was built
     std::vector<tvbx_run_cfg> cfgs_run;   // configurations the graph runs (trial runs are shorter)
     cudaStream_t stream = nullptr;
-    int32_t threads = 512;
+    int32_t threads = 512;              // of the bodies without windows, and so the next three
     size_t smem_budget = 200 * 1024;
     bool direct = false;                // register-tile bodies where a job fits
-    bool window = true;                 // windowed kernels (every job must have windows, and one model):
-                                        // the graph holds the initialisation, the turns are launched after it
+    bool only_direct = false;           // every job on register tiles
+    bool try_window = true;             // build with windows where they can be had
+    bool window = false;                // built with windows (every job has them, and one model): the
+                                        // graph holds the initialisation, the turns are launched after it
     bool packed = false;
     std::vector<BatchJob> round_jobs;   // [round][job]
     std::vector<RunPlan> plans;
     int64_t rounds = 0;
-    bool only_direct = false;           // every job on register tiles
     DevBuf d_jobs, d_items, d_head, d_ou;
     int32_t n_items = 0, grid = 0;
     cudaGraph_t graph = nullptr;
@@ -1800,6 +1801,16 @@ tvbx_status batch_build(tvbx_batch* b, int32_t threads, size_t budget, int64_t t
         for (tvbx_sweep* h : b->jobs)
             if (h->win.steps > 0 && !h->resumable) release_windows(h);
     const size_t nj = b->jobs.size();
+    if (window) {   // before anything is allocated
+        const DevModel m = to_device_model(b->jobs[0]->model, b->cfgs[0].dt_ms);
+        for (size_t j = 0; j < nj; ++j) {
+            if (sim_direct_pb(b->jobs[j]->N) == 0)
+                return fail(TVBX_E_UNSUPPORTED, "no windows for the %d regions of job %zu", b->jobs[j]->N, j);
+            const DevModel mj = to_device_model(b->jobs[j]->model, b->cfgs[j].dt_ms);
+            if (memcmp(&mj, &m, sizeof m) != 0)
+                return fail(TVBX_E_UNSUPPORTED, "windowed batch: job %zu has another model", j);
+        }
+    }
     std::vector<RunPlan> plans(nj);
     std::vector<tvbx_run_cfg> run_cfgs(b->cfgs);
     std::vector<int> pbs(nj), dirs(nj);
@@ -1832,7 +1843,7 @@ tvbx_status batch_build(tvbx_batch* b, int32_t threads, size_t budget, int64_t t
         if (c.n_steps > INT32_MAX) return fail(TVBX_E_INVALID_ARG, "batch job %zu: n_steps must be < 2^31", j);
         const int N = b->jobs[j]->N;
         // register tiles: as many 4-set quads per region as the CTA has threads for
-        const bool dj = direct && N <= threads;
+        const bool dj = direct && !window && N <= threads;
         const int pb = window ? WIN_BATCH_PB : dj ? 4 * (threads / N) : batch_pb(N, budget, threads);
         if (!pb) return fail(TVBX_E_UNSUPPORTED, "batch job %zu: %d regions do not fit %zu bytes of shared memory", j,
                              N, budget);
@@ -1842,8 +1853,6 @@ tvbx_status batch_build(tvbx_batch* b, int32_t threads, size_t budget, int64_t t
         c.chunk_steps = c.series_mode == TVBX_SERIES_STREAM ? (int32_t)S : 0;
         tvbx_status st = prepare_run(b->jobs[j], c, b->stream, pb, false, plans[j], dj, 0, window);
         if (st != TVBX_OK) return st;
-        if (window && (memcmp(&plans[j].a.m, &plans[0].a.m, sizeof(DevModel)) != 0))
-            return fail(TVBX_E_UNSUPPORTED, "windowed batch: job %zu has another model", j);
         if (!c.noise_per_set) {
             ou_off[j] = ou_floats;
             ou_floats += ((int64_t)c.n_steps * b->jobs[j]->N + 63) / 64 * 64;
@@ -1907,14 +1916,19 @@ tvbx_status batch_build(tvbx_batch* b, int32_t threads, size_t budget, int64_t t
     int dev = 0, sms = 0;
     CK(cudaGetDevice(&dev), "device");
     CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "device");
-    b->only_direct = std::all_of(dirs.begin(), dirs.end(), [](int d) { return d != 0; });
-    const int per_sm = window ? 4 : sim_batch_ctas_per_sm(threads, smem, b->only_direct);
+    const bool only_direct = std::all_of(dirs.begin(), dirs.end(), [](int d) { return d != 0; });
+    const int per_sm = window ? 1 : sim_batch_ctas_per_sm(threads, smem, only_direct);
     if (per_sm < 1) return fail(TVBX_E_UNSUPPORTED, "batch kernel does not fit %d threads / %zu bytes", threads, smem);
-    b->grid = (int32_t)std::max<int64_t>(1, std::min<int64_t>((int64_t)sms * per_sm, (int64_t)items.size()));
-    b->threads = threads;
-    b->smem_budget = budget;
-    b->direct = direct;
     b->window = window;
+    if (window) {
+        b->grid = (int32_t)items.size();   // of every turn
+    } else {
+        b->grid = (int32_t)std::max<int64_t>(1, std::min<int64_t>((int64_t)sms * per_sm, (int64_t)items.size()));
+        b->threads = threads;
+        b->smem_budget = budget;
+        b->direct = direct;
+        b->only_direct = only_direct;
+    }
     b->packed = packed;
     b->rounds = R;
     b->round_jobs.swap(jobs);
@@ -2112,6 +2126,12 @@ tvbx_status tvbx_batch_tune(tvbx_batch* b, int64_t trial_steps, int32_t* threads
         st = batch_build(b, win.threads, win.budget, 0, win.direct, false);
     }
     if (st != TVBX_OK) return st;
+    b->try_window = win.window;
+    if (win.window && best_general < INFINITY) {   // for a later build that windows do not fit
+        b->threads = general.threads;
+        b->smem_budget = general.budget;
+        b->direct = general.direct;
+    }
     if (threads_out) *threads_out = win.threads;
     if (smem_kb_out) *smem_kb_out = (int32_t)(win.budget / 1024);
     return TVBX_OK;
@@ -2125,11 +2145,10 @@ tvbx_status tvbx_batch_run(tvbx_batch* b)
     for (size_t j = 0; j < b->jobs.size() && !stale; ++j) stale = b->jobs[j]->gen != b->gens[j];
     for (size_t j = 0; j < b->jobs.size() && !stale; ++j) stale = b->cfgs_run[j].n_steps != b->cfgs[j].n_steps;
     if (stale) {
-        // untuned: windowed bodies where every job has them, else the general body
-        tvbx_status st = batch_build(b, b->window ? 128 : b->threads, b->smem_budget, 0, b->direct, b->window);
-        if (st != TVBX_OK && b->window) {
-            (void)cudaGetLastError();
-            b->window = false;
+        // untuned: windows where every job has them and they fit, else the general body
+        tvbx_status st = batch_build(b, b->threads, b->smem_budget, 0, b->direct, b->try_window);
+        if (b->try_window && (st == TVBX_E_UNSUPPORTED || st == TVBX_E_OOM)) {
+            if (st == TVBX_E_UNSUPPORTED) b->try_window = false;   // the jobs stay what they are
             st = batch_build(b, b->threads, b->smem_budget, 0, b->direct, false);
         }
         if (st != TVBX_OK) return st;
@@ -2147,8 +2166,8 @@ tvbx_status tvbx_batch_info(const tvbx_batch* b, int32_t* threads, int32_t* smem
                             int64_t* graph_nodes)
 {
     if (!b) return fail(TVBX_E_INVALID_ARG, "NULL batch");
-    if (threads) *threads = b->threads;
-    if (smem_kb) *smem_kb = (int32_t)(b->smem_budget / 1024);
+    if (threads) *threads = b->window ? 128 : b->threads;
+    if (smem_kb) *smem_kb = b->window ? 64 : (int32_t)(b->smem_budget / 1024);
     if (n_items) *n_items = b->n_items;
     if (grid) *grid = b->grid;
     if (graph_nodes) *graph_nodes = b->graph_nodes;

@@ -204,3 +204,40 @@ def test_a_batch_that_only_fits_without_windows_runs_without_them(tvbx):
                 tvbx.set_allocator()
     finally:
         tvbx.set_allocator()
+
+
+def test_a_batch_returns_to_windows_once_they_fit(tvbx):
+    """Without room for windows the untuned body is the documented one, and the
+    next rebuild tries windows again."""
+    inputs = [_window_inputs(tvbx, n, p, v) for n, p, v in ((68, 640, 100.0), (84, 512, 30.0))]
+    kw = dict(dt_ms=0.1, n_steps=100, tavg_steps=10, seed=5)
+    try:
+        peaks = [[_peak(tvbx, x, kernel, kw)[0] for kernel in (tvbx.KERNEL_GENERAL, tvbx.KERNEL_AUTO)] for x in inputs]
+        mem = CappedAllocator(tvbx)
+        sweeps = [tvbx.Sweep(W, L, points=pts) for W, L, pts in inputs]
+        b = tvbx.Batch([(sw, kw) for sw in sweeps]).run()
+        info = b.info()
+        assert info["threads"] == 128 and info["grid"] == info["items"] > 0
+        want = [sw.state() for sw in sweeps]
+        b.close()
+        for sw in sweeps:
+            sw.close()
+        assert not mem.live
+        mem = CappedAllocator(tvbx)
+        sweeps = [tvbx.Sweep(W, L, points=pts) for W, L, pts in inputs]
+        b = tvbx.Batch([(sw, kw) for sw in sweeps])
+        mem.cap = sum((g + w) // 2 for g, w in peaks)   # of the jobs; the batch's own tables are below half the difference
+        b.run()
+        info = b.info()
+        assert (info["threads"], info["smem_kb"]) == (512, 200)
+        mem.cap = None
+        sweeps[0].run(**kw)   # the job's buffers changed
+        b.run()
+        assert b.info()["threads"] == 128
+        for sw, x in zip(sweeps, want):
+            assert np.array_equal(sw.state(), x)
+        b.close()
+        for sw in sweeps:
+            sw.close()
+    finally:
+        tvbx.set_allocator()
