@@ -324,7 +324,7 @@ def run_engine(args):
     clocks = stop_clock_sampler(sampler)
     launches = tvbx.launch_count() - launches0
     sim_ms, sim_launches, sim_rs = tvbx.profile_read(sw.h)
-    kernel_id, _ = tvbx.last_kernel(sw.h)
+    kernel_name = tvbx.kernel_name(sw.h)
     tvbx.profile_enable(sw.h, False)
     t = torch.tensor([el], dtype=torch.float64, device=dev)
     if world > 1:
@@ -404,7 +404,7 @@ def run_engine(args):
         roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                     "frac": achieved / peak if achieved else None,
                     "traffic": traffic_rs * per_launch_rs if traffic_rs else None,
-                    "kernel": tvbx.KERNEL_NAMES.get(kernel_id, str(kernel_id)),
+                    "kernel": kernel_name,
                     "peak_source": "measured" if peaks else "fallback",
                     "algorithmic_bytes_per_region_step": bytes_rs,
                     "region_steps_per_launch": per_launch_rs,

@@ -162,11 +162,13 @@ typedef struct {
  *   state are those of TVBX_SERIES_KEEP, bit for bit. */
 #define TVBX_SERIES_KEEP 0
 #define TVBX_SERIES_STREAM 1
-#define TVBX_KERNEL_AUTO     0 /* fastest kernel that fits the sweep: up to 768 regions, one
-                                  step more per launch than the shortest delay, with no
-                                  thread waiting for another (tvbx_last_kernel then gives
-                                  TVBX_KERNEL_DIRECT: its state is in registers and its
-                                  coupling read straight from the ring) */
+#define TVBX_KERNEL_AUTO     0 /* fastest kernel that fits the sweep: up to 768 regions,
+                                  windows of up to one step more per launch than the
+                                  shortest delay (at most 32, rounded down to whole gather
+                                  passes), with no thread waiting for another; the other
+                                  kernels for more regions, where the windows' rings do
+                                  not fit in device memory, and where a continued run did
+                                  not start in windows */
 #define TVBX_KERNEL_DIRECT 100 /* register tiles for connectomes too large for the
                                   prefetch buffer (up to 768 regions): 4 sets of
                                   one region per thread, 16-byte ring gathers;
@@ -413,9 +415,15 @@ tvbx_status tvbx_transfer_function(const tvbx_model* model, int32_t pop, int64_t
                                    const float* x_e, const float* x_i, const float* W,
                                    const float* E_L, const float* C, float* out);
 
-/* Simulation kernel used by the last tvbx_run (TVBX_KERNEL_GENERAL or
- * TVBX_KERNEL_PREFETCH + v) and its tile size in sets. */
+/* Simulation kernel used by the last run (TVBX_KERNEL_GENERAL, TVBX_KERNEL_DIRECT
+ * or TVBX_KERNEL_PREFETCH + v) and its tile size in sets. Windows read as
+ * TVBX_KERNEL_DIRECT (their state is in registers and their coupling read straight
+ * from the ring too); tvbx_last_window tells them apart. */
 tvbx_status tvbx_last_kernel(const tvbx_sweep* h, int32_t* kernel, int32_t* sets_per_tile);
+
+/* Steps per launch of the windows that the last run or batch took (its last
+ * launches may be shorter), 0 for the other kernels. */
+tvbx_status tvbx_last_window(const tvbx_sweep* h, int32_t* steps);
 
 /* Number of kernels this library has launched in the process so far. */
 uint64_t tvbx_launch_count(void);
@@ -424,11 +432,11 @@ uint64_t tvbx_launch_count(void);
  * created (inputs uploaded by tvbx_run, outputs read to host memory). */
 tvbx_status tvbx_transfer_bytes(const tvbx_sweep* h, uint64_t* h2d, uint64_t* d2h);
 
-/* Kernel timing: when enabled, tvbx_run records a CUDA event pair around every
- * launch of the simulation kernel on the run's stream. tvbx_profile_read
- * synchronises that stream and returns the summed device time (ms), the
- * number of timed launches and the (set, region, step) updates they made,
- * accumulated since the last tvbx_profile_enable call. */
+/* Kernel timing: when enabled, tvbx_run records a CUDA event pair around the
+ * simulation launches of every chunk on the run's stream (one launch, or the
+ * chunk's windows). tvbx_profile_read synchronises that stream and returns the
+ * summed device time (ms), the number of timed launches and the (set, region,
+ * step) updates they made, accumulated since the last tvbx_profile_enable call. */
 tvbx_status tvbx_profile_enable(tvbx_sweep* h, int32_t enable);
 tvbx_status tvbx_profile_read(tvbx_sweep* h, double* sim_ms, int64_t* sim_launches,
                               double* region_steps);

@@ -245,6 +245,7 @@ struct tvbx_sweep {
     bool profiling = false;
     std::vector<cudaEvent_t> ev;    // pairs around simulation launches
     size_t ev_used = 0;
+    int64_t prof_launches = 0;
     double prof_region_steps = 0.0;
     std::vector<int64_t> perm;      // internal -> external
     std::vector<int64_t> inv;       // external -> internal
@@ -1004,8 +1005,10 @@ static tvbx_status run_chunks(tvbx_sweep* h, const tvbx_run_cfg& c, const RunPla
             }
             CK(cudaEventRecord(h->ev[h->ev_used], s), "profiling event");
         }
+        int64_t launches = 1;
         if (variant >= 0) CK(launch_sim_fast(a, variant, plan.n_tiles, plan.nnz_max, s), "simulation chunk");
         else if (plan.win.steps > 0) {
+            launches = 0;
             SimArgs aw = a;
             for (int64_t w0 = 0; w0 < a.n_chunk; w0 += aw.n_chunk) {
                 // a window stays within the steps whose far sums are at hand
@@ -1015,6 +1018,7 @@ static tvbx_status run_chunks(tvbx_sweep* h, const tvbx_run_cfg& c, const RunPla
                 aw.n_chunk = (int32_t)std::min({(int64_t)plan.win.steps, a.n_chunk - w0, most});
                 CK(launch_sim_window(aw, plan.win, plan.n_tiles, w0, h->d_far.as<float>(), (int32_t)row, s),
                    "simulation window");
+                launches += plan.win.far && row == 0 ? 2 : 1;
             }
         }
         else if (variant == -2) CK(launch_sim_direct(a, plan.n_tiles, plan.pb, s), "simulation chunk");
@@ -1022,6 +1026,7 @@ static tvbx_status run_chunks(tvbx_sweep* h, const tvbx_run_cfg& c, const RunPla
         if (h->profiling) {
             CK(cudaEventRecord(h->ev[h->ev_used + 1], s), "profiling event");
             h->ev_used += 2;
+            h->prof_launches += launches;
             h->prof_region_steps += (double)P * N * a.n_chunk;
         }
         if (streamed)
@@ -1675,6 +1680,14 @@ tvbx_status tvbx_last_kernel(const tvbx_sweep* h, int32_t* kernel, int32_t* sets
     return TVBX_OK;
 }
 
+tvbx_status tvbx_last_window(const tvbx_sweep* h, int32_t* steps)
+{
+    if (!h) return fail(TVBX_E_INVALID_ARG, "NULL handle");
+    if (!h->ran) return fail(TVBX_E_BAD_STATE, "tvbx_last_window before tvbx_run");
+    if (steps) *steps = h->win.steps;
+    return TVBX_OK;
+}
+
 tvbx_status tvbx_transfer_bytes(const tvbx_sweep* h, uint64_t* h2d, uint64_t* d2h)
 {
     if (!h) return fail(TVBX_E_INVALID_ARG, "NULL handle");
@@ -1689,6 +1702,7 @@ tvbx_status tvbx_profile_enable(tvbx_sweep* h, int32_t enable)
     if (h->stream) CK(cudaStreamSynchronize(h->stream), "synchronize");
     h->profiling = enable != 0;
     h->ev_used = 0;
+    h->prof_launches = 0;
     h->prof_region_steps = 0.0;
     return TVBX_OK;
 }
@@ -1704,7 +1718,7 @@ tvbx_status tvbx_profile_read(tvbx_sweep* h, double* sim_ms, int64_t* sim_launch
         total += ms;
     }
     if (sim_ms) *sim_ms = total;
-    if (sim_launches) *sim_launches = (int64_t)(h->ev_used / 2);
+    if (sim_launches) *sim_launches = h->prof_launches;
     if (region_steps) *region_steps = h->prof_region_steps;
     return TVBX_OK;
 }

@@ -86,7 +86,7 @@ class SurrogateCfg(ctypes.Structure):
 _lib = None
 EXPORTS = ("tvbx_version", "tvbx_last_error", "tvbx_model_defaults", "tvbx_sweep_create",
            "tvbx_sweep_create_points", "tvbx_sweep_info", "tvbx_run", "tvbx_summary", "tvbx_series",
-           "tvbx_series_range", "tvbx_series_pop_range", "tvbx_state", "tvbx_fc", "tvbx_transfer_function", "tvbx_last_kernel",
+           "tvbx_series_range", "tvbx_series_pop_range", "tvbx_state", "tvbx_fc", "tvbx_transfer_function", "tvbx_last_kernel", "tvbx_last_window",
            "tvbx_launch_count",
            "tvbx_transfer_bytes", "tvbx_profile_enable", "tvbx_profile_read", "tvbx_fc_noalloc", "tvbx_fc_series",
            "tvbx_sweep_destroy", "tvbx_surrogate_create", "tvbx_surrogate_info", "tvbx_surrogate_train",
@@ -142,6 +142,7 @@ def load(build_if_missing: bool = False):
     L.tvbx_sweep_destroy.argtypes = [vp]
     L.tvbx_launch_count.restype = ctypes.c_uint64
     L.tvbx_last_kernel.argtypes = [vp, ctypes.POINTER(i32), ctypes.POINTER(i32)]
+    L.tvbx_last_window.argtypes = [vp, ctypes.POINTER(i32)]
     L.tvbx_fc_noalloc.argtypes = [fp, i32, i64, i64, fp, fp, fp, vp]
     L.tvbx_fc_series.argtypes = [fp, i32, i64, i64, ctypes.POINTER(FcCfg), fp, fp, ctypes.POINTER(i32), fp, fp, fp,
                                  vp]
@@ -487,7 +488,7 @@ def transfer_function(pop: int, x_e, x_i, W, E_L, C=None, model: Model | None = 
     return out
 
 
-KERNEL_NAMES = {KERNEL_GENERAL: "sim_chunk_kernel", KERNEL_DIRECT: "sim_window_kernel or sim_direct_kernel"}
+KERNEL_NAMES = {KERNEL_GENERAL: "sim_chunk_kernel", KERNEL_DIRECT: "sim_direct_kernel"}
 KERNEL_NAMES.update({KERNEL_PREFETCH + v: ("sim_pack_kernel" if v in PACKED_VARIANTS else "sim_tma_kernel" if 12 <= v <= 14 else
                                           "sim_bulk_kernel" if v in (4, 5) else "sim_fast_kernel") + f" (variant {v})"
                      for v in range(N_PREFETCH_VARIANTS)})
@@ -497,6 +498,19 @@ def last_kernel(h) -> tuple[int, int]:
     k, pb = ctypes.c_int32(), ctypes.c_int32()
     _check(load().tvbx_last_kernel(h, ctypes.byref(k), ctypes.byref(pb)), "tvbx_last_kernel")
     return k.value, pb.value
+
+
+def last_window(h) -> int:
+    """Steps per launch of the last run's windows, 0 for the other kernels."""
+    n = ctypes.c_int32()
+    _check(load().tvbx_last_window(h, ctypes.byref(n)), "tvbx_last_window")
+    return n.value
+
+
+def kernel_name(h) -> str:
+    """Name of the simulation kernel of the last run."""
+    steps, kernel = last_window(h), last_kernel(h)[0]
+    return f"sim_window_kernel ({steps} steps per launch)" if steps else KERNEL_NAMES.get(kernel, str(kernel))
 
 
 def launch_count() -> int:

@@ -108,3 +108,20 @@ def test_a_set_does_not_depend_on_the_other_speeds(tvbx):
         sw.run(dt_ms=DT, n_steps=100, tavg_steps=10, seed=4)
     assert np.array_equal(both.state()[slow], alone.state())
     assert np.array_equal(both.series()[slow], alone.series())
+
+
+@pytest.mark.parametrize("d_min,steps", [(0, 1), (5, 6), (12, 8), (18, 16), (40, 32)])
+def test_reports_tell_windows_from_the_other_kernels(tvbx, d_min, steps):
+    W, L, pts = _inputs(tvbx, 30, 10, d_min)
+    sw = tvbx.Sweep(W, L, points=pts)
+    for kernel, want in ((tvbx.KERNEL_AUTO, steps), (tvbx.KERNEL_DIRECT, 0), (tvbx.KERNEL_GENERAL, 0)):
+        tvbx.profile_enable(sw.h)
+        sw.run(dt_ms=DT, n_steps=90, tavg_steps=10, kernel=kernel, chunk_steps=50)
+        _, launches, updates = tvbx.profile_read(sw.h)
+        assert tvbx.last_window(sw.h) == want and ("window" in tvbx.kernel_name(sw.h)) == (want > 0)
+        assert updates == 30 * 10 * 90
+        # far sums once every 16 steps beside windows of fewer than 8, which end with them
+        count = sum((n // 16 * -(-16 // steps) + -(-(n % 16) // steps) + -(-n // 16)) if steps < 8 else -(-n // steps)
+                    for n in (50, 40))
+        assert launches == (count if want else 2)
+    sw.close()
