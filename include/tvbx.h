@@ -386,8 +386,8 @@ tvbx_status tvbx_fc(tvbx_sweep* h, const tvbx_fc_cfg* cfg, int32_t mem, float* f
  * non-NULL), chi and mean_fc [n_sets], set_status [n_sets] (OR-ed with
  * TVBX_SET_ZERO_VAR; not cleared). The shift of each row is the mean of up to
  * 64 evenly spaced samples. Scratch of n_sets x blocks x (n_regions^2 +
- * n_regions) floats (blocks = 1 without FCD, up to 12 for few sets in FP32; else ceil(n_samples /
- * fcd_step)) is allocated stream-ordered on cuda_stream (NULL = the legacy
+ * n_regions) floats (blocks = 1 without FCD, for few sets in FP32 up to 12 where
+ * that much can be had; else ceil(n_samples / fcd_step)) is allocated stream-ordered on cuda_stream (NULL = the legacy
  * default stream) from a memory pool the library owns per device, and freed
  * into it before return; the pool keeps that memory for later calls until the
  * process exits. The call synchronises cuda_stream before it returns.

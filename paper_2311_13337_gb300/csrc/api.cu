@@ -1312,7 +1312,13 @@ static tvbx_status run_fc(tvbx_sweep* h, int32_t precision, int32_t fcd_window, 
         h->fc_valid = true;
         return TVBX_OK;
     }
-    CK(h->d_blocks.ensure(sizeof(float) * (size_t)P * n_blocks * stride_b), "FC block moments");
+    cudaError_t be = h->d_blocks.ensure(sizeof(float) * (size_t)P * n_blocks * stride_b);
+    if (be == cudaErrorMemoryAllocation && fcd_window == 0 && n_blocks > 1) {   // the same sums, added up as they are formed
+        merge = n_blocks;
+        n_blocks = 1;
+        be = h->d_blocks.ensure(sizeof(float) * (size_t)P * stride_b);
+    }
+    CK(be, "FC block moments");
     CK(h->d_fc.ensure(sizeof(float) * (size_t)P * N * N), "FC");
     CK(h->d_chi.ensure(sizeof(float) * P), "chi");
     CK(h->d_meanfc.ensure(sizeof(float) * P), "mean FC");
@@ -1452,18 +1458,26 @@ tvbx_status tvbx_fc_series(const float* series, int32_t n_regions, int64_t n_set
     cudaStream_t s = (cudaStream_t)cuda_stream;
     const size_t stride_b = (size_t)N * N + N;
     const size_t M = (size_t)N * (N - 1) / 2;
-    const size_t sz_blocks = sizeof(float) * (size_t)P * n_blocks * stride_b;
+    size_t sz_blocks = sizeof(float) * (size_t)P * n_blocks * stride_b;
     const size_t sz_shift = sizeof(float) * (size_t)N * P;
     const size_t sz_fc = fc_out ? 0 : sizeof(float) * (size_t)P * N * N;
     const size_t sz_small = sizeof(float) * (size_t)P * 3 + 256;
     const size_t sz_vec = nw > 0 && fc_reduce_needs_vec_scratch(N, n_blocks, nw) ? sizeof(float) * (size_t)P * nw * M : 0;
     const size_t sz_fcd = (nw > 0 && !fcd_out) ? sizeof(float) * (size_t)P * nw * nw : 0;
     auto up = [](size_t b) { return (b + 255) / 256 * 256; };
-    const size_t total = up(sz_blocks) + up(sz_shift) + up(sz_fc) + up(sz_small) + up(sz_vec) + up(sz_fcd);
+    const size_t others = up(sz_shift) + up(sz_fc) + up(sz_small) + up(sz_vec) + up(sz_fcd);
     void* scratch = nullptr;
     cudaMemPool_t pool;
     CK(scratch_pool(&pool), "FC scratch pool");
-    CK(cudaMallocFromPoolAsync(&scratch, total, pool, s), "FC scratch");
+    cudaError_t me = cudaMallocFromPoolAsync(&scratch, up(sz_blocks) + others, pool, s);
+    if (me == cudaErrorMemoryAllocation && nw == 0 && n_blocks > 1) {   // the same sums, added up as they are formed
+        (void)cudaGetLastError();
+        merge = n_blocks;
+        n_blocks = 1;
+        sz_blocks = sizeof(float) * (size_t)P * stride_b;
+        me = cudaMallocFromPoolAsync(&scratch, up(sz_blocks) + others, pool, s);
+    }
+    CK(me, "FC scratch");
     char* q = static_cast<char*>(scratch);
     auto take = [&](size_t b) { char* r = q; q += up(b); return r; };
     float* d_blocks = reinterpret_cast<float*>(take(sz_blocks));

@@ -241,3 +241,25 @@ def test_a_batch_returns_to_windows_once_they_fit(tvbx):
             sw.close()
     finally:
         tvbx.set_allocator()
+
+
+def test_fc_of_few_sets_without_room_for_their_moment_blocks(tvbx):
+    """Few sets store up to 12 moment blocks each; where only one fits, the same
+    sums are added up as they are formed."""
+    inputs = _window_inputs(tvbx, 68, 16, 4.0)
+    kw = dict(dt_ms=0.1, n_steps=4000, tavg_steps=1, seed=5)
+    out, grown = [], []
+    try:
+        for _ in range(2):
+            mem = CappedAllocator(tvbx)
+            sw = tvbx.Sweep(inputs[0], inputs[1], points=inputs[2]).run(**kw)
+            run = sum(mem.live.values())
+            mem.cap = run + grown[0] // 2 if grown else None
+            summ = sw.summary()
+            out.append((sw.fc(), summ["chi"], summ["mean_fc"]))
+            grown.append(sum(mem.live.values()) - run)
+            sw.close()
+            tvbx.set_allocator()
+    finally:
+        tvbx.set_allocator()
+    assert grown[0] > 4 * 12 * 16 * 68 * 69 and all(np.array_equal(a, b) for a, b in zip(*out))
