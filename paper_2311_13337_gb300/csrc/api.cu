@@ -1114,7 +1114,7 @@ uint64_t sweep_fingerprint(const tvbx_sweep* h)
 }
 
 // The ring of a windowed run to (out) or from its checkpoint layout in host
-// memory, through a staging buffer of whole slots.
+// memory, through a staging buffer of as many whole slots as fit.
 tvbx_status convert_ring(tvbx_sweep* h, bool out, int64_t n, unsigned char* host)
 {
     int64_t off = 0;   // floats into the checkpoint's ring
@@ -1123,7 +1123,8 @@ tvbx_status convert_ring(tvbx_sweep* h, bool out, int64_t n, unsigned char* host
         const int32_t H0 = h->ring_H0[gi];
         const int64_t row = (int64_t)h->N * g.stride;
         off = (off + 63) / 64 * 64;
-        const int32_t nf = (int32_t)std::min<int64_t>(H0, std::max<int64_t>(1, ((int64_t)16 << 20) / row));
+        int32_t nf = (int32_t)std::min<int64_t>(H0, std::max<int64_t>(1, ((int64_t)16 << 20) / row));
+        while (nf > 1 && h->d_tmp.ensure(sizeof(float) * (size_t)(nf * row)) != cudaSuccess) nf = (nf + 1) / 2;
         CK(h->d_tmp.ensure(sizeof(float) * (size_t)(nf * row)), "ring staging");
         float* rows = h->d_tmp.as<float>();
         for (int32_t f = 0; f < H0; f += nf) {

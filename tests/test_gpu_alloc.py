@@ -263,3 +263,32 @@ def test_fc_of_few_sets_without_room_for_their_moment_blocks(tvbx):
     finally:
         tvbx.set_allocator()
     assert grown[0] > 4 * 12 * 16 * 68 * 69 and all(np.array_equal(a, b) for a, b in zip(*out))
+
+
+def test_checkpoint_of_windows_with_little_memory_left(tvbx):
+    """The ring is converted through as few slots at a time as fit."""
+    inputs = _window_inputs(tvbx, 68, 640, 10.0)
+    kw = dict(dt_ms=0.1, n_steps=100, tavg_steps=10, seed=5)
+    cks = []
+    try:
+        for short in (False, True):
+            mem = CappedAllocator(tvbx)
+            sw = tvbx.Sweep(inputs[0], inputs[1], points=inputs[2]).run(**kw)
+            assert tvbx.last_window(sw.h) > 0
+            if short:
+                mem.cap = sum(mem.live.values()) + 3 * 4 * 68 * 672   # three slots
+            cks.append(sw.checkpoint())
+            again = tvbx.Sweep(inputs[0], inputs[1], points=inputs[2])
+            mem.cap = None
+            again.run(**kw)
+            if short:
+                mem.cap = sum(mem.live.values()) + 3 * 4 * 68 * 672
+            again.restore(cks[-1])
+            mem.cap = None
+            assert np.array_equal(again.run_continue(20).state(), sw.run_continue(20).state())
+            again.close()
+            sw.close()
+            tvbx.set_allocator()
+    finally:
+        tvbx.set_allocator()
+    assert np.array_equal(*cks)
