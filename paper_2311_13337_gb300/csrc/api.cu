@@ -1766,7 +1766,6 @@ struct tvbx_batch {
                                         // graph holds the initialisation, the turns are launched after it
     bool packed = false;
     std::vector<BatchJob> round_jobs;   // [round][job]
-    std::vector<RunPlan> plans;
     int64_t rounds = 0;
     DevBuf d_jobs, d_items, d_head, d_ou;
     int32_t n_items = 0, grid = 0;
@@ -2025,7 +2024,6 @@ tvbx_status batch_build(tvbx_batch* b, int32_t threads, size_t budget, int64_t t
     b->graph_nodes = (int64_t)nodes;
     b->graph_kernels = kernels;
     b->cfgs_run = run_cfgs;
-    b->plans.swap(plans);
     b->gens.resize(nj);
     for (size_t j = 0; j < nj; ++j) b->gens[j] = b->jobs[j]->gen;
     b->built = true;
