@@ -404,6 +404,7 @@ def run_engine(args):
         roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                     "frac": achieved / peak if achieved else None,
                     "traffic": traffic_rs * per_launch_rs if traffic_rs else None,
+                    "traffic_frac": traffic_rs * sim_rs / (sim_ms * 1e-3) / 1e9 / peak if traffic_rs and sim_ms > 0 else None,
                     "kernel": kernel_name,
                     "peak_source": "measured" if peaks else "fallback",
                     "algorithmic_bytes_per_region_step": bytes_rs,

@@ -634,8 +634,7 @@ tvbx_status tvbx_top_k(const float* values, int64_t n, int32_t k, int64_t* idx_o
  * [n_sets][TVBX_AN_COUNT], caller-owned; n_used: host, nullable. 1 <=
  * n_regions <= 752 (the phase-lag tiles of all regions must fit in shared
  * memory), n_samples >= 2. Sets are analysed in batches (the
- * analytic signals of up to 2 GiB of sets, whole waves of the phase-lag
- * kernel). A host series is uploaded batch by batch on a second stream into
+ * analytic signals and pair counts of up to 2 GiB of sets). A host series is uploaded batch by batch on a second stream into
  * two staging buffers, so the upload of one batch overlaps the analysis of
  * the previous one when the host memory is pinned (pageable memory works but
  * does not overlap); it must stay valid until cuda_stream has completed.
