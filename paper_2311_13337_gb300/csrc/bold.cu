@@ -55,6 +55,7 @@ static __device__ __forceinline__ float pow1p_m1(float v, const BoldDev& c)
         for (int k = 6; k >= 0; --k) h = fmaf(h, v, c.ca[k]);
         return h * v;
     }
+    if (v != v) return v;
     return expm1f(log1pf(v) * c.inv_alpha);
 }
 
@@ -73,6 +74,7 @@ static __device__ __forceinline__ float expm1_small(float x)
         h = fmaf(h, x, 1.0f);
         return h * x;
     }
+    if (x != x) return x;
     return expm1f(x);
 }
 
@@ -196,41 +198,52 @@ static __device__ __forceinline__ uint64_t sub2(uint64_t a, uint64_t b)
 
 // v^(1/alpha) - 1 and e^x - 1 of two elements beyond the range of the short
 // series: packed to degree 8 where both lanes are in range, else lane by lane.
-static __device__ __noinline__ void powers(const BoldDev& c, uint64_t vt, uint64_t x, uint64_t& vpa_m1, uint64_t& em1)
+// A lane that is NaN takes the other's way and stays NaN. Inlined: as a call it
+// cost 16% of the whole (2,048 x 68 x 10,000 1.82 ms, now 1.54) for what it kept
+// on the stack, and rates that are not finite were slower than without it.
+static __device__ __forceinline__ void powers(const BoldDev& c, uint64_t vt, uint64_t x, uint64_t& vpa_m1, uint64_t& em1)
 {
-    const float2 v = u2(vt), xf = u2(x);
+    const float2 v0 = u2(vt), x0 = u2(x);
+    const float2 v = make_float2(v0.x == v0.x ? v0.x : 0.0f, v0.y == v0.y ? v0.y : 0.0f);
+    const float2 xf = make_float2(x0.x == x0.x ? x0.x : 0.0f, x0.y == x0.y ? x0.y : 0.0f);
+    float2 r, e;
     if (fabsf(v.x) <= c.v_series && fabsf(v.y) <= c.v_series) {
+        const uint64_t vp = p2(v.x, v.y);
         uint64_t h = p2(c.ca[7], c.ca[7]);
 #pragma unroll
-        for (int k = 6; k >= 0; --k) h = fma2(h, vt, p2(c.ca[k], c.ca[k]));
-        vpa_m1 = mul2(h, vt);
+        for (int k = 6; k >= 0; --k) h = fma2(h, vp, p2(c.ca[k], c.ca[k]));
+        r = u2(mul2(h, vp));
     } else {
-        vpa_m1 = p2(pow1p_m1(v.x, c), pow1p_m1(v.y, c));
+        r = make_float2(pow1p_m1(v.x, c), pow1p_m1(v.y, c));
     }
     if (fabsf(xf.x) <= 0.25f && fabsf(xf.y) <= 0.25f) {
+        const uint64_t xp = p2(xf.x, xf.y);
         uint64_t h = p2(1.0f / 40320.0f, 1.0f / 40320.0f);
-        h = fma2(h, x, p2(1.0f / 5040.0f, 1.0f / 5040.0f));
-        h = fma2(h, x, p2(1.0f / 720.0f, 1.0f / 720.0f));
-        h = fma2(h, x, p2(1.0f / 120.0f, 1.0f / 120.0f));
-        h = fma2(h, x, p2(1.0f / 24.0f, 1.0f / 24.0f));
-        h = fma2(h, x, p2(1.0f / 6.0f, 1.0f / 6.0f));
-        h = fma2(h, x, p2(0.5f, 0.5f));
-        h = fma2(h, x, p2(1.0f, 1.0f));
-        em1 = mul2(h, x);
+        h = fma2(h, xp, p2(1.0f / 5040.0f, 1.0f / 5040.0f));
+        h = fma2(h, xp, p2(1.0f / 720.0f, 1.0f / 720.0f));
+        h = fma2(h, xp, p2(1.0f / 120.0f, 1.0f / 120.0f));
+        h = fma2(h, xp, p2(1.0f / 24.0f, 1.0f / 24.0f));
+        h = fma2(h, xp, p2(1.0f / 6.0f, 1.0f / 6.0f));
+        h = fma2(h, xp, p2(0.5f, 0.5f));
+        h = fma2(h, xp, p2(1.0f, 1.0f));
+        e = u2(mul2(h, xp));
     } else {
-        em1 = p2(expm1_small(xf.x), expm1_small(xf.y));
+        e = make_float2(expm1_small(xf.x), expm1_small(xf.y));
     }
+    vpa_m1 = p2(v0.x == v0.x ? r.x : v0.x, v0.y == v0.y ? r.y : v0.y);
+    em1 = p2(x0.x == x0.x ? e.x : x0.x, x0.y == x0.y ? e.y : x0.y);
 }
 
 // The same integration for two neighbouring (region, set) elements per
 // thread, i and i + 1 (i even; NP even, so every sample row starts 8-byte
 // aligned), in packed f32x2 arithmetic; reciprocals, the general forms of the
-// powers and the output are lane by lane. While v - 1 and f - 1 of both lanes
+// powers and the output are lane by lane. While v - 1 and f - 1 of a lane
 // are within v_small and f_small (rates up to about 25 Hz), both series end at
 // degree 4, which leaves the same 1e-8 of their first term as the longer ones
-// do at their bounds. The rates come BOLD_AHEAD samples ahead: one load per
+// do at their bounds; each lane by its own values, so that an element does not
+// depend on its neighbour. The rates come BOLD_AHEAD samples ahead: one load per
 // step, waited for, bound the kernel by memory latency below a full chip
-// (2,048 x 68 x 10,000: 4.58 ms; now 1.82).
+// (2,048 x 68 x 10,000: 4.58 ms; now 1.54).
 __global__ void __launch_bounds__(BOLD_THREADS)
 bold_kernel2(const float* __restrict__ series, int64_t NP, int64_t T, int decim, BoldDev c,
                              float* __restrict__ state, int reset, float* __restrict__ out)
@@ -269,6 +282,16 @@ bold_kernel2(const float* __restrict__ series, int64_t NP, int64_t T, int decim,
             em1 = mul2(fma2(fma2(fma2(e4, x, e3), x, e2), x, one), x);
         } else {
             powers(c, vt, x, vpa_m1, em1);
+            // an element's series do not depend on its neighbour
+            const bool near0 = fabsf(vtf.x) <= c.v_small && fabsf(ftf.x) <= c.f_small;
+            const bool near1 = fabsf(vtf.y) <= c.v_small && fabsf(ftf.y) <= c.f_small;
+            if (near0 || near1) {
+                const float2 vf = u2(vpa_m1), ef = u2(em1);
+                const float2 vn = u2(mul2(fma2(fma2(fma2(ca[3], vt, ca[2]), vt, ca[1]), vt, ca[0]), vt));
+                const float2 en = u2(mul2(fma2(fma2(fma2(e4, x, e3), x, e2), x, one), x));
+                vpa_m1 = p2(near0 ? vn.x : vf.x, near1 ? vn.y : vf.y);
+                em1 = p2(near0 ? en.x : ef.x, near1 ? en.y : ef.y);
+            }
         }
         const uint64_t fE_m1 = fma2(mul2(f, m_rE0), em1, ft);
         const uint64_t vq_m1 = fma2(mul2(sub2(vpa_m1, vt), rv), add2(one, qt), qt);

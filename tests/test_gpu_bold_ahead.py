@@ -38,3 +38,23 @@ def test_bold_lengths(tvbx, n_samples, n_sets):
     parts = [tvbx.bold(x[:half].contiguous(), 1.0, 1, state=st2, reset_state=True)] if half else []
     parts.append(tvbx.bold(x[half:].contiguous(), 1.0, 1, state=st2, reset_state=not half))
     assert torch.equal(torch.cat(parts), y) and torch.equal(st, st2)
+
+
+@pytest.mark.parametrize("beside", [0.0, 0.2, 3.0, float("nan"), float("inf")])
+def test_bold_of_an_element_does_not_depend_on_its_neighbour(tvbx, beside):
+    """Two elements share a thread: one at rates from 2.5 Hz to 2.7 kHz, from near
+    rest to beyond the bounds of every series, beside one of any other rates."""
+    import torch
+    T, P = 3000, 500
+    g = torch.Generator(device="cuda")
+    g.manual_seed(3)
+    amp = torch.exp(7.0 * torch.rand(P, generator=g, device="cuda") - 6.0)
+    a = amp * torch.rand((T, 1, P), generator=g, device="cuda")
+    b = beside * torch.rand((T, 1, P), generator=g, device="cuda")
+    alone = tvbx.bold(torch.stack((a, a), dim=-1).view(T, 1, 2 * P), 1.0, 10).view(-1, P, 2)
+    assert torch.equal(alone[..., 0], alone[..., 1]) and torch.isfinite(alone).all()
+    for lane in (0, 1):
+        pair = (a, b) if lane == 0 else (b, a)
+        got = tvbx.bold(torch.stack(pair, dim=-1).view(T, 1, 2 * P), 1.0, 10).view(-1, P, 2)
+        assert torch.equal(got[..., lane], alone[..., lane])
+        assert torch.isfinite(got[..., 1 - lane]).all().item() == (beside < 3.5)
