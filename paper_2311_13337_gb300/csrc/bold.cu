@@ -87,6 +87,14 @@ static __device__ __forceinline__ float rcp_approx(float x)
     return r;
 }
 
+// The signal: 1 - q = -qt, 1 - q / v = (vt - qt) / (1 + vt), 1 - v = -vt.
+static __device__ __forceinline__ float bold_of(const BoldDev& c, float vt, float qt)
+{
+    return c.V0 * fmaf(c.k3, -vt, fmaf(c.k1, -qt, c.k2 * (vt - qt) / (1.0f + vt)));
+}
+
+// One element per thread, for counts and addresses that bold_kernel2 does not
+// take: the same operations, so the same numbers.
 __global__ void bold_kernel(const float* __restrict__ series, int64_t NP, int64_t T, int decim, BoldDev c,
                             float* __restrict__ state, int reset, float* __restrict__ out)
 {
@@ -103,15 +111,22 @@ __global__ void bold_kernel(const float* __restrict__ series, int64_t NP, int64_
     int64_t o = 0;
     auto step = [&](float z) {
         const float f = 1.0f + ft;
-        const float vpa_m1 = pow1p_m1(vt, c);                                 // v^(1/alpha) - 1
+        const float x = -c.lnE * ft * rcp_approx(f);
+        float vpa_m1, em1;   // v^(1/alpha) - 1, e^x - 1
+        if (fabsf(vt) <= c.v_small && fabsf(ft) <= c.f_small) {
+            vpa_m1 = fmaf(fmaf(fmaf(c.ca[3], vt, c.ca[2]), vt, c.ca[1]), vt, c.ca[0]) * vt;
+            em1 = fmaf(fmaf(fmaf(1.0f / 24.0f, x, 1.0f / 6.0f), x, 0.5f), x, 1.0f) * x;
+        } else {
+            vpa_m1 = pow1p_m1(vt, c);
+            em1 = expm1_small(x);
+        }
         // f E(f) / E0 - 1 = ft - (1 + ft) r_E0 expm1(-ln(1 - E0) ft / f), since
         // (1 - E0)^(1/f) = (1 - E0) exp(-ln(1 - E0) ft / f): exactly 0 at rest
-        // (the argument of expm1 to 2 ulp)
-        const float fE_m1 = fmaf(-f * c.r_E0, expm1_small(__fdividef(-c.lnE * ft, f)), ft);
+        const float fE_m1 = fmaf(f * -c.r_E0, em1, ft);
         // v^(1/alpha - 1) q - 1, with v^(1/alpha - 1) - 1 = (v^(1/alpha) - v) / v
         // = (vpa_m1 - vt) / (1 + vt) (no cancellation: vpa_m1 is about vt / alpha)
         const float vq_m1 = fmaf((vpa_m1 - vt) * rcp_approx(1.0f + vt), 1.0f + qt, qt);
-        const float ds = z - c.kappa * s - c.gamma * ft;
+        const float ds = fmaf(-c.gamma, ft, fmaf(-c.kappa, s, z));
         const float nft = fmaf(c.dt, s, ft);
         const float nvt = fmaf(c.dt * c.inv_tau, ft - vpa_m1, vt);
         const float nqt = fmaf(c.dt * c.inv_tau, fE_m1 - vq_m1, qt);
@@ -121,8 +136,7 @@ __global__ void bold_kernel(const float* __restrict__ series, int64_t NP, int64_
         qt = nqt;
         if (++phase == decim) {
             phase = 0;
-            // 1 - q = -qt, 1 - q / v = (vt - qt) / (1 + vt), 1 - v = -vt
-            out[o * NP + i] = c.V0 * (c.k3 * -vt + fmaf(c.k1, -qt, c.k2 * (vt - qt) / (1.0f + vt)));
+            out[o * NP + i] = bold_of(c, vt, qt);
             ++o;
         }
     };
@@ -306,9 +320,7 @@ bold_kernel2(const float* __restrict__ series, int64_t NP, int64_t T, int decim,
         if (++phase == decim) {
             phase = 0;
             const float2 a = u2(vt), b = u2(qt);
-            const float y0 = c.V0 * (c.k3 * -a.x + fmaf(c.k1, -b.x, c.k2 * (a.x - b.x) / (1.0f + a.x)));
-            const float y1 = c.V0 * (c.k3 * -a.y + fmaf(c.k1, -b.y, c.k2 * (a.y - b.y) / (1.0f + a.y)));
-            *reinterpret_cast<float2*>(out + o * NP + i) = make_float2(y0, y1);
+            *reinterpret_cast<float2*>(out + o * NP + i) = make_float2(bold_of(c, a.x, b.x), bold_of(c, a.y, b.y));
             ++o;
         }
     };

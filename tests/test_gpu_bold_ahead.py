@@ -58,3 +58,19 @@ def test_bold_of_an_element_does_not_depend_on_its_neighbour(tvbx, beside):
         got = tvbx.bold(torch.stack(pair, dim=-1).view(T, 1, 2 * P), 1.0, 10).view(-1, P, 2)
         assert torch.equal(got[..., lane], alone[..., lane])
         assert torch.isfinite(got[..., 1 - lane]).all().item() == (beside < 3.5)
+
+
+@pytest.mark.parametrize("peak", [0.02, 0.3, 3.0])
+def test_bold_of_odd_counts_and_unaligned_rates(tvbx, peak):
+    """One element per thread gives what two give."""
+    import torch
+    T, N = 3001, 33
+    g = torch.Generator(device="cuda")
+    g.manual_seed(5)
+    a = peak * torch.rand((T, N, 1), generator=g, device="cuda")
+    st, st2 = torch.zeros((4, N, 1), device="cuda"), torch.zeros((4, N, 2), device="cuda")
+    odd, even = tvbx.bold(a, 1.0, 7, state=st), tvbx.bold(a.expand(T, N, 2).contiguous(), 1.0, 7, state=st2)
+    assert torch.equal(odd[..., 0], even[..., 0]) and torch.equal(st[..., 0], st2[..., 1])
+    x = torch.empty(T * N * 2 + 1, device="cuda")[1:].view(T, N, 2)
+    x.copy_(a.expand(T, N, 2))
+    assert x.data_ptr() % 8 == 4 and torch.equal(tvbx.bold(x, 1.0, 7), even)
