@@ -528,8 +528,8 @@ tvbx_status tvbx_batch_tune(tvbx_batch* b, int64_t trial_steps, int32_t* threads
 tvbx_status tvbx_batch_run(tvbx_batch* b);
 
 /* Current tiling, work items, persistent grid size and graph nodes. A batch built
- * with windows reads as (128, 64 KB), its work items and grid as the CTAs of every
- * turn's launch. */
+ * with windows reads as (128, 64 KB), its work items and grid as the CTAs of a
+ * turn in which no job is over. */
 tvbx_status tvbx_batch_info(const tvbx_batch* b, int32_t* threads, int32_t* smem_kb, int64_t* n_items,
                             int32_t* grid, int64_t* graph_nodes);
 

@@ -1791,6 +1791,7 @@ struct tvbx_batch {
                                         // graph holds the initialisation, the turns are launched after it
     bool packed = false;
     std::vector<BatchJob> round_jobs;   // [round][job]
+    std::vector<std::pair<int32_t, int32_t>> job_blocks;   // windowed: a job's blocks in d_items
     int64_t rounds = 0;
     DevBuf d_jobs, d_items, d_head, d_ou;
     int32_t n_items = 0, grid = 0;
@@ -1920,12 +1921,8 @@ tvbx_status batch_build(tvbx_batch* b, int32_t threads, size_t budget, int64_t t
     struct Cost { double c; int32_t job, tile; };
     std::vector<BatchItem> items;
     std::vector<int64_t> item_off((size_t)R + 1, 0);
-    int32_t win_steps = 1;
     bool packed = true;
-    for (const RunPlan& p : plans) {
-        win_steps = std::max(win_steps, p.win.steps);
-        packed = packed && p.win.packed;
-    }
+    for (const RunPlan& p : plans) packed = packed && p.win.packed;
     for (int64_t r = 0; r < R; ++r) {
         std::vector<Cost> costs;
         for (size_t j = 0; j < nj; ++j) {
@@ -1939,14 +1936,8 @@ tvbx_status batch_build(tvbx_batch* b, int32_t threads, size_t budget, int64_t t
             jobs[(size_t)r * nj + j] = BatchJob{a, pbs[j], dirs[j], plans[j].win.steps, 0,
                                                plans[j].win.far ? b->jobs[j]->d_far.as<float>() : nullptr};
             if (nc <= 0) continue;
+            if (window) continue;
             const int N = b->jobs[j]->N;
-            if (window) {
-                // one list of blocks for all rounds, the jobs with the longest windows first
-                const int32_t bpt = sim_batch_window_blocks(N, packed);
-                for (int32_t t = 0; t < plans[j].n_tiles * bpt && r == 0; ++t)
-                    costs.push_back(Cost{(double)plans[j].win.steps, (int32_t)j, t});
-                continue;
-            }
             for (int32_t t = 0; t < plans[j].n_tiles; ++t) {
                 const double per_step = (double)N * 40.0 + (double)plans[j].tile_nnz[t];   // TF work + gathers
                 costs.push_back(Cost{per_step * (double)nc * plans[j].tiles[t].nq, (int32_t)(r * nj + j), t});
@@ -1955,6 +1946,23 @@ tvbx_status batch_build(tvbx_batch* b, int32_t threads, size_t budget, int64_t t
         std::stable_sort(costs.begin(), costs.end(), [](const Cost& x, const Cost& y) { return x.c > y.c; });
         for (const Cost& c : costs) items.push_back(BatchItem{c.job, c.tile});
         item_off[(size_t)r + 1] = (int64_t)items.size();
+    }
+    b->job_blocks.assign(nj, {0, 0});
+    if (window) {
+        // one list of blocks for all rounds: the longest windows first, which are the
+        // longest blocks, of equal ones the shortest runs, so that a turn's jobs lie
+        // close together
+        std::vector<size_t> order(nj);
+        for (size_t j = 0; j < nj; ++j) order[j] = j;
+        std::stable_sort(order.begin(), order.end(), [&](size_t x, size_t y) {
+            const int32_t wx = plans[x].win.steps, wy = plans[y].win.steps;
+            return wx != wy ? wx > wy : run_cfgs[x].n_steps < run_cfgs[y].n_steps;
+        });
+        for (size_t j : order) {
+            const int32_t n = plans[j].n_tiles * sim_batch_window_blocks(b->jobs[j]->N, packed);
+            b->job_blocks[j] = {(int32_t)items.size(), (int32_t)items.size() + n};
+            for (int32_t t = 0; t < n; ++t) items.push_back(BatchItem{(int32_t)j, t});
+        }
     }
     b->n_items = (int32_t)items.size();
     CK(b->d_jobs.ensure(sizeof(BatchJob) * jobs.size()), "batch jobs");
@@ -2067,21 +2075,35 @@ tvbx_status batch_enqueue(tvbx_batch* b)
     for (int64_t r = 0; r < b->rounds; ++r) {
         const BatchJob* dev = b->d_jobs.as<BatchJob>() + (size_t)r * nj;
         const BatchJob* host = b->round_jobs.data() + (size_t)r * nj;
-        int32_t turns = 0, steps = 1;
+        std::vector<int32_t> turns(nj);
+        int32_t last = 0;
         for (size_t j = 0; j < nj; ++j) {
-            turns = std::max(turns, sim_batch_window_turns(host[j].win_steps, host[j].far != nullptr, host[j].a.n_chunk));
-            steps = std::max(steps, host[j].win_steps);
+            turns[j] = sim_batch_window_turns(host[j].win_steps, host[j].far != nullptr, host[j].a.n_chunk);
+            last = std::max(last, turns[j]);
         }
-        for (int32_t t = 0; t < turns; ++t) {
-            bool due = false;   // a job starts a far block with this turn
-            for (size_t j = 0; j < nj && !due; ++j)
-                due = host[j].far && t % ((WIN_FAR + host[j].win_steps - 1) / host[j].win_steps) == 0 &&
-                      t < sim_batch_window_turns(host[j].win_steps, true, host[j].a.n_chunk);
+        for (int32_t t = 0; t < last; ++t) {
+            // the blocks from the first to the last of the jobs that this turn concerns: a
+            // launch of all of them to the end took 58 ms where one small job with zero
+            // delays outlasts two large ones (39 ms with the persistent kernel, 41 now); eight uneven jobs
+            // 7.80 -> 7.30 ms
+            std::pair<int32_t, int32_t> live{INT32_MAX, 0}, due{INT32_MAX, 0};   // due: a far block starts
+            int32_t steps = 1;
+            for (size_t j = 0; j < nj; ++j) {
+                if (t >= turns[j]) continue;
+                const auto take = [&](std::pair<int32_t, int32_t>& r) {
+                    r = {std::min(r.first, b->job_blocks[j].first), std::max(r.second, b->job_blocks[j].second)};
+                };
+                take(live);
+                if (host[j].far && t % ((WIN_FAR + host[j].win_steps - 1) / host[j].win_steps) == 0) take(due);
+                steps = std::max(steps, host[j].win_steps);
+            }
             const BatchItem* blocks = b->d_items.as<BatchItem>();
-            if (due)
-                CK(launch_sim_batch_window(host[0].a.m, b->packed, true, dev, blocks, b->n_items, t, steps, b->stream),
+            if (due.second > due.first)
+                CK(launch_sim_batch_window(host[0].a.m, b->packed, true, dev, blocks + due.first, due.second - due.first,
+                                           t, steps, b->stream),
                    "batch far sums");
-            CK(launch_sim_batch_window(host[0].a.m, b->packed, false, dev, blocks, b->n_items, t, steps, b->stream),
+            CK(launch_sim_batch_window(host[0].a.m, b->packed, false, dev, blocks + live.first,
+                                       live.second - live.first, t, steps, b->stream),
                "batch window");
         }
         for (size_t j = 0; j < nj; ++j) {
